@@ -41,9 +41,9 @@ __device__ __forceinline__ float pt_exp2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// one lane polls a barrier (a poll reads the global timer), the warp barrier passes on what it saw
-__device__ __forceinline__ void pt_warp_wait(uint64_t *bar, uint32_t parity, volatile int *failed, int *err, int lane) {
-  if (lane == 0) tc_wait(bar, parity, failed, err);
+// the whole warp waits on a barrier
+__device__ __forceinline__ void pt_warp_wait(uint64_t *bar, uint32_t parity, volatile int *failed, int *err) {
+  tc_wait(bar, parity, failed, err);
   __syncwarp();
 }
 
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
     for (int i = 0; i < n_job; ++i) {
       // page i + 3 goes into the slot page i - 3 used, free once P V of job i - 3 has completed
       if (i >= 3) {
-        if (lane == 0) tc_wait(pv_done + ((i - 3) & 1), (uint32_t)((i - 3) >> 1) & 1u, failed, a.err);
+        tc_wait(pv_done + ((i - 3) & 1), (uint32_t)((i - 3) >> 1) & 1u, failed, a.err);
         __syncwarp();
       }
       stage(i + 3);
@@ -183,8 +183,8 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
       if (lane == 0 && i + 1 < n_job) mbar_arrive(page_full + (i + 1) % kPtSlots);
     }
   } else if (warp == 8) {
-    // ---- one thread issues the instructions to the tensor core ----
-    if (lane == 0) {
+    // ---- the warp issues the instructions to the tensor core (elect_one) ----
+    {
       const uint32_t idesc_qk = tc_instr_desc(kPtRows, 64);
       const uint32_t idesc_pv = tc_instr_desc(kPtRows, 64) | (1u << 16);   // B (= V) is MN-major: token rows of 64 dimensions
       auto qk = [&](int j) {   // S of group j % 2 = Q K^T for job j; that group holds S of its job before in registers
@@ -193,19 +193,25 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
         if (k > 0) tc_wait(s_free + g, (uint32_t)(k - 1) & 1u, failed, a.err);
         tc_fence_after_sync();
         const uint64_t dq = tc_smem_desc(Qs), dk = tc_smem_desc(slots + (size_t)(j % kPtSlots) * 16384);
+        if (elect_one()) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) tc_mma(tmem + 64u * g, dq + 2 * q, dk + 2 * q, idesc_qk, q == 0 ? 0u : 1u);   // 16 dimensions per instruction
-        tc_commit(s_full + g);
+          for (int q = 0; q < 4; ++q) tc_mma(tmem + 64u * g, dq + 2 * q, dk + 2 * q, idesc_qk, q == 0 ? 0u : 1u);   // 16 dimensions per instruction
+          tc_commit(s_full + g);
+        }
+        __syncwarp();
       };
       auto pv = [&](int j) {   // O of group j % 2 (+)= P V for job j
         const int g = j & 1, k = j >> 1;
         tc_wait(p_full + g, (uint32_t)k & 1u, failed, a.err);
         tc_fence_after_sync();
         const uint64_t dp = tc_smem_desc(Ps + g * 16384), dv = tc_smem_desc(slots + (size_t)(j % kPtSlots) * 16384 + kPageElems * 2);
+        if (elect_one()) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q)   // 16 tokens per instruction: 32 bytes along a P row, two 8-row groups (2048 bytes) down V
-          tc_mma(tmem + 128u + 64u * g, dp + 2 * q, dv + 128 * q, idesc_pv, (k == 0 && q == 0) ? 0u : 1u);
-        tc_commit(pv_done + g);
+          for (int q = 0; q < 4; ++q)   // 16 tokens per instruction: 32 bytes along a P row, two 8-row groups (2048 bytes) down V
+            tc_mma(tmem + 128u + 64u * g, dp + 2 * q, dv + 128 * q, idesc_pv, (k == 0 && q == 0) ? 0u : 1u);
+          tc_commit(pv_done + g);
+        }
+        __syncwarp();
       };
       tc_wait(q_full, 0, failed, a.err);
       if (n_job > 0) qk(0);
@@ -243,7 +249,7 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
     float m = -INFINITY, l = 0.f;
     int k = 0;
     for (int j = g; j < n_job; j += 2, ++k) {
-      pt_warp_wait(s_full + g, (uint32_t)k & 1u, failed, a.err, lane);
+      pt_warp_wait(s_full + g, (uint32_t)k & 1u, failed, a.err);
       tc_fence_after_sync();
       float s[64];
       {
@@ -280,7 +286,7 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
       const float sum = (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
       l = l * sc + sum;
       // the group's P and O belong to the tensor core until P V of the group's job before has completed
-      if (k > 0) { pt_warp_wait(pv_done + g, (uint32_t)(k - 1) & 1u, failed, a.err, lane); tc_fence_after_sync(); }
+      if (k > 0) { pt_warp_wait(pv_done + g, (uint32_t)(k - 1) & 1u, failed, a.err); tc_fence_after_sync(); }
 #pragma unroll
       for (int c8 = 0; c8 < 8; ++c8)
         *reinterpret_cast<uint4 *>(Pg + t * 128 + ((c8 ^ (t & 7)) << 4)) =
@@ -303,7 +309,7 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
     }
     trace_mark(a.trace, a.trace_slot, 3);
     // ---- the two groups' partial results: O = (O0 2^(m0 - M) + O1 2^(m1 - M)) / (l0 2^(m0 - M) + l1 2^(m1 - M)) ----
-    if (k > 0) { pt_warp_wait(pv_done + g, (uint32_t)(k - 1) & 1u, failed, a.err, lane); tc_fence_after_sync(); }
+    if (k > 0) { pt_warp_wait(pv_done + g, (uint32_t)(k - 1) & 1u, failed, a.err); tc_fence_after_sync(); }
     if (g == 1) {
       ref1_s[t] = m; l1_s[t] = l;   // without a job of its own: m = -inf, l = 0, and Ms is not read
       if (k > 0) {

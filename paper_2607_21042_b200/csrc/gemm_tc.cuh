@@ -271,12 +271,30 @@ struct GemmTcArgs {
   int trace_slot;
 };
 
-// a wait that gives up for good once any wait of the CTA has expired
+// One lane of a converged warp, known to the compiler as such.  tcgen05 and bulk-copy instructions take their operands
+// from the warp's uniform registers: issued under `if (lane == 0)` inside single-thread code, each operand is first
+// moved there for whichever lanes are active, and a k-chunk (wait, 4 MMAs, commit) took 571 cycles of the issuing
+// thread for every N; a converged warp whose elected lane issues takes 290 (measured, N = 32 .. 128, where the MMAs
+// themselves need 180-260 cycles of the tensor core).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
+// A wait that gives up for good once any wait of the CTA has expired.  The first poll decides in the common case; the
+// shared flag and the timer are read only behind it (in front of it they doubled the cost of a wait that is already
+// satisfied).
 __device__ __forceinline__ void tc_wait(uint64_t *bar, uint32_t parity, volatile int *failed, int *err) {
-  if (*failed) return;
-  if (!mbar_wait_bounded(bar, parity, kTcWaitNs)) {
-    *failed = 1;
-    if (err) atomicExch(err, 1);
+  if (mbar_try_wait(bar, parity)) return;
+  const unsigned long long t0 = global_timer_ns();
+  while (!mbar_try_wait(bar, parity)) {
+    if (*failed) return;
+    if (global_timer_ns() - t0 > kTcWaitNs) {
+      *failed = 1;
+      if (err) atomicExch(err, 1);
+      return;
+    }
   }
 }
 
@@ -364,18 +382,19 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
   trace_mark(a.trace, a.trace_slot, 1);
   if (warp == 0) {
     // ---- producer ----
-    if (lane == 0) {
-      for (int i = 0; i < pre; ++i)
-        bulk_copy_g2s(ring + (size_t)i * (kTcABytes + kTcBBytes) + kTcABytes, gB + (size_t)i * (kMaxRows * 128), kTcBBytes, full + i);
-      for (int i = pre; i < n_it; ++i) {
-        const int s = i % kTcStages;
-        tc_wait(empty + s, ((i / kTcStages) - 1) & 1, failed, a.err);
+    for (int i = 0; i < pre; ++i)
+      if (elect_one()) bulk_copy_g2s(ring + (size_t)i * (kTcABytes + kTcBBytes) + kTcABytes, gB + (size_t)i * (kMaxRows * 128), kTcBBytes, full + i);
+    for (int i = pre; i < n_it; ++i) {
+      const int s = i % kTcStages;
+      tc_wait(empty + s, ((i / kTcStages) - 1) & 1, failed, a.err);
+      if (elect_one()) {
         mbar_expect_tx(full + s, kTcABytes + kTcBBytes);
         bulk_copy_g2s(ring + (size_t)s * (kTcABytes + kTcBBytes), gA + (size_t)i * kTcABytes, kTcABytes, full + s);
         bulk_copy_g2s(ring + (size_t)s * (kTcABytes + kTcBBytes) + kTcABytes, gB + (size_t)i * (kMaxRows * 128), kTcBBytes, full + s);
       }
-      trace_mark(a.trace, a.trace_slot, 3);   // last copy issued
+      __syncwarp();
     }
+    trace_mark(a.trace, a.trace_slot, 3);   // last copy issued
     __syncwarp();   // the warp arrives at the final barrier as a whole
   } else if (warp == 1 || warp == 10) {
     // ---- MMA issuers: two threads of different warps, each with its own accumulator.  Ungrouped:
@@ -388,7 +407,7 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
     //      be told it is complete ----
     const int par = GROUPED ? 0 : (warp == 10 ? 1 : 0);
     const int stride = GROUPED ? 1 : 2;
-    if (lane == 0 && !(GROUPED && warp == 10)) {
+    if (!(GROUPED && warp == 10)) {
       const uint32_t idesc = tc_instr_desc(kTcTileM, kTcChunkN);
       for (int i = par; i < n_it; i += stride) {
         const int s = i % kTcStages;
@@ -399,15 +418,19 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
         const unsigned char *sa = ring + (size_t)s * (kTcABytes + kTcBBytes);
         const uint64_t da = tc_smem_desc(sa), db = tc_smem_desc(sa + kTcABytes);
         const uint32_t dst = GROUPED ? tmem_d + (uint32_t)(g & 1) * kTcChunkN : tmem_d + (uint32_t)par * kTcChunkN;
+        if (elect_one()) {
 #pragma unroll
-        for (int j = 0; j < kTcKChunk / 16; ++j) {  // 32 bytes further along K per step: +2 in 16-byte units
-          const bool fresh = GROUPED ? ((i & 1) == 0 && j == 0) : (i == par && j == 0);
-          tc_mma(dst, da + 2 * j, db + 2 * j, idesc, fresh ? 0u : 1u);
+          for (int j = 0; j < kTcKChunk / 16; ++j) {  // 32 bytes further along K per step: +2 in 16-byte units
+            const bool fresh = GROUPED ? ((i & 1) == 0 && j == 0) : (i == par && j == 0);
+            tc_mma(dst, da + 2 * j, db + 2 * j, idesc, fresh ? 0u : 1u);
+          }
+          tc_commit(empty + s);   // the stage may be refilled once these MMAs have read it
+          if (GROUPED && ((i & 1) == 1 || i == n_it - 1)) tc_commit(grp_done + (g & 1));
+          if (!GROUPED && i + stride >= n_it) tc_commit(acc_done);
         }
-        tc_commit(empty + s);   // the stage may be refilled once these MMAs have read it
-        if (GROUPED && ((i & 1) == 1 || i == n_it - 1)) tc_commit(grp_done + (g & 1));
+        __syncwarp();
       }
-      if (!GROUPED) tc_commit(acc_done);
+      if (!GROUPED && par >= n_it && elect_one()) tc_commit(acc_done);   // nothing issued: the barrier still counts this warp
     }
     __syncwarp();   // as above
   }
@@ -636,31 +659,35 @@ __global__ void __launch_bounds__(kTwThreads) gemm_tcw_kernel(const GemmTcArgs a
   pdl_wait();
   trace_mark(a.trace, a.trace_slot, 1);
   if (warp == 0) {
-    if (lane == 0) {
-      for (int i = 0; i < pre; ++i)
-        bulk_copy_g2s(ring + (size_t)i * kTwStageBytes, gX + (size_t)i * (kMaxRows * 128), 16384, full + i);
-      for (int i = pre; i < n_it; ++i) {
-        const int s = i % n_stage;
-        tc_wait(empty + s, ((i / n_stage) - 1) & 1, failed, a.err);
+    for (int i = 0; i < pre; ++i)
+      if (elect_one()) bulk_copy_g2s(ring + (size_t)i * kTwStageBytes, gX + (size_t)i * (kMaxRows * 128), 16384, full + i);
+    int s = 0;
+    uint32_t parity = 0;
+    for (int i = pre; i < n_it; ++i) {   // pre == n_stage here
+      tc_wait(empty + s, parity, failed, a.err);
+      if (elect_one()) {
         mbar_expect_tx(full + s, kTwStageBytes);
         bulk_copy_g2s(ring + (size_t)s * kTwStageBytes + 16384, gW + (size_t)i * kTcABytes, 16384, full + s);
         bulk_copy_g2s(ring + (size_t)s * kTwStageBytes, gX + (size_t)i * (kMaxRows * 128), 16384, full + s);
       }
-      trace_mark(a.trace, a.trace_slot, 3);   // last copy issued
+      __syncwarp();
+      if (++s == n_stage) { s = 0; parity ^= 1u; }   // no division by the runtime ring depth: it cost 0.1 us per k-chunk
     }
+    trace_mark(a.trace, a.trace_slot, 3);   // last copy issued
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = tc_instr_desc(128, 128);
-      for (int i = 0; i < n_it; ++i) {
-        const int s = i % n_stage;
-        tc_wait(full + s, (i / n_stage) & 1, failed, a.err);
-        const int g = i >> 1;
-        if (GROUPED && (i & 1) == 0 && g >= 2) tc_wait(grp_free + (g & 1), ((g >> 1) - 1) & 1, failed, a.err);
-        tc_fence_after_sync();
-        const unsigned char *sx = ring + (size_t)s * kTwStageBytes;
-        const uint64_t da = tc_smem_desc(sx), db = tc_smem_desc(sx + 16384);
-        const uint32_t dst = GROUPED ? tmem_d + (uint32_t)(g & 1) * 128u : tmem_d;
+    const uint32_t idesc = tc_instr_desc(128, 128);
+    int s = 0;
+    uint32_t parity = 0;
+    for (int i = 0; i < n_it; ++i) {
+      tc_wait(full + s, parity, failed, a.err);
+      const int g = i >> 1;
+      if (GROUPED && (i & 1) == 0 && g >= 2) tc_wait(grp_free + (g & 1), ((g >> 1) - 1) & 1, failed, a.err);
+      tc_fence_after_sync();
+      const unsigned char *sx = ring + (size_t)s * kTwStageBytes;
+      const uint64_t da = tc_smem_desc(sx), db = tc_smem_desc(sx + 16384);
+      const uint32_t dst = GROUPED ? tmem_d + (uint32_t)(g & 1) * 128u : tmem_d;
+      if (elect_one()) {
 #pragma unroll
         for (int j = 0; j < kTcKChunk / 16; ++j) {
           const bool fresh = GROUPED ? ((i & 1) == 0 && j == 0) : (i == 0 && j == 0);
@@ -668,9 +695,12 @@ __global__ void __launch_bounds__(kTwThreads) gemm_tcw_kernel(const GemmTcArgs a
         }
         tc_commit(empty + s);
         if (GROUPED && ((i & 1) == 1 || i == n_it - 1)) tc_commit(grp_done + (g & 1));
+        if (!GROUPED && i == n_it - 1) tc_commit(acc_done);
       }
-      if (!GROUPED) tc_commit(acc_done);
+      __syncwarp();
+      if (++s == n_stage) { s = 0; parity ^= 1u; }
     }
+    if (!GROUPED && n_it <= 0 && elect_one()) tc_commit(acc_done);
     __syncwarp();
   } else {
     // ---- epilogue: warp w may read accumulator lanes 32*(w%4)..+31 = batch rows; warps w and w+4 share a lane
