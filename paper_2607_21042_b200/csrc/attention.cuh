@@ -39,6 +39,7 @@ inline size_t attention_scratch_bytes(int R, int H) {
 
 struct AttnArgs {
   const float *q;            // [R][H*64]
+  const void *q_img;         // tcgen05 prefill variant: if set, q as a bf16 activation image (row tiles of 128) instead
   const uint16_t *kv_layer;  // this layer's pool slice
   const int *page_table;     // [*, pps]
   const int *row_stream, *row_pos;

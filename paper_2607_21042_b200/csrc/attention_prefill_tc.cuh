@@ -11,9 +11,14 @@
 //                   MN-major for this product); O stays in tensor memory and is rescaled there when a row's
 //                   maximum moves
 // Warps 0-3 and 4-7 are two softmax groups that take alternate pages, each with its own S, P and O (the two
-// partial results meet at the end); one thread of warp 8 issues the instructions, with Q K^T a page ahead of the
-// groups; warps 9 and 10 stage the K and V halves of the pages (16-byte asynchronous copies into six slots, with
-// the 128-byte swizzle the tensor core expects).  Every wait is bounded.
+// partial results meet at the end); warp 8 issues the instructions, with Q K^T a page ahead of the groups; warps 9 and
+// 10 stage the K and V halves of the pages (16-byte asynchronous copies into three slots each, with the 128-byte
+// swizzle the tensor core expects).  Every wait is bounded.
+//
+// What bounds it: the chain of waits between the warps of a CTA, not arithmetic or copies (with the exponentials, the
+// maxima and the copies taken out a page took the same 1.05 us).  Q arrives as one block of the activation image that
+// the linear in front wrote (fp32 rows read and packed by 128 threads cost 3 us per CTA); K slots are refilled as soon
+// as Q K^T has read them.  Per layer, 896 rows of one stream: 18.0 -> 14.8 us; 7 streams of 128 rows: 8.1 -> 7.3 us.
 #pragma once
 #include "attention_prefill.cuh"
 #include "gemm_tc.cuh"
@@ -22,7 +27,7 @@ namespace ttsgpt {
 
 constexpr int kPtRows = 128;
 constexpr int kPtThreads = 352;
-constexpr int kPtSlots = 6;
+constexpr int kPtSlots = 3;         // pages in shared memory
 constexpr int kPtMergePitch = 65;   // floats per row of the merge buffer: lane = row, conflict-free
 constexpr int kPtMaxJobs = 256;   // two partial long streams + streams of at most 128 rows
 
@@ -75,17 +80,19 @@ __device__ __forceinline__ void pt_stage(unsigned char *dst, const uint16_t *src
   pt_commit();
 }
 
-__global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const AttnArgs a, int R) {
+// PAIRED: two CTAs share an SM (grids of more than one CTA per SM)
+template <bool PAIRED>
+__global__ void __launch_bounds__(kPtThreads, PAIRED ? 2 : 1) attention_prefill_tc_kernel(const AttnArgs a, int R) {
   extern __shared__ __align__(16) unsigned char pt_smem_raw[];
   unsigned char *base = pt_smem_raw + ((1024u - (smem_u32(pt_smem_raw) & 1023u)) & 1023u);
   unsigned char *Qs = base;                   // 128 rows x 64 dimensions bf16, K-major, 128-byte swizzle
   unsigned char *Ps = base + 16384;           // [2 groups] 128 rows x 64 tokens bf16, same layout
-  unsigned char *slots = base + 49152;        // [6][K 64 tokens x 128 B | V 64 tokens x 128 B]
-  float *Ms = reinterpret_cast<float *>(slots + kPtSlots * 16384);   // [128][65] group 1's O for the merge
-  uint64_t *q_full = reinterpret_cast<uint64_t *>(Ms + kPtRows * kPtMergePitch);
+  unsigned char *slots = base + 49152;        // [kPtSlots][K 64 tokens x 128 B | V 64 tokens x 128 B]
+  float *Ms = reinterpret_cast<float *>(slots);   // [128][65] group 1's O for the merge, once every P V has completed
+  uint64_t *q_full = reinterpret_cast<uint64_t *>(slots + kPtSlots * 16384);
   uint64_t *s_full = q_full + 1, *s_free = q_full + 3, *p_full = q_full + 5, *pv_done = q_full + 7;   // [2] each, by group
-  uint64_t *page_full = q_full + 9;   // [kPtSlots] K and V of the slot's page have landed
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(q_full + 9 + kPtSlots);
+  uint64_t *page_full = q_full + 9;   // [K, V][kPtSlots] that half of the slot's page has landed
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(q_full + 9 + 2 * kPtSlots);
   volatile int *failed = reinterpret_cast<volatile int *>(tmem_slot + 1);
   __shared__ int row_s[kPtRows], row_p[kPtRows];
   __shared__ int seg_stream[kPtRows], seg_i0[kPtRows], seg_i1[kPtRows], seg_last[kPtRows];
@@ -93,9 +100,10 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
   __shared__ int n_job_s;
   __shared__ unsigned run_open[kPtRows / 32];   // bit l of word w: row 32 w + l opens a run
   __shared__ int job_ph[kPtMaxJobs];            // physical page of each job
+  __shared__ int2 job_rows[kPtMaxJobs];         // x: rows of the tile the job's run covers, first | end << 16; y: first position of its page
   __shared__ float ref1_s[kPtRows], l1_s[kPtRows];   // group 1's reference score and sum per row
 
-  const int h = blockIdx.y, r0 = blockIdx.z * kPtRows;
+  const int h = blockIdx.y, r0 = (int)(gridDim.z - 1 - blockIdx.z) * kPtRows;   // the last rows of a stream see the most pages: first
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   trace_mark(a.trace, a.trace_slot, 0);
   if (threadIdx.x < kPtRows) {
@@ -104,8 +112,8 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
     row_p[threadIdx.x] = r < R ? a.row_pos[r] : -1;
   }
   if (threadIdx.x == 0) {
-    mbar_init(q_full, kPtRows);
-    for (int sl = 0; sl < kPtSlots; ++sl) mbar_init(page_full + sl, 2);
+    mbar_init(q_full, a.q_img ? 1 : kPtRows);
+    for (int sl = 0; sl < 2 * kPtSlots; ++sl) mbar_init(page_full + sl, 1);
     for (int g = 0; g < 2; ++g) { mbar_init(s_full + g, 1); mbar_init(s_free + g, kPtRows); mbar_init(p_full + g, kPtRows); mbar_init(pv_done + g, 1); }
     *failed = 0;
   }
@@ -145,8 +153,11 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
   const int n_job = n_job_s;
   // the physical pages of all jobs up front (the page table is final before the pass's first kernel starts): a
   // page-table read in front of every page's copies would put an L2 round trip into each turn of the producer's loop
-  for (int j = threadIdx.x; j < n_job; j += kPtThreads)
-    job_ph[j] = a.page_table[(size_t)seg_stream[jobs[j] >> 8] * a.pps + (jobs[j] & 255)];
+  for (int j = threadIdx.x; j < n_job; j += kPtThreads) {
+    const int sg = jobs[j] >> 8, pg = jobs[j] & 255;
+    job_ph[j] = a.page_table[(size_t)seg_stream[sg] * a.pps + pg];
+    job_rows[j] = make_int2((seg_i0[sg] - r0) | ((seg_i1[sg] - r0) << 16), pg * kPageTokens);
+  }
   __syncthreads();
   pdl_launch_dependents();
   pdl_wait();     // Q and the K/V rows of this pass were written by the QKV kernel in front
@@ -165,22 +176,24 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
         pt_commit();   // an empty group keeps the count of groups per job uniform
       }
     };
-    stage(0); stage(1); stage(2);
-    pt_wait_but<2>();            // page 0 has landed
-    fence_proxy_async_smem();    // the tensor core reads the slots through the async proxy
-    __syncwarp();
-    if (lane == 0 && n_job > 0) mbar_arrive(page_full);
-    for (int i = 0; i < n_job; ++i) {
-      // page i + 3 goes into the slot page i - 3 used, free once P V of job i - 3 has completed
-      if (i >= 3) {
-        tc_wait(pv_done + ((i - 3) & 1), (uint32_t)((i - 3) >> 1) & 1u, failed, a.err);
-        __syncwarp();
-      }
-      stage(i + 3);
-      pt_wait_but<2>();            // everything but the two groups just committed: page i + 1 has landed
-      fence_proxy_async_smem();
+    // a K half is free once Q K^T of its page has completed, a V half once P V has
+    uint64_t *full = page_full + part * kPtSlots, *done = part == 0 ? s_full : pv_done;
+    auto announce = [&](int j) {
+      fence_proxy_async_smem();    // the tensor core reads the slots through the async proxy
       __syncwarp();
-      if (lane == 0 && i + 1 < n_job) mbar_arrive(page_full + (i + 1) % kPtSlots);
+      if (lane == 0 && j < n_job) mbar_arrive(full + j % kPtSlots);
+    };
+    static_assert(kPtSlots == 3, "the copy groups below");
+    stage(0);
+    pt_wait_but<0>();              // the first page alone: the issue of the others would hold its announcement up
+    announce(0);
+    stage(1); stage(2);
+    for (int i = 0; i < n_job; ++i) {
+      pt_wait_but<1>();            // everything but page i + 2: page i + 1 has landed
+      announce(i + 1);
+      tc_wait(done + (i & 1), (uint32_t)(i >> 1) & 1u, failed, a.err);
+      __syncwarp();
+      stage(i + 3);                // into the slot page i used
     }
   } else if (warp == 8) {
     // ---- the warp issues the instructions to the tensor core (elect_one) ----
@@ -189,7 +202,7 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
       const uint32_t idesc_pv = tc_instr_desc(kPtRows, 64) | (1u << 16);   // B (= V) is MN-major: token rows of 64 dimensions
       auto qk = [&](int j) {   // S of group j % 2 = Q K^T for job j; that group holds S of its job before in registers
         const int g = j & 1, k = j >> 1;
-        tc_wait(page_full + j % kPtSlots, (uint32_t)(j / kPtSlots) & 1u, failed, a.err);
+        tc_wait(page_full + j % kPtSlots, (uint32_t)(j / kPtSlots) & 1u, failed, a.err);   // K half
         if (k > 0) tc_wait(s_free + g, (uint32_t)(k - 1) & 1u, failed, a.err);
         tc_fence_after_sync();
         const uint64_t dq = tc_smem_desc(Qs), dk = tc_smem_desc(slots + (size_t)(j % kPtSlots) * 16384);
@@ -202,6 +215,7 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
       };
       auto pv = [&](int j) {   // O of group j % 2 (+)= P V for job j
         const int g = j & 1, k = j >> 1;
+        tc_wait(page_full + kPtSlots + j % kPtSlots, (uint32_t)(j / kPtSlots) & 1u, failed, a.err);   // V half
         tc_wait(p_full + g, (uint32_t)k & 1u, failed, a.err);
         tc_fence_after_sync();
         const uint64_t dp = tc_smem_desc(Ps + g * 16384), dv = tc_smem_desc(slots + (size_t)(j % kPtSlots) * 16384 + kPageElems * 2);
@@ -231,7 +245,13 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
     const uint32_t t_lane = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
     const uint32_t t_S = t_lane + 64u * g, t_O = t_lane + 128u + 64u * g;
     unsigned char *Pg = Ps + g * 16384;
-    if (g == 0) {
+    if (g == 0 && a.q_img) {
+      // the tile's Q of this head is one block of the image, in the layout of the swizzled tile
+      if (threadIdx.x == 0) {
+        mbar_expect_tx(q_full, 16384);
+        bulk_copy_g2s(Qs, reinterpret_cast<const unsigned char *>(a.q_img) + ((size_t)(r0 >> 7) * a.H + h) * (kMaxRows * 128), 16384, q_full);
+      }
+    } else if (g == 0) {
       // Q row of this head as bf16 into the swizzled tile (a row beyond the pass is zero)
       const float *qp = a.q + (size_t)r * a.H * kHeadDim + h * kHeadDim;
 #pragma unroll
@@ -248,33 +268,39 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
     const int pos = row_p[t];
     float m = -INFINITY, l = 0.f;
     int k = 0;
+    int2 nxt = g < n_job ? job_rows[g] : make_int2(0, 0);
     for (int j = g; j < n_job; j += 2, ++k) {
+      const int2 ji = nxt;
       pt_warp_wait(s_full + g, (uint32_t)k & 1u, failed, a.err);
       tc_fence_after_sync();
-      float s[64];
-      {
-        float lo[32], hi[32];
-        tmem_ld32(t_S, lo);
-        tmem_ld32(t_S + 32u, hi);
-#pragma unroll
-        for (int c = 0; c < 32; ++c) { s[c] = lo[c]; s[32 + c] = hi[c]; }
-      }
-      tc_fence_before_sync();
-      mbar_arrive(s_free + g);
-      const int sg = jobs[j] >> 8, pg = jobs[j] & 255;
-      const bool act = r >= seg_i0[sg] && r < seg_i1[sg];
-      const int see = act ? min(kPageTokens, pos + 1 - pg * kPageTokens) : 0;   // tokens of the page this row sees
+      if (j + 2 < n_job) nxt = job_rows[j + 2];
+      // tokens of the page this row sees
+      const int see = t >= (ji.x & 0xffff) && t < (ji.x >> 16) ? min(kPageTokens, pos + 1 - ji.y) : 0;
       // all but the last page of a row's own stream are seen whole by every row of the warp: no masks there
-      if (!__all_sync(0xFFFFFFFFu, see == kPageTokens)) {
+      const bool whole = __all_sync(0xFFFFFFFFu, see == kPageTokens);
+      // With an SM to itself the thread keeps all 64 scores in registers.  Where two CTAs share an SM (88 registers) S is
+      // read half by half, the lower half a second time behind the maximum.  Four independent chains for the maximum and
+      // for the sum; the scale (positive) is applied to the maximum and inside the exponential's argument: one
+      // multiply-add per score.
+      constexpr int HALVES = PAIRED ? 2 : 1, W = 64 / HALVES;
+      float s[W];
+      auto load = [&](int c0) {
 #pragma unroll
-        for (int c = 0; c < 64; ++c) s[c] = c < see ? s[c] : -INFINITY;
-      }
-      // four independent chains for the maximum and for the sum: one chain of 64 dependent operations per row and
-      // page was the longest thing in the loop.  The scale (positive) is applied to the maximum and inside the
-      // exponential's argument: one multiply-add per score.
+        for (int q = 0; q < W; q += 32) tmem_ld32(t_S + (uint32_t)(c0 + q), *reinterpret_cast<float (*)[32]>(s + q));
+        if (!whole) {
+#pragma unroll
+          for (int c = 0; c < W; ++c) s[c] = c0 + c < see ? s[c] : -INFINITY;
+        }
+      };
+      auto scores_read = [&]() { tc_fence_before_sync(); mbar_arrive(s_free + g); };
       float pm4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-      for (int c = 0; c < 64; ++c) pm4[c & 3] = fmaxf(pm4[c & 3], s[c]);
+      for (int hh = 0; hh < HALVES; ++hh) {
+        load(W * hh);
+        if (HALVES == 1) scores_read();
+#pragma unroll
+        for (int c = 0; c < W; ++c) pm4[c & 3] = fmaxf(pm4[c & 3], s[c]);
+      }
       const float pm = fmaxf(fmaxf(pm4[0], pm4[1]), fmaxf(pm4[2], pm4[3])) * qs;
       const float m_new = fmaxf(m, pm);
       const float ref = (m_new == -INFINITY) ? 0.f : m_new;   // a row that has seen nothing yet keeps m = -inf
@@ -282,16 +308,19 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
       m = m_new;
       float sum4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int c = 0; c < 64; ++c) { s[c] = pt_exp2(fmaf(s[c], qs, -ref)); sum4[c & 3] += s[c]; }
-      const float sum = (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
-      l = l * sc + sum;
-      // the group's P and O belong to the tensor core until P V of the group's job before has completed
-      if (k > 0) { pt_warp_wait(pv_done + g, (uint32_t)(k - 1) & 1u, failed, a.err); tc_fence_after_sync(); }
+      for (int hh = HALVES - 1; hh >= 0; --hh) {
+        if (HALVES == 2 && hh == 0) { load(0); scores_read(); }
 #pragma unroll
-      for (int c8 = 0; c8 < 8; ++c8)
-        *reinterpret_cast<uint4 *>(Pg + t * 128 + ((c8 ^ (t & 7)) << 4)) =
-            make_uint4(pack_bf16x2(s[8 * c8], s[8 * c8 + 1]), pack_bf16x2(s[8 * c8 + 2], s[8 * c8 + 3]),
-                       pack_bf16x2(s[8 * c8 + 4], s[8 * c8 + 5]), pack_bf16x2(s[8 * c8 + 6], s[8 * c8 + 7]));
+        for (int c = 0; c < W; ++c) { s[c] = pt_exp2(fmaf(s[c], qs, -ref)); sum4[c & 3] += s[c]; }
+        // the group's P and O belong to the tensor core until P V of the group's job before has completed
+        if (hh == HALVES - 1 && k > 0) { pt_warp_wait(pv_done + g, (uint32_t)(k - 1) & 1u, failed, a.err); tc_fence_after_sync(); }
+#pragma unroll
+        for (int c8 = 0; c8 < W / 8; ++c8)
+          *reinterpret_cast<uint4 *>(Pg + t * 128 + (((W / 8 * hh + c8) ^ (t & 7)) << 4)) =
+              make_uint4(pack_bf16x2(s[8 * c8], s[8 * c8 + 1]), pack_bf16x2(s[8 * c8 + 2], s[8 * c8 + 3]),
+                         pack_bf16x2(s[8 * c8 + 4], s[8 * c8 + 5]), pack_bf16x2(s[8 * c8 + 6], s[8 * c8 + 7]));
+      }
+      l = l * sc + ((sum4[0] + sum4[1]) + (sum4[2] + sum4[3]));
       __syncwarp();
       if (k > 0 && !__all_sync(0xFFFFFFFFu, sc == 1.0f)) {   // some row's maximum moved: rescale the warp's rows of O
 #pragma unroll
@@ -309,7 +338,9 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
     }
     trace_mark(a.trace, a.trace_slot, 3);
     // ---- the two groups' partial results: O = (O0 2^(m0 - M) + O1 2^(m1 - M)) / (l0 2^(m0 - M) + l1 2^(m1 - M)) ----
+    // group 1 parks its O over the slots, so it waits for the last P V of both groups
     if (k > 0) { pt_warp_wait(pv_done + g, (uint32_t)(k - 1) & 1u, failed, a.err); tc_fence_after_sync(); }
+    if (g == 1 && n_job > 0) pt_warp_wait(pv_done, (uint32_t)((n_job - 1) >> 1) & 1u, failed, a.err);
     if (g == 1) {
       ref1_s[t] = m; l1_s[t] = l;   // without a job of its own: m = -inf, l = 0, and Ms is not read
       if (k > 0) {
@@ -360,14 +391,21 @@ __global__ void __launch_bounds__(kPtThreads) attention_prefill_tc_kernel(const 
   if (warp == 8) tmem_dealloc(tmem, 256);
 }
 
-inline size_t attention_prefill_tc_smem_bytes() { return 49152 + (size_t)kPtSlots * 16384 + (size_t)kPtRows * kPtMergePitch * 4 + 1024 + 256; }
+static_assert(kPtRows * kPtMergePitch * 4 <= kPtSlots * 16384, "the merge buffer lies over the slots");
+inline size_t attention_prefill_tc_smem_bytes() { return 49152 + (size_t)kPtSlots * 16384 + 1024 + 256; }
 
-inline cudaError_t launch_attention_prefill_tc(const AttnArgs &a, int R, cudaStream_t st, bool pdl) {
+template <bool PAIRED>
+inline cudaError_t launch_attention_prefill_tc_as(const AttnArgs &a, int R, cudaStream_t st, bool pdl) {
   static PerDeviceOnce attr_once;   // per device: opt-in to more than 48 KB of dynamic shared memory
-  if (attr_once.first())
-    cudaFuncSetAttribute(attention_prefill_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attention_prefill_tc_smem_bytes());
-  const int groups = (R + kPtRows - 1) / kPtRows;
-  return launch_kernel(attention_prefill_tc_kernel, dim3(1, a.H, groups), dim3(kPtThreads), attention_prefill_tc_smem_bytes(), st, pdl, a, R);
+  const size_t smem = attention_prefill_tc_smem_bytes();
+  if (attr_once.first()) cudaFuncSetAttribute(attention_prefill_tc_kernel<PAIRED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return launch_kernel(attention_prefill_tc_kernel<PAIRED>, dim3(1, a.H, (R + kPtRows - 1) / kPtRows), dim3(kPtThreads), smem, st, pdl, a, R);
+}
+// n_sm: SMs of the device.  A grid of at most one CTA per SM takes the form whose threads hold a page's scores in registers
+// (896 rows of one stream: 1.81 against 1.84 ms per pass), a larger one the form two of which share an SM.
+inline cudaError_t launch_attention_prefill_tc(const AttnArgs &a, int R, int n_sm, cudaStream_t st, bool pdl) {
+  if (a.H * ((R + kPtRows - 1) / kPtRows) <= n_sm) return launch_attention_prefill_tc_as<false>(a, R, st, pdl);
+  return launch_attention_prefill_tc_as<true>(a, R, st, pdl);
 }
 
 }  // namespace ttsgpt

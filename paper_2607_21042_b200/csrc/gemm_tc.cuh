@@ -260,6 +260,7 @@ struct GemmTcArgs {
   int stages;               // wide kernel: ring depth, set by its launcher
   float *out_f32;           // EPI_F32: out[b*out_stride+n]; EPI_QKV: q; EPI_RESID: x (ksplit == 1) or partials [ksplit][128][N]
   int out_stride;
+  void *q_img;              // EPI_QKV, wide kernels: if set, q goes here as a bf16 activation image instead of to out_f32
   void *out_img;            // EPI_GELU: activation image of the next linear (row length N)
   int gelu_tanh;
   uint16_t *kv_layer;
@@ -559,7 +560,7 @@ constexpr int kTwMaxPartials = 4;               // k-ranges the following LayerN
 
 // bf16 destinations of the wide kernel's epilogue: four parked rows per instruction, lane = (row in the group
 // of four, 16-byte unit = 8 features).  KIND 0: tanh-GELU into the next linear's activation image, 1: erf-GELU
-// into it, 2: K/V rows into their page slots (or the staging rows of the 8-bit cache).
+// into it, 2: K/V rows into their page slots (or the staging rows of the 8-bit cache), 3: as they are into an image (q).
 template <int KIND>
 __device__ __forceinline__ void tw_rows_bf16(const unsigned char *patch, int rows, int r4, int u, int lw, const float (&sc8)[8],
                                              const float (&bi8)[8], unsigned char *blk, uint16_t *const *kv_base, size_t kv_off) {
@@ -781,7 +782,7 @@ __global__ void __launch_bounds__(kTwThreads) gemm_tcw_kernel(const GemmTcArgs a
         for (int q = 0; q < 16; ++q) mine[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
       }
       __syncwarp();
-      const bool as_bf16 = a.mode == EPI_GELU || (a.mode == EPI_QKV && n0 >= a.d);
+      const bool as_bf16 = a.mode == EPI_GELU || (a.mode == EPI_QKV && (n0 >= a.d || a.q_img));
       const bool partial = a.mode == EPI_RESID && a.ksplit > 1;
       const bool use_bias = a.bias && !partial;
       if (*failed || nv <= 0) {
@@ -795,13 +796,16 @@ __global__ void __launch_bounds__(kTwThreads) gemm_tcw_kernel(const GemmTcArgs a
         const int which = n0 >= 2 * a.d;
         const int col = n0 - (which ? 2 * a.d : a.d);
         const size_t kv_off = a.kv_stage ? (size_t)which * a.d + col : ((size_t)which * a.H + (col >> 6)) * kPageElems;
-        unsigned char *blk = reinterpret_cast<unsigned char *>(a.out_img) + ((size_t)blockIdx.z * (a.N >> 6) + (n0 >> 6)) * (kMaxRows * 128);
+        const bool q_rows = a.mode == EPI_QKV && n0 < a.d;
+        unsigned char *blk = reinterpret_cast<unsigned char *>(q_rows ? a.q_img : a.out_img) + ((size_t)blockIdx.z * ((q_rows ? a.d : a.N) >> 6) + (n0 >> 6)) * (kMaxRows * 128);
         // one loop per destination kind, so that each is straight-line code (this runs once per CTA, from a cold
         // instruction cache: a loop that chose per element between the two GELU forms took four times as long)
         if (a.mode == EPI_GELU && a.gelu_tanh)
           tw_rows_bf16<0>(patch, rows, r4, u, lw, sc8, bi8, blk, kv_base, kv_off);
         else if (a.mode == EPI_GELU)
           tw_rows_bf16<1>(patch, rows, r4, u, lw, sc8, bi8, blk, kv_base, kv_off);
+        else if (q_rows)
+          tw_rows_bf16<3>(patch, rows, r4, u, lw, sc8, bi8, blk, kv_base, kv_off);
         else
           tw_rows_bf16<2>(patch, rows, r4, u, lw, sc8, bi8, blk, kv_base, kv_off);
       } else {

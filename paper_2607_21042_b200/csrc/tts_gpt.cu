@@ -74,6 +74,7 @@ struct tts_gpt {
   uint16_t *a, *o, *hbuf, *hf;
   // tensor-core path (more than 16 rows, bf16 weights): activation images and k-split partial sums
   void *a_img = nullptr, *o_img = nullptr, *h_img = nullptr, *hf_img = nullptr;
+  void *q_img = nullptr;             // q of prefill passes of more than 128 rows
   float *partials = nullptr;
   bool have_tc = false;
   // attention scratch
@@ -257,6 +258,7 @@ size_t carve(tts_gpt *h, void *base) {
     h->hf_img = cv.take<char>(act_image_bytes(d));
     h->partials_floats = (size_t)kTiles * std::max(kTcKSplit, kTwMaxPartials) * kMaxRows * d;   // [row tile][k-range][128][d]
     h->partials = cv.take<float>(h->partials_floats);
+    h->q_img = cv.take<char>(kTiles * act_image_bytes(d));
   }
   return cv.off;
 }
@@ -338,7 +340,7 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
       if (e != cudaSuccess) return e;
       h->launches += 1;
       aa.kv_layer = h->kv_scratch; aa.page_table = h->scratch_table; aa.err = h->dev_err; aa.row_order = nullptr;
-      if (h->use_attn_tc && R > kMaxRows) return launch_attention_prefill_tc(aa, R, st, pdl);
+      if (h->use_attn_tc && R > kMaxRows) return launch_attention_prefill_tc(aa, R, h->n_sm, st, pdl);
       return launch_attention_prefill_mma(aa, R, st, pdl);
     }
     Fp8AttnArgs fa;
@@ -359,7 +361,7 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
   // prefill passes: rows of one stream share their pages (one CTA per 16 rows and head on the tensor cores;
   // the CUDA-core variant with 8 rows per CTA stays selectable)
   // (passes of several row tiles: 128 rows per CTA on tcgen05)
-  if (!aa.old_pages_final && h->use_attn_mma && h->use_attn_tc && R > kMaxRows) return launch_attention_prefill_tc(aa, R, st, pdl);
+  if (!aa.old_pages_final && h->use_attn_mma && h->use_attn_tc && R > kMaxRows) return launch_attention_prefill_tc(aa, R, h->n_sm, st, pdl);
   if (!aa.old_pages_final && h->use_attn_mma && R >= kAttnPrefillRows) return launch_attention_prefill_mma(aa, R, st, pdl);
   if (!aa.old_pages_final && h->use_attn_prefill && R >= kAttnPrefillRows) return launch_attention_prefill(aa, R, st, pdl);
   const bool stream = h->attn_stream_min_pairs > 0 ? R * aa.H >= h->attn_stream_min_pairs : attention_use_stream(R, aa.H, h->n_sm);
@@ -436,12 +438,14 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
     qa.out_f32 = h->q; qa.out_stride = d; qa.kv_layer = kvl; qa.page_table = h->ps.page_table;
     qa.row_stream = h->rt.row_stream; qa.row_pos = h->rt.row_pos; qa.pps = h->pps; qa.d = d; qa.H = c.n_head;
     qa.kv_stage = h->kv_stage;
+    const bool q_img = wide && h->use_attn_tc && h->use_attn_mma && (!h->kv_fp8 || h->pass_scratch > 0);   // the tcgen05 attention follows
+    qa.q_img = q_img ? h->q_img : nullptr;
     trace_attach(h, qa);
     if ((rc = launch_gemm(h, qa, wide, st, pdl))) return rc;
     AttnArgs aa;
     memset(&aa, 0, sizeof aa);
     aa.q = h->q; aa.kv_layer = kvl; aa.page_table = h->ps.page_table; aa.row_stream = h->rt.row_stream;
-    aa.row_pos = h->rt.row_pos; aa.out = (uint16_t *)h->o_img; aa.out_image = 1;
+    aa.row_pos = h->rt.row_pos; aa.out = (uint16_t *)h->o_img; aa.out_image = 1; aa.q_img = q_img ? h->q_img : nullptr;
     aa.H = c.n_head; aa.pps = h->pps; aa.old_pages_final = decode ? 1 : 0;
     trace_attach(h, aa);
     CUDA_TRY(h, run_attention(h, aa, R, st, pdl));
@@ -1350,7 +1354,7 @@ int32_t tts_gpt_op_attention_cluster(int32_t R, int32_t n_head, const float *q, 
     return TTS_GPT_OK;
   }
   if (cluster_size == -3) {   // rows must be stream-major with ascending positions, as in a prefill pass
-    CUDA_TRY(nullptr, launch_attention_prefill_tc(a, R, (cudaStream_t)cuda_stream, false));
+    CUDA_TRY(nullptr, launch_attention_prefill_tc(a, R, 148, (cudaStream_t)cuda_stream, false));
     return TTS_GPT_OK;
   }
   if (cluster_size == -2) {   // same requirement on the rows
