@@ -12,7 +12,9 @@ constexpr int kHeadDim = 64;
 constexpr int kPageTokens = 64;
 constexpr int kPageElems = kPageTokens * kHeadDim;  // one (page, head, K|V) block: 4096 bf16 = 8 KB
 constexpr int kMaxRows = 128;                       // rows per decode step, and rows of one row tile of a prefill pass
-constexpr int kMaxPassRows = 1024;                  // rows (streams x positions) of a prefill pass: up to 4 row tiles
+constexpr int kMaxPassRows = 4096;                  // rows (streams x positions) of a prefill pass: up to 32 row tiles
+constexpr int kMaxSplitRows = 1024;                 // rows up to which every pass may leave four k-range partial sums (or attend over e4m3 codes)
+constexpr int kMaxSplitTiles = 4 * kMaxSplitRows / kMaxRows;   // row tiles x k-ranges of a pass that leaves partial sums
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 

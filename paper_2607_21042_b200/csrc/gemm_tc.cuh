@@ -257,7 +257,8 @@ struct GemmTcArgs {
   int wfmt;                 // WF_* : bf16 = no scale, int8 = per row, int4 = per row and 128-column group
   int N, K, B, mode;        // mode: EPI_* of linear.cuh
   int ksplit;               // k-ranges (gridDim.z)
-  int stages;               // wide kernel: ring depth, set by its launcher
+  int stages;               // wide kernels: ring depth, set by the launcher
+  int bn, out_mapped;       // pair kernel: output features per tile, fp32 rows leave through a tensor map; set by its launcher
   float *out_f32;           // EPI_F32: out[b*out_stride+n]; EPI_QKV: q; EPI_RESID: x (ksplit == 1) or partials [ksplit][128][N]
   int out_stride;
   void *q_img;              // EPI_QKV, wide kernels: if set, q goes here as a bf16 activation image instead of to out_f32

@@ -151,8 +151,9 @@ struct PassParams {
 };
 
 // Row table of one prefill pass: up to kMaxPassRows (stream, position) rows taken from the prefixes.
-__global__ void __launch_bounds__(kMaxPassRows) prefill_pass_kernel(const PassParams p, PageState ps, RowTable rt, StepIO *io, int d) {
-  const int i = threadIdx.x;
+constexpr int kPassThreads = 512;
+__global__ void __launch_bounds__(kPassThreads) prefill_pass_kernel(const PassParams p, PageState ps, RowTable rt, StepIO *io, int d) {
+  const int i = blockIdx.x * kPassThreads + threadIdx.x;
   if (i < p.n_rows) {
     int j = 0;
     while (j + 1 < p.n_runs && p.run_row0[j + 1] <= i) ++j;

@@ -18,6 +18,7 @@
 #include "attention.cuh"
 #include "attention_prefill.cuh"
 #include "gemm_tc.cuh"
+#include "gemm_pw.cuh"
 #include "attention_prefill_tc.cuh"
 #include "elementwise.cuh"
 #include "kv_pages.cuh"
@@ -30,7 +31,8 @@ namespace {
 thread_local std::string g_last_error;
 
 struct PackedLinear {
-  void *w_img = nullptr;   // bf16 only: operand image for the tensor-core path (rows padded to 128)
+  void *w_img = nullptr;   // operand image for the tensor-core path (rows padded to 128)
+  CUtensorMap w_map;       // ... as the tensor the pair kernel copies from
   void *w = nullptr;
   uint16_t *s = nullptr;
   uint16_t *bias = nullptr;
@@ -75,6 +77,8 @@ struct tts_gpt {
   // tensor-core path (more than 16 rows, bf16 weights): activation images and k-split partial sums
   void *a_img = nullptr, *o_img = nullptr, *h_img = nullptr, *hf_img = nullptr;
   void *q_img = nullptr;             // q of prefill passes of more than 128 rows
+  CUtensorMap a_map, o_map, h_map;   // the images as tensors (all row tiles of a pass)
+  CUtensorMap xrow_map, part_map;    // the residual stream and the partial sums as tensors of fp32 rows
   float *partials = nullptr;
   bool have_tc = false;
   // attention scratch
@@ -95,8 +99,7 @@ struct tts_gpt {
   bool use_tc = true;   // tensor-core path for more than 16 rows (option "tc")
   bool use_attn_tc = true;   // prefill passes of more than 128 rows: attention on tcgen05 (option "attn_tc")
   bool w4_exact = false;   // int4 weights on the tensor-core path: images hold the integer codes and the kernels scale fp32 group sums (option "w4_tc_exact"); default: images hold code x group scale rounded to bf16
-  int prefill_pass_rows = 768;   // rows per prefill pass (option "prefill_pass_rows": a multiple of 128 up to 1024); set at creation
-                                 // to the most row tiles whose widest linear still runs as one wave of two CTAs per SM
+  int prefill_pass_rows = 896;   // rows per prefill pass (option "prefill_pass_rows": a multiple of 128 up to 4096); set at creation
   int tc_tail_parts = 0;  // partial sums the last FC2 of the tensor-core path left for the final LayerNorm
   bool use_attn_mma = true;      // tensor-core attention in prefill passes (option "attn_mma")
   bool use_attn_prefill = true;  // shared-page attention in prefill passes (option "attn_prefill")
@@ -246,7 +249,7 @@ size_t carve(tts_gpt *h, void *base) {
     h->scratch_src = cv.take<int>(kScratchPages);
     h->scratch_ntok = cv.take<int>(kScratchPages);
   }
-  const size_t attn_rows = h->kv_fp8 ? kMaxPassRows : kMaxRows;   // the 8-bit cache's attention kernel also serves prefill passes
+  const size_t attn_rows = h->kv_fp8 ? kMaxSplitRows : kMaxRows;   // the 8-bit cache's attention kernel also serves prefill passes
   h->attn_partials = cv.take<float>(attn_rows * c.n_head * kAttnMaxChunks * kAttnPartialFloats);
   h->attn_tickets = cv.take<unsigned int>(attn_rows * c.n_head);
   h->have_tc = true;
@@ -256,7 +259,7 @@ size_t carve(tts_gpt *h, void *base) {
     h->o_img = cv.take<char>(kTiles * act_image_bytes(d));
     h->h_img = cv.take<char>(kTiles * act_image_bytes(F));
     h->hf_img = cv.take<char>(act_image_bytes(d));
-    h->partials_floats = (size_t)kTiles * std::max(kTcKSplit, kTwMaxPartials) * kMaxRows * d;   // [row tile][k-range][128][d]
+    h->partials_floats = (size_t)kMaxSplitTiles * kMaxRows * d;   // [row tile][k-range][128][d]
     h->partials = cv.take<float>(h->partials_floats);
     h->q_img = cv.take<char>(kTiles * act_image_bytes(d));
   }
@@ -409,8 +412,17 @@ int launch_ln_tc(tts_gpt *h, int rows, const uint16_t *g, const uint16_t *b, int
   return TTS_GPT_OK;
 }
 
-int launch_gemm(tts_gpt *h, const GemmTcArgs &a, bool wide, cudaStream_t st, bool pdl) {
-  CUDA_TRY(h, wide ? launch_gemm_tcw(a, h->n_sm, st, pdl) : launch_gemm_tc(a, st, pdl));
+// Passes of up to kPairMinRows rows stay with the one-CTA wide kernel (two CTAs per SM): their tiles are too few for pairs.
+constexpr int kPairMinRows = 1024;
+bool use_pairs(const tts_gpt *h, int R) { return R > kPairMinRows && !(h->cfg.wfmt == WF_INT4 && h->w4_exact); }
+
+int launch_gemm(tts_gpt *h, const GemmTcArgs &a, const CUtensorMap &w_map, const CUtensorMap &x_map, bool wide, cudaStream_t st, bool pdl) {
+  if (!wide) CUDA_TRY(h, launch_gemm_tc(a, st, pdl));
+  else if (!use_pairs(h, a.B)) CUDA_TRY(h, launch_gemm_tcw(a, h->n_sm, st, pdl));
+  else {
+    const CUtensorMap *out = a.mode != EPI_RESID ? nullptr : a.ksplit > 1 ? &h->part_map : &h->xrow_map;
+    CUDA_TRY(h, launch_gemm_pw(a, w_map, x_map, out, pw_plan(a.N, a.K, a.B, a.mode == EPI_RESID, h->n_sm, a.ksplit).bn, h->n_sm, st, pdl));
+  }
   return TTS_GPT_OK;
 }
 
@@ -423,8 +435,9 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
   cudaStream_t st = h->stream;
   const bool pdl = h->use_pdl;
   const bool wide = R > kMaxRows;
-  const int o_ks = wide ? tcw_ksplit_resid(d) : kTcKSplit;
-  const int f2_ks = wide ? tcw_ksplit_resid(c.d_ff) : kTcKSplit;
+  const bool pairs = use_pairs(h, R);
+  const int o_ks = !wide ? kTcKSplit : pairs ? pw_plan(d, d, R, true, h->n_sm).ksplit : tcw_ksplit_resid(d);
+  const int f2_ks = !wide ? kTcKSplit : pairs ? pw_plan(d, c.d_ff, R, true, h->n_sm).ksplit : tcw_ksplit_resid(c.d_ff);
   const int o_parts = o_ks > 1 ? o_ks : 0, f2_parts = f2_ks > 1 ? f2_ks : 0;   // 0: the linear added into x itself
   for (int l = 0; l < c.n_layer; ++l) {
     LayerW &L = h->layers[l];
@@ -441,7 +454,7 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
     const bool q_img = wide && h->use_attn_tc && h->use_attn_mma && (!h->kv_fp8 || h->pass_scratch > 0);   // the tcgen05 attention follows
     qa.q_img = q_img ? h->q_img : nullptr;
     trace_attach(h, qa);
-    if ((rc = launch_gemm(h, qa, wide, st, pdl))) return rc;
+    if ((rc = launch_gemm(h, qa, L.qkv.w_map, h->a_map, wide, st, pdl))) return rc;
     AttnArgs aa;
     memset(&aa, 0, sizeof aa);
     aa.q = h->q; aa.kv_layer = kvl; aa.page_table = h->ps.page_table; aa.row_stream = h->rt.row_stream;
@@ -452,17 +465,17 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
     GemmTcArgs oa = gemm_args(h, L.o, h->o_img, R, EPI_RESID, o_ks);
     oa.out_f32 = o_parts ? h->partials : h->x; oa.out_stride = d;
     trace_attach(h, oa);
-    if ((rc = launch_gemm(h, oa, wide, st, pdl))) return rc;
+    if ((rc = launch_gemm(h, oa, L.o.w_map, h->o_map, wide, st, pdl))) return rc;
     rc = launch_ln_tc(h, R, L.ln2_g, L.ln2_b, o_parts, L.o.bias, h->a_img, nullptr, nullptr, nullptr, nullptr, 1);
     if (rc) return rc;
     GemmTcArgs f1 = gemm_args(h, L.fc1, h->a_img, R, EPI_GELU, 1);
     f1.out_img = h->h_img; f1.gelu_tanh = c.gelu_tanh;
     trace_attach(h, f1);
-    if ((rc = launch_gemm(h, f1, wide, st, pdl))) return rc;
+    if ((rc = launch_gemm(h, f1, L.fc1.w_map, h->a_map, wide, st, pdl))) return rc;
     GemmTcArgs f2 = gemm_args(h, L.fc2, h->h_img, R, EPI_RESID, f2_ks);
     f2.out_f32 = f2_parts ? h->partials : h->x; f2.out_stride = d;
     trace_attach(h, f2);
-    if ((rc = launch_gemm(h, f2, wide, st, pdl))) return rc;
+    if ((rc = launch_gemm(h, f2, L.fc2.w_map, h->h_map, wide, st, pdl))) return rc;
     h->launches += 5;
   }
   h->tc_tail_parts = f2_parts;
@@ -701,10 +714,29 @@ int32_t tts_gpt_create(const tts_gpt_config_t *cfg, const tts_gpt_weights_t *w, 
     TRY_(load_linear(h, L.fc2, c.wfmt, w->fc2_w[l], qz ? w->fc2_s[l] : nullptr, w->fc2_b[l], "fc2"));
   }
   if (c.wfmt == WF_INT4) TRY_(write_int4_images(h));
+  {   // operand images, residual stream and partial sums as tensors, for the linears of large prefill passes
+    auto image = [&](CUtensorMap *m, const void *img, size_t blocks) -> int {
+      CUDA_TRY(h, pw_image_map(m, img, blocks));
+      return TTS_GPT_OK;
+    };
+    auto rows = [&](CUtensorMap *m, const float *base, size_t n) -> int {
+      CUDA_TRY(h, pw_rows_map(m, base, d, n));
+      return TTS_GPT_OK;
+    };
+    const size_t tiles = kMaxPassRows / kMaxRows;
+    TRY_(image(&h->a_map, h->a_img, tiles * (d / 64)));
+    TRY_(image(&h->o_map, h->o_img, tiles * (d / 64)));
+    TRY_(image(&h->h_map, h->h_img, tiles * (c.d_ff / 64)));
+    TRY_(rows(&h->xrow_map, h->x, kMaxPassRows));
+    TRY_(rows(&h->part_map, h->partials, (size_t)kMaxSplitTiles * kMaxRows));
+    for (auto &L : h->layers)
+      for (PackedLinear *pl : {&L.qkv, &L.o, &L.fc1, &L.fc2})
+        TRY_(image(&pl->w_map, pl->w_img, (size_t)((pl->N + 127) / 128) * (pl->K / 64)));
+  }
 #undef TRY_
   const int init_n = std::max(std::max(c.n_pages, c.max_streams * h->pps), c.max_streams);
   init_pages_kernel<<<(init_n + 255) / 256, 256, 0, h->stream>>>(h->ps);
-  cudaError_t e = cudaMemsetAsync(h->attn_tickets, 0, (size_t)(h->kv_fp8 ? kMaxPassRows : kMaxRows) * c.n_head * sizeof(unsigned int), h->stream);
+  cudaError_t e = cudaMemsetAsync(h->attn_tickets, 0, (size_t)(h->kv_fp8 ? kMaxSplitRows : kMaxRows) * c.n_head * sizeof(unsigned int), h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->canary_lo, kCanaryByte, kCanaryBytes, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->canary_hi, kCanaryByte, kCanaryBytes, h->stream);
   if (e == cudaSuccess) {
@@ -735,12 +767,10 @@ int32_t tts_gpt_create(const tts_gpt_config_t *cfg, const tts_gpt_weights_t *w, 
   if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
     h->n_sm = sms;
   {
-    // rows per prefill pass: the wide linears run two CTAs per SM; a pass of t row tiles gives the widest linear
-    // t x (features / 128) x k-ranges CTAs, and one CTA too many doubles its time.  Measured on 148 SMs with this
-    // model (FC1: 40 feature tiles): 88946 prefix rows in 301 / 279 / 308 ms at 6 / 7 / 8 row tiles.
-    const tts_gpt_config_t &c = h->cfg;
-    const int widest = std::max(std::max((c.d_ff + 127) / 128, (3 * c.d_model + 127) / 128), tcw_ksplit_resid(c.d_ff) * ((c.d_model + 127) / 128));
-    const int t = std::max(1, std::min(kMaxPassRows / kMaxRows, 2 * h->n_sm / std::max(1, widest)));
+    // rows per prefill pass: the most row tiles whose model-wide linears (O projection, FC2) still run as one wave of
+    // one 256 x 256 tile per pair of SMs; QKV and FC1 then take 3 and 4 nearly full waves.  28 tiles with this model on
+    // 148 SMs.
+    const int t = std::max(1, std::min(kMaxPassRows / kMaxRows, 2 * (h->n_sm / 2 / ((h->cfg.d_model + 255) / 256))));
     h->prefill_pass_rows = t * kMaxRows;
   }
   *out = h;
@@ -814,7 +844,8 @@ static int prefill_impl(tts_gpt_t *h, int32_t n, const void *const *emb, const i
   io.out_hidden = (uint16_t *)out_hidden; io.top_k = top_k; io.temperature = temperature; io.n_out = 0;
   // rows in stream-major order; a pass takes up to `pass_rows` of them (several row tiles of 128 when the
   // tensor-core path is available, else one)
-  const int pass_rows = (h->have_tc && h->use_tc) ? h->prefill_pass_rows : kMaxRows;
+  int pass_rows = (h->have_tc && h->use_tc) ? h->prefill_pass_rows : kMaxRows;
+  if ((c.wfmt == WF_INT4 && h->w4_exact) || (h->kv_fp8 && !h->use_attn_mma)) pass_rows = std::min(pass_rows, kMaxSplitRows);
   PassParams ps;
   memset(&ps, 0, sizeof ps);
   ps.io = io;
@@ -829,7 +860,7 @@ static int prefill_impl(tts_gpt_t *h, int32_t n, const void *const *emb, const i
     ps.run_scratch0[ps.n_runs] = (short)scratch_pages;
     ps.scratch_table = h->scratch_table; ps.scratch_src = h->scratch_src; ps.scratch_ntok = h->scratch_ntok;
     h->pass_scratch = scratch_pages;
-    prefill_pass_kernel<<<1, kMaxPassRows, 0, h->stream>>>(ps, h->ps, h->rt, h->io, c.d_model);
+    prefill_pass_kernel<<<(std::max(ps.n_rows, scratch_pages) + kPassThreads - 1) / kPassThreads, kPassThreads, 0, h->stream>>>(ps, h->ps, h->rt, h->io, c.d_model);
     CUDA_TRY(h, cudaGetLastError());
     h->launches += 1;
     int r = run_embed(h, ps.n_rows);
@@ -1104,7 +1135,7 @@ int32_t tts_gpt_debug_set_option(tts_gpt_t *h, const char *name, int32_t value) 
   if (k == "graph") h->use_graph = on && h->stream != nullptr && h->stream != cudaStreamLegacy;
   else if (k == "pdl") h->use_pdl = on;
   else if (k == "tc") h->use_tc = on;
-  else if (k == "prefill_pass_rows") { if (value < kMaxRows || value > kMaxPassRows || value % kMaxRows) return fail(h, TTS_GPT_E_ARG, "prefill_pass_rows must be a multiple of 128 from 128 to 1024"); h->prefill_pass_rows = value; }
+  else if (k == "prefill_pass_rows") { if (value < kMaxRows || value > kMaxPassRows || value % kMaxRows) return fail(h, TTS_GPT_E_ARG, "prefill_pass_rows must be a multiple of 128 from 128 to %d", kMaxPassRows); h->prefill_pass_rows = value; }
   else if (k == "tc_min_rows") { if (value < 1 || value > kMaxRows) return fail(h, TTS_GPT_E_ARG, "tc_min_rows must be in 1..%d", kMaxRows); h->tc_min_rows = value; }
   else if (k == "attn_tc") h->use_attn_tc = on;
   else if (k == "w4_tc_exact") {
@@ -1205,6 +1236,15 @@ int32_t tts_gpt_op_linear_tc_scratch_bytes(int32_t N, int32_t K, size_t *bytes) 
   return TTS_GPT_OK;
 }
 
+// the wide kernels on one row tile: int4 codes with group sums on the one-CTA kernel, the rest on the pair kernel
+static cudaError_t launch_wide(const GemmTcArgs &a, cudaStream_t st) {
+  if (a.wfmt == WF_INT4) return launch_gemm_tcw(a, 148, st, false);
+  CUtensorMap w_map, x_map;
+  cudaError_t e = pw_image_map(&w_map, a.w_img, (size_t)((a.N + 127) / 128) * (a.K / 64));
+  if (e == cudaSuccess) e = pw_image_map(&x_map, a.act_img, a.K / 64);
+  return e != cudaSuccess ? e : launch_gemm_pw(a, w_map, x_map, nullptr, pw_plan(a.N, a.K, a.B, a.mode == EPI_RESID, 148, a.ksplit).bn, 148, st, false);
+}
+
 int32_t tts_gpt_op_linear_tc(int32_t wfmt, int32_t N, int32_t K, const void *w, const void *s, const void *bias,
                              int32_t B, const void *act, float *out, int32_t ksplit, void *scratch, void *cuda_stream) {
   size_t bytes;
@@ -1236,10 +1276,10 @@ int32_t tts_gpt_op_linear_tc(int32_t wfmt, int32_t N, int32_t K, const void *w, 
   a.w_img = wimg; a.act_img = aimg; a.N = N; a.K = K; a.B = B; a.ksplit = ksplit; a.wfmt = wfmt; a.scales = tiled_s;
   if (ksplit == 1) {
     a.mode = EPI_F32; a.bias = (const uint16_t *)bias; a.out_f32 = out; a.out_stride = N;
-    CUDA_TRY(nullptr, wide ? launch_gemm_tcw(a, 148, st, false) : launch_gemm_tc(a, st, false));
+    CUDA_TRY(nullptr, wide ? launch_wide(a, st) : launch_gemm_tc(a, st, false));
   } else {   // partial sums per k-range, then folded in range order (what the following LayerNorm does in the engine)
     a.mode = EPI_RESID; a.out_f32 = part; a.out_stride = N;
-    CUDA_TRY(nullptr, wide ? launch_gemm_tcw(a, 148, st, false) : launch_gemm_tc(a, st, false));
+    CUDA_TRY(nullptr, wide ? launch_wide(a, st) : launch_gemm_tc(a, st, false));
     fold_partials_kernel<<<(unsigned)(((size_t)B * N + 255) / 256), 256, 0, st>>>(part, ksplit, B, N, (const uint16_t *)bias, out);
     CUDA_TRY(nullptr, cudaGetLastError());
   }
