@@ -126,6 +126,97 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }   // sources may be overwritten
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }         // writes are done
 
+// 32 lanes x 8 columns of 32-bit
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// Where a group of 64 features of a warp's 32 rows goes.
+enum { PW_GELU_TANH = 0, PW_GELU_ERF = 1, PW_BF16 = 2, PW_F32 = 3 };
+// One group out of tensor memory, through bias (and int8 scale) and GELU, into the warp's patch: [32 rows][128 bytes],
+// 16-byte unit u at u ^ (row % 8); bf16 kinds leave the 64 columns there, fp32 leaves in two blocks of 32 columns.
+// The loop is kept rolled, eight columns a turn: unrolled over 32 columns this code ran at ten cycles an instruction,
+// fetched from beyond the instruction cache for every block (10.7 us of epilogue for a tile of the O projection).
+// bs, sc: two features per lane and register, columns 0..31 and 32..63 of the group, dealt out by shuffles.
+template <int KIND>
+__device__ __forceinline__ void pw_group(const GemmTcArgs &a, uint32_t t_grp, unsigned char *patch, int lane, const uint32_t (&bs)[2], const uint32_t (&sc)[2],
+                                         bool empty_range, bool store, const CUtensorMap *out_map, bool add, int col, int map_row, float *plain, size_t pitch, int rows) {
+#pragma unroll 1
+  for (int c8 = 0; c8 < 8; ++c8) {
+    float v[8];
+    tmem_ld8(t_grp + 8u * c8, v);
+    if (empty_range) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) v[c] = 0.f;
+    }
+    const uint32_t b_mine = c8 < 4 ? bs[0] : bs[1];
+    if (a.wfmt == WF_INT8) {
+      const uint32_t s_mine = c8 < 4 ? sc[0] : sc[1];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t b = __shfl_sync(0xFFFFFFFFu, b_mine, 4 * (c8 & 3) + q), s = __shfl_sync(0xFFFFFFFFu, s_mine, 4 * (c8 & 3) + q);
+        v[2 * q] = fmaf(v[2 * q], bf16_lo(s), bf16_lo(b));
+        v[2 * q + 1] = fmaf(v[2 * q + 1], bf16_hi(s), bf16_hi(b));
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t b = __shfl_sync(0xFFFFFFFFu, b_mine, 4 * (c8 & 3) + q);
+        v[2 * q] += bf16_lo(b);
+        v[2 * q + 1] += bf16_hi(b);
+      }
+    }
+    if (KIND == PW_GELU_TANH) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) v[c] = gelu_tanh_f(v[c]);
+    }
+    if (KIND == PW_GELU_ERF) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) v[c] = gelu_erf_f(v[c]);
+    }
+    if (c8 == 0 || (KIND == PW_F32 && c8 == 4)) {   // the patch is free once the copy engine has read it
+      if (elect_one()) bulk_wait_read();
+      __syncwarp();
+    }
+    if (KIND != PW_F32) {
+      *reinterpret_cast<uint4 *>(patch + lane * 128 + ((c8 ^ (lane & 7)) << 4)) =
+          make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
+      continue;
+    }
+    const int u = 2 * (c8 & 3);
+    *reinterpret_cast<float4 *>(patch + lane * 128 + ((u ^ (lane & 7)) << 4)) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float4 *>(patch + lane * 128 + (((u + 1) ^ (lane & 7)) << 4)) = make_float4(v[4], v[5], v[6], v[7]);
+    if ((c8 & 3) != 3) continue;
+    const int c32 = 32 * (c8 >> 2);
+    if (out_map) {
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (store && elect_one()) {
+        if (add) block_store<true>(out_map, col + c32, map_row, patch);
+        else block_store<false>(out_map, col + c32, map_row, patch);
+        bulk_commit();
+      }
+      __syncwarp();
+    } else {   // rows the copy engine cannot address (a caller's own array): eight lanes per row
+      __syncwarp();
+      for (int rr = lane >> 3; rr < rows && store; rr += 4) {
+        const float4 x = *reinterpret_cast<const float4 *>(patch + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4));
+        const float xs[4] = {x.x, x.y, x.z, x.w};
+        float *dst = plain + (size_t)rr * pitch + c32 + 4 * (lane & 7);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (col + c32 + 4 * (lane & 7) + e < a.N) dst[e] = add ? dst[e] + xs[e] : xs[e];   // the last features may be ragged
+      }
+      __syncwarp();
+    }
+  }
+}
+
 __global__ void __launch_bounds__(kPwThreads, 1) gemm_pw_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap x_map,
                                                               const __grid_constant__ CUtensorMap out_map, const GemmTcArgs a) {
   extern __shared__ __align__(16) unsigned char pw_smem_raw[];
@@ -251,14 +342,20 @@ __global__ void __launch_bounds__(kPwThreads, 1) gemm_pw_kernel(const __grid_con
         }
       }
       // bias and scales of this warp's (up to two) groups, two features per lane and register, fetched ahead of the
-      // accumulator and dealt out by shuffles: a load behind it takes over 1000 cycles while every SM streams operands
-      uint32_t bias2[4], scale2[4];
+      // accumulator: a load behind it takes over 1000 cycles while every SM streams operands
+      uint32_t bias2[2][2], scale2[2][2];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int n = p.n0 + grp * 64 + (q >> 1) * 128 + (q & 1) * 32 + 2 * (lane & 15);
-        const bool there = n < min(n_end, a.N & ~31);
-        bias2[q] = use_bias && there ? __ldg(reinterpret_cast<const uint32_t *>(a.bias + n)) : 0u;
-        scale2[q] = a.wfmt == WF_INT8 && there ? __ldg(reinterpret_cast<const uint32_t *>(a.scales + n)) : 0u;
+        uint32_t bw = 0u, sw = 0u;
+        if (n + 1 < n_end) {
+          if (use_bias) bw = __ldg(reinterpret_cast<const uint32_t *>(a.bias + n));
+          if (a.wfmt == WF_INT8) sw = __ldg(reinterpret_cast<const uint32_t *>(a.scales + n));
+        } else if (n < n_end) {
+          if (use_bias) bw = a.bias[n];
+          if (a.wfmt == WF_INT8) sw = a.scales[n];
+        }
+        bias2[q >> 1][q & 1] = bw; scale2[q >> 1][q & 1] = sw;
       }
       tc_wait(acc_full + (k & 1), (uint32_t)(k >> 1) & 1u, failed, a.err);   // committed by CTA 0 to both CTAs
       if (k == 0) trace_mark(a.trace, a.trace_slot, 4, 64);   // first accumulator complete
@@ -266,112 +363,48 @@ __global__ void __launch_bounds__(kPwThreads, 1) gemm_pw_kernel(const __grid_con
       __syncwarp();
       const uint32_t t_row = tmem_d + 256u * (uint32_t)(k & 1) + ((uint32_t)(lw * 32) << 16);
       const bool store = rows > 0 && !__any_sync(0xFFFFFFFFu, *failed);   // nothing is stored after an expired wait
+#pragma unroll 1
       for (int n64 = p.n0 + grp * 64; n64 < n_end; n64 += 128) {
-        const bool to_img = a.mode == EPI_GELU || (a.mode == EPI_QKV && n64 < a.d && a.q_img);
-        const bool as_bf16 = to_img || (a.mode == EPI_QKV && n64 >= a.d);
         const bool second = n64 - p.n0 >= 128;
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-          const int nb = n64 + 32 * hh;
-          float v[32];
-          tmem_ld32(t_row + (uint32_t)(nb - p.n0), v);
-          if (p.n_it <= 0) {
-#pragma unroll
-            for (int c = 0; c < 32; ++c) v[c] = 0.f;
-          }
-          if (nb + 32 > a.N) {   // ragged last features: fp32 rows written one by one
-#pragma unroll
-            for (int c = 0; c < 32; ++c)
-              if (store && lane < rows && nb + c < a.N) {
-                const float b = use_bias ? bf16_bits_to_float(a.bias[nb + c]) : 0.f, s1 = a.wfmt == WF_INT8 ? bf16_bits_to_float(a.scales[nb + c]) : 1.f;
-                float *dst = (partial ? a.out_f32 + (((size_t)(p.row0 >> 7) * a.ksplit + p.ks) * kMaxRows + lw * 32 + lane) * a.N : a.out_f32 + (size_t)r * a.out_stride) + nb + c;
-                const float y = fmaf(v[c], s1, b);
-                *dst = add ? *dst + y : y;
-              }
-            __syncwarp();
-            continue;
-          }
-          const uint32_t b_mine = second ? bias2[2 + hh] : bias2[hh], s_mine = second ? scale2[2 + hh] : scale2[hh];
-          if (a.wfmt == WF_INT8) {
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-              const uint32_t b = __shfl_sync(0xFFFFFFFFu, b_mine, c), sc = __shfl_sync(0xFFFFFFFFu, s_mine, c);
-              v[2 * c] = fmaf(v[2 * c], bf16_lo(sc), bf16_lo(b));
-              v[2 * c + 1] = fmaf(v[2 * c + 1], bf16_hi(sc), bf16_hi(b));
-            }
-          } else if (use_bias) {
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-              const uint32_t b = __shfl_sync(0xFFFFFFFFu, b_mine, c);
-              v[2 * c] += bf16_lo(b);
-              v[2 * c + 1] += bf16_hi(b);
-            }
-          }
-          if (a.mode == EPI_GELU) {
-            if (a.gelu_tanh) {
-#pragma unroll
-              for (int c = 0; c < 32; ++c) v[c] = gelu_tanh_f(v[c]);
-            } else {
-#pragma unroll 4
-              for (int c = 0; c < 32; ++c) v[c] = gelu_erf_f(v[c]);
-            }
-          }
-          if (!as_bf16 || hh == 0) {   // the patch is free once the copy engine has read it
-            if (elect_one()) bulk_wait_read();
-            __syncwarp();
-          }
-          if (as_bf16) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              *reinterpret_cast<uint4 *>(patch + lane * 128 + (((4 * hh + q) ^ (lane & 7)) << 4)) =
-                  make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]), pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
-                             pack_bf16x2(v[8 * q + 4], v[8 * q + 5]), pack_bf16x2(v[8 * q + 6], v[8 * q + 7]));
-          } else {
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-              *reinterpret_cast<float4 *>(patch + lane * 128 + ((q ^ (lane & 7)) << 4)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-            if (a.out_mapped) {
-              fence_proxy_async_smem();
-              __syncwarp();
-              if (store && elect_one()) {
-                if (add) block_store<true>(&out_map, nb, p.row0 + lw * 32, patch);
-                else block_store<false>(&out_map, nb, partial ? ((p.row0 >> 7) * a.ksplit + p.ks) * kMaxRows + lw * 32 : p.row0 + lw * 32, patch);
-                bulk_commit();
-              }
-            } else {   // rows the copy engine cannot address (a caller's own array): eight lanes per row
-              __syncwarp();
-              for (int rr = lane >> 3; rr < rows && store; rr += 4) {
-                const float4 x = *reinterpret_cast<const float4 *>(patch + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4));
-                float *dst = (partial ? a.out_f32 + (((size_t)(p.row0 >> 7) * a.ksplit + p.ks) * kMaxRows + lw * 32 + rr) * a.N
-                                      : a.out_f32 + (size_t)(p.row0 + lw * 32 + rr) * a.out_stride) + nb + 4 * (lane & 7);
-                dst[0] = add ? dst[0] + x.x : x.x; dst[1] = add ? dst[1] + x.y : x.y; dst[2] = add ? dst[2] + x.z : x.z; dst[3] = add ? dst[3] + x.w : x.w;
-              }
-              __syncwarp();
-            }
-          }
+        const uint32_t bs[2] = {second ? bias2[1][0] : bias2[0][0], second ? bias2[1][1] : bias2[0][1]};
+        const uint32_t sc[2] = {second ? scale2[1][0] : scale2[0][0], second ? scale2[1][1] : scale2[0][1]};
+        const uint32_t t_grp = t_row + (uint32_t)(n64 - p.n0);
+        const bool to_img = a.mode == EPI_GELU || (a.mode == EPI_QKV && n64 < a.d && a.q_img);
+        const bool none = p.n_it <= 0;
+        if (a.mode == EPI_GELU) {
+          if (a.gelu_tanh) pw_group<PW_GELU_TANH>(a, t_grp, patch, lane, bs, sc, none, store, nullptr, false, 0, 0, nullptr, 0, 0);
+          else pw_group<PW_GELU_ERF>(a, t_grp, patch, lane, bs, sc, none, store, nullptr, false, 0, 0, nullptr, 0, 0);
+        } else if (to_img || (a.mode == EPI_QKV && n64 >= a.d)) {
+          pw_group<PW_BF16>(a, t_grp, patch, lane, bs, sc, none, store, nullptr, false, 0, 0, nullptr, 0, 0);
+        } else {
+          const int prow = ((p.row0 >> 7) * a.ksplit + p.ks) * kMaxRows + lw * 32;
+          float *plain = partial ? a.out_f32 + (size_t)prow * a.N + n64 : a.out_f32 + (size_t)(p.row0 + lw * 32) * a.out_stride + n64;
+          pw_group<PW_F32>(a, t_grp, patch, lane, bs, sc, none, store, a.out_mapped ? &out_map : nullptr, add, n64, partial ? prow : p.row0 + lw * 32, plain,
+                           partial ? (size_t)a.N : (size_t)a.out_stride, rows);
+          continue;
         }
-        if (as_bf16) {
-          if (to_img) fence_proxy_async_smem();
+        if (to_img) {   // 32 rows x 64 columns are 4 KB of the image; rows past the pass are never read
+          fence_proxy_async_smem();
           __syncwarp();
-          if (to_img) {   // 32 rows x 64 columns are 4 KB of the image; rows past the pass are never read
-            unsigned char *img = reinterpret_cast<unsigned char *>(a.mode == EPI_GELU ? a.out_img : a.q_img);
-            const int cols64 = (a.mode == EPI_GELU ? a.N : a.d) >> 6;
-            if (store && elect_one()) {
-              bulk_store(img + ((size_t)(p.row0 >> 7) * cols64 + (n64 >> 6)) * (kMaxRows * 128) + (size_t)lw * 4096, patch, 4096);
-              bulk_commit();
-            }
-          } else {        // K/V rows: eight lanes write the 128 bytes of a row into its page slot or staging row
-            const int which = n64 >= 2 * a.d, col = n64 - (which ? 2 * a.d : a.d);
-            const size_t kv_off = a.kv_stage ? (size_t)which * a.d + col : ((size_t)which * a.H + (col >> 6)) * kPageElems;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int rr = 4 * i + (lane >> 3);
-              const uint4 y = *reinterpret_cast<const uint4 *>(patch + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4));
-              uint16_t *dst = reinterpret_cast<uint16_t *>(__shfl_sync(0xFFFFFFFFu, reinterpret_cast<unsigned long long>(kv_mine), rr));
-              if (rr < rows && store) *reinterpret_cast<uint4 *>(dst + kv_off + 8 * (lane & 7)) = y;
-            }
-            __syncwarp();
+          unsigned char *img = reinterpret_cast<unsigned char *>(a.mode == EPI_GELU ? a.out_img : a.q_img);
+          const int cols64 = (a.mode == EPI_GELU ? a.N : a.d) >> 6;
+          if (store && elect_one()) {
+            bulk_store(img + ((size_t)(p.row0 >> 7) * cols64 + (n64 >> 6)) * (kMaxRows * 128) + (size_t)lw * 4096, patch, 4096);
+            bulk_commit();
           }
+          __syncwarp();
+        } else {        // K/V rows: eight lanes write the 128 bytes of a row into its page slot or staging row
+          __syncwarp();
+          const int which = n64 >= 2 * a.d, col = n64 - (which ? 2 * a.d : a.d);
+          const size_t kv_off = a.kv_stage ? (size_t)which * a.d + col : ((size_t)which * a.H + (col >> 6)) * kPageElems;
+#pragma unroll 2
+          for (int i = 0; i < 8; ++i) {
+            const int rr = 4 * i + (lane >> 3);
+            const uint4 y = *reinterpret_cast<const uint4 *>(patch + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4));
+            uint16_t *dst = reinterpret_cast<uint16_t *>(__shfl_sync(0xFFFFFFFFu, reinterpret_cast<unsigned long long>(kv_mine), rr));
+            if (rr < rows && store) *reinterpret_cast<uint4 *>(dst + kv_off + 8 * (lane & 7)) = y;
+          }
+          __syncwarp();
         }
       }
       // this warp has read its part of the accumulator, which may take the tile after next
