@@ -402,7 +402,12 @@ int launch_ln_tc(tts_gpt *h, int rows, const uint16_t *g, const uint16_t *b, int
   if (rows > kMaxRows && h->cfg.d_model % 8 == 0) {
     // the many rows of a large prefill pass: one warp per row
     const dim3 rgrid((rows + kLnRowsWarps - 1) / kLnRowsWarps), rblock(kLnRowsWarps * 32);
-    if (np <= 1) CUDA_TRY(h, launch_kernel(layernorm_rows_kernel<2>, rgrid, rblock, 0, h->stream, h->use_pdl, la, rows));
+    if (n_part == 0 && !add_bias && out_img && !out_plain && !gather && !io) {   // nothing to fold: the pair kernel's passes
+      la.err = h->dev_err;
+      CUDA_TRY(h, launch_kernel(layernorm_big_kernel, dim3((rows + kLnBigWarps - 1) / kLnBigWarps), dim3(kLnBigWarps * 32),
+                                layernorm_big_smem_bytes(h->cfg.d_model), h->stream, h->use_pdl, la, rows));
+    }
+    else if (np <= 1) CUDA_TRY(h, launch_kernel(layernorm_rows_kernel<2>, rgrid, rblock, 0, h->stream, h->use_pdl, la, rows));
     else if (np <= 5) CUDA_TRY(h, launch_kernel(layernorm_rows_kernel<10>, rgrid, rblock, 0, h->stream, h->use_pdl, la, rows));
     else CUDA_TRY(h, launch_kernel(layernorm_rows_kernel<2 * kLnMaxPerThread>, rgrid, rblock, 0, h->stream, h->use_pdl, la, rows));
   } else if (np <= 1) CUDA_TRY(h, launch_kernel(layernorm_tc_kernel<1>, grid, block, 0, h->stream, h->use_pdl, la));
@@ -444,7 +449,7 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
     uint16_t *kvl = h->kv + h->kv_layer_elems * l;
     int rc;
     // fold the previous layer's FC2 partial sums into x, then LN1 -> image
-    rc = launch_ln_tc(h, R, L.ln1_g, L.ln1_b, l == 0 ? 0 : f2_parts, l == 0 ? nullptr : h->layers[l - 1].fc2.bias,
+    rc = launch_ln_tc(h, R, L.ln1_g, L.ln1_b, l == 0 ? 0 : f2_parts, l == 0 || !f2_parts ? nullptr : h->layers[l - 1].fc2.bias,
                       h->a_img, nullptr, nullptr, nullptr, nullptr, 1);
     if (rc) return rc;
     GemmTcArgs qa = gemm_args(h, L.qkv, h->a_img, R, EPI_QKV, 1);
@@ -466,7 +471,7 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
     oa.out_f32 = o_parts ? h->partials : h->x; oa.out_stride = d;
     trace_attach(h, oa);
     if ((rc = launch_gemm(h, oa, L.o.w_map, h->o_map, wide, st, pdl))) return rc;
-    rc = launch_ln_tc(h, R, L.ln2_g, L.ln2_b, o_parts, L.o.bias, h->a_img, nullptr, nullptr, nullptr, nullptr, 1);
+    rc = launch_ln_tc(h, R, L.ln2_g, L.ln2_b, o_parts, o_parts ? L.o.bias : nullptr, h->a_img, nullptr, nullptr, nullptr, nullptr, 1);
     if (rc) return rc;
     GemmTcArgs f1 = gemm_args(h, L.fc1, h->a_img, R, EPI_GELU, 1);
     f1.out_img = h->h_img; f1.gelu_tanh = c.gelu_tanh;
