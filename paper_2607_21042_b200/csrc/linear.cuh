@@ -17,7 +17,7 @@
 // previous kernel, so under programmatic dependent launch the copy overlaps the predecessor's
 // tail and occupies no registers.  Only then does the CTA wait for its predecessor, stage (or
 // layer-normalise) the activation rows, wait for the weights (bounded wait, error word on
-// expiry), form the products — fp32 FMAs for up to 4 batch rows, the tensor pipe above — and the
+// expiry), form the products — fp32 FMAs for one batch row, the tensor pipe above — and the
 // warps' partial sums meet in shared memory in warp order (results do not depend on timing).
 // Batches above 16 loop over m-tiles re-using the weights in shared memory.
 #pragma once
@@ -32,8 +32,8 @@ enum { EPI_F32 = 0, EPI_QKV = 1, EPI_RESID = 2, EPI_GELU = 3 };
 constexpr int kLinearWarps = 10;  // divides the k-tile counts of K=1280 and K=5120 in every format
 constexpr int kLinearThreads = kLinearWarps * 32;
 constexpr int kSmallKSplit = 4;     // k-ranges of FC2 between 5 and 16 rows (partial sums folded by the next LayerNorm)
-constexpr int kLnFuseMaxRows = 4;   // LayerNorm is fused into the linear up to this batch: every CTA repeats
-                                    // it, which beats a separate launch only while the rows are few
+constexpr int kLnFuseMaxRows = 1;   // LayerNorm is fused into the linear up to this batch: every CTA repeats it, which
+                                    // beats a separate launch for a single row only
 
 __host__ __device__ inline int k_per_tile(int wf) { return wf == WF_BF16 ? 32 : (wf == WF_INT8 ? 64 : 128); }
 __host__ __device__ inline int row_tiles(int N) { return (N + 7) / 8; }
@@ -176,10 +176,10 @@ enum { ACT_DIRECT = 0, ACT_STAGED = 1, ACT_LN = 2 };
 constexpr int kStageMaxBytes = 44 * 1024;
 constexpr int kLinearSmemBudget = 108 * 1024;  // per CTA, so that two CTAs share an SM
 
-// NB: 0 = tensor-pipe path (any batch, 16 rows per m-tile); 1 or 4 = CUDA-core path for batches of
-// at most NB rows.  On this part one warp-level MMA occupies the tensor pipe of its SM partition
-// for about 32 cycles whatever the number of real batch rows, so below 5 rows plain fp32 FMAs on
-// the widened weights are cheaper.
+// NB: 0 = tensor-pipe path (any batch, 16 rows per m-tile); 1 = CUDA-core path for a single row, whose fp32 FMAs
+// on the widened weights are cheaper than MMAs that are fifteen sixteenths padding.  From two rows on the MMAs win:
+// the FMA path with LayerNorm fused in took 0.77 / 0.90 / 1.04 ms per step at 2 / 3 / 4 rows (bf16, context 530),
+// MMAs behind LayerNorm kernels of their own 0.59 / 0.63 / 0.71.
 template <int WF, int RT, int MODE, int NB>
 __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearArgs a) {
   constexpr bool LN = MODE == ACT_LN;
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
   //      (mean = (ma+mb)/2, M2 = M2a + M2b + (mb-ma)^2 * n/2), first by shuffles, then across the
   //      warps through shared memory: one block barrier, no cancellation.
   const int stride = ln_stage_stride(WF, KB * KT);   // staged columns: this CTA's k-range
-  constexpr int RPR = NB == 1 ? 1 : 4;  // rows per LayerNorm round (a one-row launch carries the code of one row only)
+  constexpr int RPR = kLnFuseMaxRows;   // rows per LayerNorm round
   if (LN) {
     float2 *lnred = reinterpret_cast<float2 *>(red);  // [warps][RPR] (mean, M2), reused later for the partial sums
     const int nw_used = (a.K / 4 + 31) / 32;           // warps that hold columns (K is a multiple of 128)
@@ -626,9 +626,8 @@ inline cudaError_t launch_linear_nb(const LinearArgs &a, int grid, cudaStream_t 
 
 template <int WF, int RT, int MODE>
 inline cudaError_t launch_linear_inst(const LinearArgs &a, int grid, cudaStream_t st, bool pdl) {
-  if (MODE != ACT_DIRECT) {  // batches of up to 4 rows always fit the staging buffer
+  if (MODE != ACT_DIRECT) {  // one row always fits the staging buffer
     if (a.B == 1) return launch_linear_nb<WF, RT, (MODE == ACT_DIRECT ? ACT_STAGED : MODE), 1>(a, grid, st, pdl);
-    if (a.B <= 4) return launch_linear_nb<WF, RT, (MODE == ACT_DIRECT ? ACT_STAGED : MODE), 4>(a, grid, st, pdl);
   }
   return launch_linear_nb<WF, RT, MODE, 0>(a, grid, st, pdl);
 }

@@ -93,7 +93,7 @@ struct tts_gpt {
   std::map<int, int> graph_nodes;
   bool use_graph;
   bool use_pdl;
-  bool use_fc2_ksplit = true;   // 5-16 rows: FC2 splits K (option "fc2_ksplit")
+  bool use_fc2_ksplit = true;   // 2-16 rows: FC2 splits K (option "fc2_ksplit")
   int pending_parts = 0;        // k-range partial sums of the last FC2 still to be folded into x
   size_t partials_floats = 0;
   bool use_tc = true;   // tensor-core path for more than 16 rows (option "tc")
@@ -527,7 +527,7 @@ int run_layers(tts_gpt *h, int R, bool decode) {
   cudaStream_t st = h->stream;
   const bool pdl = h->use_pdl;
   const bool fuse_ln = can_fuse_ln(c.wfmt, R, d);
-  // 5 to 16 rows: FC2 (K = d_ff) splits K over kSmallKSplit CTAs per row tile, so that a CTA stages a
+  // 2 to 16 rows: FC2 (K = d_ff) splits K over kSmallKSplit CTAs per row tile, so that a CTA stages a
   // quarter of the wide activation rows; its partial sums are folded into x by the next LayerNorm
   const int fc2_ks = (!fuse_ln && h->use_fc2_ksplit && (c.d_ff / k_per_tile(c.wfmt)) % kSmallKSplit == 0 &&
                       (size_t)kSmallKSplit * kMaxRows * d <= h->partials_floats) ? kSmallKSplit : 1;
