@@ -19,6 +19,7 @@
 #include "attention_prefill.cuh"
 #include "gemm_tc.cuh"
 #include "gemm_pw.cuh"
+#include "attention_decode.cuh"
 #include "attention_prefill_tc.cuh"
 #include "elementwise.cuh"
 #include "kv_pages.cuh"
@@ -78,6 +79,7 @@ struct tts_gpt {
   void *a_img = nullptr, *o_img = nullptr, *h_img = nullptr, *hf_img = nullptr;
   void *q_img = nullptr;             // q of prefill passes of more than 128 rows
   CUtensorMap a_map, o_map, h_map;   // the images as tensors (all row tiles of a pass)
+  CUtensorMap kv_map;                // the KV pool (all layers) as token rows: attention_decode_kernel
   CUtensorMap xrow_map, part_map;    // the residual stream and the partial sums as tensors of fp32 rows
   float *partials = nullptr;
   bool have_tc = false;
@@ -103,6 +105,7 @@ struct tts_gpt {
   int tc_tail_parts = 0;  // partial sums the last FC2 of the tensor-core path left for the final LayerNorm
   bool use_attn_mma = true;      // tensor-core attention in prefill passes (option "attn_mma")
   bool use_attn_prefill = true;  // shared-page attention in prefill passes (option "attn_prefill")
+  bool use_attn_decode = true;   // unit-split tensor-pipe attention of decode steps (option "attn_decode")
   bool use_attn_stream = true;   // streaming attention for large batches (option "attn_stream")
   int attn_cluster_fill = 1;     // clusters grow until the grid covers the GPU this many times
   int attn_stream_min_pairs = 0; // (row, head) pairs from which it is used; 0: attention_use_stream decides
@@ -367,6 +370,8 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
   if (!aa.old_pages_final && h->use_attn_mma && h->use_attn_tc && R > kMaxRows) return launch_attention_prefill_tc(aa, R, h->n_sm, st, pdl);
   if (!aa.old_pages_final && h->use_attn_mma && R >= kAttnPrefillRows) return launch_attention_prefill_mma(aa, R, st, pdl);
   if (!aa.old_pages_final && h->use_attn_prefill && R >= kAttnPrefillRows) return launch_attention_prefill(aa, R, st, pdl);
+  if (aa.old_pages_final && h->use_attn_decode && h->attn_stream_min_pairs == 0 && attention_use_decode(R, aa.H, h->n_sm))
+    return launch_attention_decode(aa, R, h->kv_map, (int)((aa.kv_layer - h->kv) / kHeadDim), h->n_sm, st, pdl);
   const bool stream = h->attn_stream_min_pairs > 0 ? R * aa.H >= h->attn_stream_min_pairs : attention_use_stream(R, aa.H, h->n_sm);
   if (h->use_attn_stream && stream) return launch_attention_stream(aa, R, st, pdl);
   return launch_attention(aa, R, attention_cluster_size(R, aa.H, h->n_sm, h->attn_cluster_fill), st, pdl);
@@ -732,6 +737,7 @@ int32_t tts_gpt_create(const tts_gpt_config_t *cfg, const tts_gpt_weights_t *w, 
     TRY_(image(&h->a_map, h->a_img, tiles * (d / 64)));
     TRY_(image(&h->o_map, h->o_img, tiles * (d / 64)));
     TRY_(image(&h->h_map, h->h_img, tiles * (c.d_ff / 64)));
+    if (!h->kv_fp8) TRY_([&]() -> int { CUDA_TRY(h, attention_decode_map(&h->kv_map, h->kv, h->kv_layer_elems * c.n_layer / kHeadDim)); return TTS_GPT_OK; }());
     TRY_(rows(&h->xrow_map, h->x, kMaxPassRows));
     TRY_(rows(&h->part_map, h->partials, (size_t)kMaxSplitTiles * kMaxRows));
     for (auto &L : h->layers)
@@ -1152,6 +1158,7 @@ int32_t tts_gpt_debug_set_option(tts_gpt_t *h, const char *name, int32_t value) 
   }
   else if (k == "attn_mma") h->use_attn_mma = on;
   else if (k == "attn_prefill") h->use_attn_prefill = on;
+  else if (k == "attn_decode") h->use_attn_decode = on;
   else if (k == "attn_stream") h->use_attn_stream = on;
   else if (k == "attn_stream_min_pairs") h->attn_stream_min_pairs = value > 0 ? value : 0;
   else if (k == "attn_cluster_fill") h->attn_cluster_fill = value > 0 ? value : 1;

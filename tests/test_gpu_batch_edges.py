@@ -1,0 +1,87 @@
+"""Sizes at which the kernels of middle decode batches and of the largest prefill passes can go wrong: 32-token units and
+pages that begin or end with the newest token, (row, head) pairs cut over warps, row tiles without rows, ragged tiles;
+each against the fp64 oracle on identical history."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import gpt_oracle as O
+from paper_2607_21042_b200 import binding as B
+from paper_2607_21042_b200 import cases as C
+from helpers import assert_logits_close, bits_dev, check_tokens
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _run(eng, prefixes, n_steps):
+    S, V = len(prefixes), eng.cfg.vocab
+    toks = torch.zeros((n_steps + 1, S), dtype=torch.int32, device=DEV)
+    logits = torch.zeros((n_steps + 1, S, V), dtype=torch.float32, device=DEV)
+    ids, _ = eng.prefill([bits_dev(p) for p in prefixes], out_tokens=toks[0], out_logits=logits[0])
+    for k in range(1, n_steps + 1):
+        eng.decode_step(ids, toks[k], out_logits=logits[k])
+    eng.sync()
+    for s in ids:
+        eng.release_stream(s)
+    return logits.cpu().numpy().transpose(1, 0, 2), toks.cpu().numpy().T
+
+
+def _check(model, prefixes, lg, tk, streams, what):
+    for s in streams:
+        ref, _ = O.replay_full(model, O.bf16_to_f64(prefixes[s]), tk[s][:-1])
+        assert_logits_close(lg[s], ref, "%s, stream %d" % (what, s))
+        check_tokens(tk[s], ref, 0, 1.0, None, "%s, stream %d" % (what, s))
+
+
+@pytest.mark.parametrize("S", [75, 100, 128])
+def test_unit_split_decode_attention(S):
+    """300, 400 and 512 (row, head) pairs on one CTA per SM: contexts that cross 32-token and page edges while they decode,
+    one long context among short ones, stale pages full of NaN behind every context."""
+    edges = [1, 30, 31, 32, 33, 62, 63, 64, 65, 95, 96, 127, 128, 700]
+    lens = [edges[i % len(edges)] if i < 28 else 2 + (11 * i) % 60 for i in range(S)]
+    cfg = C.tiny_config(max_streams=S, n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=768)
+    w = C.make_weights(cfg, seed=21)
+    model = O.OracleModel(cfg, w)
+    eng = B.TtsGpt(cfg, w, DEV)
+    eng.set_option("poison_free_pages", 1)
+    prefixes = C.make_prefixes(cfg, lens, seed=22)
+    lg, tk = _run(eng, prefixes, 4)
+    _check(model, prefixes, lg, tk, list(range(14)) + [S - 1], "unit-split attention")
+    lg2, _ = _run(eng, prefixes, 4)
+    assert np.array_equal(lg, lg2)
+    eng.set_option("attn_decode", 0)      # one CTA per pair
+    lg3, _ = _run(eng, prefixes, 4)
+    assert np.max(np.abs(lg3[:, :2] - lg[:, :2])) < 3e-2
+    eng.destroy()
+
+
+@pytest.mark.parametrize("wfmt", [C.W_BF16, C.W_INT8_PC, C.W_INT4_G128])
+@pytest.mark.parametrize("lens", [[1025], [700, 3, 450, 128, 1], [1279, 1281, 5, 31]])
+def test_prefill_passes_of_the_pair_kernel(wfmt, lens):
+    """Passes of more than 1024 rows: an odd number of row tiles (a pair whose second tile has no rows), tiles of one row,
+    streams that end inside a tile; then decode steps over the pages they wrote."""
+    S = len(lens)
+    cfg = C.tiny_config(wfmt=wfmt, max_streams=S, n_pages=S * 22, max_context=1408, max_pos=1408)
+    w = C.make_weights(cfg, seed=23)
+    model = O.OracleModel(cfg, w)
+    eng = B.TtsGpt(cfg, w, DEV)
+    prefixes = C.make_prefixes(cfg, lens, seed=24)
+    lg, tk = _run(eng, prefixes, 3)
+    _check(model, prefixes, lg, tk, range(S), "pair kernel")
+    assert eng.check_canaries() == 0
+    eng.destroy()
+
+
+def test_prefill_pair_kernel_with_the_8bit_cache_and_k_ranges():
+    """A model width at which the residual linears of a large pass take k-ranges, K/V rows through the staging array."""
+    cfg = C.tiny_config(d_model=512, n_head=8, d_ff=2048, kv_fmt=C.KV_FP8_E4M3, max_streams=2, n_pages=40, max_context=1216, max_pos=1216)
+    w = C.make_weights(cfg, seed=25)
+    prefixes = C.make_prefixes(cfg, [1100, 77], seed=26)
+    eng = B.TtsGpt(cfg, w, DEV)
+    lg, _ = _run(eng, prefixes, 2)
+    eng.set_option("prefill_pass_rows", 512)
+    lg2, _ = _run(eng, prefixes, 2)
+    assert np.max(np.abs(lg[:, 0] - lg2[:, 0])) < 4.5e-2
+    assert eng.check_canaries() == 0
+    eng.destroy()
