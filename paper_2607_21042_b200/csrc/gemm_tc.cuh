@@ -28,16 +28,10 @@
 
 namespace ttsgpt {
 
-// Measured on B200 (FC1 shape, 128 rows): chunks of 32 rows with a 5-stage ring (160 CTAs, two per
-// SM) beat chunks of 64 rows with 4 or 8 stages by 6-13 us per linear although the latter re-read
-// the weights from L2 only twice: more CTAs keep more copies in flight and overlap their epilogues.
-constexpr int kTcStages = 4;            // even: a stage is always consumed by the same MMA issuer (see the issuers); 4 x 20 KB
+constexpr int kTcStages = 4, kTcMaxStages = 8;   // ring depth where CTAs share an SM / where a CTA has it to itself
 constexpr int kTcTileM = 128;          // weight rows per CTA
-constexpr int kTcChunkN = 32;          // batch rows per CTA (the N operand; weights are re-read once per chunk)
 constexpr int kTcKChunk = 64;          // columns per pipeline stage (128 bytes of bf16)
 constexpr uint32_t kTcABytes = kTcTileM * 128;   // 16 KB
-constexpr uint32_t kTcBBytes = kTcChunkN * 128;  // 4 KB
-static_assert(kTcChunkN == 32, "the epilogue reads one 32-column accumulator slice per thread");
 constexpr int kTcThreads = 352;          // warp 0: producer, warp 1: MMA issuer, warps 2-9: epilogue
 constexpr int kTcEpiThreads = 256;
 constexpr int kTcEpiCols = 16;           // accumulator columns (batch rows) per epilogue thread: two warps share a lane quarter
@@ -308,20 +302,24 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 // tensor-memory buffers; while the next group runs in the other buffer, the epilogue warps read the
 // finished group out, multiply it by the group's scale of their weight row and add it to fp32
 // registers.  Otherwise one 32-column accumulator collects the whole k-range.
-template <bool GROUPED>
+// CN: batch rows per CTA (the N operand), 32 or 64.
+template <bool GROUPED, int CN>
 __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a) {
+  static_assert(CN == 32 || !GROUPED, "the group buffers hold 32 columns");
+  constexpr uint32_t kStage = kTcABytes + CN * 128;   // a stage: 128 weight rows | CN batch rows
+  const int n_stage = a.stages;                       // even: a stage is always consumed by the same issuer
   extern __shared__ __align__(16) unsigned char tc_smem_raw[];
-  // [stages x (A 16 KB | B 4 KB)] on a 1024-byte boundary (the swizzle pattern repeats every 1024
+  // [stages x (A 16 KB | B CN x 128 bytes)] on a 1024-byte boundary (the swizzle pattern repeats every 1024
   // bytes of shared-memory address), then barriers and small state
   unsigned char *ring = tc_smem_raw + ((1024u - (smem_u32(tc_smem_raw) & 1023u)) & 1023u);
-  uint64_t *full = reinterpret_cast<uint64_t *>(ring + kTcStages * (kTcABytes + kTcBBytes));
-  uint64_t *empty = full + kTcStages;
-  uint64_t *acc_done = empty + kTcStages;
+  uint64_t *full = reinterpret_cast<uint64_t *>(ring + n_stage * kStage);
+  uint64_t *empty = full + kTcMaxStages;
+  uint64_t *acc_done = empty + kTcMaxStages;
   uint64_t *grp_done = acc_done + 1;   // [2] group buffer filled (MMA warp -> all)
   uint64_t *grp_free = grp_done + 2;   // [2] group buffer read out (all epilogue threads -> MMA warp)
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(grp_free + 2);
   volatile int *failed = reinterpret_cast<volatile int *>(tmem_slot + 1);
-  uint16_t **kv_base = reinterpret_cast<uint16_t **>(tmem_slot + 4);   // [32] EPI_QKV: page slot of each batch row
+  uint16_t **kv_base = reinterpret_cast<uint16_t **>(tmem_slot + 4);   // [CN] EPI_QKV: page slot of each batch row
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nt = blockIdx.x, bc = blockIdx.y, ks = blockIdx.z;
@@ -333,16 +331,16 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
   const int n_it = kc1 - kc0;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kTcStages; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, 1); }
+    for (int s = 0; s < n_stage; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, 1); }
     mbar_init(acc_done, GROUPED ? 1 : 2);   // both MMA issuers commit to it
     mbar_init(grp_done, 1); mbar_init(grp_done + 1, 1);
     mbar_init(grp_free, kTcEpiThreads); mbar_init(grp_free + 1, kTcEpiThreads);
     *failed = 0;
   }
-  if (warp == 0) tmem_alloc(tmem_slot, 2 * kTcChunkN);
-  if (a.mode == EPI_QKV && threadIdx.x >= 64 && threadIdx.x < 64 + kTcChunkN) {   // page slots of this chunk's batch rows
+  if (warp == 0) tmem_alloc(tmem_slot, 2 * CN);
+  if (a.mode == EPI_QKV && threadIdx.x >= 64 && threadIdx.x < 64 + CN) {   // page slots of this chunk's batch rows
     const int bl = threadIdx.x - 64;
-    const int b = bc * kTcChunkN + bl;
+    const int b = bc * CN + bl;
     uint16_t *p = nullptr;
     if (b < a.B) {
       if (a.kv_stage) {
@@ -361,13 +359,13 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
   const uint32_t tmem_d = *tmem_slot;
 
   const unsigned char *gA = reinterpret_cast<const unsigned char *>(a.w_img) + ((size_t)nt * KC + kc0) * kTcABytes;
-  const unsigned char *gB = reinterpret_cast<const unsigned char *>(a.act_img) + (size_t)kc0 * (kMaxRows * 128) + (size_t)bc * kTcBBytes;
+  const unsigned char *gB = reinterpret_cast<const unsigned char *>(a.act_img) + (size_t)kc0 * (kMaxRows * 128) + (size_t)bc * (CN * 128);
 
-  const int pre = min(n_it, kTcStages);
+  const int pre = min(n_it, n_stage);
   if (threadIdx.x == 0) {
     for (int i = 0; i < pre; ++i) {   // weights do not depend on the previous kernel
-      mbar_expect_tx(full + i, kTcABytes + kTcBBytes);
-      bulk_copy_g2s(ring + (size_t)i * (kTcABytes + kTcBBytes), gA + (size_t)i * kTcABytes, kTcABytes, full + i);
+      mbar_expect_tx(full + i, kStage);
+      bulk_copy_g2s(ring + (size_t)i * kStage, gA + (size_t)i * kTcABytes, kTcABytes, full + i);
     }
   }
   // per-row epilogue constants do not depend on the kernel in front either
@@ -385,16 +383,18 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
   if (warp == 0) {
     // ---- producer ----
     for (int i = 0; i < pre; ++i)
-      if (elect_one()) bulk_copy_g2s(ring + (size_t)i * (kTcABytes + kTcBBytes) + kTcABytes, gB + (size_t)i * (kMaxRows * 128), kTcBBytes, full + i);
-    for (int i = pre; i < n_it; ++i) {
-      const int s = i % kTcStages;
-      tc_wait(empty + s, ((i / kTcStages) - 1) & 1, failed, a.err);
+      if (elect_one()) bulk_copy_g2s(ring + (size_t)i * kStage + kTcABytes, gB + (size_t)i * (kMaxRows * 128), CN * 128, full + i);
+    int s = 0;
+    uint32_t parity = 0;
+    for (int i = pre; i < n_it; ++i) {   // pre == n_stage here
+      tc_wait(empty + s, parity, failed, a.err);
       if (elect_one()) {
-        mbar_expect_tx(full + s, kTcABytes + kTcBBytes);
-        bulk_copy_g2s(ring + (size_t)s * (kTcABytes + kTcBBytes), gA + (size_t)i * kTcABytes, kTcABytes, full + s);
-        bulk_copy_g2s(ring + (size_t)s * (kTcABytes + kTcBBytes) + kTcABytes, gB + (size_t)i * (kMaxRows * 128), kTcBBytes, full + s);
+        mbar_expect_tx(full + s, kStage);
+        bulk_copy_g2s(ring + (size_t)s * kStage, gA + (size_t)i * kTcABytes, kTcABytes, full + s);
+        bulk_copy_g2s(ring + (size_t)s * kStage + kTcABytes, gB + (size_t)i * (kMaxRows * 128), CN * 128, full + s);
       }
       __syncwarp();
+      if (++s == n_stage) { s = 0; parity ^= 1u; }
     }
     trace_mark(a.trace, a.trace_slot, 3);   // last copy issued
     __syncwarp();   // the warp arrives at the final barrier as a whole
@@ -410,16 +410,17 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
     const int par = GROUPED ? 0 : (warp == 10 ? 1 : 0);
     const int stride = GROUPED ? 1 : 2;
     if (!(GROUPED && warp == 10)) {
-      const uint32_t idesc = tc_instr_desc(kTcTileM, kTcChunkN);
+      const uint32_t idesc = tc_instr_desc(kTcTileM, CN);
+      int s = par;
+      uint32_t parity = 0;
       for (int i = par; i < n_it; i += stride) {
-        const int s = i % kTcStages;
-        tc_wait(full + s, (i / kTcStages) & 1, failed, a.err);
+        tc_wait(full + s, parity, failed, a.err);
         const int g = i >> 1;   // group of this k-chunk inside the k-range
         if (GROUPED && (i & 1) == 0 && g >= 2) tc_wait(grp_free + (g & 1), ((g >> 1) - 1) & 1, failed, a.err);
         tc_fence_after_sync();
-        const unsigned char *sa = ring + (size_t)s * (kTcABytes + kTcBBytes);
+        const unsigned char *sa = ring + (size_t)s * kStage;
         const uint64_t da = tc_smem_desc(sa), db = tc_smem_desc(sa + kTcABytes);
-        const uint32_t dst = GROUPED ? tmem_d + (uint32_t)(g & 1) * kTcChunkN : tmem_d + (uint32_t)par * kTcChunkN;
+        const uint32_t dst = GROUPED ? tmem_d + (uint32_t)(g & 1) * 32u : tmem_d + (uint32_t)par * CN;
         if (elect_one()) {
 #pragma unroll
           for (int j = 0; j < kTcKChunk / 16; ++j) {  // 32 bytes further along K per step: +2 in 16-byte units
@@ -431,6 +432,7 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
           if (!GROUPED && i + stride >= n_it) tc_commit(acc_done);
         }
         __syncwarp();
+        if ((s += stride) >= n_stage) { s -= n_stage; parity ^= 1u; }
       }
       if (!GROUPED && par >= n_it && elect_one()) tc_commit(acc_done);   // nothing issued: the barrier still counts this warp
     }
@@ -441,8 +443,16 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
   //      rows n; columns = batch rows ----
   if (warp >= 2 && warp < 10) {
   const int lw = warp & 3;
-  const int c0 = ((warp - 2) >> 2) * kTcEpiCols;   // this thread's first accumulator column
   const int n = nt * kTcTileM + lw * 32 + lane;
+  if (!GROUPED) {
+    tc_wait(acc_done, 0, failed, a.err);
+    trace_mark(a.trace, a.trace_slot, 4, 64);   // accumulator complete
+    tc_fence_after_sync();
+    __syncwarp();
+  }
+#pragma unroll 1   // 32 columns a turn, 16 per warp: the code of one turn is fetched once
+  for (int turn = 0; turn < CN / 32; ++turn) {
+  const int c0 = 32 * turn + ((warp - 2) >> 2) * kTcEpiCols;   // this thread's first accumulator column
   float v[kTcEpiCols];
   if (GROUPED) {
 #pragma unroll
@@ -464,14 +474,10 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
       for (int c = 0; c < kTcEpiCols; ++c) v[c] = fmaf(sc, t[c], v[c]);
     }
   } else {
-    tc_wait(acc_done, 0, failed, a.err);
-    trace_mark(a.trace, a.trace_slot, 4, 64);   // accumulator complete
-    tc_fence_after_sync();
-    __syncwarp();
     tmem_ld16(tmem_d + ((uint32_t)(lw * 32) << 16) + (uint32_t)c0, v);
     if (n_it >= 2) {   // the odd k-chunks' accumulator
       float t2[kTcEpiCols];
-      tmem_ld16(tmem_d + ((uint32_t)(lw * 32) << 16) + (uint32_t)kTcChunkN + (uint32_t)c0, t2);
+      tmem_ld16(tmem_d + ((uint32_t)(lw * 32) << 16) + (uint32_t)CN + (uint32_t)c0, t2);
 #pragma unroll
       for (int c = 0; c < kTcEpiCols; ++c) v[c] += t2[c];
     }
@@ -481,10 +487,10 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
 #pragma unroll
     for (int c = 0; c < kTcEpiCols; ++c) v[c] = 0.f;
   }
-  if (n < a.N && !*failed) {
+  if (n < a.N && bc * CN + c0 < a.B && !*failed) {
     // one straight-line store loop per destination kind: a single loop that branches on the epilogue
     // mode for every batch row compiled into code whose speed varied 2-4x with unrelated edits
-    const int nb = min(kTcEpiCols, a.B - bc * kTcChunkN - c0);   // real batch rows among this thread's columns
+    const int nb = min(kTcEpiCols, a.B - bc * CN - c0);   // real batch rows among this thread's columns
 #pragma unroll
     for (int c = 0; c < kTcEpiCols; ++c) v[c] = fmaf(v[c], e_rsc, e_bias);   // int8: per-row scale (1 otherwise), then bias
     if (a.mode == EPI_GELU) {
@@ -501,7 +507,7 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
       const int u = (n & 63) >> 3;
 #pragma unroll
       for (int c = 0; c < kTcEpiCols; ++c) {
-        const int b = bc * kTcChunkN + c0 + c;
+        const int b = bc * CN + c0 + c;
         if (c < nb) *reinterpret_cast<uint16_t *>(img + (size_t)b * 128 + (size_t)((u ^ (b & 7)) << 4)) = float_to_bf16_bits(v[c]);
       }
     } else if (a.mode == EPI_QKV && n >= a.d) {
@@ -514,8 +520,8 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
     } else {
       // fp32 rows: logits, q, the residual stream, or this k-range's partial sums
       const bool partial = a.mode == EPI_RESID && a.ksplit > 1;
-      float *dst = partial ? a.out_f32 + ((size_t)ks * kMaxRows + bc * kTcChunkN + c0) * a.N + n
-                           : a.out_f32 + (size_t)(bc * kTcChunkN + c0) * a.out_stride + n;
+      float *dst = partial ? a.out_f32 + ((size_t)ks * kMaxRows + bc * CN + c0) * a.N + n
+                           : a.out_f32 + (size_t)(bc * CN + c0) * a.out_stride + n;
       const size_t step = partial ? (size_t)a.N : (size_t)a.out_stride;
       if (a.mode == EPI_RESID && !partial) {
 #pragma unroll
@@ -528,12 +534,14 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
       }
     }
   }
+  __syncwarp();   // the next turn reads tensor memory as a warp
+  }
   trace_mark(a.trace, a.trace_slot, 6, 64);     // this thread's epilogue done
   }
   tc_fence_before_sync();
   __syncthreads();
   trace_mark(a.trace, a.trace_slot, 2, 64);   // by an epilogue thread: its own stores precede the mark
-  if (warp == 0) tmem_dealloc(tmem_d, 2 * kTcChunkN);
+  if (warp == 0) tmem_dealloc(tmem_d, 2 * CN);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -887,18 +895,26 @@ __global__ void fold_partials_kernel(const float *__restrict__ part, int n_part,
   out[i] = v;
 }
 
-inline size_t gemm_tc_smem_bytes() { return (size_t)kTcStages * (kTcABytes + kTcBBytes) + 1024 + 512; }
+inline size_t gemm_tc_smem_bytes(int cn, int stages) { return (size_t)stages * (kTcABytes + cn * 128) + 1024 + 1024; }
 
-inline cudaError_t launch_gemm_tc(const GemmTcArgs &a, cudaStream_t st, bool pdl) {
+template <bool GROUPED, int CN>
+inline cudaError_t launch_gemm_tc_as(GemmTcArgs a, int stages, cudaStream_t st, bool pdl) {
   static PerDeviceOnce attr_once;   // per device: opt-in to more than 48 KB of dynamic shared memory
-  if (attr_once.first()) {
-    cudaFuncSetAttribute(gemm_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_tc_smem_bytes());
-    cudaFuncSetAttribute(gemm_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_tc_smem_bytes());
-  }
-  dim3 grid((a.N + kTcTileM - 1) / kTcTileM, (a.B + kTcChunkN - 1) / kTcChunkN, a.ksplit);
-  if (a.wfmt == WF_INT4)
-    return launch_kernel(gemm_tc_kernel<true>, grid, dim3(kTcThreads), gemm_tc_smem_bytes(), st, pdl, a);
-  return launch_kernel(gemm_tc_kernel<false>, grid, dim3(kTcThreads), gemm_tc_smem_bytes(), st, pdl, a);
+  if (attr_once.first())
+    cudaFuncSetAttribute(gemm_tc_kernel<GROUPED, CN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_tc_smem_bytes(CN, kTcMaxStages));
+  a.stages = stages;
+  dim3 grid((a.N + kTcTileM - 1) / kTcTileM, (a.B + CN - 1) / CN, a.ksplit);
+  return launch_kernel(gemm_tc_kernel<GROUPED, CN>, grid, dim3(kTcThreads), gemm_tc_smem_bytes(CN, stages), st, pdl, a);
+}
+
+// n_sm: SMs of the device.  With chunks of 32 batch rows a linear of more than 64 rows has more CTAs than SMs, which share
+// an SM, its bandwidth from L2 (20 KB per k-chunk and CTA, the weights four times over) and a ring of half the depth;
+// chunks of 64 rows leave one CTA per SM with eight stages in flight.
+inline cudaError_t launch_gemm_tc(const GemmTcArgs &a, int n_sm, cudaStream_t st, bool pdl) {
+  if (a.wfmt == WF_INT4) return launch_gemm_tc_as<true, 32>(a, kTcStages, st, pdl);
+  const int tiles = (a.N + kTcTileM - 1) / kTcTileM * a.ksplit;
+  if (tiles * ((a.B + 31) / 32) <= n_sm) return launch_gemm_tc_as<false, 32>(a, kTcMaxStages, st, pdl);
+  return launch_gemm_tc_as<false, 64>(a, tiles * ((a.B + 63) / 64) <= n_sm ? kTcMaxStages : kTcStages, st, pdl);
 }
 
 }  // namespace ttsgpt

@@ -427,7 +427,7 @@ constexpr int kPairMinRows = 1024;
 bool use_pairs(const tts_gpt *h, int R) { return R > kPairMinRows && !(h->cfg.wfmt == WF_INT4 && h->w4_exact); }
 
 int launch_gemm(tts_gpt *h, const GemmTcArgs &a, const CUtensorMap &w_map, const CUtensorMap &x_map, bool wide, cudaStream_t st, bool pdl) {
-  if (!wide) CUDA_TRY(h, launch_gemm_tc(a, st, pdl));
+  if (!wide) CUDA_TRY(h, launch_gemm_tc(a, h->n_sm, st, pdl));
   else if (!use_pairs(h, a.B)) CUDA_TRY(h, launch_gemm_tcw(a, h->n_sm, st, pdl));
   else {
     const CUtensorMap *out = a.mode != EPI_RESID ? nullptr : a.ksplit > 1 ? &h->part_map : &h->xrow_map;
@@ -504,7 +504,7 @@ int run_head_tc(tts_gpt *h, int n_out) {
   if (big) {
     GemmTcArgs ha = gemm_args(h, h->head, h->hf_img, n_out, EPI_F32, 1);
     ha.out_f32 = h->logits; ha.out_stride = c.vocab;
-    CUDA_TRY(h, launch_gemm_tc(ha, st, pdl));
+    CUDA_TRY(h, launch_gemm_tc(ha, h->n_sm, st, pdl));
   } else {
     LinearArgs ha = linear_args(h, h->head, h->hf, n_out, EPI_F32);
     ha.out_f32 = h->logits; ha.out_stride = c.vocab;
@@ -1288,10 +1288,10 @@ int32_t tts_gpt_op_linear_tc(int32_t wfmt, int32_t N, int32_t K, const void *w, 
   a.w_img = wimg; a.act_img = aimg; a.N = N; a.K = K; a.B = B; a.ksplit = ksplit; a.wfmt = wfmt; a.scales = tiled_s;
   if (ksplit == 1) {
     a.mode = EPI_F32; a.bias = (const uint16_t *)bias; a.out_f32 = out; a.out_stride = N;
-    CUDA_TRY(nullptr, wide ? launch_wide(a, st) : launch_gemm_tc(a, st, false));
+    CUDA_TRY(nullptr, wide ? launch_wide(a, st) : launch_gemm_tc(a, 148, st, false));
   } else {   // partial sums per k-range, then folded in range order (what the following LayerNorm does in the engine)
     a.mode = EPI_RESID; a.out_f32 = part; a.out_stride = N;
-    CUDA_TRY(nullptr, wide ? launch_wide(a, st) : launch_gemm_tc(a, st, false));
+    CUDA_TRY(nullptr, wide ? launch_wide(a, st) : launch_gemm_tc(a, 148, st, false));
     fold_partials_kernel<<<(unsigned)(((size_t)B * N + 255) / 256), 256, 0, st>>>(part, ksplit, B, N, (const uint16_t *)bias, out);
     CUDA_TRY(nullptr, cudaGetLastError());
   }
