@@ -11,7 +11,7 @@
 // registers (exact) and the bf16 scale multiplies the fp32 partial sums (per row for int8, per row
 // and 128-column group for int4).
 //
-// A CTA owns 1, 2 or 4 adjacent 8-row tiles (one contiguous block of the streaming layout) and
+// A CTA owns 1 to 4 adjacent 8-row tiles (one contiguous block of the streaming layout) and
 // splits K over its 10 warps.  Its very first action is one bulk asynchronous copy (TMA, untiled,
 // completion on an mbarrier) of that whole block into shared memory: weights do not depend on the
 // previous kernel, so under programmatic dependent launch the copy overlaps the predecessor's
@@ -228,6 +228,7 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
   }
 
   // ---- everything else that no kernel of the step writes: LN gamma/beta, bias, scales, KV slots ----
+  constexpr int EPT = kLinearThreads / C * C;   // threads of the epilogue: a whole number of batch rows per round
   const int ecol = threadIdx.x % C;             // this thread's output column in every epilogue round
   const int en = tile0 * 8 + ecol;              // = output feature n
   float e_bias = 0.f, e_scale = 1.f;
@@ -237,12 +238,12 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
   }
   // EPI_QKV: where this thread's K/V outputs go (row table and page table are final before the
   // first kernel of the step starts); batches above 16 rows look the slot up in the epilogue
-  constexpr int ER = (16 * C + kLinearThreads - 1) / kLinearThreads;  // epilogue rounds
+  constexpr int ER = (16 * C + EPT - 1) / EPT;  // epilogue rounds
   uint16_t *kv_dst[ER];
 #pragma unroll
   for (int e = 0; e < ER; ++e) {
     kv_dst[e] = nullptr;
-    const int b = (threadIdx.x + e * kLinearThreads) / C;
+    const int b = (threadIdx.x + e * EPT) / C;
     if (a.mode == EPI_QKV && en >= a.d && en < a.N && b < a.B && b < 16) {
       const int which = en >= 2 * a.d;  // 0 = K, 1 = V
       const int col = en - (which ? 2 * a.d : a.d);
@@ -373,7 +374,7 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
 #pragma unroll
     for (int e = 0; e < ER; ++e) {
       e_old[e] = 0.f;
-      const int o = threadIdx.x + e * kLinearThreads;
+      const int o = threadIdx.x < EPT ? threadIdx.x + e * EPT : 16 * C;
       const int b = m0 + o / C;
       if (a.mode == EPI_RESID && gridDim.y == 1 && o < 16 * C && b < a.B && en < a.N) e_old[e] = a.out_f32[(size_t)b * a.out_stride + en];
     }
@@ -544,7 +545,7 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
     trace_mark(a.trace, a.trace_slot, 5);
 #pragma unroll
     for (int e = 0; e < ER; ++e) {
-      const int o = threadIdx.x + e * kLinearThreads;
+      const int o = threadIdx.x < EPT ? threadIdx.x + e * EPT : 16 * C;
       const int bl = o / C;
       const int n = en, b = m0 + bl;
       if (o < 16 * C && n < a.N && b < a.B) {
@@ -605,10 +606,12 @@ struct LinearPlan { int rt, grid; };
 inline LinearPlan plan_linear(int wf, int N, int K, int B, int mode, int max_ctas) {   // K, max_ctas: per k-range
   const int tiles = row_tiles(N);
   LinearPlan p;
+  // The fewest tiles per CTA with which one wave takes the launch: a second wave starts its copies late (bf16 FC1 at
+  // 8 rows on two tiles per CTA, 320 CTAs for 296 places: 5.9 us; on three: 3.75 us).  One row of bf16 weights doubles
+  // instead: what it waits for is its copies, and four tiles in one copy are the faster (a step 0.468 ms, on three 0.476).
   p.rt = 1;
-  while (p.rt < 4 && (tiles + p.rt - 1) / p.rt > max_ctas &&
-         linear_smem_bytes(wf, p.rt * 2, mode, B, K) <= (size_t)kLinearSmemBudget)
-    p.rt *= 2;
+  for (int rt = 2; rt <= 4 && (tiles + p.rt - 1) / p.rt > max_ctas && linear_smem_bytes(wf, rt, mode, B, K) <= (size_t)kLinearSmemBudget; ++rt)
+    if (rt != 3 || B > 1 || wf != WF_BF16) p.rt = rt;
   p.grid = (tiles + p.rt - 1) / p.rt;
   return p;
 }
@@ -639,6 +642,7 @@ inline cudaError_t launch_linear_wf(const LinearArgs &a, int max_ctas, cudaStrea
   if (linear_smem_bytes(WF, p.rt, MODE, a.B, a.K / ks) > 200 * 1024) return cudaErrorInvalidValue;
   if (p.rt == 1) return launch_linear_inst<WF, 1, MODE>(a, p.grid, st, pdl);
   if (p.rt == 2) return launch_linear_inst<WF, 2, MODE>(a, p.grid, st, pdl);
+  if (p.rt == 3) return launch_linear_inst<WF, 3, MODE>(a, p.grid, st, pdl);
   return launch_linear_inst<WF, 4, MODE>(a, p.grid, st, pdl);
 }
 
