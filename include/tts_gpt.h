@@ -145,7 +145,9 @@ int32_t tts_gpt_prefill_tokens(tts_gpt_t *h, int32_t n, const void *const *cond_
  * step, appends that token's K/V at position ctx_i, attends over ctx_i + 1 keys, and returns the
  * logits of the next token, the sampled next token and optionally the final-LayerNorm hidden row.
  * top_k 0 or 1 = greedy (lowest index on ties); top_k in 2..64 = softmax over the top_k logits
- * at `temperature`, inverse CDF with uniforms[i].  Afterwards ctx_i += 1.
+ * at `temperature`, inverse CDF with uniforms[i].  Sampled calls (prefill and decode, top_k > 1) form
+ * their sums in one fixed order, so that the same uniforms give the same tokens; greedy calls may take
+ * faster kernels with another order of sums.  Afterwards ctx_i += 1.
  * Errors: E_ARG, E_STREAM (unknown / duplicate id), E_CTX_OVERFLOW (ctx_i + 1 > max_context),
  * E_NO_PAGES.  All-or-nothing; nothing is enqueued on error. */
 int32_t tts_gpt_decode_step(tts_gpt_t *h, int32_t n, const int32_t *stream_ids,

@@ -34,6 +34,7 @@ constexpr int kLinearThreads = kLinearWarps * 32;
 constexpr int kSmallKSplit = 4;     // k-ranges of FC2 between 5 and 16 rows (partial sums folded by the next LayerNorm)
 constexpr int kLnFuseMaxRows = 1;   // LayerNorm is fused into the linear up to this batch: every CTA repeats it, which
                                     // beats a separate launch for a single row only
+constexpr int kLnFuseMaxRowsOrdered = 4;   // the same for launches that keep the order of sums of the FMA path
 
 __host__ __device__ inline int k_per_tile(int wf) { return wf == WF_BF16 ? 32 : (wf == WF_INT8 ? 64 : 128); }
 __host__ __device__ inline int row_tiles(int N) { return (N + 7) / 8; }
@@ -127,7 +128,8 @@ struct LinearArgs {
   const uint16_t *bias;   // bf16 [N] or null
   const uint16_t *act;    // bf16 [B][K]  (unused when ln_x is set)
   int N, K, B, mode;
-  // fused LayerNorm in front (B <= kLnFuseMaxRows, K <= kLnFuseMaxK): act = LN(ln_x[gather[b]])
+  int ordered;           // 1: up to 4 rows take the FMA path (a fixed order of sums)
+  // fused LayerNorm in front (see can_fuse_ln): act = LN(ln_x[gather[b]])
   const float *ln_x;      // fp32 [*][K] or null
   const uint16_t *ln_g, *ln_b;
   float ln_eps;
@@ -176,10 +178,11 @@ enum { ACT_DIRECT = 0, ACT_STAGED = 1, ACT_LN = 2 };
 constexpr int kStageMaxBytes = 44 * 1024;
 constexpr int kLinearSmemBudget = 108 * 1024;  // per CTA, so that two CTAs share an SM
 
-// NB: 0 = tensor-pipe path (any batch, 16 rows per m-tile); 1 = CUDA-core path for a single row, whose fp32 FMAs
-// on the widened weights are cheaper than MMAs that are fifteen sixteenths padding.  From two rows on the MMAs win:
-// the FMA path with LayerNorm fused in took 0.77 / 0.90 / 1.04 ms per step at 2 / 3 / 4 rows (bf16, context 530),
-// MMAs behind LayerNorm kernels of their own 0.59 / 0.63 / 0.71.
+// NB: 0 = tensor-pipe path (any batch, 16 rows per m-tile); 1 or 4 = CUDA-core path for at most NB rows.  The fp32 FMAs
+// on the widened weights are cheaper for a single row, where MMAs are fifteen sixteenths padding.  From two rows on the
+// MMAs win: FMAs with LayerNorm fused in took 0.77 / 0.90 / 1.04 ms per step at 2 / 3 / 4 rows (bf16, context 530),
+// MMAs behind LayerNorm kernels of their own 0.59 / 0.63 / 0.71.  FMAs remain up to 4 rows where LinearArgs::ordered asks
+// for their order of sums.
 template <int WF, int RT, int MODE, int NB>
 __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearArgs a) {
   constexpr bool LN = MODE == ACT_LN;
@@ -273,7 +276,7 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
   //      (mean = (ma+mb)/2, M2 = M2a + M2b + (mb-ma)^2 * n/2), first by shuffles, then across the
   //      warps through shared memory: one block barrier, no cancellation.
   const int stride = ln_stage_stride(WF, KB * KT);   // staged columns: this CTA's k-range
-  constexpr int RPR = kLnFuseMaxRows;   // rows per LayerNorm round
+  constexpr int RPR = NB == 1 ? 1 : kLnFuseMaxRowsOrdered;   // rows per LayerNorm round (a one-row launch carries the code of one row only)
   if (LN) {
     float2 *lnred = reinterpret_cast<float2 *>(red);  // [warps][RPR] (mean, M2), reused later for the partial sums
     const int nw_used = (a.K / 4 + 31) / 32;           // warps that hold columns (K is a multiple of 128)
@@ -629,8 +632,10 @@ inline cudaError_t launch_linear_nb(const LinearArgs &a, int grid, cudaStream_t 
 
 template <int WF, int RT, int MODE>
 inline cudaError_t launch_linear_inst(const LinearArgs &a, int grid, cudaStream_t st, bool pdl) {
-  if (MODE != ACT_DIRECT) {  // one row always fits the staging buffer
-    if (a.B == 1) return launch_linear_nb<WF, RT, (MODE == ACT_DIRECT ? ACT_STAGED : MODE), 1>(a, grid, st, pdl);
+  if (MODE != ACT_DIRECT) {  // batches of up to 4 rows always fit the staging buffer
+    constexpr int M = MODE == ACT_DIRECT ? ACT_STAGED : MODE;
+    if (a.B == 1) return launch_linear_nb<WF, RT, M, 1>(a, grid, st, pdl);
+    if (a.ordered && a.B <= kLnFuseMaxRowsOrdered) return launch_linear_nb<WF, RT, M, 4>(a, grid, st, pdl);
   }
   return launch_linear_nb<WF, RT, MODE, 0>(a, grid, st, pdl);
 }
@@ -647,9 +652,8 @@ inline cudaError_t launch_linear_wf(const LinearArgs &a, int max_ctas, cudaStrea
 }
 
 // Whether LayerNorm can be fused in front of a linear with this shape (one float4 of the row per thread).
-inline bool can_fuse_ln(int wf, int B, int K) {
-  (void)wf;
-  return B <= kLnFuseMaxRows && K <= 4 * kLinearThreads;
+inline bool can_fuse_ln(int B, int K, bool ordered) {
+  return B <= (ordered ? kLnFuseMaxRowsOrdered : kLnFuseMaxRows) && K <= 4 * kLinearThreads;
 }
 
 template <int WF>
@@ -662,7 +666,7 @@ inline cudaError_t launch_linear_mode(const LinearArgs &a, int max_ctas, cudaStr
 
 // K must be a multiple of 128.
 inline cudaError_t launch_linear(int wf, const LinearArgs &a, cudaStream_t st, bool pdl = false, int max_ctas = 296) {
-  if (a.ln_x && !can_fuse_ln(wf, a.B, a.K)) return cudaErrorInvalidValue;
+  if (a.ln_x && !can_fuse_ln(a.B, a.K, a.ordered)) return cudaErrorInvalidValue;
   if (a.ksplit > 1 && (a.ln_x || a.mode != EPI_RESID || (a.K / k_per_tile(wf)) % a.ksplit != 0)) return cudaErrorInvalidValue;
   if (wf == WF_BF16) return launch_linear_mode<WF_BF16>(a, max_ctas, st, pdl);
   if (wf == WF_INT8) return launch_linear_mode<WF_INT8>(a, max_ctas, st, pdl);

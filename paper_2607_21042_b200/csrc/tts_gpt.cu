@@ -90,7 +90,7 @@ struct tts_gpt {
   std::vector<char> open;
   std::vector<int> ctx, pos_next;
   int n_free;
-  // step graphs by row count
+  // step graphs by row count, those of sampled steps under its negative
   std::map<int, cudaGraphExec_t> graphs;
   std::map<int, int> graph_nodes;
   bool use_graph;
@@ -105,6 +105,13 @@ struct tts_gpt {
   int tc_tail_parts = 0;  // partial sums the last FC2 of the tensor-core path left for the final LayerNorm
   bool use_attn_mma = true;      // tensor-core attention in prefill passes (option "attn_mma")
   bool use_attn_prefill = true;  // shared-page attention in prefill passes (option "attn_prefill")
+  // Sampled calls (top_k > 1) keep one order of sums: the FMA linears up to 4 rows, prefill passes of `ordered_pass_rows`,
+  // the CUDA-core decode attention.  A sampled token hangs on the last bits of its logits (neighbours in the tail of the
+  // distribution lie closer than bf16 rounding moves them, and the token feeds every later step), so a caller who replays
+  // a sequence of uniforms gets the same utterance only if the sums run in the same order.  Greedy calls are free of that
+  // and take the faster kernels.
+  bool ordered = false;          // set by each prefill and decode call
+  int ordered_pass_rows = 896;
   bool use_attn_decode = true;   // unit-split tensor-pipe attention of decode steps (option "attn_decode")
   bool use_attn_stream = true;   // streaming attention for large batches (option "attn_stream")
   int attn_cluster_fill = 1;     // clusters grow until the grid covers the GPU this many times
@@ -320,6 +327,7 @@ LinearArgs linear_args(tts_gpt *h, const PackedLinear &pl, const uint16_t *act, 
 LinearArgs linear_args(tts_gpt *h, const PackedLinear &pl, const uint16_t *act, int B, int mode) {
   LinearArgs a = linear_args(pl, act, B, mode);
   a.err = h->dev_err;
+  a.ordered = h->ordered ? 1 : 0;
   return a;
 }
 
@@ -370,7 +378,7 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
   if (!aa.old_pages_final && h->use_attn_mma && h->use_attn_tc && R > kMaxRows) return launch_attention_prefill_tc(aa, R, h->n_sm, st, pdl);
   if (!aa.old_pages_final && h->use_attn_mma && R >= kAttnPrefillRows) return launch_attention_prefill_mma(aa, R, st, pdl);
   if (!aa.old_pages_final && h->use_attn_prefill && R >= kAttnPrefillRows) return launch_attention_prefill(aa, R, st, pdl);
-  if (aa.old_pages_final && h->use_attn_decode && h->attn_stream_min_pairs == 0 && attention_use_decode(R, aa.H, h->n_sm))
+  if (aa.old_pages_final && h->use_attn_decode && !h->ordered && h->attn_stream_min_pairs == 0 && attention_use_decode(R, aa.H, h->n_sm))
     return launch_attention_decode(aa, R, h->kv_map, (int)((aa.kv_layer - h->kv) / kHeadDim), h->n_sm, st, pdl);
   const bool stream = h->attn_stream_min_pairs > 0 ? R * aa.H >= h->attn_stream_min_pairs : attention_use_stream(R, aa.H, h->n_sm);
   if (h->use_attn_stream && stream) return launch_attention_stream(aa, R, st, pdl);
@@ -393,6 +401,10 @@ GemmTcArgs gemm_args(tts_gpt *h, const PackedLinear &pl, const void *act_img, in
   return a;
 }
 
+// Passes of up to kPairMinRows rows stay with the one-CTA wide kernel (two CTAs per SM): their tiles are too few for pairs.
+constexpr int kPairMinRows = 1024;
+bool use_pairs(const tts_gpt *h, int R) { return R > kPairMinRows && !(h->cfg.wfmt == WF_INT4 && h->w4_exact); }
+
 int launch_ln_tc(tts_gpt *h, int rows, const uint16_t *g, const uint16_t *b, int n_part, const uint16_t *add_bias,
                  void *out_img, uint16_t *out_plain, const int *gather, const int *out_slot, const StepIO *io,
                  int write_back) {
@@ -407,7 +419,7 @@ int launch_ln_tc(tts_gpt *h, int rows, const uint16_t *g, const uint16_t *b, int
   if (rows > kMaxRows && h->cfg.d_model % 8 == 0) {
     // the many rows of a large prefill pass: one warp per row
     const dim3 rgrid((rows + kLnRowsWarps - 1) / kLnRowsWarps), rblock(kLnRowsWarps * 32);
-    if (n_part == 0 && !add_bias && out_img && !out_plain && !gather && !io) {   // nothing to fold: the pair kernel's passes
+    if (use_pairs(h, rows) && n_part == 0 && !add_bias && out_img && !out_plain && !gather && !io) {   // nothing to fold: the pair kernel's passes
       la.err = h->dev_err;
       CUDA_TRY(h, launch_kernel(layernorm_big_kernel, dim3((rows + kLnBigWarps - 1) / kLnBigWarps), dim3(kLnBigWarps * 32),
                                 layernorm_big_smem_bytes(h->cfg.d_model), h->stream, h->use_pdl, la, rows));
@@ -421,10 +433,6 @@ int launch_ln_tc(tts_gpt *h, int rows, const uint16_t *g, const uint16_t *b, int
   h->launches += 1;
   return TTS_GPT_OK;
 }
-
-// Passes of up to kPairMinRows rows stay with the one-CTA wide kernel (two CTAs per SM): their tiles are too few for pairs.
-constexpr int kPairMinRows = 1024;
-bool use_pairs(const tts_gpt *h, int R) { return R > kPairMinRows && !(h->cfg.wfmt == WF_INT4 && h->w4_exact); }
 
 int launch_gemm(tts_gpt *h, const GemmTcArgs &a, const CUtensorMap &w_map, const CUtensorMap &x_map, bool wide, cudaStream_t st, bool pdl) {
   if (!wide) CUDA_TRY(h, launch_gemm_tc(a, h->n_sm, st, pdl));
@@ -531,7 +539,7 @@ int run_layers(tts_gpt *h, int R, bool decode) {
   const int d = c.d_model;
   cudaStream_t st = h->stream;
   const bool pdl = h->use_pdl;
-  const bool fuse_ln = can_fuse_ln(c.wfmt, R, d);
+  const bool fuse_ln = can_fuse_ln(R, d, h->ordered);
   // 2 to 16 rows: FC2 (K = d_ff) splits K over kSmallKSplit CTAs per row tile, so that a CTA stages a
   // quarter of the wide activation rows; its partial sums are folded into x by the next LayerNorm
   const int fc2_ks = (!fuse_ln && h->use_fc2_ksplit && (c.d_ff / k_per_tile(c.wfmt)) % kSmallKSplit == 0 &&
@@ -609,7 +617,7 @@ int run_head(tts_gpt *h, int n_out, int R) {
                           h->rt.out_slot, h->io, 0);
     if (rc) return rc;
     h->pending_parts = 0;
-  } else if (can_fuse_ln(WF_BF16, n_out, c.d_model)) {
+  } else if (can_fuse_ln(n_out, c.d_model, h->ordered)) {
     ha.ln_x = h->x; ha.ln_g = h->lnf_g; ha.ln_b = h->lnf_b; ha.ln_eps = c.ln_eps;
     ha.ln_gather = h->rt.out_rows; ha.ln_out_slot = h->rt.out_slot; ha.ln_io = h->io;
   } else {
@@ -783,6 +791,9 @@ int32_t tts_gpt_create(const tts_gpt_config_t *cfg, const tts_gpt_weights_t *w, 
     // 148 SMs.
     const int t = std::max(1, std::min(kMaxPassRows / kMaxRows, 2 * (h->n_sm / 2 / ((h->cfg.d_model + 255) / 256))));
     h->prefill_pass_rows = t * kMaxRows;
+    // ordered passes: the most row tiles whose widest linear of one-CTA tiles, two per SM, is one wave (7 tiles with this model)
+    const int widest = std::max(std::max((h->cfg.d_ff + 127) / 128, (3 * h->cfg.d_model + 127) / 128), tcw_ksplit_resid(h->cfg.d_ff) * ((h->cfg.d_model + 127) / 128));
+    h->ordered_pass_rows = std::max(1, std::min(kMaxSplitRows / kMaxRows, 2 * h->n_sm / std::max(1, widest))) * kMaxRows;
   }
   *out = h;
   return TTS_GPT_OK;
@@ -856,6 +867,8 @@ static int prefill_impl(tts_gpt_t *h, int32_t n, const void *const *emb, const i
   // rows in stream-major order; a pass takes up to `pass_rows` of them (several row tiles of 128 when the
   // tensor-core path is available, else one)
   int pass_rows = (h->have_tc && h->use_tc) ? h->prefill_pass_rows : kMaxRows;
+  h->ordered = top_k > 1;
+  if (h->ordered) pass_rows = std::min(pass_rows, h->ordered_pass_rows);
   if ((c.wfmt == WF_INT4 && h->w4_exact) || (h->kv_fp8 && !h->use_attn_mma)) pass_rows = std::min(pass_rows, kMaxSplitRows);
   PassParams ps;
   memset(&ps, 0, sizeof ps);
@@ -950,8 +963,10 @@ int32_t tts_gpt_decode_step(tts_gpt_t *h, int32_t n, const int32_t *stream_ids, 
   // The step's graph is captured (nothing runs during capture) before anything of the call is committed: a
   // failure to capture or instantiate leaves the engine exactly as it was.
   cudaGraphExec_t exec = nullptr;
+  h->ordered = top_k > 1;
+  const int key = h->ordered ? -n : n;
   if (h->use_graph) {
-    auto it = h->graphs.find(n);
+    auto it = h->graphs.find(key);
     if (it == h->graphs.end()) {
       cudaGraph_t g = nullptr;
       const unsigned long long before = h->launches;
@@ -968,8 +983,8 @@ int32_t tts_gpt_decode_step(tts_gpt_t *h, int32_t n, const int32_t *stream_ids, 
       e = cudaGraphInstantiate(&ge, g, 0);
       cudaGraphDestroy(g);
       if (e != cudaSuccess) return fail(h, TTS_GPT_E_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
-      it = h->graphs.emplace(n, ge).first;
-      h->graph_nodes[n] = nodes;
+      it = h->graphs.emplace(key, ge).first;
+      h->graph_nodes[key] = nodes;
     }
     exec = it->second;
   }
@@ -987,7 +1002,7 @@ int32_t tts_gpt_decode_step(tts_gpt_t *h, int32_t n, const int32_t *stream_ids, 
 
   if (exec) {
     CUDA_TRY(h, cudaGraphLaunch(exec, h->stream));
-    h->launches += h->graph_nodes[n];
+    h->launches += h->graph_nodes[key];
     return TTS_GPT_OK;
   }
   rc = run_embed(h, n);

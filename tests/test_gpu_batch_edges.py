@@ -14,13 +14,13 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-def _run(eng, prefixes, n_steps):
+def _run(eng, prefixes, n_steps, **kw):
     S, V = len(prefixes), eng.cfg.vocab
     toks = torch.zeros((n_steps + 1, S), dtype=torch.int32, device=DEV)
     logits = torch.zeros((n_steps + 1, S, V), dtype=torch.float32, device=DEV)
-    ids, _ = eng.prefill([bits_dev(p) for p in prefixes], out_tokens=toks[0], out_logits=logits[0])
+    ids, _ = eng.prefill([bits_dev(p) for p in prefixes], out_tokens=toks[0], out_logits=logits[0], **kw)
     for k in range(1, n_steps + 1):
-        eng.decode_step(ids, toks[k], out_logits=logits[k])
+        eng.decode_step(ids, toks[k], out_logits=logits[k], **kw)
     eng.sync()
     for s in ids:
         eng.release_stream(s)
@@ -83,5 +83,25 @@ def test_prefill_pair_kernel_with_the_8bit_cache_and_k_ranges():
     eng.set_option("prefill_pass_rows", 512)
     lg2, _ = _run(eng, prefixes, 2)
     assert np.max(np.abs(lg[:, 0] - lg2[:, 0])) < 4.5e-2
+    assert eng.check_canaries() == 0
+    eng.destroy()
+
+
+@pytest.mark.parametrize("S", [1, 2, 4, 5, 75])
+def test_sampled_calls_keep_their_order_of_sums(S):
+    """Sampled calls have step graphs, pass sizes and (2 to 4 rows, middle batches) kernels of their own: with uniforms of
+    zero they take the first of the top k, the greedy token, and greedy calls in between change nothing."""
+    lens = [1030 if i == 0 else 2 + (11 * i) % 60 for i in range(S)]
+    cfg = C.tiny_config(max_streams=S, n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=1152, max_pos=1152)
+    w = C.make_weights(cfg, seed=27)
+    model = O.OracleModel(cfg, w)
+    eng = B.TtsGpt(cfg, w, DEV)
+    prefixes = C.make_prefixes(cfg, lens, seed=28)
+    kw = dict(top_k=4, uniforms=torch.zeros(S, device=DEV))
+    lg, tk = _run(eng, prefixes, 4, **kw)
+    _check(model, prefixes, lg, tk, sorted({0, S // 2, S - 1}), "sampled")
+    _run(eng, prefixes, 2)
+    lg2, tk2 = _run(eng, prefixes, 4, **kw)
+    assert np.array_equal(lg, lg2) and np.array_equal(tk, tk2)
     assert eng.check_canaries() == 0
     eng.destroy()
