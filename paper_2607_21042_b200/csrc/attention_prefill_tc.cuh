@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kPtThreads, PAIRED ? 2 : 1) attention_prefill_
       // all but the last page of a row's own stream are seen whole by every row of the warp: no masks there
       const bool whole = __all_sync(0xFFFFFFFFu, see == kPageTokens);
       // With an SM to itself the thread keeps all 64 scores in registers.  Where two CTAs share an SM (88 registers) S is
-      // read half by half, the lower half a second time behind the maximum.  Four independent chains for the maximum and
+      // read half by half, the upper half a second time behind the maximum.  Four independent chains for the maximum and
       // for the sum; the scale (positive) is applied to the maximum and inside the exponential's argument: one
       // multiply-add per score.
       constexpr int HALVES = PAIRED ? 2 : 1, W = 64 / HALVES;
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(kPtThreads, PAIRED ? 2 : 1) attention_prefill_
       auto scores_read = [&]() { tc_fence_before_sync(); mbar_arrive(s_free + g); };
       float pm4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-      for (int hh = 0; hh < HALVES; ++hh) {
+      for (int hh = HALVES - 1; hh >= 0; --hh) {
         load(W * hh);
         if (HALVES == 1) scores_read();
 #pragma unroll
@@ -308,12 +308,12 @@ __global__ void __launch_bounds__(kPtThreads, PAIRED ? 2 : 1) attention_prefill_
       m = m_new;
       float sum4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int hh = HALVES - 1; hh >= 0; --hh) {
-        if (HALVES == 2 && hh == 0) { load(0); scores_read(); }
+      for (int hh = 0; hh < HALVES; ++hh) {   // tokens in ascending order in both forms: the same sums
+        if (HALVES == 2 && hh == 1) { load(W); scores_read(); }
 #pragma unroll
         for (int c = 0; c < W; ++c) { s[c] = pt_exp2(fmaf(s[c], qs, -ref)); sum4[c & 3] += s[c]; }
         // the group's P and O belong to the tensor core until P V of the group's job before has completed
-        if (hh == HALVES - 1 && k > 0) { pt_warp_wait(pv_done + g, (uint32_t)(k - 1) & 1u, failed, a.err); tc_fence_after_sync(); }
+        if (hh == 0 && k > 0) { pt_warp_wait(pv_done + g, (uint32_t)(k - 1) & 1u, failed, a.err); tc_fence_after_sync(); }
 #pragma unroll
         for (int c8 = 0; c8 < W / 8; ++c8)
           *reinterpret_cast<uint4 *>(Pg + t * 128 + (((W / 8 * hh + c8) ^ (t & 7)) << 4)) =

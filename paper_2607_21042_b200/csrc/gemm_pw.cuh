@@ -435,7 +435,7 @@ inline PwPlan pw_plan(int N, int K, int rows, bool resid, int n_sm, int fixed_ks
     for (int ks = 1; ks <= (resid ? kTwMaxPartials : 1); ++ks) {
       const int per = (KC + ks - 1) / ks;
       if (fixed_ks > 0 && ks != fixed_ks) continue;
-      if (fixed_ks <= 0 && ks > 1 && (per < 4 || per * (ks - 1) >= KC || (rows + kMaxRows - 1) / kMaxRows * ks > kMaxSplitTiles)) break;
+      if (fixed_ks <= 0 && ks > 1 && (per < 4 || per * (ks - 1) >= KC || (rows + kMaxRows - 1) / kMaxRows * ks > 4 * kMaxSplitRows / kMaxRows)) break;
       const int tiles = n_rp * ((N + bn - 1) / bn) * ks, waves = (tiles + n_pair - 1) / n_pair;
       const float tile_us = std::max(per * chunk_us, epi_us);
       const float us = waves * tile_us + epi_us + (ks > 1 ? 0.4f + 0.0005f * rows * ks : 0.f);

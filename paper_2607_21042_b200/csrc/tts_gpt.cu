@@ -105,11 +105,11 @@ struct tts_gpt {
   int tc_tail_parts = 0;  // partial sums the last FC2 of the tensor-core path left for the final LayerNorm
   bool use_attn_mma = true;      // tensor-core attention in prefill passes (option "attn_mma")
   bool use_attn_prefill = true;  // shared-page attention in prefill passes (option "attn_prefill")
-  // Sampled calls (top_k > 1) keep one order of sums: the FMA linears up to 4 rows, prefill passes of `ordered_pass_rows`,
-  // the CUDA-core decode attention.  A sampled token hangs on the last bits of its logits (neighbours in the tail of the
-  // distribution lie closer than bf16 rounding moves them, and the token feeds every later step), so a caller who replays
-  // a sequence of uniforms gets the same utterance only if the sums run in the same order.  Greedy calls are free of that
-  // and take the faster kernels.
+  // Sampled calls (top_k > 1) keep one order of sums: the FMA linears up to 4 rows, prefill passes with the k-ranges and
+  // tails of passes of `ordered_pass_rows`, the CUDA-core decode attention.  A sampled token hangs on the last bits of its
+  // logits (neighbours in the tail of the distribution lie closer than bf16 rounding moves them, and the token feeds every
+  // later step), so a caller who replays a sequence of uniforms gets the same utterance only if the sums run in the same
+  // order.  Greedy calls are free of that and take the faster kernels.
   bool ordered = false;          // set by each prefill and decode call
   int ordered_pass_rows = 896;
   bool use_attn_decode = true;   // unit-split tensor-pipe attention of decode steps (option "attn_decode")
@@ -419,7 +419,7 @@ int launch_ln_tc(tts_gpt *h, int rows, const uint16_t *g, const uint16_t *b, int
   if (rows > kMaxRows && h->cfg.d_model % 8 == 0) {
     // the many rows of a large prefill pass: one warp per row
     const dim3 rgrid((rows + kLnRowsWarps - 1) / kLnRowsWarps), rblock(kLnRowsWarps * 32);
-    if (use_pairs(h, rows) && n_part == 0 && !add_bias && out_img && !out_plain && !gather && !io) {   // nothing to fold: the pair kernel's passes
+    if (use_pairs(h, rows) && !h->ordered && n_part == 0 && !add_bias && out_img && !out_plain && !gather && !io) {   // nothing to fold: the pair kernel's passes
       la.err = h->dev_err;
       CUDA_TRY(h, launch_kernel(layernorm_big_kernel, dim3((rows + kLnBigWarps - 1) / kLnBigWarps), dim3(kLnBigWarps * 32),
                                 layernorm_big_smem_bytes(h->cfg.d_model), h->stream, h->use_pdl, la, rows));
@@ -454,8 +454,9 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
   const bool pdl = h->use_pdl;
   const bool wide = R > kMaxRows;
   const bool pairs = use_pairs(h, R);
-  const int o_ks = !wide ? kTcKSplit : pairs ? pw_plan(d, d, R, true, h->n_sm).ksplit : tcw_ksplit_resid(d);
-  const int f2_ks = !wide ? kTcKSplit : pairs ? pw_plan(d, c.d_ff, R, true, h->n_sm).ksplit : tcw_ksplit_resid(c.d_ff);
+  const bool free_ks = pairs && !h->ordered;   // ordered passes keep the k-ranges of the one-CTA wide kernel
+  const int o_ks = !wide ? kTcKSplit : free_ks ? pw_plan(d, d, R, true, h->n_sm).ksplit : tcw_ksplit_resid(d);
+  const int f2_ks = !wide ? kTcKSplit : free_ks ? pw_plan(d, c.d_ff, R, true, h->n_sm).ksplit : tcw_ksplit_resid(c.d_ff);
   const int o_parts = o_ks > 1 ? o_ks : 0, f2_parts = f2_ks > 1 ? f2_ks : 0;   // 0: the linear added into x itself
   for (int l = 0; l < c.n_layer; ++l) {
     LayerW &L = h->layers[l];
@@ -867,9 +868,16 @@ static int prefill_impl(tts_gpt_t *h, int32_t n, const void *const *emb, const i
   // rows in stream-major order; a pass takes up to `pass_rows` of them (several row tiles of 128 when the
   // tensor-core path is available, else one)
   int pass_rows = (h->have_tc && h->use_tc) ? h->prefill_pass_rows : kMaxRows;
-  h->ordered = top_k > 1;
-  if (h->ordered) pass_rows = std::min(pass_rows, h->ordered_pass_rows);
   if ((c.wfmt == WF_INT4 && h->w4_exact) || (h->kv_fp8 && !h->use_attn_mma)) pass_rows = std::min(pass_rows, kMaxSplitRows);
+  h->ordered = top_k > 1;
+  // Ordered passes: what a row's sums look like depends on the pass of `unit` rows it lies in by its last tile (a pass of up
+  // to 128 rows has kernels of its own) and by the rows whose logits are wanted together.  Several units run as one pass,
+  // with a last unit of up to 128 rows apart and the head unit by unit.  (Over the 8-bit cache a pass is one unit: how many
+  // pages it reaches decides which attention it takes.)
+  const int unit = h->ordered ? std::min(pass_rows, h->ordered_pass_rows) : 0;
+  if (unit) pass_rows = h->kv_fp8 ? unit : pass_rows / unit * unit;
+  int left = 0;            // rows not yet in a pass
+  for (int i = 0; i < n; ++i) left += plen[i];
   PassParams ps;
   memset(&ps, 0, sizeof ps);
   ps.io = io;
@@ -891,7 +899,19 @@ static int prefill_impl(tts_gpt_t *h, int32_t n, const void *const *emb, const i
     if (r) return r;
     r = run_layers(h, ps.n_rows, false);
     if (r) return r;
-    if (ps.n_out > 0) r = run_head(h, ps.n_out, ps.n_rows);
+    if (unit == 0 || ps.n_rows <= unit) {
+      if (ps.n_out > 0) r = run_head(h, ps.n_out, ps.n_rows);
+    } else {
+      const RowTable rt = h->rt;
+      for (int j0 = 0, j = 0; j0 < ps.n_out && !r; j0 = j) {
+        while (j < ps.n_out && ps.out_rows[j] / unit == ps.out_rows[j0] / unit) ++j;
+        h->rt.out_rows = rt.out_rows + j0;
+        h->rt.out_slot = rt.out_slot + j0;
+        r = run_head(h, j - j0, ps.n_rows);
+      }
+      h->rt = rt;
+    }
+    left -= ps.n_rows;
     ps.n_rows = 0; ps.n_out = 0; ps.n_runs = 0;
     scratch_pages = 0; h->pass_scratch = 0;
     return r;
@@ -899,7 +919,9 @@ static int prefill_impl(tts_gpt_t *h, int32_t n, const void *const *emb, const i
   for (int i = 0; i < n; ++i) {
     int t = 0;
     while (t < plen[i]) {
-      const int take = std::min(plen[i] - t, pass_rows - ps.n_rows);
+      const bool tail_apart = unit && left > unit && left <= pass_rows && left % unit != 0 && left % unit <= kMaxRows;
+      const int end = tail_apart ? left - left % unit : pass_rows;   // rows of this pass
+      const int take = std::min(plen[i] - t, end - ps.n_rows);
       ps.run_stream[ps.n_runs] = (short)pp.stream_ids[i];
       ps.run_pos0[ps.n_runs] = (short)t;
       ps.run_row0[ps.n_runs] = (short)ps.n_rows;
@@ -913,7 +935,7 @@ static int prefill_impl(tts_gpt_t *h, int32_t n, const void *const *emb, const i
         ps.out_slot[ps.n_out] = (short)i;
         ++ps.n_out;
       }
-      if (ps.n_rows == pass_rows) { rc = flush(); if (rc) return rc; }
+      if (ps.n_rows == end) { rc = flush(); if (rc) return rc; }
     }
   }
   return flush();
