@@ -33,6 +33,7 @@ struct RowTable {
 // their own range of the position table; prefix embeddings are used as given: Section II-C)
 __global__ void embed_kernel(RowTable rt, const uint16_t *__restrict__ tok_emb, const uint16_t *__restrict__ pos_emb,
                              int d, int vocab, int max_pos, float *__restrict__ x) {
+  pdl_wait();   // for the set-up kernel in front; the next kernel may not start before this one ends: it relies on the tables
   const int r = blockIdx.x;
   int tok = rt.row_token[r];
   float *xr = x + (size_t)r * d;
@@ -431,8 +432,6 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(const SampleArgs
   __shared__ float sel_v[kMaxTopK]; __shared__ int sel_i[kMaxTopK];
   __shared__ float srt_v[kMaxTopK]; __shared__ int srt_i[kMaxTopK];
 
-  pdl_launch_dependents();
-  pdl_wait();
   const int j = blockIdx.x;
   const int slot = a.out_slot ? a.out_slot[j] : j;
   const int V = a.V;
@@ -443,6 +442,10 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(const SampleArgs
     top_k = a.io->top_k; temperature = a.io->temperature; uniforms = a.io->uniforms;
     out_tokens = a.io->out_tokens; out_logits = a.io->out_logits;
   }
+  const float u = top_k > 1 && uniforms ? uniforms[slot] : 0.f;   // (may lie in host memory)
+  // everything above is final before the step's first kernel starts
+  pdl_launch_dependents();
+  pdl_wait();
   for (int i = threadIdx.x; i < V; i += blockDim.x) {
     const float v = src[i];
     lg[i] = v;
@@ -567,7 +570,6 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(const SampleArgs
     float w[kMaxTopK];
     float total = 0.f;
     for (int r = 0; r < k; ++r) { w[r] = expf((srt_v[r] - srt_v[0]) * inv_t); total += w[r]; }
-    const float u = uniforms ? uniforms[slot] : 0.f;
     float cum = 0.f;
     token = srt_i[k - 1];
     for (int r = 0; r < k; ++r) {

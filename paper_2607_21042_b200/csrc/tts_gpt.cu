@@ -91,8 +91,13 @@ struct tts_gpt {
   std::vector<int> ctx, pos_next;
   int n_free;
   // step graphs by row count, those of sampled steps under its negative
-  std::map<int, cudaGraphExec_t> graphs;
-  std::map<int, int> graph_nodes;
+  struct StepGraph {
+    cudaGraph_t graph;
+    cudaGraphExec_t exec;
+    cudaGraphNode_t setup;   // step_setup_kernel, the root: its parameters are replaced for every step
+    int launches;            // kernels in the graph
+  };
+  std::map<int, StepGraph> graphs;
   bool use_graph;
   bool use_pdl;
   bool use_fc2_ksplit = true;   // 2-16 rows: FC2 splits K (option "fc2_ksplit")
@@ -642,10 +647,15 @@ int run_head(tts_gpt *h, int n_out, int R) {
 
 int run_embed(tts_gpt *h, int R) {
   const tts_gpt_config_t &c = h->cfg;
-  embed_kernel<<<R, 256, 0, h->stream>>>(h->rt, h->tok_emb, h->pos_emb, c.d_model, emb_rows_of(c), c.max_pos, h->x);
-  CUDA_TRY(h, cudaGetLastError());
+  CUDA_TRY(h, launch_kernel(embed_kernel, dim3(R), dim3(256), 0, h->stream, h->use_pdl, h->rt, (const uint16_t *)h->tok_emb, (const uint16_t *)h->pos_emb,
+                            c.d_model, emb_rows_of(c), c.max_pos, h->x));
   h->launches += 1;
   return TTS_GPT_OK;
+}
+
+void drop_graphs(tts_gpt *h) {
+  for (auto &kv : h->graphs) { cudaGraphExecDestroy(kv.second.exec); cudaGraphDestroy(kv.second.graph); }
+  h->graphs.clear();
 }
 
 // Output rows are written with vector stores: the hidden rows need 16-byte alignment, the rest their
@@ -982,55 +992,58 @@ int32_t tts_gpt_decode_step(tts_gpt_t *h, int32_t n, const int32_t *stream_ids, 
   }
   if (pages > h->n_free) return fail(h, TTS_GPT_E_NO_PAGES, "decode_step: %d pages needed, %d free", pages, h->n_free);
 
-  // The step's graph is captured (nothing runs during capture) before anything of the call is committed: a
-  // failure to capture or instantiate leaves the engine exactly as it was.
-  cudaGraphExec_t exec = nullptr;
-  h->ordered = top_k > 1;
-  const int key = h->ordered ? -n : n;
-  if (h->use_graph) {
-    auto it = h->graphs.find(key);
-    if (it == h->graphs.end()) {
-      cudaGraph_t g = nullptr;
-      const unsigned long long before = h->launches;
-      CUDA_TRY(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-      rc = run_embed(h, n);
-      if (!rc) rc = run_layers(h, n, true);
-      if (!rc) rc = run_head(h, n, n);
-      cudaError_t e = cudaStreamEndCapture(h->stream, &g);
-      const int nodes = (int)(h->launches - before);
-      h->launches = before;  // captured, not run
-      if (rc) { if (g) cudaGraphDestroy(g); return rc; }
-      if (e != cudaSuccess) return fail(h, TTS_GPT_E_CUDA, "graph capture: %s", cudaGetErrorString(e));
-      cudaGraphExec_t ge = nullptr;
-      e = cudaGraphInstantiate(&ge, g, 0);
-      cudaGraphDestroy(g);
-      if (e != cudaSuccess) return fail(h, TTS_GPT_E_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
-      it = h->graphs.emplace(key, ge).first;
-      h->graph_nodes[key] = nodes;
-    }
-    exec = it->second;
-  }
-
   StepParams sp;
   sp.n = n;
   memcpy(sp.stream_ids, stream_ids, (size_t)n * sizeof(int));
   sp.io.in_tokens = in_tokens; sp.io.uniforms = uniforms; sp.io.out_tokens = out_tokens; sp.io.out_logits = out_logits;
   sp.io.out_hidden = (uint16_t *)out_hidden; sp.io.top_k = top_k; sp.io.temperature = temperature; sp.io.n_out = n;
-  step_setup_kernel<<<1, kMaxRows, 0, h->stream>>>(sp, h->ps, h->rt, h->io);
-  CUDA_TRY(h, cudaGetLastError());
-  h->launches += 1;
+  h->ordered = top_k > 1;
+  auto enqueue = [&]() -> int {
+    step_setup_kernel<<<1, kMaxRows, 0, h->stream>>>(sp, h->ps, h->rt, h->io);
+    CUDA_TRY(h, cudaGetLastError());
+    h->launches += 1;
+    int r = run_embed(h, n);
+    if (!r) r = run_layers(h, n, true);
+    return r ? r : run_head(h, n, n);
+  };
+  // The step's graph is captured (nothing runs during capture) before anything of the call is committed: a
+  // failure to capture or instantiate leaves the engine exactly as it was.  The set-up kernel is the graph's first
+  // node and gets the step's parameters there (a launch of its own in front of the graph: 2 us more per step).
+  const tts_gpt::StepGraph *sg = nullptr;
+  if (h->use_graph) {
+    const int key = h->ordered ? -n : n;
+    auto it = h->graphs.find(key);
+    if (it == h->graphs.end()) {
+      tts_gpt::StepGraph ng;
+      memset(&ng, 0, sizeof ng);
+      const unsigned long long before = h->launches;
+      CUDA_TRY(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
+      rc = enqueue();
+      cudaError_t e = cudaStreamEndCapture(h->stream, &ng.graph);
+      ng.launches = (int)(h->launches - before);
+      h->launches = before;  // captured, not run
+      if (!rc && e != cudaSuccess) rc = fail(h, TTS_GPT_E_CUDA, "graph capture: %s", cudaGetErrorString(e));
+      size_t roots = 1;
+      if (!rc && ((e = cudaGraphGetRootNodes(ng.graph, &ng.setup, &roots)) != cudaSuccess || roots != 1))
+        rc = fail(h, TTS_GPT_E_CUDA, "graph capture: no single root (%s)", cudaGetErrorString(e));
+      if (!rc && (e = cudaGraphInstantiate(&ng.exec, ng.graph, 0)) != cudaSuccess) rc = fail(h, TTS_GPT_E_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
+      if (rc) { if (ng.graph) cudaGraphDestroy(ng.graph); return rc; }
+      it = h->graphs.emplace(key, ng).first;
+    }
+    sg = &it->second;
+    void *args[] = {&sp, &h->ps, &h->rt, &h->io};
+    cudaKernelNodeParams kp;
+    memset(&kp, 0, sizeof kp);
+    kp.func = (void *)step_setup_kernel;
+    kp.gridDim = dim3(1); kp.blockDim = dim3(kMaxRows); kp.kernelParams = args;
+    CUDA_TRY(h, cudaGraphExecKernelNodeSetParams(sg->exec, sg->setup, &kp));
+  }
   for (int i = 0; i < n; ++i) { h->ctx[stream_ids[i]] += 1; h->pos_next[stream_ids[i]] += 1; }
   h->n_free -= pages;
-
-  if (exec) {
-    CUDA_TRY(h, cudaGraphLaunch(exec, h->stream));
-    h->launches += h->graph_nodes[key];
-    return TTS_GPT_OK;
-  }
-  rc = run_embed(h, n);
-  if (!rc) rc = run_layers(h, n, true);
-  if (!rc) rc = run_head(h, n, n);
-  return rc;
+  if (!sg) return enqueue();
+  CUDA_TRY(h, cudaGraphLaunch(sg->exec, h->stream));
+  h->launches += sg->launches;
+  return TTS_GPT_OK;
 }
 
 int32_t tts_gpt_decode_steps(tts_gpt_t *h, int32_t n, const int32_t *stream_ids, const int32_t *in_tokens,
@@ -1093,16 +1106,33 @@ int32_t tts_gpt_decode_step_host(tts_gpt_t *h, int32_t n, const int32_t *stream_
   const tts_gpt_config_t &c = h->cfg;
   if (n < 1 || n > c.max_streams || !stream_ids || !out_tokens) return fail(h, TTS_GPT_E_ARG, "decode_step_host: bad n or null argument");
   if (top_k > 1 && !uniforms) return fail(h, TTS_GPT_E_ARG, "decode_step_host: top-k sampling needs uniforms");
-  if (in_tokens) CUDA_TRY(h, cudaMemcpyAsync(h->st_in, in_tokens, (size_t)n * sizeof(int), cudaMemcpyHostToDevice, h->stream));
-  if (top_k > 1) CUDA_TRY(h, cudaMemcpyAsync(h->st_uni, uniforms, (size_t)n * sizeof(float), cudaMemcpyHostToDevice, h->stream));
-  const int rc = tts_gpt_decode_step(h, n, stream_ids, in_tokens ? h->st_in : nullptr, top_k, temperature,
-                                     top_k > 1 ? h->st_uni : nullptr, h->st_tok, out_logits ? h->st_log : nullptr,
-                                     out_hidden ? h->st_hid : nullptr);
+  // Pinned buffers are read and written by the step's kernels over the bus, the others through staging arrays and copies
+  // on the stream (a copy costs the stream 3 to 5 us on either side of the step's kernels).
+  auto mapped = [](const void *p, size_t align) -> void * {
+    cudaPointerAttributes at;
+    if (!p || cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    return at.type == cudaMemoryTypeHost && (uintptr_t)at.devicePointer % align == 0 ? at.devicePointer : nullptr;
+  };
+  const int *in = (const int *)mapped(in_tokens, 4);
+  const float *uni = top_k > 1 ? (const float *)mapped(uniforms, 4) : nullptr;
+  int *tok = (int *)mapped(out_tokens, 4);
+  float *log = (float *)mapped(out_logits, 4);
+  void *hid = mapped(out_hidden, 16);
+  if (in_tokens && !in) {
+    CUDA_TRY(h, cudaMemcpyAsync(h->st_in, in_tokens, (size_t)n * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+    in = h->st_in;
+  }
+  if (top_k > 1 && !uni) {
+    CUDA_TRY(h, cudaMemcpyAsync(h->st_uni, uniforms, (size_t)n * sizeof(float), cudaMemcpyHostToDevice, h->stream));
+    uni = h->st_uni;
+  }
+  const int rc = tts_gpt_decode_step(h, n, stream_ids, in, top_k, temperature, uni, tok ? tok : h->st_tok,
+                                     log || !out_logits ? log : h->st_log, hid || !out_hidden ? hid : h->st_hid);
   if (rc) return rc;
-  CUDA_TRY(h, cudaMemcpyAsync(out_tokens, h->st_tok, (size_t)n * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  if (out_logits)
+  if (!tok) CUDA_TRY(h, cudaMemcpyAsync(out_tokens, h->st_tok, (size_t)n * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  if (out_logits && !log)
     CUDA_TRY(h, cudaMemcpyAsync(out_logits, h->st_log, (size_t)n * c.vocab * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
-  if (out_hidden)
+  if (out_hidden && !hid)
     CUDA_TRY(h, cudaMemcpyAsync(out_hidden, h->st_hid, (size_t)n * c.d_model * sizeof(uint16_t), cudaMemcpyDeviceToHost, h->stream));
   return tts_gpt_sync(h);
 }
@@ -1120,7 +1150,7 @@ int32_t tts_gpt_sync(tts_gpt_t *h) {
 int32_t tts_gpt_destroy(tts_gpt_t *h) {
   if (!h) return fail(nullptr, TTS_GPT_E_ARG, "null handle");
   cudaStreamSynchronize(h->stream);
-  for (auto &kv : h->graphs) cudaGraphExecDestroy(kv.second);
+  drop_graphs(h);
   if (h->host_err) cudaFreeHost((void *)h->host_err);
   delete h;
   return TTS_GPT_OK;
@@ -1144,9 +1174,7 @@ int32_t tts_gpt_debug_kernel_launches(const tts_gpt_t *h, uint64_t *n) {
 int32_t tts_gpt_debug_set_trace(tts_gpt_t *h, void *trace, int32_t *n_slots) {
   if (!h) return fail(nullptr, TTS_GPT_E_ARG, "null handle");
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  for (auto &kv : h->graphs) cudaGraphExecDestroy(kv.second);  // slots are baked into captured graphs
-  h->graphs.clear();
-  h->graph_nodes.clear();
+  drop_graphs(h);   // slots are baked into captured graphs
   h->trace = (unsigned long long *)trace;
   if (n_slots) *n_slots = 7 * h->cfg.n_layer + 2;   // upper bound: the tensor-core path traces 7 kernels per layer
   return TTS_GPT_OK;
@@ -1175,9 +1203,7 @@ int32_t tts_gpt_debug_expire_wait(tts_gpt_t *h, uint32_t limit_us) {
 int32_t tts_gpt_debug_set_option(tts_gpt_t *h, const char *name, int32_t value) {
   if (!h || !name) return fail(nullptr, TTS_GPT_E_ARG, "null argument");
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  for (auto &kv : h->graphs) cudaGraphExecDestroy(kv.second);   // the choice is baked into captured step graphs
-  h->graphs.clear();
-  h->graph_nodes.clear();
+  drop_graphs(h);   // the choice is baked into captured step graphs
   const std::string k(name);
   const bool on = value != 0;
   if (k == "graph") h->use_graph = on && h->stream != nullptr && h->stream != cudaStreamLegacy;
