@@ -6,18 +6,19 @@
 // core wants them in shared memory (K-major, 128-byte swizzle): a k-chunk of 64 columns of 128
 // rows is one 16 KB block in which row r sits at byte r*128 and the 16-byte unit u of that row is
 // stored at unit (u ^ (r % 8)).  Weights [N,K] become blocks [n/128][k/64]; activations of up to
-// 128 rows become blocks [k/64] (rows are batch rows, so the 32 rows of a batch chunk are 4 KB
+// 128 rows become blocks [k/64] (rows are batch rows, so the 32 or 64 rows of a batch chunk are
 // contiguous inside a block).  A stage of the pipeline is therefore filled by two plain bulk
-// asynchronous copies (16 KB of weights, 4 KB of activations): no tensor maps, no alignment rules
+// asynchronous copies (16 KB of weights, 4 or 8 KB of activations): no tensor maps, no alignment rules
 // beyond 16 bytes.  The kernels that produce activations (LayerNorm, attention, the GELU epilogue
 // below) write this image directly.
 //
-// A CTA owns a 128-row weight tile (the M operand), one chunk of 32 batch rows (the N operand) and
-// a contiguous range of k-chunks; with 4 batch chunks of 32 and, for the two linears that feed the
-// residual stream, 4 k-ranges, every linear of the block runs on 120-160 CTAs.  Warp 0 produces
-// (bulk copies into a 4-stage ring guarded by full/empty mbarriers; the weight copies of the first
+// A CTA owns a 128-row weight tile (the M operand), one chunk of 32 or 64 batch rows (the N operand) and
+// a contiguous range of k-chunks (4 k-ranges for the two linears that feed the residual stream); chunks of 64
+// rows where chunks of 32 would take more CTAs than there are SMs.  Warp 0 produces (bulk copies into a ring of 4
+// or, with an SM to itself, 8 stages guarded by full/empty mbarriers; the weight copies of the first
 // stages are issued before the dependency wait), warps 1 and 10 issue the MMAs (4 per k-chunk, M=128,
-// N=32, K=16; even and odd k-chunks into two accumulators) and commit each stage back to the producer, and warps 2-9 read the 128x32 fp32
+// N=32 or 64, K=16; even and odd k-chunks into two accumulators) and commit each stage back to the producer, and
+// warps 2-9 read the fp32
 // accumulator out of tensor memory and run the epilogue.  K-split partial sums go to a scratch
 // array that the following LayerNorm kernel folds into the residual stream in a fixed order.
 // Every wait is bounded; on expiry the CTA sets the error word, stops waiting and still releases

@@ -9,8 +9,9 @@
 // [n_pages][2 (K|V)][n_head] blocks of 4352 bytes: 64 tokens x 64 codes, then the 64 scales of the block.
 //
 // Path.  The QKV linear writes the step's new K/V rows as bf16 into a small staging area;
-// `kv_quantize_kernel` encodes them into their page slots (one warp per token, head and K|V);
-// `attention_fp8_kernel` is the split-KV decode attention over such pages: a CTA per (row, head, split),
+// `kv_quantize_kernel` encodes them into their page slots (one warp per token, head and K|V; in small decode
+// batches `attention_fp8_decode_kernel` does it on the way);
+// `attention_fp8_kernel` is the split-KV attention over such pages: a CTA per (row, head, split),
 // a warp per page, a lane on 16 codes of one of 8 tokens per load; scores, online softmax and outputs in
 // fp32, the scale applied to the 64-term dot product (K) and to the softmax weight (V) rather than to
 // every element; partial results of the splits meet through global scratch and the CTA that takes the
@@ -39,6 +40,14 @@ __device__ __forceinline__ void e4m3x16_to_float(const uint4 &w, float (&f)[16])
   }
 }
 
+// One staged row of K or V of one head as codes: lane l returns those of values 2l and 2l + 1, s the row's scale.
+__device__ __forceinline__ uint16_t e4m3_encode_row(uint32_t pair, float &s) {
+  const float x0 = bf16_lo(pair), x1 = bf16_hi(pair);
+  const float amax = warp_max(fmaxf(fabsf(x0), fabsf(x1)));
+  s = amax > 0.f ? amax / kE4m3Max : 1.0f;
+  return (uint16_t)__nv_cvt_float2_to_fp8x2(make_float2(__fdiv_rn(x0, s), __fdiv_rn(x1, s)), __NV_SATFINITE, __NV_E4M3);
+}
+
 // Encodes the staged K/V rows of a pass into their page slots.  stage: bf16 [R][2][H*64].  grid (H, R),
 // 64 threads: warp 0 takes K, warp 1 takes V; a lane takes two neighbouring values.
 __global__ void __launch_bounds__(64) kv_quantize_kernel(const uint16_t *__restrict__ stage, unsigned char *__restrict__ kv_layer,
@@ -48,15 +57,12 @@ __global__ void __launch_bounds__(64) kv_quantize_kernel(const uint16_t *__restr
   pdl_wait();
   const int h = blockIdx.x, r = blockIdx.y, which = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int d = H * kHeadDim;
-  const uint32_t pair = *reinterpret_cast<const uint32_t *>(stage + ((size_t)r * 2 + which) * d + h * kHeadDim + 2 * lane);
-  const float x0 = bf16_lo(pair), x1 = bf16_hi(pair);
-  const float amax = warp_max(fmaxf(fabsf(x0), fabsf(x1)));
-  const float s = amax > 0.f ? amax / kE4m3Max : 1.0f;
-  const __nv_fp8x2_storage_t codes = __nv_cvt_float2_to_fp8x2(make_float2(__fdiv_rn(x0, s), __fdiv_rn(x1, s)), __NV_SATFINITE, __NV_E4M3);
+  float s;
+  const uint16_t codes = e4m3_encode_row(*reinterpret_cast<const uint32_t *>(stage + ((size_t)r * 2 + which) * d + h * kHeadDim + 2 * lane), s);
   const int pos = row_pos[r];
   const int page = page_table[(size_t)row_stream[r] * pps + (pos >> 6)];
   unsigned char *blk = kv_layer + (((size_t)page * 2 + which) * H + h) * kFp8BlockBytes;
-  *reinterpret_cast<uint16_t *>(blk + (size_t)(pos & 63) * kHeadDim + 2 * lane) = (uint16_t)codes;
+  *reinterpret_cast<uint16_t *>(blk + (size_t)(pos & 63) * kHeadDim + 2 * lane) = codes;
   if (lane == 0) *reinterpret_cast<float *>(blk + kPageTokens * kHeadDim + 4 * (pos & 63)) = s;
 }
 
@@ -85,12 +91,10 @@ __global__ void __launch_bounds__(kQrWarps * 32) kv_quantize_rows_kernel(const u
       const int it = it0 + b * kQrWarps;
       if (it < n_items) {   // uniform in the warp
         const int which = it / H, h = it - which * H;
-        const float x0 = bf16_lo(pair[b]), x1 = bf16_hi(pair[b]);
-        const float amax = warp_max(fmaxf(fabsf(x0), fabsf(x1)));
-        const float sc = amax > 0.f ? amax / kE4m3Max : 1.0f;
-        const __nv_fp8x2_storage_t codes = __nv_cvt_float2_to_fp8x2(make_float2(__fdiv_rn(x0, sc), __fdiv_rn(x1, sc)), __NV_SATFINITE, __NV_E4M3);
+        float sc;
+        const uint16_t codes = e4m3_encode_row(pair[b], sc);
         unsigned char *blk = kv_layer + (((size_t)page * 2 + which) * H + h) * kFp8BlockBytes;
-        *reinterpret_cast<uint16_t *>(blk + (size_t)(pos & 63) * kHeadDim + 2 * lane) = (uint16_t)codes;
+        *reinterpret_cast<uint16_t *>(blk + (size_t)(pos & 63) * kHeadDim + 2 * lane) = codes;
         if (lane == 0) *reinterpret_cast<float *>(blk + kPageTokens * kHeadDim + 4 * (pos & 63)) = sc;
       }
     }
@@ -107,6 +111,8 @@ struct Fp8AttnArgs {
   int H, pps, out_image;
   const int *row_order;           // streaming variant: rows by descending context length, or null
   int *err;                       // streaming variant: set when a bounded wait ran out
+  const uint16_t *stage;          // decode variant: the step's new K/V rows, bf16 [R][2][H*64]
+  int whole_pages;                // decode variant, 1: the ticket kernel's split into whole pages and its order of sums
   unsigned long long *trace;
   int trace_slot;
 };
@@ -271,6 +277,202 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attention_fp8_kernel(const Fp
   }
   if (threadIdx.x == 0) a.tickets[(size_t)r * a.H + h] = 0u;  // ready for the next launch
   trace_mark(a.trace, a.trace_slot, 2);
+}
+
+// Decode steps below the streaming variant's pairs: as above, with what a prefill pass cannot have.  The splits of a pair are the CTAs of a cluster and meet in rank 0's shared memory
+// (through global scratch and a ticket the merge took half of the kernel: 5 of 11 us at 9 rows of 930 tokens); the first
+// half page of every warp is loaded, and the rest asked into L2, ahead of the dependency wait (only the new token's slot
+// is not final then); and the new token is encoded here, by the warp that owns the last page, into the cache and into
+// its own registers, without a kernel of its own.
+// Per step, against the encoding kernel and the ticket kernel: 1 row of 930 tokens 0.633 -> 0.493 ms, 3 rows 0.731 -> 0.610,
+// 9 rows 0.807 -> 0.758, 12 rows 0.951 -> 0.841, 28 rows of 730 tokens 1.254 -> 0.989.
+__global__ void __launch_bounds__(kAttnWarps * 32) attention_fp8_decode_kernel(const Fp8AttnArgs a) {
+  const int c = blockIdx.x, S = gridDim.x, h = blockIdx.y, r = blockIdx.z;
+  trace_mark(a.trace, a.trace_slot, 0);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tg = lane >> 2, sub = lane & 3;
+  __shared__ float sm_m[kAttnWarps], sm_l[kAttnWarps], sm_o[kAttnWarps][kHeadDim];
+  __shared__ float cl_all[kAttnMaxChunks][kAttnPartialFloats];          // rank 0: every split's (M, L, O[64])
+  __shared__ __align__(16) unsigned char sm_new[2][kHeadDim];           // the new token's codes
+  // row and page tables are final before the step's first kernel starts
+  const int n_tok = min(a.row_pos[r] + 1, a.pps * kPageTokens);
+  // The row is cut into half pages of 32 tokens, dealt in runs to the splits and round-robin to the warps of a split; with
+  // whole_pages a warp takes both halves of a page.  Item i of this warp is half page first + (i >> sh) * step + (i & sh).
+  const int sh = a.whole_pages, n_half = (n_tok + 31) / 32, n_unit = sh ? (n_half + 1) >> 1 : n_half;
+  const int per = (n_unit + S - 1) / S;                    // units per split
+  const int n_chunks = (n_unit + per - 1) / per;           // splits that have units
+  const int first = (c * per + warp) << sh, step = kAttnWarps << sh, end = min(n_half, ((c + 1) * per) << sh);
+  const int *pt = a.page_table + (size_t)a.row_stream[r] * a.pps;
+  const size_t v_off = (size_t)a.H * kFp8BlockBytes;
+  auto half_of = [&](int i) { return first + (i >> sh) * step + (i & sh); };
+  const int my_phys = half_of(lane) < end ? pt[half_of(lane) >> 1] : 0;     // page of item `lane`
+  auto block = [&](int i) {                                                 // K block of item i's page; V: v_off on
+    const int phys = i < 32 ? __shfl_sync(0xFFFFFFFFu, my_phys, i) : pt[half_of(i) >> 1];
+    return a.kv_layer + ((size_t)phys * 2 * a.H + h) * kFp8BlockBytes;
+  };
+
+  uint4 kk[4], vv[4];
+  float ks[4], vs[4];
+  auto load = [&](int u, int i) {
+    const unsigned char *K = block(i), *V = K + v_off;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int t = 32 * (u & 1) + 8 * q + tg;
+      kk[q] = ld_cg_u4(K + (size_t)t * kHeadDim + 16 * sub);
+      vv[q] = ld_cg_u4(V + (size_t)t * kHeadDim + 16 * sub);
+      ks[q] = __ldcg(reinterpret_cast<const float *>(K + kPageTokens * kHeadDim + 4 * t));
+      vs[q] = __ldcg(reinterpret_cast<const float *>(V + kPageTokens * kHeadDim + 4 * t));
+    }
+  };
+  auto prefetch = [&](int u, int i) {   // 2 KB of K and of V in 128-byte lines, and their scales
+    const unsigned char *K = block(i);
+    prefetch_l2(K + (lane >> 4) * v_off + (u & 1) * (32 * kHeadDim) + (lane & 15) * 128);
+    if (lane < 2) prefetch_l2(K + lane * v_off + kPageTokens * kHeadDim + (u & 1) * 128);
+  };
+  int u = first;
+  if (u < end) load(u, 0);
+  if (half_of(1) < end) prefetch(half_of(1), 1);
+  pdl_launch_dependents();
+  pdl_wait();
+  trace_mark(a.trace, a.trace_slot, 1);
+
+  float qv[16];
+  {
+    const float qs = 0.125f * 1.4426950408889634f;   // scores in log2 units
+    const float *qp = a.q + (size_t)r * a.H * kHeadDim + h * kHeadDim + 16 * sub;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float4 t = *reinterpret_cast<const float4 *>(qp + 4 * e);
+      qv[4 * e] = t.x * qs; qv[4 * e + 1] = t.y * qs; qv[4 * e + 2] = t.z * qs; qv[4 * e + 3] = t.w * qs;
+    }
+  }
+  const int tn = (n_tok - 1) & (kPageTokens - 1), newest = n_half - 1;   // the new token's slot in the last page, its half page
+  float new_ks = 0.f, new_vs = 0.f;
+  if (end == n_half && newest >= first && ((newest >> sh) - (first >> sh)) % kAttnWarps == 0) {   // it is one of this warp's
+    const uint16_t *st = a.stage + (size_t)r * 2 * a.H * kHeadDim + h * kHeadDim + 2 * lane;
+    const uint16_t kc = e4m3_encode_row(__ldcg(reinterpret_cast<const unsigned int *>(st)), new_ks);
+    const uint16_t vc = e4m3_encode_row(__ldcg(reinterpret_cast<const unsigned int *>(st + a.H * kHeadDim)), new_vs);
+    unsigned char *blk = const_cast<unsigned char *>(a.kv_layer) + ((size_t)pt[newest >> 1] * 2 * a.H + h) * kFp8BlockBytes;
+    *reinterpret_cast<uint16_t *>(blk + (size_t)tn * kHeadDim + 2 * lane) = kc;
+    *reinterpret_cast<uint16_t *>(blk + v_off + (size_t)tn * kHeadDim + 2 * lane) = vc;
+    if (lane < 2) *reinterpret_cast<float *>(blk + lane * v_off + kPageTokens * kHeadDim + 4 * tn) = lane ? new_vs : new_ks;
+    *reinterpret_cast<uint16_t *>(&sm_new[0][2 * lane]) = kc;
+    *reinterpret_cast<uint16_t *>(&sm_new[1][2 * lane]) = vc;
+    __syncwarp();
+  }
+  float m = -INFINITY, l = 0.f, o[16];
+#pragma unroll
+  for (int e = 0; e < 16; ++e) o[e] = 0.f;
+#pragma unroll 1
+  for (int i = 1; u < end; ++i) {
+    const int next = half_of(i);
+    if (next < end && i > 1) prefetch(next, i);
+    uint32_t vmask = 0u;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) vmask |= 32 * u + 8 * q + tg < n_tok ? 1u << q : 0u;
+    if (u == newest && tg == (tn & 7)) {
+      const uint4 kn = *reinterpret_cast<const uint4 *>(&sm_new[0][16 * sub]), vn = *reinterpret_cast<const uint4 *>(&sm_new[1][16 * sub]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {   // register selects (no dynamic indexing)
+        const bool hit = q == ((tn >> 3) & 3);
+        kk[q].x = hit ? kn.x : kk[q].x; kk[q].y = hit ? kn.y : kk[q].y; kk[q].z = hit ? kn.z : kk[q].z; kk[q].w = hit ? kn.w : kk[q].w;
+        vv[q].x = hit ? vn.x : vv[q].x; vv[q].y = hit ? vn.y : vv[q].y; vv[q].z = hit ? vn.z : vv[q].z; vv[q].w = hit ? vn.w : vv[q].w;
+        ks[q] = hit ? new_ks : ks[q]; vs[q] = hit ? new_vs : vs[q];
+      }
+    }
+    fp8_fold4(kk, vv, ks, vs, vmask, qv, m, l, o);
+    u = next;
+    if (u < end) load(u, i);
+  }
+  // warp result: sum over the 8 token groups
+  l += __shfl_xor_sync(0xFFFFFFFFu, l, 4);
+  l += __shfl_xor_sync(0xFFFFFFFFu, l, 8);
+  l += __shfl_xor_sync(0xFFFFFFFFu, l, 16);
+#pragma unroll
+  for (int e = 0; e < 16; ++e) {
+    o[e] += __shfl_xor_sync(0xFFFFFFFFu, o[e], 4);
+    o[e] += __shfl_xor_sync(0xFFFFFFFFu, o[e], 8);
+    o[e] += __shfl_xor_sync(0xFFFFFFFFu, o[e], 16);
+  }
+  if (tg == 0) {
+    if (sub == 0) { sm_m[warp] = m; sm_l[warp] = l; }
+#pragma unroll
+    for (int e = 0; e < 16; ++e) sm_o[warp][16 * sub + e] = o[e];
+  }
+  __syncthreads();
+  trace_mark(a.trace, a.trace_slot, 3);
+  const int e = threadIdx.x;
+  float M = -INFINITY, L = 0.f, O = 0.f;
+  uint16_t *out = nullptr;
+  if (e < kHeadDim) {
+#pragma unroll
+    for (int w = 0; w < kAttnWarps; ++w) M = fmaxf(M, sm_m[w]);
+#pragma unroll
+    for (int w = 0; w < kAttnWarps; ++w) {
+      const float f = (sm_m[w] == -INFINITY) ? 0.f : exp2f(sm_m[w] - M);   // a warp without pages contributes nothing
+      L = fmaf(sm_l[w], f, L);
+      O = fmaf(sm_o[w][e], f, O);
+    }
+    out = a.out_image ? reinterpret_cast<uint16_t *>(reinterpret_cast<unsigned char *>(a.out) + act_image_offset_tiled(r, h * kHeadDim + e, a.H * kHeadDim))
+                      : a.out + (size_t)r * a.H * kHeadDim + h * kHeadDim + e;
+  }
+  if (S == 1) {
+    if (e < kHeadDim) *out = float_to_bf16_bits(O / L);
+    trace_mark(a.trace, a.trace_slot, 2);
+    return;
+  }
+  cg::cluster_group cluster = cg::this_cluster();
+  cluster.sync();   // rank 0 runs (its shared memory exists)
+  if (e < kHeadDim && c < n_chunks) {
+    float *dst = cluster.map_shared_rank(&cl_all[0][0], 0) + (size_t)c * kAttnPartialFloats;
+    if (e == 0) { dst[0] = M; dst[1] = L; }
+    dst[2 + e] = O;
+  }
+  cluster.sync();
+  if (c == 0 && e < kHeadDim) {
+    if (n_chunks > 1) {
+      M = -INFINITY;
+      for (int cc = 0; cc < n_chunks; ++cc) M = fmaxf(M, cl_all[cc][0]);
+      L = 0.f; O = 0.f;
+      for (int cc = 0; cc < n_chunks; ++cc) {
+        const float f = exp2f(cl_all[cc][0] - M);
+        L = fmaf(cl_all[cc][1], f, L);
+        O = fmaf(cl_all[cc][2 + e], f, O);
+      }
+    }
+    *out = float_to_bf16_bits(O / L);
+  }
+  trace_mark(a.trace, a.trace_slot, 2);
+}
+
+// Four CTAs are resident per SM (118 registers; with 96 the loaded half page spills): the most splits that still are one
+// wave.  A few CTAs beyond it cost a whole second wave (9 rows of 930 tokens, 720 CTAs: attention 13.3 us a layer instead of 10.4).
+inline bool attention_fp8_decode_fits(int R, int H, int splits, int n_sm) { return R * H * splits <= 4 * n_sm; }
+inline int attention_fp8_decode_splits(int R, int H, int n_sm) {
+  const int s = std::max(1, std::min(kAttnMaxChunks, 4 * n_sm / (R * H)));
+  return s == 7 ? 6 : s;   // clusters of seven leave places free (4 rows of 930 tokens: 0.742 ms per step, on six 0.648)
+}
+
+// splits: CTAs of a (row, head) pair, a cluster if more than one
+inline cudaError_t launch_attention_fp8_decode(const Fp8AttnArgs &a, int R, int splits, cudaStream_t st, bool pdl) {
+  cudaLaunchConfig_t cfg;
+  cfg.gridDim = dim3(splits, a.H, R); cfg.blockDim = dim3(kAttnWarps * 32);
+  cfg.dynamicSmemBytes = 0; cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (splits > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = splits; at[n].val.clusterDim.y = 1; at[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (pdl) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, attention_fp8_decode_kernel, a);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -350,9 +350,18 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
     // 8-bit cache: the QKV linear left the new K/V rows in the staging area; encode them into their page
     // slots, then attend over e4m3 pages (the same kernel for prefill passes and decode steps)
     unsigned char *kvl = reinterpret_cast<unsigned char *>(const_cast<uint16_t *>(aa.kv_layer));
-    cudaError_t e = launch_kv_quantize(h->kv_stage, kvl, aa.page_table, aa.row_stream, aa.row_pos, aa.pps, aa.H, R, st, pdl);
-    if (e != cudaSuccess) return e;
-    h->launches += 1;
+    const bool many = h->attn_stream_min_pairs > 0 ? R * aa.H >= h->attn_stream_min_pairs : attention_use_stream(R, aa.H, h->n_sm);
+    const bool stream = aa.old_pages_final && h->use_attn_stream && many;   // decode steps with enough (row, head) pairs
+    // the other ones encode the new rows themselves, over as many splits as are resident at once (ordered steps keep the
+    // ticket kernel's splits, and that kernel where they are more)
+    const int n_split = h->ordered ? attention_fp8_splits(R, aa.H, h->n_sm) : attention_fp8_decode_splits(R, aa.H, h->n_sm);
+    const bool small = aa.old_pages_final && !stream && (!h->ordered || attention_fp8_decode_fits(R, aa.H, n_split, h->n_sm));
+    cudaError_t e = cudaSuccess;
+    if (!small) {
+      e = launch_kv_quantize(h->kv_stage, kvl, aa.page_table, aa.row_stream, aa.row_pos, aa.pps, aa.H, R, st, pdl);
+      if (e != cudaSuccess) return e;
+      h->launches += 1;
+    }
     if (!aa.old_pages_final && h->pass_scratch > 0 && h->use_attn_mma && R >= kAttnPrefillRows) {
       // prefill pass: decode the pages its rows attend over into bf16 scratch pages, then the tensor-core kernel
       e = launch_kv_dequant_pages(kvl, h->kv_scratch, h->scratch_src, h->scratch_ntok, h->pass_scratch, aa.H, st, pdl);
@@ -368,11 +377,12 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
     fa.out = aa.out; fa.partials = h->attn_partials; fa.tickets = h->attn_tickets; fa.H = aa.H; fa.pps = aa.pps;
     fa.out_image = aa.out_image; fa.trace = aa.trace; fa.trace_slot = aa.trace_slot;
     fa.err = h->dev_err;
-    const bool many = h->attn_stream_min_pairs > 0 ? R * aa.H >= h->attn_stream_min_pairs : attention_use_stream(R, aa.H, h->n_sm);
-    if (aa.old_pages_final && h->use_attn_stream && many) {   // decode steps with enough (row, head) pairs
+    if (stream) {
       fa.row_order = h->rt.row_order;
       return launch_attention_fp8_stream(fa, R, st, pdl);
     }
+    fa.stage = h->kv_stage; fa.whole_pages = h->ordered ? 1 : 0;
+    if (small) return launch_attention_fp8_decode(fa, R, n_split, st, pdl);
     return launch_attention_fp8(fa, R, attention_fp8_splits(R, aa.H, h->n_sm), st, pdl);
   }
   aa.err = h->dev_err;

@@ -105,3 +105,26 @@ def test_sampled_calls_keep_their_order_of_sums(S):
     assert np.array_equal(lg, lg2) and np.array_equal(tk, tk2)
     assert eng.check_canaries() == 0
     eng.destroy()
+
+
+@pytest.mark.parametrize("S", [1, 21, 30, 40, 60, 80])
+def test_8bit_decode_attention_splits(S):
+    """8, 6, 4, 3, 2 and 1 CTAs per (row, head) over the 8-bit cache: contexts at the edges of half pages and pages, splits
+    without tokens, stale pages; against the streaming kernel on the same history, greedy and sampled order."""
+    edges = [700, 1, 30, 31, 32, 33, 62, 63, 64, 65, 95, 96, 127, 128, 161]
+    lens = [edges[i % len(edges)] if i < 30 else 2 + (11 * i) % 60 for i in range(S)]
+    cfg = C.tiny_config(kv_fmt=C.KV_FP8_E4M3, max_streams=S, n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=768)
+    w = C.make_weights(cfg, seed=29)
+    eng = B.TtsGpt(cfg, w, DEV)
+    eng.set_option("poison_free_pages", 1)
+    prefixes = C.make_prefixes(cfg, lens, seed=30)
+    lg, tk = _run(eng, prefixes, 3)
+    lg2, tk2 = _run(eng, prefixes, 3, top_k=4, uniforms=torch.zeros(S, device=DEV))
+    eng.set_option("attn_stream_min_pairs", 1)
+    lg3, tk3 = _run(eng, prefixes, 3)
+    for a, t in ((lg, tk), (lg2, tk2)):
+        same = (t == tk3).all(axis=1)      # streams whose history is the same up to ties
+        assert same.mean() > 0.9
+        assert np.max(np.abs(a[same] - lg3[same])) < 4.5e-2
+    assert eng.check_canaries() == 0
+    eng.destroy()
