@@ -72,8 +72,8 @@ __device__ __forceinline__ void load_page(PageLoad &pl, const uint16_t *K, const
 // token); m and l are warp-uniform, o[e] is the lane's partial over its tokens (summed over tg at
 // the very end).  At least one slot of the warp must be valid.
 // first half: scores of NS slots (log2 units, -inf for slots without a token) and their maximum over the warp
-template <int NS>
-__device__ __forceinline__ float score_slots(const uint4 (&kk)[16], const float (&qv)[8], uint32_t vmask, float (&s)[16]) {
+template <int NS, int N>
+__device__ __forceinline__ float score_slots(const uint4 (&kk)[N], const float (&qv)[8], uint32_t vmask, float (&s)[N]) {
   float pm = -INFINITY;
 #pragma unroll
   for (int i = 0; i < NS; ++i) {
@@ -97,8 +97,8 @@ __device__ __forceinline__ float score_slots(const uint4 (&kk)[16], const float 
 }
 
 // second half: rescale the running (m, l, o) to the new maximum and add the NS slots' weighted values
-template <int NS>
-__device__ __forceinline__ void accum_slots(uint4 (&vv)[16], const float (&s)[16], float pm, uint32_t vmask, float &m,
+template <int NS, int N>
+__device__ __forceinline__ void accum_slots(uint4 (&vv)[N], const float (&s)[N], float pm, uint32_t vmask, float &m,
                                             float &l, float (&o)[8]) {
   const float m_new = fmaxf(m, pm);           // finite: the caller only folds batches with a valid token
   const float rescale = exp2f(m - m_new);     // first batch: exp2(-inf) = 0
@@ -383,6 +383,134 @@ inline int attention_cluster_size(int R, int H, int n_sm, int fill = 1) {
   int s = 1;
   while (s < kAttnMaxCluster && R * H * s < fill * n_sm) s *= 2;
   return s;
+}
+
+// ------------------------------------------------------------------------------------------
+// half-page variant (decode steps whose sums need no fixed order, see attention_use_half): a pair's
+// half pages of 32 tokens dealt in runs to up to eight CTAs of a cluster, round-robin to the warps of a CTA.  A warp
+// holds 32 tokens in registers, not 64, so that four CTAs are resident per SM instead of two and the split is no longer
+// between one CTA per pair and twice as many as fit; its next half page is asked into L2 ahead of the dependency wait.
+// Per step: 8 rows of 530 tokens 0.687 -> 0.640 ms, of 1530 tokens 0.881 -> 0.763, 4 rows of 530 0.638 -> 0.583.
+// ------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(kAttnWarps * 32, 4) attention_half_kernel(const AttnArgs a) {
+  const int S = gridDim.x, c = blockIdx.x, h = blockIdx.y, r = blockIdx.z;
+  trace_mark(a.trace, a.trace_slot, 0);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tg = lane >> 3, sub = lane & 7;
+  __shared__ float sm_m[kAttnWarps], sm_l[kAttnWarps], sm_o[kAttnWarps][kHeadDim];
+  __shared__ float cl_all[kAttnMaxCluster][kAttnPartialFloats];   // rank 0: every split's (M, L, O[64])
+  // row and page tables are final before the step's first kernel starts
+  const int n_tok = a.row_pos[r] + 1, n_half = (n_tok + 31) >> 5;
+  const int per = (n_half + S - 1) / S, n_chunks = (n_half + per - 1) / per;   // half pages per split, splits that have some
+  const int first = c * per + warp, end = min(n_half, (c + 1) * per);
+  const int *pt = a.page_table + (size_t)a.row_stream[r] * a.pps;
+  auto half_of = [&](int i) { return first + i * kAttnWarps; };
+  const int my_phys = half_of(lane) < end ? pt[half_of(lane) >> 1] : 0;        // page of the warp's item `lane`
+  auto block = [&](int i) {                                                    // K rows of item i; V: v_off elements on
+    const int u = half_of(i), phys = i < 32 ? __shfl_sync(0xFFFFFFFFu, my_phys, i) : pt[u >> 1];
+    return a.kv_layer + ((size_t)phys * 2 * a.H + h) * kPageElems + (u & 1) * (32 * kHeadDim);
+  };
+  const size_t v_off = (size_t)a.H * kPageElems;
+  uint4 kk[8], vv[8];
+  auto load = [&](int i) {
+    const uint16_t *K = block(i) + tg * kHeadDim + 8 * sub;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) kk[q] = ld_cg_u4(K + (size_t)4 * q * kHeadDim);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) vv[q] = ld_cg_u4(K + v_off + (size_t)4 * q * kHeadDim);
+  };
+  auto prefetch = [&](int i) {   // 32 rows of 128 bytes of K and of V
+    const uint16_t *K = block(i) + lane * kHeadDim;
+    prefetch_l2(K);
+    prefetch_l2(K + v_off);
+  };
+  // The newest token's rows are the only ones that the step writes: everything is requested ahead of the wait, and those
+  // two are read again behind it.
+  if (half_of(0) < end) load(0);
+  if (half_of(1) < end) prefetch(1);
+  cg::cluster_group cluster = cg::this_cluster();
+  if (S > 1) cluster_arrive_relaxed();
+  pdl_launch_dependents();
+  pdl_wait();
+  trace_mark(a.trace, a.trace_slot, 1);
+  float qv[8], m = -INFINITY, l = 0.f, o[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) o[e] = 0.f;
+  load_q(qv, a.q + (size_t)r * a.H * kHeadDim + h * kHeadDim + 8 * sub);
+  const int newest = n_half - 1, tn = (n_tok - 1) & 31;
+  uint4 kn = make_uint4(0, 0, 0, 0), vn = kn;
+  if (end == n_half && newest >= first && (newest - first) % kAttnWarps == 0) {
+    const uint16_t *K = block((newest - first) / kAttnWarps) + tn * kHeadDim + 8 * sub;
+    kn = ld_cg_u4(K);
+    vn = ld_cg_u4(K + v_off);
+  }
+#pragma unroll 1
+  for (int i = 0; half_of(i) < end; ++i) {
+    const int u = half_of(i);
+    if (i > 0 && half_of(i + 1) < end) prefetch(i + 1);
+    uint32_t vmask = 0u;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) vmask |= 32 * u + 4 * q + tg < n_tok ? 1u << q : 0u;
+    if (u == newest && tg == (tn & 3)) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {   // register selects (no dynamic indexing)
+        const bool hit = q == (tn >> 2);
+        kk[q].x = hit ? kn.x : kk[q].x; kk[q].y = hit ? kn.y : kk[q].y; kk[q].z = hit ? kn.z : kk[q].z; kk[q].w = hit ? kn.w : kk[q].w;
+        vv[q].x = hit ? vn.x : vv[q].x; vv[q].y = hit ? vn.y : vv[q].y; vv[q].z = hit ? vn.z : vv[q].z; vv[q].w = hit ? vn.w : vv[q].w;
+      }
+    }
+    float s[8];
+    const float pm = score_slots<8>(kk, qv, vmask, s);
+    accum_slots<8>(vv, s, pm, vmask, m, l, o);
+    if (half_of(i + 1) < end) load(i + 1);
+  }
+  trace_mark(a.trace, a.trace_slot, 3);
+  float M, L, O;
+  cta_merge(m, l, o, warp, tg, sub, sm_m, sm_l, sm_o, M, L, O);
+  const int e = threadIdx.x;
+  uint16_t *out = a.out_image ? reinterpret_cast<uint16_t *>(reinterpret_cast<unsigned char *>(a.out) + act_image_offset_tiled(r, h * kHeadDim + (e & 63), a.H * kHeadDim))
+                              : a.out + (size_t)r * a.H * kHeadDim + h * kHeadDim + (e & 63);
+  if (S == 1) {
+    if (e < kHeadDim) *out = float_to_bf16_bits(O / L);
+    trace_mark(a.trace, a.trace_slot, 2);
+    return;
+  }
+  cluster_wait();   // every CTA of the cluster runs, so that its shared memory exists
+  if (e < kHeadDim && c < n_chunks) {
+    float *dst = cluster.map_shared_rank(&cl_all[0][0], 0) + (size_t)c * kAttnPartialFloats;
+    if (e == 0) { dst[0] = M; dst[1] = L; }
+    dst[2 + e] = O;
+  }
+  trace_mark(a.trace, a.trace_slot, 4);
+  cluster.sync();
+  if (c == 0 && e < kHeadDim) {
+    M = -INFINITY;
+    for (int k = 0; k < n_chunks; ++k) M = fmaxf(M, cl_all[k][0]);
+    L = 0.f; O = 0.f;
+    for (int k = 0; k < n_chunks; ++k) {
+      const float f = exp2f(cl_all[k][0] - M);
+      L = fmaf(cl_all[k][1], f, L);
+      O = fmaf(cl_all[k][2 + e], f, O);
+    }
+    *out = float_to_bf16_bits(O / L);
+  }
+  trace_mark(a.trace, a.trace_slot, 2);
+}
+
+// Four CTAs of the half-page kernels are resident per SM: the most splits that still are one wave.
+inline bool attention_half_fits(int R, int H, int splits, int n_sm) { return R * H * splits <= 4 * n_sm; }
+inline int attention_half_splits(int R, int H, int n_sm) {
+  const int s = std::max(1, std::min(kAttnMaxCluster, 4 * n_sm / (R * H)));
+  return s == 7 ? 6 : s;   // clusters of seven leave places free (8-bit cache, 4 rows of 930 tokens: 0.742 ms per step, on six 0.648)
+}
+// Where power-of-two clusters of the kernel above fill at most two thirds of its places, two per SM (160 CTAs at 2, 4
+// and 8 rows of 20 heads, 180 at 9), yet every SM; one row is as fast on the kernel above.  Where they fill more the halves gain nothing (3 rows of 530 tokens 0.591 against
+// 0.601 ms per step, 6 rows of 930 0.727 against 0.733, 12 rows of 530 0.808 against 0.819).
+inline bool attention_use_half(int R, int H, int n_sm) {
+  const int grid = R * H * attention_cluster_size(R, H, n_sm);
+  return R > 1 && grid >= n_sm && 3 * grid <= 4 * n_sm;
+}
+inline cudaError_t launch_attention_half(const AttnArgs &a, int R, int splits, cudaStream_t st, bool pdl) {
+  return launch_kernel_cluster(attention_half_kernel, dim3(splits, a.H, R), dim3(kAttnWarps * 32), splits, st, pdl, a);
 }
 
 inline cudaError_t launch_attention(const AttnArgs &a, int R, int cluster, cudaStream_t st, bool pdl) {

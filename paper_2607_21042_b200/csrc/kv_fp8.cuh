@@ -332,6 +332,8 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attention_fp8_decode_kernel(c
   int u = first;
   if (u < end) load(u, 0);
   if (half_of(1) < end) prefetch(half_of(1), 1);
+  cg::cluster_group cluster = cg::this_cluster();
+  if (S > 1) cluster_arrive_relaxed();
   pdl_launch_dependents();
   pdl_wait();
   trace_mark(a.trace, a.trace_slot, 1);
@@ -421,8 +423,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attention_fp8_decode_kernel(c
     trace_mark(a.trace, a.trace_slot, 2);
     return;
   }
-  cg::cluster_group cluster = cg::this_cluster();
-  cluster.sync();   // rank 0 runs (its shared memory exists)
+  cluster_wait();   // every CTA of the cluster runs, so that its shared memory exists
   if (e < kHeadDim && c < n_chunks) {
     float *dst = cluster.map_shared_rank(&cl_all[0][0], 0) + (size_t)c * kAttnPartialFloats;
     if (e == 0) { dst[0] = M; dst[1] = L; }
@@ -445,34 +446,10 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attention_fp8_decode_kernel(c
   trace_mark(a.trace, a.trace_slot, 2);
 }
 
-// Four CTAs are resident per SM (118 registers; with 96 the loaded half page spills): the most splits that still are one
-// wave.  A few CTAs beyond it cost a whole second wave (9 rows of 930 tokens, 720 CTAs: attention 13.3 us a layer instead of 10.4).
-inline bool attention_fp8_decode_fits(int R, int H, int splits, int n_sm) { return R * H * splits <= 4 * n_sm; }
-inline int attention_fp8_decode_splits(int R, int H, int n_sm) {
-  const int s = std::max(1, std::min(kAttnMaxChunks, 4 * n_sm / (R * H)));
-  return s == 7 ? 6 : s;   // clusters of seven leave places free (4 rows of 930 tokens: 0.742 ms per step, on six 0.648)
-}
-
-// splits: CTAs of a (row, head) pair, a cluster if more than one
+// (9 rows of 930 tokens as 720 CTAs, a few beyond one wave: attention 13.3 us a layer instead of 10.4; with 96 registers
+// and five CTAs per SM the loaded half page spills)
 inline cudaError_t launch_attention_fp8_decode(const Fp8AttnArgs &a, int R, int splits, cudaStream_t st, bool pdl) {
-  cudaLaunchConfig_t cfg;
-  cfg.gridDim = dim3(splits, a.H, R); cfg.blockDim = dim3(kAttnWarps * 32);
-  cfg.dynamicSmemBytes = 0; cfg.stream = st;
-  cudaLaunchAttribute at[2];
-  int n = 0;
-  if (splits > 1) {
-    at[n].id = cudaLaunchAttributeClusterDimension;
-    at[n].val.clusterDim.x = splits; at[n].val.clusterDim.y = 1; at[n].val.clusterDim.z = 1;
-    ++n;
-  }
-  if (pdl) {
-    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[n].val.programmaticStreamSerializationAllowed = 1;
-    ++n;
-  }
-  cfg.attrs = at;
-  cfg.numAttrs = n;
-  return cudaLaunchKernelEx(&cfg, attention_fp8_decode_kernel, a);
+  return launch_kernel_cluster(attention_fp8_decode_kernel, dim3(splits, a.H, R), dim3(kAttnWarps * 32), splits, st, pdl, a);
 }
 
 // ------------------------------------------------------------------------------------------

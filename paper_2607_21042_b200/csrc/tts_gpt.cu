@@ -117,6 +117,7 @@ struct tts_gpt {
   // order.  Greedy calls are free of that and take the faster kernels.
   bool ordered = false;          // set by each prefill and decode call
   int ordered_pass_rows = 896;
+  bool use_attn_half = true;     // half-page attention of decode steps (option "attn_half")
   bool use_attn_decode = true;   // unit-split tensor-pipe attention of decode steps (option "attn_decode")
   bool use_attn_stream = true;   // streaming attention for large batches (option "attn_stream")
   int attn_cluster_fill = 1;     // clusters grow until the grid covers the GPU this many times
@@ -350,12 +351,15 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
     // 8-bit cache: the QKV linear left the new K/V rows in the staging area; encode them into their page
     // slots, then attend over e4m3 pages (the same kernel for prefill passes and decode steps)
     unsigned char *kvl = reinterpret_cast<unsigned char *>(const_cast<uint16_t *>(aa.kv_layer));
-    const bool many = h->attn_stream_min_pairs > 0 ? R * aa.H >= h->attn_stream_min_pairs : attention_use_stream(R, aa.H, h->n_sm);
+    // streaming: beyond the bf16 cache's line, and (steps free in their sums) where its pairs are one wave of three CTAs per
+    // SM and no split fits the other kernel (18 rows of 930 tokens 0.939 against 1.037 ms per step)
+    const bool one_wave = !h->ordered && R * aa.H > 2 * h->n_sm && R * aa.H <= 3 * h->n_sm;
+    const bool many = h->attn_stream_min_pairs > 0 ? R * aa.H >= h->attn_stream_min_pairs : one_wave || attention_use_stream(R, aa.H, h->n_sm);
     const bool stream = aa.old_pages_final && h->use_attn_stream && many;   // decode steps with enough (row, head) pairs
     // the other ones encode the new rows themselves, over as many splits as are resident at once (ordered steps keep the
     // ticket kernel's splits, and that kernel where they are more)
-    const int n_split = h->ordered ? attention_fp8_splits(R, aa.H, h->n_sm) : attention_fp8_decode_splits(R, aa.H, h->n_sm);
-    const bool small = aa.old_pages_final && !stream && (!h->ordered || attention_fp8_decode_fits(R, aa.H, n_split, h->n_sm));
+    const int n_split = h->ordered ? attention_fp8_splits(R, aa.H, h->n_sm) : attention_half_splits(R, aa.H, h->n_sm);
+    const bool small = aa.old_pages_final && !stream && (!h->ordered || attention_half_fits(R, aa.H, n_split, h->n_sm));
     cudaError_t e = cudaSuccess;
     if (!small) {
       e = launch_kv_quantize(h->kv_stage, kvl, aa.page_table, aa.row_stream, aa.row_pos, aa.pps, aa.H, R, st, pdl);
@@ -395,6 +399,8 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
   if (!aa.old_pages_final && h->use_attn_prefill && R >= kAttnPrefillRows) return launch_attention_prefill(aa, R, st, pdl);
   if (aa.old_pages_final && h->use_attn_decode && !h->ordered && h->attn_stream_min_pairs == 0 && attention_use_decode(R, aa.H, h->n_sm))
     return launch_attention_decode(aa, R, h->kv_map, (int)((aa.kv_layer - h->kv) / kHeadDim), h->n_sm, st, pdl);
+  if (aa.old_pages_final && h->use_attn_half && !h->ordered && h->attn_stream_min_pairs == 0 && attention_use_half(R, aa.H, h->n_sm))
+    return launch_attention_half(aa, R, attention_half_splits(R, aa.H, h->n_sm), st, pdl);
   const bool stream = h->attn_stream_min_pairs > 0 ? R * aa.H >= h->attn_stream_min_pairs : attention_use_stream(R, aa.H, h->n_sm);
   if (h->use_attn_stream && stream) return launch_attention_stream(aa, R, st, pdl);
   return launch_attention(aa, R, attention_cluster_size(R, aa.H, h->n_sm, h->attn_cluster_fill), st, pdl);
@@ -1232,6 +1238,7 @@ int32_t tts_gpt_debug_set_option(tts_gpt_t *h, const char *name, int32_t value) 
   else if (k == "attn_mma") h->use_attn_mma = on;
   else if (k == "attn_prefill") h->use_attn_prefill = on;
   else if (k == "attn_decode") h->use_attn_decode = on;
+  else if (k == "attn_half") h->use_attn_half = on;
   else if (k == "attn_stream") h->use_attn_stream = on;
   else if (k == "attn_stream_min_pairs") h->attn_stream_min_pairs = value > 0 ? value : 0;
   else if (k == "attn_cluster_fill") h->attn_cluster_fill = value > 0 ? value : 1;

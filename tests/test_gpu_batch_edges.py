@@ -128,3 +128,22 @@ def test_8bit_decode_attention_splits(S):
         assert np.max(np.abs(a[same] - lg3[same])) < 4.5e-2
     assert eng.check_canaries() == 0
     eng.destroy()
+
+
+@pytest.mark.parametrize("S", [5, 21, 37, 49])
+def test_half_page_decode_attention(S):
+    """8, 6, 4 and 3 CTAs per (row, head) over the bf16 cache: contexts at the edges of half pages and pages, splits without
+    tokens, stale pages full of NaN behind every context."""
+    edges = [700, 1, 30, 31, 32, 33, 62, 63, 64, 65, 95, 96, 127, 128, 161]
+    lens = [edges[i % len(edges)] if i < 30 else 2 + (11 * i) % 60 for i in range(S)]
+    cfg = C.tiny_config(max_streams=S, n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=768)
+    w = C.make_weights(cfg, seed=31)
+    model = O.OracleModel(cfg, w)
+    eng = B.TtsGpt(cfg, w, DEV)
+    eng.set_option("poison_free_pages", 1)
+    prefixes = C.make_prefixes(cfg, lens, seed=32)
+    lg, tk = _run(eng, prefixes, 4)
+    _check(model, prefixes, lg, tk, sorted(set(range(min(S, 15))) | {S - 1}), "half-page attention")
+    lg2, _ = _run(eng, prefixes, 4)
+    assert np.array_equal(lg, lg2)
+    eng.destroy()
