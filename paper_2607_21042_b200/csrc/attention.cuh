@@ -390,7 +390,8 @@ inline int attention_cluster_size(int R, int H, int n_sm, int fill = 1) {
 // half pages of 32 tokens dealt in runs to up to eight CTAs of a cluster, round-robin to the warps of a CTA.  A warp
 // holds 32 tokens in registers, not 64, so that four CTAs are resident per SM instead of two and the split is no longer
 // between one CTA per pair and twice as many as fit; its next half page is asked into L2 ahead of the dependency wait.
-// Per step: 8 rows of 530 tokens 0.687 -> 0.640 ms, of 1530 tokens 0.881 -> 0.763, 4 rows of 530 0.638 -> 0.583.
+// Per step: 8 rows of 530 tokens 0.687 -> 0.640 ms, of 1530 tokens 0.881 -> 0.763, 4 rows of 530 0.638 -> 0.583, 3 rows of
+// 1730 (int4 weights) 0.674 -> 0.640, 10 rows of 930 0.895 -> 0.843.
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kAttnWarps * 32, 4) attention_half_kernel(const AttnArgs a) {
   const int S = gridDim.x, c = blockIdx.x, h = blockIdx.y, r = blockIdx.z;
@@ -502,12 +503,11 @@ inline int attention_half_splits(int R, int H, int n_sm) {
   const int s = std::max(1, std::min(kAttnMaxCluster, 4 * n_sm / (R * H)));
   return s == 7 ? 6 : s;   // clusters of seven leave places free (8-bit cache, 4 rows of 930 tokens: 0.742 ms per step, on six 0.648)
 }
-// Where power-of-two clusters of the kernel above fill at most two thirds of its places, two per SM (160 CTAs at 2, 4
-// and 8 rows of 20 heads, 180 at 9), yet every SM; one row is as fast on the kernel above.  Where they fill more the halves gain nothing (3 rows of 530 tokens 0.591 against
-// 0.601 ms per step, 6 rows of 930 0.727 against 0.733, 12 rows of 530 0.808 against 0.819).
+// Two rows and more whose pairs the kernel above spreads over every SM, up to the middle batches' kernel.  One row is as
+// fast there, and so are short contexts (3 rows of 230 tokens 0.569 against 0.574 ms per step, 10 rows of 230 0.654
+// against 0.662; 10 rows of 930 0.895 against 0.843).
 inline bool attention_use_half(int R, int H, int n_sm) {
-  const int grid = R * H * attention_cluster_size(R, H, n_sm);
-  return R > 1 && grid >= n_sm && 3 * grid <= 4 * n_sm;
+  return R > 1 && R * H <= 2 * n_sm && R * H * attention_cluster_size(R, H, n_sm) >= n_sm;
 }
 inline cudaError_t launch_attention_half(const AttnArgs &a, int R, int splits, cudaStream_t st, bool pdl) {
   return launch_kernel_cluster(attention_half_kernel, dim3(splits, a.H, R), dim3(kAttnWarps * 32), splits, st, pdl, a);
