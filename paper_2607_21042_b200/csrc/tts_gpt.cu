@@ -901,7 +901,7 @@ static int prefill_impl(tts_gpt_t *h, int32_t n, const void *const *emb, const i
   // with a last unit of up to 128 rows apart and the head unit by unit.  (Over the 8-bit cache a pass is one unit: how many
   // pages it reaches decides which attention it takes.)
   const int unit = h->ordered ? std::min(pass_rows, h->ordered_pass_rows) : 0;
-  if (unit) pass_rows = h->kv_fp8 ? unit : pass_rows / unit * unit;
+  if (unit) pass_rows = h->kv_fp8 ? unit : std::max(unit, std::min(pass_rows, kMaxOrderedRows) / unit * unit);
   int left = 0;            // rows not yet in a pass
   for (int i = 0; i < n; ++i) left += plen[i];
   PassParams ps;
