@@ -247,7 +247,6 @@ size_t carve(tts_gpt *h, void *base) {
   rt.row_order = cv.take<int>(kMaxRows);
   h->io = cv.take<StepIO>(1);
   h->x = cv.take<float>((size_t)kMaxPassRows * d);
-  h->q = cv.take<float>((size_t)kMaxPassRows * d);
   h->logits = cv.take<float>((size_t)kMaxRows * V);
   h->st_in = cv.take<int>(kMaxRows);
   h->st_tok = cv.take<int>(kMaxRows);
@@ -276,8 +275,12 @@ size_t carve(tts_gpt *h, void *base) {
     h->h_img = cv.take<char>(kTiles * act_image_bytes(F));
     h->hf_img = cv.take<char>(act_image_bytes(d));
     h->partials_floats = (size_t)kMaxSplitTiles * kMaxRows * d;   // [row tile][k-range][128][d]
+    // q lives from the QKV linear to the attention, partial sums from a residual linear to the LayerNorm behind it: never
+    // at the same time, so q's rows and q's image lie in the partial sums' memory
+    static_assert(kMaxSplitTiles * kMaxRows * 4 >= kMaxPassRows * 4 + kMaxPassRows * 2, "q rows and q image fit");
     h->partials = cv.take<float>(h->partials_floats);
-    h->q_img = cv.take<char>(kTiles * act_image_bytes(d));
+    h->q = h->partials;
+    h->q_img = reinterpret_cast<char *>(h->q + (size_t)kMaxPassRows * d);
   }
   return cv.off;
 }
