@@ -241,6 +241,14 @@ int32_t tts_gpt_debug_set_option(tts_gpt_t *h, const char *name, int32_t value);
  * clears the word; the engine and the CUDA context stay usable.  Nothing hangs or faults. */
 int32_t tts_gpt_debug_expire_wait(tts_gpt_t *h, uint32_t limit_us);
 
+/* Test aid for the same path inside the linear of large prefill passes: runs the QKV linear of layer 0 on the
+ * activation rows of the last prefill pass, rows (1..256) of them, into out (DEVICE fp32 [rows][3d], 16-byte
+ * aligned), as tiles of rows x 128 features on two pairs of CTAs, each pair taking every second tile.  tile >= 0: that
+ * tile's copies are announced 16 bytes longer than they are, its pair's issuing warp gives up after limit_us
+ * microseconds (1..100000), and neither that tile nor the pair's later ones are stored; the next tts_gpt_sync returns
+ * TTS_GPT_E_TIMEOUT once.  tile -1: a whole run.  Nothing hangs or faults. */
+int32_t tts_gpt_debug_expire_pair(tts_gpt_t *h, int32_t rows, int32_t tile, uint32_t limit_us, float *out);
+
 /* ---------------------------------------------------------------------------------------------
  * Single-kernel entry points: the building blocks of the step, callable on their own (unit parity
  * tests, micro-benchmarks).  All pointers DEVICE unless marked HOST; `cuda_stream` as above; each

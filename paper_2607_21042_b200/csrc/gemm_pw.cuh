@@ -7,7 +7,12 @@
 // CTA 0's issuer waits on one barrier per stage for both CTAs' copies.  A pair of CTAs walks the tiles; warp 0 of each
 // keeps a ring of stages full across tile boundaries, warp 1 of CTA 0 issues the instructions, and warps 2-9 of each
 // drain one of two accumulators in tensor memory while the other fills, so that the epilogue of a tile and the first
-// copies of the next run under the instructions.  Every wait is bounded.
+// copies of the next run under the instructions.
+//
+// Every wait is bounded.  A role acts only behind a wait that was satisfied; where one expires, the roles of both CTAs
+// stop (going on would arrive on barriers whose phase is still open, which is a fault).  The issuer then commits
+// nothing more, so that a tile is stored, by either CTA, only if every wait in front of its accumulator was satisfied.
+// A pair that gave up stays until the copies it requested have landed in its shared memory.
 //
 // What bounds it.  One CTA per 128 x 256 tile is bound by shared memory: an instruction of K = 16 reads 12 KB of
 // operands in 128 cycles and its copies write another 12 KB, 192 of 128 bytes per cycle; measured 0.40 us per k-chunk
@@ -27,6 +32,7 @@ constexpr int kPwThreads = 320;             // warp 0 producer, warp 1 issuer, w
 constexpr int kPwMaxStages = 8;
 constexpr uint32_t kPwRingBytes = 6 * 32768;             // per CTA: 6 stages at BN = 256, 8 at BN = 128
 constexpr uint32_t kPwPatchBytes = 8 * 4096;             // 4 KB per epilogue warp
+constexpr unsigned long long kPwLingerNs = 10000000ull;  // a pair that gave up: a copy in flight needs microseconds
 inline size_t pw_smem_bytes() { return (size_t)kPwRingBytes + kPwPatchBytes + 1024 + 512; }
 inline int pw_stages(int bn) { return std::min(kPwMaxStages, (int)(kPwRingBytes / (16384u + (uint32_t)bn * 64u))); }
 
@@ -51,8 +57,9 @@ __device__ __forceinline__ PwTile pw_tile(const GemmTcArgs &a, int t, int n_rp, 
 // half lies in one 128-row block of the image); a half past the last feature is not copied: its accumulator columns are
 // not stored
 __device__ __forceinline__ bool pw_half_exists(const GemmTcArgs &a, int n0, int rank) { return n0 + rank * (a.bn >> 1) < a.N; }
-__device__ __forceinline__ uint32_t pw_pair_bytes(const GemmTcArgs &a, const PwTile &p) {   // of a stage, both CTAs together; p: CTA 0's view
-  return 16384u + (a.B > p.row0 + kMaxRows ? 16384u : 0u) + (uint32_t)(a.bn >> 1) * 128u * (pw_half_exists(a, p.n0, 1) ? 2u : 1u);
+__device__ __forceinline__ uint32_t pw_pair_bytes(const GemmTcArgs &a, const PwTile &p, int t) {   // of a stage of tile t, both CTAs together; p: CTA 0's view
+  const uint32_t starved = t + 1 == a.starve ? 16u : 0u;   // test aid: bytes that never arrive
+  return 16384u + (a.B > p.row0 + kMaxRows ? 16384u : 0u) + (uint32_t)(a.bn >> 1) * 128u * (pw_half_exists(a, p.n0, 1) ? 2u : 1u) + starved;
 }
 // An operand image as a two-dimensional tensor: rows of 64 bf16 (128 bytes), blocks one behind the other.  The bytes
 // are already in the order the tensor core wants, so the copy itself does not swizzle.  Both CTAs of a pair complete
@@ -74,23 +81,10 @@ __device__ __forceinline__ void mbar_arrive_remote(uint64_t *bar, uint32_t rank)
   asm volatile("{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, %1;\n\tmbarrier.arrive.release.cluster.shared::cluster.b64 _, [ra];\n\t}"
                ::"r"(smem_u32(bar)), "r"(rank) : "memory");
 }
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t *bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-               : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ void tc_wait_cluster(uint64_t *bar, uint32_t parity, volatile int *failed, int *err) {
-  if (mbar_try_wait_cluster(bar, parity)) return;
-  const unsigned long long t0 = global_timer_ns();
-  while (!mbar_try_wait_cluster(bar, parity)) {
-    if (*failed) return;
-    if (global_timer_ns() - t0 > kTcWaitNs) {
-      *failed = 1;
-      if (err) atomicExch(err, 1);
-      return;
-    }
-  }
+// sets the flag of CTA `rank` of the pair
+__device__ __forceinline__ void pw_tell(volatile int *failed, uint32_t rank) {
+  asm volatile("{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, %1;\n\tst.relaxed.cluster.shared::cluster.u32 [ra], 1;\n\t}"
+               ::"r"(smem_u32(const_cast<const int *>(failed))), "r"(rank) : "memory");
 }
 __device__ __forceinline__ void tmem_alloc2(uint32_t *dst_smem, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)), "r"(ncols) : "memory");
@@ -256,7 +250,7 @@ __global__ void __launch_bounds__(kPwThreads, 1) gemm_pw_kernel(const __grid_con
     pre = min(p.n_it, n_stage);
     for (int i = 0; i < pre; ++i)
       if (elect_one()) {
-        if (rank == 0) mbar_expect_tx(full + i, pw_pair_bytes(a, p));
+        if (rank == 0) mbar_expect_tx(full + i, pw_pair_bytes(a, p, pair));
         if (pw_half_exists(a, p.n0, rank)) pw_copy_weights(&w_map, a, p.n0, rank, p.kc0 + i, KC, ring + (size_t)i * stage_bytes + 16384, full0 + 8u * i);
       }
     __syncwarp();
@@ -268,14 +262,15 @@ __global__ void __launch_bounds__(kPwThreads, 1) gemm_pw_kernel(const __grid_con
   if (warp == 0) {
     int it = 0, s = 0;         // stages handed out so far, over all tiles; the next stage
     uint32_t parity = 1;       // of the phase that frees it (a fresh barrier's phase before its first counts as complete)
-    for (int t = pair; t < n_tile; t += n_pair) {
+    bool go = true;
+    for (int t = pair; go && t < n_tile; t += n_pair) {
       const PwTile p = pw_tile(a, t, n_rp, rank, KC);
       const int xrow = ((p.row0 >> 7) * KC + p.kc0) * kMaxRows;
-      const uint32_t bytes = pw_pair_bytes(a, p);   // used by CTA 0 only
+      const uint32_t bytes = pw_pair_bytes(a, p, t);   // used by CTA 0 only
       const bool w_mine = pw_half_exists(a, p.n0, rank);
       for (int i = 0; i < p.n_it; ++i, ++it) {
         unsigned char *st = ring + (size_t)s * stage_bytes;
-        tc_wait(empty + s, parity, failed, a.err);
+        if (!(go = tc_wait_warp<false>(empty + s, parity, failed, a.err))) break;
         if (elect_one()) {
           if (it >= pre) {
             if (rank == 0) mbar_expect_tx(full + s, bytes);
@@ -297,12 +292,14 @@ __global__ void __launch_bounds__(kPwThreads, 1) gemm_pw_kernel(const __grid_con
       const uint32_t idesc = tc_instr_desc(256, a.bn);
       int s = 0, k = 0;
       uint32_t parity = 0;
-      for (int t = pair; t < n_tile; t += n_pair, ++k) {
+      const unsigned long long limit = a.issue_wait_ns ? a.issue_wait_ns : kTcWaitNs;
+      bool go = true;
+      for (int t = pair; go && t < n_tile; t += n_pair, ++k) {
         const PwTile p = pw_tile(a, t, n_rp, rank, KC);
         const uint32_t dst = tmem_d + 256u * (uint32_t)(k & 1);
-        if (k >= 2) tc_wait_cluster(acc_free + (k & 1), (uint32_t)((k >> 1) - 1) & 1u, failed, a.err);
+        if (k >= 2 && !tc_wait_warp<true>(acc_free + (k & 1), (uint32_t)((k >> 1) - 1) & 1u, failed, a.err, limit)) break;
         for (int i = 0; i < p.n_it; ++i) {
-          tc_wait_cluster(full + s, parity, failed, a.err);
+          if (!(go = tc_wait_warp<true>(full + s, parity, failed, a.err, limit))) break;
           tc_fence_after_sync();
           const unsigned char *st = ring + (size_t)s * stage_bytes;
           const uint64_t da = tc_smem_desc(st), db = tc_smem_desc(st + 16384);
@@ -357,12 +354,12 @@ __global__ void __launch_bounds__(kPwThreads, 1) gemm_pw_kernel(const __grid_con
         }
         bias2[q >> 1][q & 1] = bw; scale2[q >> 1][q & 1] = sw;
       }
-      tc_wait(acc_full + (k & 1), (uint32_t)(k >> 1) & 1u, failed, a.err);   // committed by CTA 0 to both CTAs
+      if (!tc_wait_warp<false>(acc_full + (k & 1), (uint32_t)(k >> 1) & 1u, failed, a.err)) break;   // committed by CTA 0 to both CTAs
       if (k == 0) trace_mark(a.trace, a.trace_slot, 4, 64);   // first accumulator complete
       tc_fence_after_sync();
       __syncwarp();
       const uint32_t t_row = tmem_d + 256u * (uint32_t)(k & 1) + ((uint32_t)(lw * 32) << 16);
-      const bool store = rows > 0 && !__any_sync(0xFFFFFFFFu, *failed);   // nothing is stored after an expired wait
+      const bool store = rows > 0;
 #pragma unroll 1
       for (int n64 = p.n0 + grp * 64; n64 < n_end; n64 += 128) {
         const bool second = n64 - p.n0 >= 128;
@@ -417,6 +414,11 @@ __global__ void __launch_bounds__(kPwThreads, 1) gemm_pw_kernel(const __grid_con
   }
   tc_fence_before_sync();
   __syncthreads();
+  if (warp == 0 && __any_sync(0xFFFFFFFFu, *failed)) {
+    pw_tell(failed, rank ^ 1);
+    const unsigned long long t0 = global_timer_ns();
+    while (__any_sync(0xFFFFFFFFu, global_timer_ns() - t0 <= kPwLingerNs)) {}
+  }
   cluster_barrier();   // neither CTA leaves, nor frees tensor memory, while the other still arrives on its barriers or computes
   trace_mark(a.trace, a.trace_slot, 2, 64);
   if (warp == 0) tmem_dealloc2(tmem_d, 512);

@@ -264,6 +264,8 @@ struct GemmTcArgs {
   const int *page_table, *row_stream, *row_pos;
   int pps, d, H;
   int *err;
+  int starve;                 // pair kernel, test aid: 1 + the tile whose copies are never complete (0: none) ...
+  unsigned long long issue_wait_ns;   // ... and how long its issuer then waits (0: as long as everything else)
   unsigned long long *trace;  // optional timeline trace (see trace_mark)
   int trace_slot;
 };
@@ -293,6 +295,31 @@ __device__ __forceinline__ void tc_wait(uint64_t *bar, uint32_t parity, volatile
       return;
     }
   }
+}
+
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t *bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+  return ok != 0;
+}
+// A warp's wait, the same answer in every lane: whether the barrier's phase has completed.  False once a wait of the CTA
+// has expired, or after limit_ns.  CLUSTER: the other CTA's threads arrive on the barrier too.  (The vote belongs here: as a
+// vote of the caller's behind the wait it cost 0.7 us a launch, and an issuing lane that goes by its own answer as much.)
+template <bool CLUSTER>
+__device__ __forceinline__ bool tc_wait_warp(uint64_t *bar, uint32_t parity, volatile int *failed, int *err, unsigned long long limit_ns = kTcWaitNs) {
+  auto complete = [&]() { return __all_sync(0xFFFFFFFFu, CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity)) != 0; };
+  if (complete()) return true;
+  const unsigned long long t0 = global_timer_ns();
+  while (!complete()) {
+    if (__any_sync(0xFFFFFFFFu, *failed)) return false;
+    if (__any_sync(0xFFFFFFFFu, global_timer_ns() - t0 > limit_ns)) {
+      *failed = 1;
+      if (err) atomicExch(err, 1);
+      return false;
+    }
+  }
+  return true;
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {

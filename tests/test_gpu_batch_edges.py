@@ -73,6 +73,39 @@ def test_prefill_passes_of_the_pair_kernel(wfmt, lens):
     eng.destroy()
 
 
+@pytest.mark.parametrize("rows,tile", [(200, 0), (200, 2), (256, 3), (100, 5)])
+def test_pair_kernel_stores_nothing_behind_an_expired_wait(rows, tile):
+    """The issuing warp of one pair of CTAs gives up on a tile: neither CTA stores that tile or a later one of the pair,
+    the other pair's tiles and the earlier ones are whole, the error is reported once and the engine goes on."""
+    cfg = C.tiny_config(max_streams=1, n_pages=8)       # QKV: 768 features, six tiles, three for each of the two pairs
+    eng = B.TtsGpt(cfg, C.make_weights(cfg, seed=33), DEV)
+    prefix = C.make_prefixes(cfg, [256], seed=34)
+    lg, tk = _run(eng, prefix, 0)
+    mark = -12345.0
+    whole = torch.full((rows, 768), mark, device=DEV)
+    out = torch.full((rows, 768), mark, device=DEV)
+    torch.cuda.synchronize()
+    eng.debug_expire_pair(rows, -1, 1000, whole)
+    eng.sync()
+    assert not bool((whole == mark).any()) and bool(torch.isfinite(whole).all())
+    eng.debug_expire_pair(rows, tile, 1000, out)
+    with pytest.raises(B.TtsGptError) as e:
+        eng.sync()
+    assert e.value.code == B.E_TIMEOUT
+    for t in range(6):
+        got, want = out[:, 128 * t:128 * t + 128], whole[:, 128 * t:128 * t + 128]
+        lost = t >= tile and (t - tile) % 2 == 0
+        assert bool((got == mark).all()) if lost else bool(torch.equal(got, want)), t
+    eng.sync()
+    lg2, tk2 = _run(eng, prefix, 0)
+    assert np.array_equal(lg, lg2) and np.array_equal(tk, tk2)
+    for bad in ((0, 0, 1000), (257, 0, 1000), (200, 6, 1000), (200, 0, 0)):
+        with pytest.raises(B.TtsGptError) as e:
+            eng.debug_expire_pair(*bad, out)
+        assert e.value.code == B.E_ARG
+    eng.destroy()
+
+
 def test_prefill_pair_kernel_with_the_8bit_cache_and_k_ranges():
     """A model width at which the residual linears of a large pass take k-ranges, K/V rows through the staging array."""
     cfg = C.tiny_config(d_model=512, n_head=8, d_ff=2048, kv_fmt=C.KV_FP8_E4M3, max_streams=2, n_pages=40, max_context=1216, max_pos=1216)
