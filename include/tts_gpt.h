@@ -246,7 +246,8 @@ int32_t tts_gpt_debug_expire_wait(tts_gpt_t *h, uint32_t limit_us);
  * aligned), as tiles of rows x 128 features on two pairs of CTAs, each pair taking every second tile.  tile >= 0: that
  * tile's copies are announced 16 bytes longer than they are, its pair's issuing warp gives up after limit_us
  * microseconds (1..100000), and neither that tile nor the pair's later ones are stored; the next tts_gpt_sync returns
- * TTS_GPT_E_TIMEOUT once.  tile -1: a whole run.  Nothing hangs or faults. */
+ * TTS_GPT_E_TIMEOUT once.  tile -1: a whole run.  tile -2: a whole run, on tiles of 256 features, in
+ * which the second CTA of a pair comes to each of its tiles limit_us late (nothing expires).  Nothing hangs or faults. */
 int32_t tts_gpt_debug_expire_pair(tts_gpt_t *h, int32_t rows, int32_t tile, uint32_t limit_us, float *out);
 
 /* ---------------------------------------------------------------------------------------------

@@ -32,6 +32,7 @@ constexpr int kPwThreads = 320;             // warp 0 producer, warp 1 issuer, w
 constexpr int kPwMaxStages = 8;
 constexpr uint32_t kPwRingBytes = 6 * 32768;             // per CTA: 6 stages at BN = 256, 8 at BN = 128
 constexpr uint32_t kPwPatchBytes = 8 * 4096;             // 4 KB per epilogue warp
+constexpr uint32_t kPwTokenBytes = 8192;                 // a CTA with neither rows nor weights in a tile copies one box all the same
 constexpr unsigned long long kPwLingerNs = 10000000ull;  // a pair that gave up: a copy in flight needs microseconds
 inline size_t pw_smem_bytes() { return (size_t)kPwRingBytes + kPwPatchBytes + 1024 + 512; }
 inline int pw_stages(int bn) { return std::min(kPwMaxStages, (int)(kPwRingBytes / (16384u + (uint32_t)bn * 64u))); }
@@ -59,7 +60,8 @@ __device__ __forceinline__ PwTile pw_tile(const GemmTcArgs &a, int t, int n_rp, 
 __device__ __forceinline__ bool pw_half_exists(const GemmTcArgs &a, int n0, int rank) { return n0 + rank * (a.bn >> 1) < a.N; }
 __device__ __forceinline__ uint32_t pw_pair_bytes(const GemmTcArgs &a, const PwTile &p, int t) {   // of a stage of tile t, both CTAs together; p: CTA 0's view
   const uint32_t starved = t + 1 == a.starve ? 16u : 0u;   // test aid: bytes that never arrive
-  return 16384u + (a.B > p.row0 + kMaxRows ? 16384u : 0u) + (uint32_t)(a.bn >> 1) * 128u * (pw_half_exists(a, p.n0, 1) ? 2u : 1u) + starved;
+  const bool half1 = pw_half_exists(a, p.n0, 1);
+  return 16384u + (a.B > p.row0 + kMaxRows ? 16384u : half1 ? 0u : kPwTokenBytes) + (uint32_t)(a.bn >> 1) * 128u * (half1 ? 2u : 1u) + starved;
 }
 // An operand image as a two-dimensional tensor: rows of 64 bf16 (128 bytes), blocks one behind the other.  The bytes
 // are already in the order the tensor core wants, so the copy itself does not swizzle.  Both CTAs of a pair complete
@@ -260,29 +262,43 @@ __global__ void __launch_bounds__(kPwThreads, 1) gemm_pw_kernel(const __grid_con
   trace_mark(a.trace, a.trace_slot, 1);
 
   if (warp == 0) {
+    // A stage's release is waited for by its parity, so a producer may not fall two releases behind the issuer.  It does not
+    // as long as the issuer needs something of each chunk from it: a CTA with neither rows nor weights in a tile copies a
+    // box of the other's rows.  In the first lap that does not hold (its weights were requested above, and CTA 1 may have
+    // no rows), so the first lap, whose stages are free, does not wait.  (A wait there for the phase before a fresh barrier's
+    // first found that first phase complete in one launch in 10^6, and stood still.)
     int it = 0, s = 0;         // stages handed out so far, over all tiles; the next stage
-    uint32_t parity = 1;       // of the phase that frees it (a fresh barrier's phase before its first counts as complete)
+    uint32_t parity = 1;       // of the phase that frees it
     bool go = true;
     for (int t = pair; go && t < n_tile; t += n_pair) {
       const PwTile p = pw_tile(a, t, n_rp, rank, KC);
-      const int xrow = ((p.row0 >> 7) * KC + p.kc0) * kMaxRows;
       const uint32_t bytes = pw_pair_bytes(a, p, t);   // used by CTA 0 only
       const bool w_mine = pw_half_exists(a, p.n0, rank);
-      for (int i = 0; i < p.n_it; ++i, ++it) {
+      const int n_box = p.rows > 0 ? 2 : w_mine ? 0 : 1;
+      const int xrow = (((p.row0 >> 7) - (n_box == 1 ? 1 : 0)) * KC + p.kc0) * kMaxRows;
+      if (a.starve < 0 && rank == 1) {                 // test aid: CTA 1's producer is late
+        const unsigned long long t0 = global_timer_ns();
+        while (__any_sync(0xFFFFFFFFu, global_timer_ns() - t0 <= a.issue_wait_ns)) {}
+      }
+      auto chunk = [&](int i) {
         unsigned char *st = ring + (size_t)s * stage_bytes;
-        if (!(go = tc_wait_warp<false>(empty + s, parity, failed, a.err))) break;
         if (elect_one()) {
           if (it >= pre) {
             if (rank == 0) mbar_expect_tx(full + s, bytes);
             if (w_mine) pw_copy_weights(&w_map, a, p.n0, rank, p.kc0 + i, KC, st + 16384, full0 + 8u * s);
           }
-          if (p.rows > 0) {
-            pw_copy_rows(&x_map, xrow + i * kMaxRows, st, full0 + 8u * s);
-            pw_copy_rows(&x_map, xrow + i * kMaxRows + kPwBoxRows, st + kPwBoxRows * 128, full0 + 8u * s);
-          }
+          if (n_box > 0) pw_copy_rows(&x_map, xrow + i * kMaxRows, st, full0 + 8u * s);
+          if (n_box > 1) pw_copy_rows(&x_map, xrow + i * kMaxRows + kPwBoxRows, st + kPwBoxRows * 128, full0 + 8u * s);
         }
         __syncwarp();
         if (++s == n_stage) { s = 0; parity ^= 1u; }   // no division by the runtime ring depth
+        ++it;
+      };
+      int i = 0;   // two loops: one that asks in every turn whether to wait takes 0.7 us more per launch
+      for (; i < p.n_it && it < n_stage; ++i) chunk(i);
+      for (; i < p.n_it; ++i) {
+        if (!(go = tc_wait_warp<false>(empty + s, parity, failed, a.err))) break;
+        chunk(i);
       }
     }
     trace_mark(a.trace, a.trace_slot, 3);   // last copy issued
@@ -292,7 +308,7 @@ __global__ void __launch_bounds__(kPwThreads, 1) gemm_pw_kernel(const __grid_con
       const uint32_t idesc = tc_instr_desc(256, a.bn);
       int s = 0, k = 0;
       uint32_t parity = 0;
-      const unsigned long long limit = a.issue_wait_ns ? a.issue_wait_ns : kTcWaitNs;
+      const unsigned long long limit = a.starve > 0 ? a.issue_wait_ns : kTcWaitNs;
       bool go = true;
       for (int t = pair; go && t < n_tile; t += n_pair, ++k) {
         const PwTile p = pw_tile(a, t, n_rp, rank, KC);

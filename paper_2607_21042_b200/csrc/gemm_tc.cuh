@@ -264,8 +264,8 @@ struct GemmTcArgs {
   const int *page_table, *row_stream, *row_pos;
   int pps, d, H;
   int *err;
-  int starve;                 // pair kernel, test aid: 1 + the tile whose copies are never complete (0: none) ...
-  unsigned long long issue_wait_ns;   // ... and how long its issuer then waits (0: as long as everything else)
+  int starve;                 // pair kernel, test aid: 1 + the tile whose copies are never complete (its issuer waits issue_wait_ns);
+  unsigned long long issue_wait_ns;   // -1: CTA 1's producer comes to each of its tiles that much late; 0: none
   unsigned long long *trace;  // optional timeline trace (see trace_mark)
   int trace_slot;
 };

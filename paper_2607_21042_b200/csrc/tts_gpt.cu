@@ -1226,11 +1226,12 @@ int32_t tts_gpt_debug_expire_pair(tts_gpt_t *h, int32_t rows, int32_t tile, uint
     return fail(h, TTS_GPT_E_ARG, "expire_pair: bad or misaligned argument");
   if (c.wfmt == WF_INT4 && h->w4_exact) return fail(h, TTS_GPT_E_UNSUPPORTED, "expire_pair: no pair kernel for integer codes with group sums");
   const PackedLinear &pl = h->layers[0].qkv;
-  if (tile < -1 || tile >= (pl.N + 127) / 128) return fail(h, TTS_GPT_E_ARG, "expire_pair: no such tile");
+  if (tile < -2 || tile >= (pl.N + 127) / 128) return fail(h, TTS_GPT_E_ARG, "expire_pair: no such tile");
   GemmTcArgs a = gemm_args(h, pl, h->a_img, rows, EPI_F32, 1);
   a.out_f32 = out; a.out_stride = pl.N;
   if (tile >= 0) { a.starve = tile + 1; a.issue_wait_ns = (unsigned long long)limit_us * 1000ull; }
-  CUDA_TRY(h, launch_gemm_pw(a, pl.w_map, h->a_map, nullptr, 128, 4, h->stream, false));
+  if (tile == -2) { a.starve = -1; a.issue_wait_ns = (unsigned long long)limit_us * 1000ull; }
+  CUDA_TRY(h, launch_gemm_pw(a, pl.w_map, h->a_map, nullptr, tile == -2 ? 256 : 128, 4, h->stream, false));
   return TTS_GPT_OK;
 }
 

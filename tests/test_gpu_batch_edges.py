@@ -106,6 +106,27 @@ def test_pair_kernel_stores_nothing_behind_an_expired_wait(rows, tile):
     eng.destroy()
 
 
+@pytest.mark.parametrize("rows", [100, 200])
+@pytest.mark.parametrize("heads", [4, 6])
+def test_pair_kernel_waits_for_a_late_second_cta(heads, rows):
+    """The second CTA of a pair comes late to every tile: with rows of its own, with weights only (100 rows), and with neither
+    (100 rows, last tile of 1152 features): nothing expires and every value is that of an undisturbed run."""
+    d = 64 * heads
+    cfg = C.tiny_config(d_model=d, n_head=heads, d_ff=4 * d, max_streams=1, n_pages=8)
+    eng = B.TtsGpt(cfg, C.make_weights(cfg, seed=35), DEV)
+    _run(eng, C.make_prefixes(cfg, [256], seed=36), 0)
+    whole, late = torch.zeros((rows, 3 * d), device=DEV), torch.full((rows, 3 * d), float("nan"), device=DEV)
+    torch.cuda.synchronize()
+    eng.debug_expire_pair(rows, -1, 1000, whole)
+    for _ in range(3):
+        eng.debug_expire_pair(rows, -2, 50, late)
+        eng.sync()
+        assert torch.equal(late, whole)
+        late.fill_(float("nan"))
+        torch.cuda.synchronize()
+    eng.destroy()
+
+
 def test_prefill_pair_kernel_with_the_8bit_cache_and_k_ranges():
     """A model width at which the residual linears of a large pass take k-ranges, K/V rows through the staging array."""
     cfg = C.tiny_config(d_model=512, n_head=8, d_ff=2048, kv_fmt=C.KV_FP8_E4M3, max_streams=2, n_pages=40, max_context=1216, max_pos=1216)
