@@ -241,14 +241,15 @@ int32_t tts_gpt_debug_set_option(tts_gpt_t *h, const char *name, int32_t value);
  * clears the word; the engine and the CUDA context stay usable.  Nothing hangs or faults. */
 int32_t tts_gpt_debug_expire_wait(tts_gpt_t *h, uint32_t limit_us);
 
-/* Test aid for the same path inside the linear of large prefill passes: runs the QKV linear of layer 0 on the
- * activation rows of the last prefill pass, rows (1..256) of them, into out (DEVICE fp32 [rows][3d], 16-byte
- * aligned), as tiles of rows x 128 features on two pairs of CTAs, each pair taking every second tile.  tile >= 0: that
- * tile's copies are announced 16 bytes longer than they are, its pair's issuing warp gives up after limit_us
- * microseconds (1..100000), and neither that tile nor the pair's later ones are stored; the next tts_gpt_sync returns
- * TTS_GPT_E_TIMEOUT once.  tile -1: a whole run.  tile -2: a whole run, on tiles of 256 features, in
- * which the second CTA of a pair comes to each of its tiles limit_us late (nothing expires).  Nothing hangs or faults. */
-int32_t tts_gpt_debug_expire_pair(tts_gpt_t *h, int32_t rows, int32_t tile, uint32_t limit_us, float *out);
+/* Test aid for the same path inside the tensor-core linears: runs the QKV linear of layer 0 on the activation rows of the
+ * last prefill pass, `rows` of them, into out (DEVICE fp32 [rows][3d], 16-byte aligned).  kernel 0: that of decode steps
+ * (1..128 rows), 1: that of prefill passes of several row tiles (1..256 rows), 2: that of large passes (1..256 rows), here
+ * on two pairs of CTAs that take every second tile of 128 features each.  tile >= 0: the copies of that 128-feature tile
+ * are announced 16 bytes longer than they are, its issuing warps give up after limit_us microseconds (1..100000;
+ * kernel 1: after the 2 s that every wait has), the tile is not stored, nor (kernel 2) are the pair's later ones, and the next tts_gpt_sync returns TTS_GPT_E_TIMEOUT once.
+ * tile -1: a whole run.  tile -2 (kernel 2): a whole run, on tiles of 256 features, in which the second CTA of a pair
+ * comes to each of its tiles limit_us late (nothing expires).  Nothing hangs or faults. */
+int32_t tts_gpt_debug_expire_linear(tts_gpt_t *h, int32_t kernel, int32_t rows, int32_t tile, uint32_t limit_us, float *out);
 
 /* ---------------------------------------------------------------------------------------------
  * Single-kernel entry points: the building blocks of the step, callable on their own (unit parity

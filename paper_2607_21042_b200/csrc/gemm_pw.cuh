@@ -33,7 +33,6 @@ constexpr int kPwMaxStages = 8;
 constexpr uint32_t kPwRingBytes = 6 * 32768;             // per CTA: 6 stages at BN = 256, 8 at BN = 128
 constexpr uint32_t kPwPatchBytes = 8 * 4096;             // 4 KB per epilogue warp
 constexpr uint32_t kPwTokenBytes = 8192;                 // a CTA with neither rows nor weights in a tile copies one box all the same
-constexpr unsigned long long kPwLingerNs = 10000000ull;  // a pair that gave up: a copy in flight needs microseconds
 inline size_t pw_smem_bytes() { return (size_t)kPwRingBytes + kPwPatchBytes + 1024 + 512; }
 inline int pw_stages(int bn) { return std::min(kPwMaxStages, (int)(kPwRingBytes / (16384u + (uint32_t)bn * 64u))); }
 
@@ -308,14 +307,13 @@ __global__ void __launch_bounds__(kPwThreads, 1) gemm_pw_kernel(const __grid_con
       const uint32_t idesc = tc_instr_desc(256, a.bn);
       int s = 0, k = 0;
       uint32_t parity = 0;
-      const unsigned long long limit = a.starve > 0 ? a.issue_wait_ns : kTcWaitNs;
       bool go = true;
       for (int t = pair; go && t < n_tile; t += n_pair, ++k) {
         const PwTile p = pw_tile(a, t, n_rp, rank, KC);
         const uint32_t dst = tmem_d + 256u * (uint32_t)(k & 1);
-        if (k >= 2 && !tc_wait_warp<true>(acc_free + (k & 1), (uint32_t)((k >> 1) - 1) & 1u, failed, a.err, limit)) break;
+        if (k >= 2 && !tc_wait_warp<true>(acc_free + (k & 1), (uint32_t)((k >> 1) - 1) & 1u, failed, a.err, &a)) break;
         for (int i = 0; i < p.n_it; ++i) {
-          if (!(go = tc_wait_warp<true>(full + s, parity, failed, a.err, limit))) break;
+          if (!(go = tc_wait_warp<true>(full + s, parity, failed, a.err, &a))) break;
           tc_fence_after_sync();
           const unsigned char *st = ring + (size_t)s * stage_bytes;
           const uint64_t da = tc_smem_desc(st), db = tc_smem_desc(st + 16384);
@@ -430,11 +428,11 @@ __global__ void __launch_bounds__(kPwThreads, 1) gemm_pw_kernel(const __grid_con
   }
   tc_fence_before_sync();
   __syncthreads();
-  if (warp == 0 && __any_sync(0xFFFFFFFFu, *failed)) {
-    pw_tell(failed, rank ^ 1);
-    const unsigned long long t0 = global_timer_ns();
-    while (__any_sync(0xFFFFFFFFu, global_timer_ns() - t0 <= kPwLingerNs)) {}
+  if (warp == 0) {
+    if (__any_sync(0xFFFFFFFFu, *failed)) pw_tell(failed, rank ^ 1);
+    tc_linger(failed);
   }
+  __syncwarp();
   cluster_barrier();   // neither CTA leaves, nor frees tensor memory, while the other still arrives on its barriers or computes
   trace_mark(a.trace, a.trace_slot, 2, 64);
   if (warp == 0) tmem_dealloc2(tmem_d, 512);

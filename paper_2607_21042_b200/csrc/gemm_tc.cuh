@@ -21,8 +21,9 @@
 // warps 2-9 read the fp32
 // accumulator out of tensor memory and run the epilogue.  K-split partial sums go to a scratch
 // array that the following LayerNorm kernel folds into the residual stream in a fixed order.
-// Every wait is bounded; on expiry the CTA sets the error word, stops waiting and still releases
-// its tensor memory.
+// Every wait is bounded.  Where one expires, the error word and the CTA's flag are set, the producer requests nothing more
+// (it would arrive on a stage's barrier whose phase is still open, which is a fault), nothing is stored, and the CTA stays
+// until the copies it requested have landed before it releases its tensor memory.
 #pragma once
 #include "common.cuh"
 #include "linear.cuh"
@@ -264,8 +265,8 @@ struct GemmTcArgs {
   const int *page_table, *row_stream, *row_pos;
   int pps, d, H;
   int *err;
-  int starve;                 // pair kernel, test aid: 1 + the tile whose copies are never complete (its issuer waits issue_wait_ns);
-  unsigned long long issue_wait_ns;   // -1: CTA 1's producer comes to each of its tiles that much late; 0: none
+  int starve;                 // test aid: 1 + the tile (pair kernel; else feature tile) whose copies are never complete (its issuers wait issue_wait_ns);
+  unsigned long long issue_wait_ns;   // -1: the producer of a pair's CTA 1 comes to each of its tiles that much late; 0: none
   unsigned long long *trace;  // optional timeline trace (see trace_mark)
   int trace_slot;
 };
@@ -281,15 +282,16 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0;
 }
 
-// A wait that gives up for good once any wait of the CTA has expired.  The first poll decides in the common case; the
+// `test`: an issuer's wait, shorter where a test starves it (not in the wide kernel: there it cost 1.5 % of a prefill call of
+// 777 rows).  A wait that gives up for good once any wait of the CTA has expired.  The first poll decides in the common case; the
 // shared flag and the timer are read only behind it (in front of it they doubled the cost of a wait that is already
 // satisfied).
-__device__ __forceinline__ void tc_wait(uint64_t *bar, uint32_t parity, volatile int *failed, int *err) {
+__device__ __forceinline__ void tc_wait(uint64_t *bar, uint32_t parity, volatile int *failed, int *err, const GemmTcArgs *test = nullptr) {
   if (mbar_try_wait(bar, parity)) return;
   const unsigned long long t0 = global_timer_ns();
   while (!mbar_try_wait(bar, parity)) {
     if (*failed) return;
-    if (global_timer_ns() - t0 > kTcWaitNs) {
+    if (global_timer_ns() - t0 > (test && test->starve > 0 ? test->issue_wait_ns : kTcWaitNs)) {
       *failed = 1;
       if (err) atomicExch(err, 1);
       return;
@@ -304,22 +306,31 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t *bar, uint32_t pa
   return ok != 0;
 }
 // A warp's wait, the same answer in every lane: whether the barrier's phase has completed.  False once a wait of the CTA
-// has expired, or after limit_ns.  CLUSTER: the other CTA's threads arrive on the barrier too.  (The vote belongs here: as a
+// has expired.  `test` as above.  CLUSTER: the other CTA's threads arrive on the barrier too.  (The vote belongs here: as a
 // vote of the caller's behind the wait it cost 0.7 us a launch, and an issuing lane that goes by its own answer as much.)
 template <bool CLUSTER>
-__device__ __forceinline__ bool tc_wait_warp(uint64_t *bar, uint32_t parity, volatile int *failed, int *err, unsigned long long limit_ns = kTcWaitNs) {
+__device__ __forceinline__ bool tc_wait_warp(uint64_t *bar, uint32_t parity, volatile int *failed, int *err, const GemmTcArgs *test = nullptr) {
   auto complete = [&]() { return __all_sync(0xFFFFFFFFu, CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity)) != 0; };
   if (complete()) return true;
   const unsigned long long t0 = global_timer_ns();
   while (!complete()) {
     if (__any_sync(0xFFFFFFFFu, *failed)) return false;
-    if (__any_sync(0xFFFFFFFFu, global_timer_ns() - t0 > limit_ns)) {
+    if (__any_sync(0xFFFFFFFFu, global_timer_ns() - t0 > (test && test->starve > 0 ? test->issue_wait_ns : kTcWaitNs))) {
       *failed = 1;
       if (err) atomicExch(err, 1);
       return false;
     }
   }
   return true;
+}
+
+// A warp of a CTA that gave up, ahead of its end: no copy may be in flight towards a CTA that has left.  A copy takes
+// microseconds, and a barrier whose phase stays open would not tell.
+constexpr unsigned long long kTcLingerNs = 10000000ull;
+__device__ __forceinline__ void tc_linger(volatile int *failed) {
+  if (!__any_sync(0xFFFFFFFFu, *failed)) return;
+  const unsigned long long t0 = global_timer_ns();
+  while (__any_sync(0xFFFFFFFFu, global_timer_ns() - t0 <= kTcLingerNs)) {}
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
@@ -390,9 +401,10 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
   const unsigned char *gB = reinterpret_cast<const unsigned char *>(a.act_img) + (size_t)kc0 * (kMaxRows * 128) + (size_t)bc * (CN * 128);
 
   const int pre = min(n_it, n_stage);
+  const uint32_t stage_bytes = kStage + (a.starve == nt + 1 ? 16u : 0u);
   if (threadIdx.x == 0) {
     for (int i = 0; i < pre; ++i) {   // weights do not depend on the previous kernel
-      mbar_expect_tx(full + i, kStage);
+      mbar_expect_tx(full + i, stage_bytes);
       bulk_copy_g2s(ring + (size_t)i * kStage, gA + (size_t)i * kTcABytes, kTcABytes, full + i);
     }
   }
@@ -416,8 +428,9 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
     uint32_t parity = 0;
     for (int i = pre; i < n_it; ++i) {   // pre == n_stage here
       tc_wait(empty + s, parity, failed, a.err);
+      if (__any_sync(0xFFFFFFFFu, *failed)) break;   // also where an issuer gave up: its release then came behind the flag
       if (elect_one()) {
-        mbar_expect_tx(full + s, kStage);
+        mbar_expect_tx(full + s, stage_bytes);
         bulk_copy_g2s(ring + (size_t)s * kStage, gA + (size_t)i * kTcABytes, kTcABytes, full + s);
         bulk_copy_g2s(ring + (size_t)s * kStage + kTcABytes, gB + (size_t)i * (kMaxRows * 128), CN * 128, full + s);
       }
@@ -442,9 +455,9 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
       int s = par;
       uint32_t parity = 0;
       for (int i = par; i < n_it; i += stride) {
-        tc_wait(full + s, parity, failed, a.err);
+        tc_wait(full + s, parity, failed, a.err, &a);
         const int g = i >> 1;   // group of this k-chunk inside the k-range
-        if (GROUPED && (i & 1) == 0 && g >= 2) tc_wait(grp_free + (g & 1), ((g >> 1) - 1) & 1, failed, a.err);
+        if (GROUPED && (i & 1) == 0 && g >= 2) tc_wait(grp_free + (g & 1), ((g >> 1) - 1) & 1, failed, a.err, &a);
         tc_fence_after_sync();
         const unsigned char *sa = ring + (size_t)s * kStage;
         const uint64_t da = tc_smem_desc(sa), db = tc_smem_desc(sa + kTcABytes);
@@ -569,7 +582,10 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
   tc_fence_before_sync();
   __syncthreads();
   trace_mark(a.trace, a.trace_slot, 2, 64);   // by an epilogue thread: its own stores precede the mark
-  if (warp == 0) tmem_dealloc(tmem_d, 2 * CN);
+  if (warp == 0) {
+    tc_linger(failed);
+    tmem_dealloc(tmem_d, 2 * CN);
+  }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -687,9 +703,10 @@ __global__ void __launch_bounds__(kTwThreads) gemm_tcw_kernel(const GemmTcArgs a
   const unsigned char *gX = reinterpret_cast<const unsigned char *>(a.act_img) + ((size_t)blockIdx.z * KC + kc0) * (kMaxRows * 128);
 
   const int pre = min(n_it, n_stage);
+  const uint32_t stage_bytes = kTwStageBytes + (a.starve == nt + 1 ? 16u : 0u);
   if (threadIdx.x == 0) {
     for (int i = 0; i < pre; ++i) {   // weights do not depend on the previous kernel
-      mbar_expect_tx(full + i, kTwStageBytes);
+      mbar_expect_tx(full + i, stage_bytes);
       bulk_copy_g2s(ring + (size_t)i * kTwStageBytes + 16384, gW + (size_t)i * kTcABytes, 16384, full + i);
     }
   }
@@ -703,8 +720,9 @@ __global__ void __launch_bounds__(kTwThreads) gemm_tcw_kernel(const GemmTcArgs a
     uint32_t parity = 0;
     for (int i = pre; i < n_it; ++i) {   // pre == n_stage here
       tc_wait(empty + s, parity, failed, a.err);
+      if (__any_sync(0xFFFFFFFFu, *failed)) break;   // as above
       if (elect_one()) {
-        mbar_expect_tx(full + s, kTwStageBytes);
+        mbar_expect_tx(full + s, stage_bytes);
         bulk_copy_g2s(ring + (size_t)s * kTwStageBytes + 16384, gW + (size_t)i * kTcABytes, 16384, full + s);
         bulk_copy_g2s(ring + (size_t)s * kTwStageBytes, gX + (size_t)i * (kMaxRows * 128), 16384, full + s);
       }
@@ -889,7 +907,10 @@ __global__ void __launch_bounds__(kTwThreads) gemm_tcw_kernel(const GemmTcArgs a
   tc_fence_before_sync();
   __syncthreads();
   trace_mark(a.trace, a.trace_slot, 2, 64);
-  if (warp == 0) tmem_dealloc(tmem_d, kCols);
+  if (warp == 0) {
+    tc_linger(failed);
+    tmem_dealloc(tmem_d, kCols);
+  }
 }
 
 inline size_t gemm_tcw_smem_bytes(int stages) { return (size_t)stages * kTwStageBytes + 1024 + 2304; }

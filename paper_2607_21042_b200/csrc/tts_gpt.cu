@@ -1219,19 +1219,21 @@ int32_t tts_gpt_debug_expire_wait(tts_gpt_t *h, uint32_t limit_us) {
   return TTS_GPT_OK;
 }
 
-int32_t tts_gpt_debug_expire_pair(tts_gpt_t *h, int32_t rows, int32_t tile, uint32_t limit_us, float *out) {
+int32_t tts_gpt_debug_expire_linear(tts_gpt_t *h, int32_t kernel, int32_t rows, int32_t tile, uint32_t limit_us, float *out) {
   if (!h) return fail(nullptr, TTS_GPT_E_ARG, "null handle");
   const tts_gpt_config_t &c = h->cfg;
-  if (rows < 1 || rows > 2 * kMaxRows || limit_us < 1 || limit_us > 100000 || !out || (uintptr_t)out % 16)
-    return fail(h, TTS_GPT_E_ARG, "expire_pair: bad or misaligned argument");
-  if (c.wfmt == WF_INT4 && h->w4_exact) return fail(h, TTS_GPT_E_UNSUPPORTED, "expire_pair: no pair kernel for integer codes with group sums");
+  if (kernel < 0 || kernel > 2 || rows < 1 || rows > (kernel == 0 ? 1 : 2) * kMaxRows || limit_us < 1 || limit_us > 100000 || !out || (uintptr_t)out % 16)
+    return fail(h, TTS_GPT_E_ARG, "expire_linear: bad or misaligned argument");
+  if (kernel == 2 && c.wfmt == WF_INT4 && h->w4_exact) return fail(h, TTS_GPT_E_UNSUPPORTED, "expire_linear: no pair kernel for integer codes with group sums");
   const PackedLinear &pl = h->layers[0].qkv;
-  if (tile < -2 || tile >= (pl.N + 127) / 128) return fail(h, TTS_GPT_E_ARG, "expire_pair: no such tile");
+  if (tile < (kernel == 2 ? -2 : -1) || tile >= (pl.N + 127) / 128) return fail(h, TTS_GPT_E_ARG, "expire_linear: no such tile");
   GemmTcArgs a = gemm_args(h, pl, h->a_img, rows, EPI_F32, 1);
   a.out_f32 = out; a.out_stride = pl.N;
   if (tile >= 0) { a.starve = tile + 1; a.issue_wait_ns = (unsigned long long)limit_us * 1000ull; }
   if (tile == -2) { a.starve = -1; a.issue_wait_ns = (unsigned long long)limit_us * 1000ull; }
-  CUDA_TRY(h, launch_gemm_pw(a, pl.w_map, h->a_map, nullptr, tile == -2 ? 256 : 128, 4, h->stream, false));
+  if (kernel == 0) CUDA_TRY(h, launch_gemm_tc(a, h->n_sm, h->stream, false));
+  else if (kernel == 1) CUDA_TRY(h, launch_gemm_tcw(a, h->n_sm, h->stream, false));
+  else CUDA_TRY(h, launch_gemm_pw(a, pl.w_map, h->a_map, nullptr, tile == -2 ? 256 : 128, 4, h->stream, false));
   return TTS_GPT_OK;
 }
 

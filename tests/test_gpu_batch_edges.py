@@ -73,36 +73,40 @@ def test_prefill_passes_of_the_pair_kernel(wfmt, lens):
     eng.destroy()
 
 
-@pytest.mark.parametrize("rows,tile", [(200, 0), (200, 2), (256, 3), (100, 5)])
-def test_pair_kernel_stores_nothing_behind_an_expired_wait(rows, tile):
-    """The issuing warp of one pair of CTAs gives up on a tile: neither CTA stores that tile or a later one of the pair,
-    the other pair's tiles and the earlier ones are whole, the error is reported once and the engine goes on."""
-    cfg = C.tiny_config(max_streams=1, n_pages=8)       # QKV: 768 features, six tiles, three for each of the two pairs
+@pytest.mark.parametrize("wfmt", [C.W_BF16, C.W_INT4_G128])
+@pytest.mark.parametrize("kernel,rows,tile", [(0, 17, 0), (0, 128, 5), (1, 256, 4), (2, 200, 0), (2, 200, 2), (2, 256, 3), (2, 100, 5)])
+def test_tensor_core_linears_store_nothing_behind_an_expired_wait(wfmt, kernel, rows, tile):
+    """The warps that issue a tile's instructions give up: that tile is not stored (by either CTA of a pair), nor are a
+    pair's later ones; all others are whole, the error is reported once and the engine goes on (20 k-chunks: the rings wrap).
+    int4: the kernels that scale group sums, and the pair kernel on dequantized images."""
+    cfg = C.tiny_config(d_model=1280, n_head=20, d_ff=1280, wfmt=wfmt, max_streams=1, n_pages=8)   # QKV: 30 tiles, 20 k-chunks
     eng = B.TtsGpt(cfg, C.make_weights(cfg, seed=33), DEV)
+    if wfmt == C.W_INT4_G128 and kernel < 2:
+        eng.set_option("w4_tc_exact", 1)
     prefix = C.make_prefixes(cfg, [256], seed=34)
     lg, tk = _run(eng, prefix, 0)
     mark = -12345.0
-    whole = torch.full((rows, 768), mark, device=DEV)
-    out = torch.full((rows, 768), mark, device=DEV)
+    whole = torch.full((rows, 3840), mark, device=DEV)
+    out = torch.full((rows, 3840), mark, device=DEV)
     torch.cuda.synchronize()
-    eng.debug_expire_pair(rows, -1, 1000, whole)
+    eng.debug_expire_linear(kernel, rows, -1, 1000, whole)
     eng.sync()
     assert not bool((whole == mark).any()) and bool(torch.isfinite(whole).all())
-    eng.debug_expire_pair(rows, tile, 1000, out)
+    eng.debug_expire_linear(kernel, rows, tile, 1000, out)
     with pytest.raises(B.TtsGptError) as e:
         eng.sync()
     assert e.value.code == B.E_TIMEOUT
-    for t in range(6):
+    for t in range(30):
         got, want = out[:, 128 * t:128 * t + 128], whole[:, 128 * t:128 * t + 128]
-        lost = t >= tile and (t - tile) % 2 == 0
+        lost = t == tile or (kernel == 2 and t > tile and (t - tile) % 2 == 0)
         assert bool((got == mark).all()) if lost else bool(torch.equal(got, want)), t
     eng.sync()
     lg2, tk2 = _run(eng, prefix, 0)
     assert np.array_equal(lg, lg2) and np.array_equal(tk, tk2)
-    for bad in ((0, 0, 1000), (257, 0, 1000), (200, 6, 1000), (200, 0, 0)):
+    for bad in ((3, 100, 0, 1000), (0, 129, 0, 1000), (1, 0, 0, 1000), (1, 100, -2, 1000), (2, 257, 0, 1000), (2, 200, 30, 1000), (2, 200, 0, 0)):
         with pytest.raises(B.TtsGptError) as e:
-            eng.debug_expire_pair(*bad, out)
-        assert e.value.code == B.E_ARG
+            eng.debug_expire_linear(*bad, out)
+        assert e.value.code in (B.E_ARG, B.E_UNSUPPORTED)   # group sums have no pair kernel
     eng.destroy()
 
 
@@ -117,9 +121,9 @@ def test_pair_kernel_waits_for_a_late_second_cta(heads, rows):
     _run(eng, C.make_prefixes(cfg, [256], seed=36), 0)
     whole, late = torch.zeros((rows, 3 * d), device=DEV), torch.full((rows, 3 * d), float("nan"), device=DEV)
     torch.cuda.synchronize()
-    eng.debug_expire_pair(rows, -1, 1000, whole)
+    eng.debug_expire_linear(2, rows, -1, 1000, whole)
     for _ in range(3):
-        eng.debug_expire_pair(rows, -2, 50, late)
+        eng.debug_expire_linear(2, rows, -2, 50, late)
         eng.sync()
         assert torch.equal(late, whole)
         late.fill_(float("nan"))
