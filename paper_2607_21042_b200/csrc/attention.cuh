@@ -765,7 +765,7 @@ __global__ void __launch_bounds__(kAttnPrefillRows * 32, 3) attention_prefill_ke
     for (int p = 0; p < n_pages; ++p, ++j) {
       const int slot = j % kAttnPrefillStages;
       // the stage job j-1 used is free since the barrier that ended its iteration
-      if (threadIdx.x == 0) issue_next((j + kAttnPrefillStages - 1) % kAttnPrefillStages);
+      if (threadIdx.x == 0 && !dead) issue_next((j + kAttnPrefillStages - 1) % kAttnPrefillStages);
       const uint32_t parity = (uint32_t)(j / kAttnPrefillStages) & 1u;
       if (!dead && !mbar_wait_bounded(bars + slot, parity, kAttnWaitNs)) {
         if (a.err) atomicExch(a.err, 1);

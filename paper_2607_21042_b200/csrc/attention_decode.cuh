@@ -46,6 +46,7 @@ struct AdShared {
   uint64_t bar[kAdWarps][kAdStages];
   int first_unit[kAdMaxPairs + 1];                 // running unit counts of the CTA's pairs
   int row[kAdMaxPairs], n_tok[kAdMaxPairs];
+  int dead;                                        // some warp's wait has expired: parts are not merged
 };
 inline size_t attention_decode_smem_bytes() { return (size_t)kAdWarps * kAdStages * 2 * kAdHalf + sizeof(AdShared) + 1024; }
 
@@ -90,6 +91,7 @@ __global__ void __launch_bounds__(kAdWarps * 32, 1) attention_decode_kernel(cons
     sh.n_tok[threadIdx.x] = n;
   }
   if (lane < kAdStages) mbar_init(&sh.bar[warp][lane], 1);
+  if (threadIdx.x == 0) sh.dead = 0;
   for (int i = lane; i < 8 * kAdPitchP / 4; i += 32) reinterpret_cast<uint32_t *>(sh.p[warp])[i] = 0u;
   __syncthreads();
   if (warp == 0) {   // running unit counts, two pairs per lane
@@ -226,6 +228,7 @@ __global__ void __launch_bounds__(kAdWarps * 32, 1) attention_decode_kernel(cons
       dead = true;
     }
     dead = __any_sync(0xFFFFFFFFu, dead);
+    if (dead) sh.dead = 1;
     phase ^= 1u << s;
     const bool last = left <= kAdUnit;          // the unit holds the pair's newest token
     if (last) {
@@ -294,7 +297,7 @@ __global__ void __launch_bounds__(kAdWarps * 32, 1) attention_decode_kernel(cons
     // every lane has read the stage (the MMAs consumed what it loaded): refill it
     fence_proxy_async_smem();
     __syncwarp();
-    if (issued < u_end) {
+    if (issued < u_end && !dead) {              // (behind an expired wait the stage's barrier may still be in its old phase)
       if (issued - base < 32) {
         issue(issued - base, s);
       } else {                                  // beyond the described units: describe ahead, then return to the present ones
@@ -328,7 +331,7 @@ __global__ void __launch_bounds__(kAdWarps * 32, 1) attention_decode_kernel(cons
       O0 = fmaf(f, o[lane], O0);
       O1 = fmaf(f, o[lane + 32], O1);
     }
-    if (!dead) {
+    if (!sh.dead) {
       const int h = (cid + pair * n_cta) % a.H, r = sh.row[pair];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
@@ -339,6 +342,7 @@ __global__ void __launch_bounds__(kAdWarps * 32, 1) attention_decode_kernel(cons
       }
     }
   }
+  if (dead) tc_linger(&sh.dead);                // copies of the warp may still be in flight
   trace_mark(a.trace, a.trace_slot, 2);
 }
 
