@@ -15,7 +15,6 @@ constexpr int kMaxRows = 128;                       // rows per decode step, and
 constexpr int kMaxPassRows = 4096;                  // rows (streams x positions) of a prefill pass: up to 32 row tiles
 constexpr int kMaxSplitRows = 1024;                 // rows up to which every pass may leave four k-range partial sums (or attend over e4m3 codes)
 constexpr int kMaxOrderedRows = 2688;               // rows of a sampled pass, all of which leave up to four partial sums: 55 MB of them at width 1280
-constexpr int kMaxSplitTiles = 4 * kMaxOrderedRows / kMaxRows;   // row tiles x k-ranges of a pass that leaves partial sums
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 

@@ -173,7 +173,18 @@ int check_config(const tts_gpt_config_t *c) {
 // rows of the embedding table: the semantic codes and specials the head predicts, then the text region if any
 inline int emb_rows_of(const tts_gpt_config_t &c) { return c.emb_rows > 0 ? c.emb_rows : c.vocab; }
 
+// Rows the largest pass of an engine can have: those of a call, which the streams' contexts and the page pool bound, up to
+// kMaxPassRows.  Activations and partial sums are sized for it (in whole row tiles; a decode step has up to one).
+inline int pass_rows_of(const tts_gpt_config_t &c) {
+  const long long rows = std::min((long long)c.max_streams * c.max_context, (long long)c.n_pages * kPageTokens);
+  return (int)std::min<long long>(kMaxPassRows, (rows + kMaxRows - 1) / kMaxRows * kMaxRows);
+}
+// row tiles x k-ranges of a pass that leaves partial sums
+inline int split_tiles_of(const tts_gpt_config_t &c) { return 4 * std::min(pass_rows_of(c), kMaxOrderedRows) / kMaxRows; }
+
 constexpr int kScratchPages = 256;          // decoded pages a prefill pass over the 8-bit cache may need
+// rows of the split attention's scratch (the 8-bit cache's kernel also serves prefill passes)
+inline size_t attn_rows_of(const tts_gpt_config_t &c) { return c.kv_fmt == TTS_GPT_KV_FP8_E4M3 ? std::min(kMaxSplitRows, pass_rows_of(c)) : kMaxRows; }
 constexpr size_t kCanaryBytes = 4096;      // guard region in front of and behind the KV pool
 constexpr unsigned char kCanaryByte = 0xA5;
 
@@ -202,6 +213,7 @@ void carve_linear(Carver &cv, PackedLinear &pl, int wf, int N, int K) {
 size_t carve(tts_gpt *h, void *base) {
   const tts_gpt_config_t &c = h->cfg;
   const int d = c.d_model, F = c.d_ff, V = c.vocab, S = c.max_streams;
+  const size_t pass_rows = pass_rows_of(c);
   h->pps = c.max_context / 64;
   Carver cv(base);
   h->tok_emb = cv.take<uint16_t>((size_t)emb_rows_of(c) * d);
@@ -246,7 +258,7 @@ size_t carve(tts_gpt *h, void *base) {
   rt.out_slot = cv.take<int>(kMaxRows);
   rt.row_order = cv.take<int>(kMaxRows);
   h->io = cv.take<StepIO>(1);
-  h->x = cv.take<float>((size_t)kMaxPassRows * d);
+  h->x = cv.take<float>(pass_rows * d);
   h->logits = cv.take<float>((size_t)kMaxRows * V);
   h->st_in = cv.take<int>(kMaxRows);
   h->st_tok = cv.take<int>(kMaxRows);
@@ -257,30 +269,30 @@ size_t carve(tts_gpt *h, void *base) {
   h->o = cv.take<uint16_t>((size_t)kMaxRows * d);
   h->hbuf = cv.take<uint16_t>((size_t)kMaxRows * F);
   h->hf = cv.take<uint16_t>((size_t)kMaxRows * d);
-  h->kv_stage = h->kv_fp8 ? cv.take<uint16_t>((size_t)kMaxPassRows * 2 * d) : nullptr;
+  h->kv_stage = h->kv_fp8 ? cv.take<uint16_t>(pass_rows * 2 * d) : nullptr;
   if (h->kv_fp8) {
     h->kv_scratch = cv.take<uint16_t>((size_t)kScratchPages * 2 * c.n_head * kPageElems);
     h->scratch_table = cv.take<int>((size_t)S * h->pps);
     h->scratch_src = cv.take<int>(kScratchPages);
     h->scratch_ntok = cv.take<int>(kScratchPages);
   }
-  const size_t attn_rows = h->kv_fp8 ? kMaxSplitRows : kMaxRows;   // the 8-bit cache's attention kernel also serves prefill passes
+  const size_t attn_rows = attn_rows_of(c);   // the 8-bit cache's attention kernel also serves prefill passes
   h->attn_partials = cv.take<float>(attn_rows * c.n_head * kAttnMaxChunks * kAttnPartialFloats);
   h->attn_tickets = cv.take<unsigned int>(attn_rows * c.n_head);
   h->have_tc = true;
   if (h->have_tc) {
-    constexpr int kTiles = kMaxPassRows / kMaxRows;   // row tiles of a prefill pass
-    h->a_img = cv.take<char>(kTiles * act_image_bytes(d));
-    h->o_img = cv.take<char>(kTiles * act_image_bytes(d));
-    h->h_img = cv.take<char>(kTiles * act_image_bytes(F));
+    const size_t tiles = pass_rows / kMaxRows;   // row tiles of a prefill pass
+    h->a_img = cv.take<char>(tiles * act_image_bytes(d));
+    h->o_img = cv.take<char>(tiles * act_image_bytes(d));
+    h->h_img = cv.take<char>(tiles * act_image_bytes(F));
     h->hf_img = cv.take<char>(act_image_bytes(d));
-    h->partials_floats = (size_t)kMaxSplitTiles * kMaxRows * d;   // [row tile][k-range][128][d]
+    h->partials_floats = (size_t)split_tiles_of(c) * kMaxRows * d;   // [row tile][k-range][128][d]
     // q lives from the QKV linear to the attention, partial sums from a residual linear to the LayerNorm behind it: never
     // at the same time, so q's rows and q's image lie in the partial sums' memory
-    static_assert(kMaxSplitTiles * kMaxRows * 4 >= kMaxPassRows * 4 + kMaxPassRows * 2, "q rows and q image fit");
+    static_assert(4 * kMaxOrderedRows * 4 >= kMaxPassRows * 4 + kMaxPassRows * 2, "q rows and q image fit (smaller passes: 16 against 6 bytes a row)");
     h->partials = cv.take<float>(h->partials_floats);
     h->q = h->partials;
-    h->q_img = reinterpret_cast<char *>(h->q + (size_t)kMaxPassRows * d);
+    h->q_img = reinterpret_cast<char *>(h->q + pass_rows * d);
   }
   return cv.off;
 }
@@ -771,13 +783,13 @@ int32_t tts_gpt_create(const tts_gpt_config_t *cfg, const tts_gpt_weights_t *w, 
       CUDA_TRY(h, pw_rows_map(m, base, d, n));
       return TTS_GPT_OK;
     };
-    const size_t tiles = kMaxPassRows / kMaxRows;
+    const size_t tiles = pass_rows_of(c) / kMaxRows;
     TRY_(image(&h->a_map, h->a_img, tiles * (d / 64)));
     TRY_(image(&h->o_map, h->o_img, tiles * (d / 64)));
     TRY_(image(&h->h_map, h->h_img, tiles * (c.d_ff / 64)));
     if (!h->kv_fp8) TRY_([&]() -> int { CUDA_TRY(h, attention_decode_map(&h->kv_map, h->kv, h->kv_layer_elems * c.n_layer / kHeadDim)); return TTS_GPT_OK; }());
-    TRY_(rows(&h->xrow_map, h->x, kMaxPassRows));
-    TRY_(rows(&h->part_map, h->partials, (size_t)kMaxSplitTiles * kMaxRows));
+    TRY_(rows(&h->xrow_map, h->x, pass_rows_of(c)));
+    TRY_(rows(&h->part_map, h->partials, (size_t)split_tiles_of(c) * kMaxRows));
     for (auto &L : h->layers)
       for (PackedLinear *pl : {&L.qkv, &L.o, &L.fc1, &L.fc2})
         TRY_(image(&pl->w_map, pl->w_img, (size_t)((pl->N + 127) / 128) * (pl->K / 64)));
@@ -785,7 +797,7 @@ int32_t tts_gpt_create(const tts_gpt_config_t *cfg, const tts_gpt_weights_t *w, 
 #undef TRY_
   const int init_n = std::max(std::max(c.n_pages, c.max_streams * h->pps), c.max_streams);
   init_pages_kernel<<<(init_n + 255) / 256, 256, 0, h->stream>>>(h->ps);
-  cudaError_t e = cudaMemsetAsync(h->attn_tickets, 0, (size_t)(h->kv_fp8 ? kMaxSplitRows : kMaxRows) * c.n_head * sizeof(unsigned int), h->stream);
+  cudaError_t e = cudaMemsetAsync(h->attn_tickets, 0, attn_rows_of(c) * c.n_head * sizeof(unsigned int), h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->canary_lo, kCanaryByte, kCanaryBytes, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->canary_hi, kCanaryByte, kCanaryBytes, h->stream);
   if (e == cudaSuccess) {
@@ -1222,7 +1234,7 @@ int32_t tts_gpt_debug_expire_wait(tts_gpt_t *h, uint32_t limit_us) {
 int32_t tts_gpt_debug_expire_linear(tts_gpt_t *h, int32_t kernel, int32_t rows, int32_t tile, uint32_t limit_us, float *out) {
   if (!h) return fail(nullptr, TTS_GPT_E_ARG, "null handle");
   const tts_gpt_config_t &c = h->cfg;
-  if (kernel < 0 || kernel > 2 || rows < 1 || rows > (kernel == 0 ? 1 : 2) * kMaxRows || limit_us < 1 || limit_us > 100000 || !out || (uintptr_t)out % 16)
+  if (kernel < 0 || kernel > 2 || rows < 1 || rows > std::min((kernel == 0 ? 1 : 2) * kMaxRows, pass_rows_of(c)) || limit_us < 1 || limit_us > 100000 || !out || (uintptr_t)out % 16)
     return fail(h, TTS_GPT_E_ARG, "expire_linear: bad or misaligned argument");
   if (kernel == 2 && c.wfmt == WF_INT4 && h->w4_exact) return fail(h, TTS_GPT_E_UNSUPPORTED, "expire_linear: no pair kernel for integer codes with group sums");
   const PackedLinear &pl = h->layers[0].qkv;

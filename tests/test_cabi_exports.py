@@ -43,6 +43,23 @@ def test_binding_lists_every_declared_symbol():
     assert sorted(binding.EXPORTS) == _declared()
 
 
+@pytest.mark.parametrize("kv_fmt", [0, 1])
+def test_workspace_holds_the_rows_a_pass_can_have(lib, kv_fmt):
+    """Activations are sized by the rows that the streams' contexts and the page pool allow, up to 4096."""
+    from paper_2607_21042_b200 import binding, cases
+    ws = lambda **kw: binding.query_workspace(cases.full_config(kv_fmt=kv_fmt, **kw))  # noqa: E731
+    d, f, layers, heads = 1280, 5120, 24, 20
+    page = layers * 2 * heads * (8192 if kv_fmt == 0 else 4352)
+    # bytes a row: x and four partial sums in fp32, the images of three linears' inputs; 8-bit cache: staged K/V rows
+    row = 4 * d + 4 * 4 * d + 2 * (d + d + f) + (4 * d if kv_fmt else 0)
+    one = ws(max_streams=1, max_context=2048, n_pages=32)
+    assert abs(one - ws(max_streams=1, max_context=2048, n_pages=16) - 16 * page - 1024 * row) < 8192
+    assert ws(max_streams=1, max_context=2048, n_pages=64) - one - 32 * page < 8192      # the context bounds the rows
+    big = ws(max_streams=4, max_context=2048, n_pages=64)
+    assert abs(ws(max_streams=4, max_context=2048, n_pages=128) - big - 64 * page) < 8192      # 4096 rows
+    assert one < ws(max_streams=4, max_context=2048, n_pages=32) + 8192
+
+
 def test_query_workspace_and_config_errors_need_no_gpu(lib):
     from paper_2607_21042_b200 import binding, cases
     cfg = cases.workload(2).cfg
