@@ -8,7 +8,7 @@ import torch
 from oracle import gpt_oracle as O
 from paper_2607_21042_b200 import binding as B
 from paper_2607_21042_b200 import cases as C
-from helpers import assert_logits_close, bits_dev, check_tokens
+from helpers import E4M3_MAX_ABS, E4M3_REL_L2, E4M3_REL_L2_SHORT, assert_logits_close, bits_dev, check_tokens, logits_errors
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -32,6 +32,17 @@ def _check(model, prefixes, lg, tk, streams, what):
         ref, _ = O.replay_full(model, O.bf16_to_f64(prefixes[s]), tk[s][:-1])
         assert_logits_close(lg[s], ref, "%s, stream %d" % (what, s))
         check_tokens(tk[s], ref, 0, 1.0, None, "%s, stream %d" % (what, s))
+
+
+def _check_e4m3(model, prefixes, lg, tk, streams, what):
+    """The bars of the 8-bit cache: the relative one is wider below 32 attended tokens (see helpers)."""
+    for s in streams:
+        ref, _ = O.replay_full(model, O.bf16_to_f64(prefixes[s]), tk[s][:-1])
+        ctx = prefixes[s].shape[0] + np.arange(len(ref))
+        for i in range(len(ref)):
+            ma, rl = logits_errors(lg[s][i], ref[i])
+            bar = E4M3_REL_L2 if ctx[i] >= 32 else E4M3_REL_L2_SHORT
+            assert ma <= E4M3_MAX_ABS and rl <= bar, "%s, stream %d, step %d: max-abs %.4g, relative L2 %.4g" % (what, s, i, ma, rl)
 
 
 @pytest.mark.parametrize("S", [75, 100, 128])
@@ -137,7 +148,8 @@ def test_prefill_pair_kernel_with_the_8bit_cache_and_k_ranges():
     w = C.make_weights(cfg, seed=25)
     prefixes = C.make_prefixes(cfg, [1100, 77], seed=26)
     eng = B.TtsGpt(cfg, w, DEV)
-    lg, _ = _run(eng, prefixes, 2)
+    lg, tk = _run(eng, prefixes, 2)
+    _check_e4m3(O.OracleModel(cfg, w), prefixes, lg, tk, range(2), "pair kernel, 8-bit cache")
     eng.set_option("prefill_pass_rows", 512)
     lg2, _ = _run(eng, prefixes, 2)
     assert np.max(np.abs(lg[:, 0] - lg2[:, 0])) < 4.5e-2
@@ -165,6 +177,40 @@ def test_sampled_calls_keep_their_order_of_sums(S):
     eng.destroy()
 
 
+ONE_UNIT_OF_MORE = {   # model, rows of a unit, prefix lengths
+    "tail of 1 row": ("tiny", 1024, [1025]),
+    "tail of 128 rows": ("tiny", 1024, [1100, 1000, 76]),
+    "tail of 129 rows": ("tiny", 1024, [1153, 1024]),
+    "two whole units": ("tiny", 1024, [2048]),
+    "three units in two passes, tail of 5 rows": ("tiny", 1024, [1500, 1000, 577]),
+    "many streams, heads of more than 16 rows": ("tiny", 1024, [30 + 7 * (i % 11) for i in range(40)]),
+    "wide model, three units": ("wide", 896, [1900, 20, 700, 64]),
+    "wide model, tail of 100 rows": ("wide", 896, [896, 996]),
+    "wide model, four units": ("wide", 896, [2000, 1300]),
+}
+
+
+@pytest.mark.parametrize("wfmt", [C.W_BF16, C.W_INT8_PC, C.W_INT4_G128])
+@pytest.mark.parametrize("form", list(ONE_UNIT_OF_MORE))
+def test_sampled_passes_of_several_units_give_the_bits_of_single_units(form, wfmt):
+    """A sampled prefill runs several units of rows as one pass and the last few rows apart: the same bits, tokens and
+    cache (decoded from afterwards) as with passes of one unit."""
+    model, unit, lens = ONE_UNIT_OF_MORE[form]
+    kw = dict(wfmt=wfmt, max_streams=len(lens), n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=2048, max_pos=2048)
+    if model == "wide":
+        kw.update(d_model=1280, n_head=20, d_ff=5120)
+    cfg = C.tiny_config(**kw)
+    eng = B.TtsGpt(cfg, C.make_weights(cfg, seed=37), DEV)
+    prefixes = C.make_prefixes(cfg, lens, seed=38)
+    u = dict(top_k=30, uniforms=torch.rand(len(lens), generator=torch.Generator(DEV).manual_seed(3), device=DEV))
+    steps = 2 if max(lens) <= 2040 else 0
+    lg, tk = _run(eng, prefixes, steps, **u)
+    eng.set_option("prefill_pass_rows", unit)
+    lg1, tk1 = _run(eng, prefixes, steps, **u)
+    assert np.array_equal(lg, lg1) and np.array_equal(tk, tk1)
+    eng.destroy()
+
+
 @pytest.mark.parametrize("S", [1, 21, 30, 40, 60, 80])
 def test_8bit_decode_attention_splits(S):
     """8, 6, 4, 3, 2 and 1 CTAs per (row, head) over the 8-bit cache: contexts at the edges of half pages and pages, splits
@@ -173,11 +219,15 @@ def test_8bit_decode_attention_splits(S):
     lens = [edges[i % len(edges)] if i < 30 else 2 + (11 * i) % 60 for i in range(S)]
     cfg = C.tiny_config(kv_fmt=C.KV_FP8_E4M3, max_streams=S, n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=768)
     w = C.make_weights(cfg, seed=29)
+    model = O.OracleModel(cfg, w)
     eng = B.TtsGpt(cfg, w, DEV)
     eng.set_option("poison_free_pages", 1)
     prefixes = C.make_prefixes(cfg, lens, seed=30)
     lg, tk = _run(eng, prefixes, 3)
     lg2, tk2 = _run(eng, prefixes, 3, top_k=4, uniforms=torch.zeros(S, device=DEV))
+    streams = sorted(set(range(min(S, 15))) | {S - 1})
+    _check_e4m3(model, prefixes, lg, tk, streams, "8-bit cache, greedy")
+    _check_e4m3(model, prefixes, lg2, tk2, streams, "8-bit cache, sampled order")
     eng.set_option("attn_stream_min_pairs", 1)
     lg3, tk3 = _run(eng, prefixes, 3)
     for a, t in ((lg, tk), (lg2, tk2)):
