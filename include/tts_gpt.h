@@ -145,9 +145,15 @@ int32_t tts_gpt_prefill_tokens(tts_gpt_t *h, int32_t n, const void *const *cond_
  * step, appends that token's K/V at position ctx_i, attends over ctx_i + 1 keys, and returns the
  * logits of the next token, the sampled next token and optionally the final-LayerNorm hidden row.
  * top_k 0 or 1 = greedy (lowest index on ties); top_k in 2..64 = softmax over the top_k logits
- * at `temperature`, inverse CDF with uniforms[i].  Sampled calls (prefill and decode, top_k > 1) form
- * their sums in one fixed order, so that the same uniforms give the same tokens; greedy calls may take
- * faster kernels with another order of sums.  Afterwards ctx_i += 1.
+ * at `temperature`, inverse CDF with uniforms[i].  Afterwards ctx_i += 1.
+ * Reproducibility: the same sequence of calls on a fresh engine gives the same results bit for bit, greedy or
+ * sampled (same library, same kind of GPU); no sum depends on timing.  The order of a sum does depend on the rows of
+ * the call (decode: 1, 2-4, 5-16, 17 and more rows, in some kernels the contexts of the other rows too; prefill: the rows
+ * prefilled together), so a stream that goes on in a
+ * batch of another size sees logits rounded differently (about 0.5 % relative after 24 layers), and a sampled token
+ * whose uniform falls that close to an edge of the distribution may change.  Sampled calls (prefill and decode, top_k > 1)
+ * keep, for each number of rows, the orders of sums of earlier versions of this library; greedy calls take faster
+ * kernels with other orders where there are some.
  * Errors: E_ARG, E_STREAM (unknown / duplicate id), E_CTX_OVERFLOW (ctx_i + 1 > max_context),
  * E_NO_PAGES.  All-or-nothing; nothing is enqueued on error. */
 int32_t tts_gpt_decode_step(tts_gpt_t *h, int32_t n, const int32_t *stream_ids,
@@ -226,7 +232,7 @@ int32_t tts_gpt_debug_check_canaries(tts_gpt_t *h, int32_t *bad_bytes);
  * step graphs.  Names: "graph", "pdl", "tc" and "tc_min_rows" (tensor-core
  * linears), "prefill_pass_rows" (rows per prefill pass: a multiple of 128 up to 4096; the default is chosen at creation
  * from the SM count and the model width, 3584 for the 24-layer model on 148 SMs; passes of more than 128 rows need
- * the tensor-core path; sampled calls take a multiple of 896 of them), "w4_tc_exact" (int4 weights only: by default the operand images of the tensor-core path, used for more than 16 rows,
+ * the tensor-core path; sampled calls take a multiple of a unit of rows, 896 for the 24-layer model), "w4_tc_exact" (int4 weights only: by default the operand images of the tensor-core path, used for more than 16 rows,
  * hold code x group scale rounded once to bf16; 1 rewrites them as integer codes and the kernels scale fp32 sums per
  * 128-column group, 0 writes the default back), "attn_tc", "attn_mma", "attn_prefill", "attn_half", "attn_decode", "attn_stream", "attn_stream_min_pairs", "attn_cluster_fill",
  * "fc2_ksplit"; "poison_free_pages" (test aid standing in for a memory checker: every free page, and

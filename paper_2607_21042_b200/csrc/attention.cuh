@@ -501,11 +501,16 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 4) attention_half_kernel(cons
 inline bool attention_half_fits(int R, int H, int splits, int n_sm) { return R * H * splits <= 4 * n_sm; }
 inline int attention_half_splits(int R, int H, int n_sm) {
   const int s = std::max(1, std::min(kAttnMaxCluster, 4 * n_sm / (R * H)));
-  return s == 7 ? 6 : s;   // clusters of seven leave places free (8-bit cache, 4 rows of 930 tokens: 0.742 ms per step, on six 0.648)
+  // clusters of seven leave places free: 4 rows, on seven / on six, ms per step at 100, 530 and 1400 tokens: 0.642 / 0.586, 0.653 /
+  // 0.605, 0.733 / 0.678; 8-bit cache 0.671 / 0.587, 0.680 / 0.607, 0.747 / 0.663
+  return s == 7 ? 6 : s;
 }
-// Two rows and more whose pairs the kernel above spreads over every SM, up to the middle batches' kernel.  One row is as
-// fast there, and so are short contexts (3 rows of 230 tokens 0.569 against 0.574 ms per step, 10 rows of 230 0.654
-// against 0.662; 10 rows of 930 0.895 against 0.843).
+// Two rows and more whose pairs the kernel above spreads over every SM, up to the middle batches' kernel.  Here / clusters of
+// whole pages (attention_kernel), ms per step at contexts of 100, 530 and 1400 tokens: 1 row 0.467 / 0.470, 0.470 / 0.484,
+// 0.497 / 0.509; 2 rows 0.546 / 0.548, 0.554 / 0.570, 0.597 / 0.636; 4 rows 0.578 / 0.585, 0.608 / 0.639, 0.684 / 0.760; 8 rows
+// 0.594 / 0.592, 0.662 / 0.700, 0.778 / 0.923; 14 rows 0.833 / 0.841, 0.948 / 0.959, 1.155 / 1.212.  (One row stays with
+// clusters of whole pages, whose sums greedy and sampled steps share.)  Against the middle batches' kernel: 10 rows 0.645 /
+// 0.693, 0.774 / 0.773, 0.952 / 0.933; 14 rows 0.833 / 0.910, 0.948 / 0.982, 1.155 / 1.212; beyond the line see there.
 inline bool attention_use_half(int R, int H, int n_sm) {
   return R > 1 && R * H <= 2 * n_sm && R * H * attention_cluster_size(R, H, n_sm) >= n_sm;
 }
@@ -659,8 +664,8 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 3) attention_stream_kernel(co
   trace_mark(a.trace, a.trace_slot, 2);
 }
 
-// (row, head) pairs from which the streaming variant is used: the GPU is then covered four times
-// over with one CTA per pair (at 16 rows of 20 heads the cluster variant still measured faster)
+// (row, head) pairs from which the streaming variant is used where the kernels above and that of the middle batches are not
+// (sampled steps, batches of more than ten pairs per SM): the GPU is then covered four times over with one CTA per pair.
 inline bool attention_use_stream(int R, int H, int n_sm) { return R * H >= 4 * n_sm; }
 
 inline cudaError_t launch_attention_stream(const AttnArgs &a, int R, cudaStream_t st, bool pdl) {

@@ -346,8 +346,15 @@ __global__ void __launch_bounds__(kAdWarps * 32, 1) attention_decode_kernel(cons
   trace_mark(a.trace, a.trace_slot, 2);
 }
 
-// (row, head) pairs for which the kernel is used.  Up to two per SM the register-load kernel's one CTA per pair still
-// fits in one wave (8 rows at 530 tokens: 0.754 against 0.773 ms per step); beyond ten the streaming kernel is ahead.
+// (row, head) pairs for which the kernel is used: between the half-page kernel, of which up to two pairs per SM are one wave,
+// and the streaming kernel.  ms per step, here / half pages / streaming, rows of one context of 100, 530 and 1400 tokens:
+// 15 rows 0.901 / 0.834 / 0.861, 0.973 / 0.990 / 1.007, 1.195 / 1.268 / 1.311; 24 rows 0.853 / 0.793 / 0.894, 1.027 / 0.979 /
+// 1.151, 1.425 / 1.339 / 1.741; 37 rows 0.934 / 0.912 / 0.987, 1.224 / 1.264 / 1.288, 1.777 / 1.939 / 1.965; 64 rows 1.063 / 1.081 /
+// 1.194, 1.528 / 1.622 / 1.668, 2.579 / 2.664 / 2.692; 74 rows 1.133 / 1.146 / 1.280, 1.677 / 1.725 / 1.861, 2.857 / 2.846 / 3.202;
+// 96 rows 1.329 / 1.278 / 1.418, 2.078 / 2.043 / 2.133, 3.613 / 3.609 / 3.819; 128 rows 1.611 / 1.469 / 1.678, 2.613 / 2.425 / 2.599,
+// 4.71 / 4.48 / 4.78 (the three took turns, each with contexts up to 70 tokens longer than the one before).  For rows of
+// equal length half pages are ahead where their splits fill the places (24, 48 rows) and from 80 rows on; the line at ten
+// pairs per SM was drawn with the ragged batch of 128 rows (2.747 streaming, 2.792 here).
 inline bool attention_use_decode(int R, int H, int n_sm) { return R * H > 2 * n_sm && R * H <= 10 * n_sm; }
 
 // layer_row: first row of the layer in kv_map, the whole pool as rows of 64 bf16 (attention_decode_map)

@@ -592,15 +592,13 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
 // Wide variant for passes of more than 128 rows (prefill): all 128 rows of a row tile in one
 // instruction.
 //
-// A tcgen05.mma with M = 128 takes about 72 ns on this part whether its N extent is 32 or 128, so
-// the kernel above, whose instructions are 32 batch rows wide, wastes three quarters of each.  It
-// still wins while a pass has at most 128 rows, because it spreads a linear over four times as many
+// The kernel above re-reads the weights once per 32 or 64 batch rows and issues instructions of 32 or 64 columns.  It
+// still wins while a pass has at most 128 rows, because it spreads a linear over two to four times as many
 // CTAs without any merge.  A prefill pass of several row tiles has enough independent output tiles
 // for the wide shape: here the operand roles are swapped, the activation block of a k-chunk (128
 // rows x 64 columns, 16 KB) is the M operand, a 128-row weight block the N operand, and one CTA
 // computes a whole [128 rows] x [128 output features] tile for its k-range: K/16 instructions where
-// four CTAs of the kernel above issue K/16 each, and the weights cross from L2 once per 128 rows
-// instead of once per 32.  Grid = feature tiles x k-ranges x row tiles.  Accumulator lane = row,
+// two to four CTAs of the kernel above issue K/16 each, and the weights cross from L2 once per 128 rows.  Grid = feature tiles x k-ranges x row tiles.  Accumulator lane = row,
 // column = output feature; the epilogue parks the accumulator rows in the idle ring and writes
 // them out with the lanes along the row.  The residual linears split K over up to 4 CTAs whose
 // partial sums the next LayerNorm folds (partials [row tile][range][128][N]); the others take all

@@ -31,7 +31,7 @@ enum { EPI_F32 = 0, EPI_QKV = 1, EPI_RESID = 2, EPI_GELU = 3 };
 
 constexpr int kLinearWarps = 10;  // divides the k-tile counts of K=1280 and K=5120 in every format
 constexpr int kLinearThreads = kLinearWarps * 32;
-constexpr int kSmallKSplit = 4;     // k-ranges of FC2 between 5 and 16 rows (partial sums folded by the next LayerNorm)
+constexpr int kSmallKSplit = 4;     // k-ranges of FC2 from 2 to 16 rows (partial sums folded by the next LayerNorm)
 constexpr int kLnFuseMaxRows = 1;   // LayerNorm is fused into the linear up to this batch: every CTA repeats it, which
                                     // beats a separate launch for a single row only
 constexpr int kLnFuseMaxRowsOrdered = 4;   // the same for launches that keep the order of sums of the FMA path
@@ -128,7 +128,7 @@ struct LinearArgs {
   const uint16_t *bias;   // bf16 [N] or null
   const uint16_t *act;    // bf16 [B][K]  (unused when ln_x is set)
   int N, K, B, mode;
-  int ordered;           // 1: up to 4 rows take the FMA path (a fixed order of sums)
+  int ordered;           // 1: up to 4 rows take the FMA path (the order of sums of sampled calls)
   // fused LayerNorm in front (see can_fuse_ln): act = LN(ln_x[gather[b]])
   const float *ln_x;      // fp32 [*][K] or null
   const uint16_t *ln_g, *ln_b;
@@ -610,8 +610,11 @@ inline LinearPlan plan_linear(int wf, int N, int K, int B, int mode, int max_cta
   const int tiles = row_tiles(N);
   LinearPlan p;
   // The fewest tiles per CTA with which one wave takes the launch: a second wave starts its copies late (bf16 FC1 at
-  // 8 rows on two tiles per CTA, 320 CTAs for 296 places: 5.9 us; on three: 3.75 us).  One row of bf16 weights doubles
-  // instead: what it waits for is its copies, and four tiles in one copy are the faster (a step 0.468 ms, on three 0.476).
+  // 8 rows on two tiles per CTA, 320 CTAs for 296 places: 5.9 us; on three: 3.75 us).  A step with and without three
+  // tiles (contexts of 530 tokens, ms): bf16 2 rows 0.552 / 0.589, 4 rows 0.607 / 0.698, 8 rows 0.659 / 0.727, 16 rows
+  // 0.925 / 0.931; int8 1 row 0.497 / 0.509, 4 rows 0.617 / 0.641, 16 rows 0.869 / 0.907; int4 1 row 0.533 / 0.539, 8 rows
+  // 0.650 / 0.699.  One row of bf16 weights doubles instead: what it waits for is its copies, and four tiles in one copy are
+  // slightly the faster (0.481 against 0.484).
   p.rt = 1;
   for (int rt = 2; rt <= 4 && (tiles + p.rt - 1) / p.rt > max_ctas && linear_smem_bytes(wf, rt, mode, B, K) <= (size_t)kLinearSmemBudget; ++rt)
     if (rt != 3 || B > 1 || wf != WF_BF16) p.rt = rt;

@@ -75,7 +75,7 @@ struct tts_gpt {
   float *st_uni, *st_log;       // uniforms, logits [kMaxRows][vocab]
   uint16_t *st_hid;             // hidden rows [kMaxRows][d]
   uint16_t *a, *o, *hbuf, *hf;
-  // tensor-core path (more than 16 rows, bf16 weights): activation images and k-split partial sums
+  // tensor-core path (more than 16 rows): activation images and k-split partial sums
   void *a_img = nullptr, *o_img = nullptr, *h_img = nullptr, *hf_img = nullptr;
   void *q_img = nullptr;             // q of prefill passes of more than 128 rows
   CUtensorMap a_map, o_map, h_map;   // the images as tensors (all row tiles of a pass)
@@ -110,11 +110,15 @@ struct tts_gpt {
   int tc_tail_parts = 0;  // partial sums the last FC2 of the tensor-core path left for the final LayerNorm
   bool use_attn_mma = true;      // tensor-core attention in prefill passes (option "attn_mma")
   bool use_attn_prefill = true;  // shared-page attention in prefill passes (option "attn_prefill")
-  // Sampled calls (top_k > 1) keep one order of sums: the FMA linears up to 4 rows, prefill passes with the k-ranges and
-  // tails of passes of `ordered_pass_rows`, the CUDA-core decode attention.  A sampled token hangs on the last bits of its
-  // logits (neighbours in the tail of the distribution lie closer than bf16 rounding moves them, and the token feeds every
-  // later step), so a caller who replays a sequence of uniforms gets the same utterance only if the sums run in the same
-  // order.  Greedy calls are free of that and take the faster kernels.
+  // Sampled calls (top_k > 1) keep, for each number of rows, the order of sums that earlier versions of the library had: the
+  // FMA linears up to 4 rows, prefill passes with the k-ranges and tails of passes of `ordered_pass_rows`, the CUDA-core
+  // decode attention.  A sampled token hangs on the last bits of its logits (neighbours in the tail of the distribution lie
+  // closer than bf16 rounding moves them, and the token feeds every later step), so a recorded sequence of uniforms
+  // replayed on a newer library gives the same utterance only if the sums run in the same order.  (Replaying the same calls
+  // on one library gives the same bits with either set of kernels; across batch sizes neither keeps an order.)  It costs
+  // (24-layer model, bf16, contexts of 530 tokens, ms per step, greedy / sampled): 2 rows 0.554 / 0.746, 3 rows 0.591 /
+  // 0.900, 4 rows 0.605 / 0.971, 8 rows 0.656 / 0.702, 21 rows 0.967 / 1.052, 64 rows 1.487 / 1.636, 128 rows level; over
+  // the 8-bit cache 4 rows 0.607 / 1.088, 21 rows 0.885 / 1.184.
   bool ordered = false;          // set by each prefill and decode call
   int ordered_pass_rows = 896;
   bool use_attn_half = true;     // half-page attention of decode steps (option "attn_half")
@@ -367,7 +371,11 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
     // slots, then attend over e4m3 pages (the same kernel for prefill passes and decode steps)
     unsigned char *kvl = reinterpret_cast<unsigned char *>(const_cast<uint16_t *>(aa.kv_layer));
     // streaming: beyond the bf16 cache's line, and (steps free in their sums) where its pairs are one wave of three CTAs per
-    // SM and no split fits the other kernel (18 rows of 930 tokens 0.939 against 1.037 ms per step)
+    // SM and no split fits the other kernel.  ms per step, streaming / split, at contexts of 100, 530, 930 and 1400 tokens:
+    // 14 rows (two per SM: split) 0.849 / 0.842, 0.944 / 0.934, 1.034 / 0.999, 1.103 / 1.066; 15 rows 0.826 / 0.811, 0.922 /
+    // 0.998, 1.015 / 1.126, 1.094 / 1.263; 22 rows 0.804 / 0.799, 0.898 / 0.938, 0.999 / 1.079, 1.100 / 1.224; 23 rows (more
+    // than one wave of it: split) 0.838 / 0.805, 0.986 / 0.934, 1.134 / 1.076, 1.256 / 1.218; 30 rows (beyond the line) 0.874 /
+    // 0.871, 1.058 / 1.118, 1.190 / 1.301, 1.336 / 1.493.  Short contexts are level on both sides of every line.
     const bool one_wave = !h->ordered && R * aa.H > 2 * h->n_sm && R * aa.H <= 3 * h->n_sm;
     const bool many = h->attn_stream_min_pairs > 0 ? R * aa.H >= h->attn_stream_min_pairs : one_wave || attention_use_stream(R, aa.H, h->n_sm);
     const bool stream = aa.old_pages_final && h->use_attn_stream && many;   // decode steps with enough (row, head) pairs
@@ -424,7 +432,7 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
 // The transformer blocks for R rows already described by the row table, x holding the input rows.
 // Every kernel after the first of a step is launched with programmatic dependent launch, so its
 // weight loads overlap the tail of its predecessor.
-// ---- tensor-core path: more than 16 rows, bf16 weights ----
+// ---- tensor-core path: more than 16 rows ----
 GemmTcArgs gemm_args(tts_gpt *h, const PackedLinear &pl, const void *act_img, int B, int mode, int ksplit) {
   GemmTcArgs a;
   memset(&a, 0, sizeof a);
@@ -438,6 +446,11 @@ GemmTcArgs gemm_args(tts_gpt *h, const PackedLinear &pl, const void *act_img, in
 }
 
 // Passes of up to kPairMinRows rows stay with the one-CTA wide kernel (two CTAs per SM): their tiles are too few for pairs.
+// One prefill call of the 24-layer model, one-CTA kernel / pairs, ms: one stream of 300 rows 1.42 / 1.69, 640 1.71 / 1.95,
+// 777 1.80 / 2.24, 896 1.83 / 2.28, 1000 2.47 / 2.48, 1024 2.45 / 2.46, 1100 2.64 / 2.80, 1280 2.84 / 2.91, 1400 3.07 / 3.04,
+// 1536 3.15 / 3.09, 2000 4.22 / 4.09; eight streams of 640 rows together 1.67 / 1.91, 1024 2.18 / 2.14, 1152 2.28 / 2.49, 1536
+// 2.87 / 2.66, 1792 3.03 / 2.79 (int8 weights within 2 % of these).  The two cross between 1000 and 1400 rows, up and down
+// with how full the last wave of either is; a rule by the two kernels' waves could gain up to 9 % there.
 constexpr int kPairMinRows = 1024;
 bool use_pairs(const tts_gpt *h, int R) { return R > kPairMinRows && !(h->cfg.wfmt == WF_INT4 && h->w4_exact); }
 
