@@ -668,7 +668,7 @@ inline cudaError_t launch_linear_mode(const LinearArgs &a, int max_ctas, cudaStr
 }
 
 // K must be a multiple of 128.
-inline cudaError_t launch_linear(int wf, const LinearArgs &a, cudaStream_t st, bool pdl = false, int max_ctas = 296) {
+inline cudaError_t launch_linear(int wf, const LinearArgs &a, cudaStream_t st, bool pdl, int max_ctas) {
   if (a.ln_x && !can_fuse_ln(a.B, a.K, a.ordered)) return cudaErrorInvalidValue;
   if (a.ksplit > 1 && (a.ln_x || a.mode != EPI_RESID || (a.K / k_per_tile(wf)) % a.ksplit != 0)) return cudaErrorInvalidValue;
   if (wf == WF_BF16) return launch_linear_mode<WF_BF16>(a, max_ctas, st, pdl);

@@ -139,6 +139,13 @@ struct tts_gpt {
 
 namespace {
 
+// SMs of the current device
+int device_sms() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) return sms;
+  return 148;
+}
+
 int fail(tts_gpt *h, int code, const char *fmt, ...) {
   char buf[512];
   va_list ap;
@@ -837,9 +844,7 @@ int32_t tts_gpt_create(const tts_gpt_config_t *cfg, const tts_gpt_weights_t *w, 
   // the legacy default stream cannot be captured
   h->use_graph = h->stream != nullptr && h->stream != cudaStreamLegacy;
   h->use_pdl = true;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
-    h->n_sm = sms;
+  h->n_sm = device_sms();
   {
     // rows per prefill pass: the most row tiles whose model-wide linears (O projection, FC2) still run as one wave of
     // one 256 x 256 tile per pair of SMs; QKV and FC1 then take 3 and 4 nearly full waves.  28 tiles with this model on
@@ -1363,7 +1368,7 @@ int32_t tts_gpt_op_linear(int32_t wfmt, int32_t N, int32_t K, const void *packed
   pl.bias = (uint16_t *)bias;
   LinearArgs a = linear_args(pl, (const uint16_t *)act, B, EPI_F32);
   a.out_f32 = out; a.out_stride = N;
-  CUDA_TRY(nullptr, launch_linear(wfmt, a, (cudaStream_t)cuda_stream, false));
+  CUDA_TRY(nullptr, launch_linear(wfmt, a, (cudaStream_t)cuda_stream, false, 2 * device_sms()));
   return TTS_GPT_OK;
 }
 
@@ -1376,11 +1381,12 @@ int32_t tts_gpt_op_linear_tc_scratch_bytes(int32_t N, int32_t K, size_t *bytes) 
 
 // the wide kernels on one row tile: int4 codes with group sums on the one-CTA kernel, the rest on the pair kernel
 static cudaError_t launch_wide(const GemmTcArgs &a, cudaStream_t st) {
-  if (a.wfmt == WF_INT4) return launch_gemm_tcw(a, 148, st, false);
+  const int n_sm = device_sms();
+  if (a.wfmt == WF_INT4) return launch_gemm_tcw(a, n_sm, st, false);
   CUtensorMap w_map, x_map;
   cudaError_t e = pw_image_map(&w_map, a.w_img, (size_t)((a.N + 127) / 128) * (a.K / 64));
   if (e == cudaSuccess) e = pw_image_map(&x_map, a.act_img, a.K / 64);
-  return e != cudaSuccess ? e : launch_gemm_pw(a, w_map, x_map, nullptr, pw_plan(a.N, a.K, a.B, a.mode == EPI_RESID, 148, a.ksplit).bn, 148, st, false);
+  return e != cudaSuccess ? e : launch_gemm_pw(a, w_map, x_map, nullptr, pw_plan(a.N, a.K, a.B, a.mode == EPI_RESID, n_sm, a.ksplit).bn, n_sm, st, false);
 }
 
 int32_t tts_gpt_op_linear_tc(int32_t wfmt, int32_t N, int32_t K, const void *w, const void *s, const void *bias,
@@ -1414,10 +1420,10 @@ int32_t tts_gpt_op_linear_tc(int32_t wfmt, int32_t N, int32_t K, const void *w, 
   a.w_img = wimg; a.act_img = aimg; a.N = N; a.K = K; a.B = B; a.ksplit = ksplit; a.wfmt = wfmt; a.scales = tiled_s;
   if (ksplit == 1) {
     a.mode = EPI_F32; a.bias = (const uint16_t *)bias; a.out_f32 = out; a.out_stride = N;
-    CUDA_TRY(nullptr, wide ? launch_wide(a, st) : launch_gemm_tc(a, 148, st, false));
+    CUDA_TRY(nullptr, wide ? launch_wide(a, st) : launch_gemm_tc(a, device_sms(), st, false));
   } else {   // partial sums per k-range, then folded in range order (what the following LayerNorm does in the engine)
     a.mode = EPI_RESID; a.out_f32 = part; a.out_stride = N;
-    CUDA_TRY(nullptr, wide ? launch_wide(a, st) : launch_gemm_tc(a, 148, st, false));
+    CUDA_TRY(nullptr, wide ? launch_wide(a, st) : launch_gemm_tc(a, device_sms(), st, false));
     fold_partials_kernel<<<(unsigned)(((size_t)B * N + 255) / 256), 256, 0, st>>>(part, ksplit, B, N, (const uint16_t *)bias, out);
     CUDA_TRY(nullptr, cudaGetLastError());
   }
@@ -1532,7 +1538,7 @@ int32_t tts_gpt_op_attention_cluster(int32_t R, int32_t n_head, const float *q, 
     return TTS_GPT_OK;
   }
   if (cluster_size == -3) {   // rows must be stream-major with ascending positions, as in a prefill pass
-    CUDA_TRY(nullptr, launch_attention_prefill_tc(a, R, 148, (cudaStream_t)cuda_stream, false));
+    CUDA_TRY(nullptr, launch_attention_prefill_tc(a, R, device_sms(), (cudaStream_t)cuda_stream, false));
     return TTS_GPT_OK;
   }
   if (cluster_size == -2) {   // same requirement on the rows
