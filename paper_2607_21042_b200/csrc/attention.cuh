@@ -669,11 +669,9 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 3) attention_stream_kernel(co
 inline bool attention_use_stream(int R, int H, int n_sm) { return R * H >= 4 * n_sm; }
 
 inline cudaError_t launch_attention_stream(const AttnArgs &a, int R, cudaStream_t st, bool pdl) {
-  static PerDeviceOnce attr_once;   // per device: opt-in to more than 48 KB of dynamic shared memory
+  static SmemOptIn opt_in;
   const size_t smem = (size_t)kAttnWarps * kAttnStageBytes;
-  if (attr_once.first()) {
-    cudaFuncSetAttribute(attention_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  }
+  if (const cudaError_t e = opt_in(attention_stream_kernel, smem)) return e;
   return launch_kernel(attention_stream_kernel, dim3(1, a.H, R), dim3(kAttnWarps * 32), smem, st, pdl, a);
 }
 
@@ -806,11 +804,9 @@ __global__ void __launch_bounds__(kAttnPrefillRows * 32, 3) attention_prefill_ke
 }
 
 inline cudaError_t launch_attention_prefill(const AttnArgs &a, int R, cudaStream_t st, bool pdl) {
-  static PerDeviceOnce attr_once;   // per device: opt-in to more than 48 KB of dynamic shared memory
+  static SmemOptIn opt_in;
   const size_t smem = (size_t)kAttnPrefillStages * kAttnStageBytes;
-  if (attr_once.first()) {
-    cudaFuncSetAttribute(attention_prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  }
+  if (const cudaError_t e = opt_in(attention_prefill_kernel, smem)) return e;
   const int groups = (R + kAttnPrefillRows - 1) / kAttnPrefillRows;
   return launch_kernel(attention_prefill_kernel, dim3(1, a.H, groups), dim3(kAttnPrefillRows * 32), smem, st, pdl, a, R);
 }

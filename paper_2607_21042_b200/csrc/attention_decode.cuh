@@ -359,8 +359,8 @@ inline bool attention_use_decode(int R, int H, int n_sm) { return R * H > 2 * n_
 
 // layer_row: first row of the layer in kv_map, the whole pool as rows of 64 bf16 (attention_decode_map)
 inline cudaError_t launch_attention_decode(const AttnArgs &a, int R, const CUtensorMap &kv_map, int layer_row, int n_sm, cudaStream_t st, bool pdl) {
-  static PerDeviceOnce attr_once;   // per device: opt-in to more than 48 KB of dynamic shared memory
-  if (attr_once.first()) cudaFuncSetAttribute(attention_decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attention_decode_smem_bytes());
+  static SmemOptIn opt_in;
+  if (const cudaError_t e = opt_in(attention_decode_kernel, attention_decode_smem_bytes())) return e;
   AdArgs ad;
   ad.at = a; ad.layer_row = layer_row; ad.n_pair = R * a.H;
   const int n_cta = std::min(n_sm, ad.n_pair);

@@ -396,9 +396,9 @@ inline size_t attention_prefill_tc_smem_bytes() { return 49152 + (size_t)kPtSlot
 
 template <bool PAIRED>
 inline cudaError_t launch_attention_prefill_tc_as(const AttnArgs &a, int R, cudaStream_t st, bool pdl) {
-  static PerDeviceOnce attr_once;   // per device: opt-in to more than 48 KB of dynamic shared memory
+  static SmemOptIn opt_in;
   const size_t smem = attention_prefill_tc_smem_bytes();
-  if (attr_once.first()) cudaFuncSetAttribute(attention_prefill_tc_kernel<PAIRED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (const cudaError_t e = opt_in(attention_prefill_tc_kernel<PAIRED>, smem)) return e;
   return launch_kernel(attention_prefill_tc_kernel<PAIRED>, dim3(1, a.H, (R + kPtRows - 1) / kPtRows), dim3(kPtThreads), smem, st, pdl, a, R);
 }
 // n_sm: SMs of the device.  A grid of at most one CTA per SM takes the form whose threads hold a page's scores in registers

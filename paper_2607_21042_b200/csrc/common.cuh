@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <atomic>
 
 namespace ttsgpt {
 
@@ -108,17 +109,20 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
 // orders this thread's earlier generic-proxy accesses of shared memory before its later bulk copies
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// A function attribute (the opt-in to more than 48 KB of dynamic shared memory) belongs to one device:
-// returns true the first time it is asked about the current device through this flag set.
-struct PerDeviceOnce {
-  bool done[64] = {};
-  bool first() {
+// The opt-in to more than 48 KB of dynamic shared memory, a function attribute that belongs to one device: made by every
+// thread that comes before one of them has made it, so that none launches ahead of it.
+struct SmemOptIn {
+  std::atomic<bool> done[64] = {};
+  template <typename... KArgs>
+  cudaError_t operator()(void (*kernel)(KArgs...), size_t bytes) {
     int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) return true;
-    if (done[dev]) return false;
-    done[dev] = true;
-    return true;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool known = dev >= 0 && dev < 64;
+    if (known && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && known) done[dev].store(true, std::memory_order_release);
+    return e;
   }
 };
 

@@ -463,7 +463,8 @@ inline PwPlan pw_plan(int N, int K, int rows, bool resid, int n_sm, int fixed_ks
 
 inline cudaError_t pw_encode(CUtensorMap *map, CUtensorMapDataType type, const void *base, size_t cols, size_t rows, size_t pitch_bytes, int box_cols,
                              int box_rows, CUtensorMapSwizzle swizzle) {
-  static PFN_cuTensorMapEncodeTiled encode = nullptr;   // the same address whoever looks it up first
+  static std::atomic<PFN_cuTensorMapEncodeTiled> known{nullptr};   // the same address whoever looks it up first
+  PFN_cuTensorMapEncodeTiled encode = known.load(std::memory_order_acquire);
   if (!encode) {
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult found;
@@ -471,6 +472,7 @@ inline cudaError_t pw_encode(CUtensorMap *map, CUtensorMapDataType type, const v
     if (e != cudaSuccess) return e;
     if (found != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
     encode = (PFN_cuTensorMapEncodeTiled)fn;
+    known.store(encode, std::memory_order_release);
   }
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, strides[1] = {(cuuint64_t)pitch_bytes};
   const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows}, step[2] = {1, 1};
@@ -490,8 +492,8 @@ inline cudaError_t pw_rows_map(CUtensorMap *map, const float *base, size_t cols,
 // w_map, x_map: pw_image_map of a0.w_img and a0.act_img; out_map: pw_rows_map of a0.out_f32 (null: plain stores)
 inline cudaError_t launch_gemm_pw(const GemmTcArgs &a0, const CUtensorMap &w_map, const CUtensorMap &x_map, const CUtensorMap *out_map, int bn, int n_sm,
                                   cudaStream_t st, bool pdl) {
-  static PerDeviceOnce attr_once;   // per device: opt-in to more than 48 KB of dynamic shared memory
-  if (attr_once.first()) cudaFuncSetAttribute(gemm_pw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pw_smem_bytes());
+  static SmemOptIn opt_in;
+  if (const cudaError_t e = opt_in(gemm_pw_kernel, pw_smem_bytes())) return e;
   GemmTcArgs a = a0;
   a.bn = bn;
   a.stages = pw_stages(bn);

@@ -918,11 +918,9 @@ inline int tcw_ksplit_resid(int K) { return std::max(1, std::min(kTwMaxPartials,
 
 // n_sm: SMs of the device; a grid that fits at one CTA per SM gets the deep ring
 inline cudaError_t launch_gemm_tcw(const GemmTcArgs &a0, int n_sm, cudaStream_t st, bool pdl) {
-  static PerDeviceOnce attr_once;
-  if (attr_once.first()) {
-    cudaFuncSetAttribute(gemm_tcw_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_tcw_smem_bytes(kTwMaxStages));
-    cudaFuncSetAttribute(gemm_tcw_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_tcw_smem_bytes(kTwMaxStages));
-  }
+  static SmemOptIn opt_in, opt_in_grouped;
+  if (const cudaError_t e = opt_in(gemm_tcw_kernel<false>, gemm_tcw_smem_bytes(kTwMaxStages))) return e;
+  if (const cudaError_t e = opt_in_grouped(gemm_tcw_kernel<true>, gemm_tcw_smem_bytes(kTwMaxStages))) return e;
   GemmTcArgs a = a0;
   dim3 grid((a.N + 127) / 128, a.ksplit, (a.B + kMaxRows - 1) / kMaxRows);
   a.stages = (int)(grid.x * grid.y * grid.z) <= n_sm ? kTwMaxStages : 3;
@@ -946,9 +944,8 @@ inline size_t gemm_tc_smem_bytes(int cn, int stages) { return (size_t)stages * (
 
 template <bool GROUPED, int CN>
 inline cudaError_t launch_gemm_tc_as(GemmTcArgs a, int stages, cudaStream_t st, bool pdl) {
-  static PerDeviceOnce attr_once;   // per device: opt-in to more than 48 KB of dynamic shared memory
-  if (attr_once.first())
-    cudaFuncSetAttribute(gemm_tc_kernel<GROUPED, CN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_tc_smem_bytes(CN, kTcMaxStages));
+  static SmemOptIn opt_in;
+  if (const cudaError_t e = opt_in(gemm_tc_kernel<GROUPED, CN>, gemm_tc_smem_bytes(CN, kTcMaxStages))) return e;
   a.stages = stages;
   dim3 grid((a.N + kTcTileM - 1) / kTcTileM, (a.B + CN - 1) / CN, a.ksplit);
   return launch_kernel(gemm_tc_kernel<GROUPED, CN>, grid, dim3(kTcThreads), gemm_tc_smem_bytes(CN, stages), st, pdl, a);

@@ -630,9 +630,9 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 3) attention_fp8_stream_kerne
 }
 
 inline cudaError_t launch_attention_fp8_stream(const Fp8AttnArgs &a, int R, cudaStream_t st, bool pdl) {
-  static PerDeviceOnce attr_once;   // per device: opt-in to more than 48 KB of dynamic shared memory
+  static SmemOptIn opt_in;
   const size_t smem = (size_t)kAttnWarps * kFp8Stages * kFp8StageBytes;
-  if (attr_once.first()) cudaFuncSetAttribute(attention_fp8_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (const cudaError_t e = opt_in(attention_fp8_stream_kernel, smem)) return e;
   return launch_kernel(attention_fp8_stream_kernel, dim3(1, a.H, R), dim3(kAttnWarps * 32), smem, st, pdl, a);
 }
 

@@ -626,10 +626,8 @@ template <int WF, int RT, int MODE, int NB>
 inline cudaError_t launch_linear_nb(const LinearArgs &a, int grid, cudaStream_t st, bool pdl) {
   const int ks = a.ksplit > 1 ? a.ksplit : 1;
   const size_t smem = linear_smem_bytes(WF, RT, MODE, a.B, a.K / ks);
-  static PerDeviceOnce attr_once;   // per device: opt-in to more than 48 KB of dynamic shared memory
-  if (attr_once.first()) {
-    cudaFuncSetAttribute(linear_kernel<WF, RT, MODE, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  }
+  static SmemOptIn opt_in;
+  if (const cudaError_t e = opt_in(linear_kernel<WF, RT, MODE, NB>, 200 * 1024)) return e;
   return launch_kernel(linear_kernel<WF, RT, MODE, NB>, dim3(grid, ks), dim3(kLinearThreads), smem, st, pdl, a);
 }
 

@@ -1,6 +1,10 @@
 """Sizes at which the kernels of middle decode batches and of the largest prefill passes can go wrong: 32-token units and
 pages that begin or end with the newest token, (row, head) pairs cut over warps, row tiles without rows, ragged tiles;
 each against the fp64 oracle on identical history."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -255,3 +259,41 @@ def test_half_page_decode_attention(S):
     lg2, _ = _run(eng, prefixes, 4)
     assert np.array_equal(lg, lg2)
     eng.destroy()
+
+
+THREADS = """
+import threading, numpy as np, torch
+from paper_2607_21042_b200 import binding as B, cases as C
+cfgs = [C.tiny_config(wfmt=f, kv_fmt=k, max_streams=2, n_pages=48, max_context=2048, max_pos=2048) for f in (0, 1, 2) for k in (0, 1)]
+weights = [C.make_weights(c, seed=41) for c in cfgs]
+prefixes = [torch.from_numpy(p.view(np.int16)).to("cuda:0") for p in C.make_prefixes(cfgs[0], [1300, 70], seed=42)]
+torch.cuda.synchronize()
+gate, got = threading.Barrier(len(cfgs)), {}
+def work(i, wait):
+    torch.cuda.set_device(0)
+    eng = B.TtsGpt(cfgs[i], weights[i], "cuda:0")
+    lg = torch.zeros((3, 2, cfgs[i].vocab), device="cuda:0")
+    tok = torch.zeros((3, 2), dtype=torch.int32, device="cuda:0")
+    torch.cuda.synchronize()
+    if wait:
+        gate.wait(60)
+    ids, _ = eng.prefill(prefixes, out_tokens=tok[0], out_logits=lg[0])
+    eng.decode_steps(ids, 2, tok[1:], out_logits=lg[1:])
+    eng.sync()
+    got[i, wait] = lg.cpu().numpy()
+ts = [threading.Thread(target=work, args=(i, True)) for i in range(len(cfgs))]
+[t.start() for t in ts]
+[t.join() for t in ts]
+for i in range(len(cfgs)):
+    work(i, False)
+    assert np.array_equal(got[i, True], got[i, False]), i
+print("threads ok")
+"""
+
+
+def test_first_calls_from_several_threads():
+    """Six engines make a process's first launches at the same moment, each on a thread and stream of its own: every kernel's
+    shared-memory opt-in is in place for each of them, and the results are those of one engine after the other."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", THREADS], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "threads ok" in r.stdout, r.stdout + r.stderr
