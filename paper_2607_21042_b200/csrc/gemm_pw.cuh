@@ -301,6 +301,13 @@ __global__ void __launch_bounds__(kPwThreads, 1) gemm_pw_kernel(const __grid_con
       }
     }
     trace_mark(a.trace, a.trace_slot, 3);   // last copy issued
+    // The issuer's releases of the last stages are arrivals in this CTA's shared memory, which is the next CTA's once this
+    // one has left: they are waited for too.
+    if (it < n_stage) { s = 0; parity = 0; }
+    for (int i = 0; go && i < min(it, n_stage); ++i) {
+      go = tc_wait_warp<false>(empty + s, parity, failed, a.err);
+      if (++s == n_stage) { s = 0; parity ^= 1u; }
+    }
     __syncwarp();
   } else if (warp == 1) {
     if (rank == 0) {
