@@ -20,6 +20,7 @@
 // cluster launch and backs the stand-alone entry points.
 #pragma once
 #include <cooperative_groups.h>
+#include <algorithm>
 #include "common.cuh"
 #include "elementwise.cuh"
 
@@ -51,8 +52,31 @@ struct AttnArgs {
   int trace_slot;
   int out_image;             // 1: `out` is an activation image for the tensor-core linear (see act_image_offset)
   int old_pages_final;       // 1: one row per stream (decode step), pages before a row's last are not written by this step
-  const int *row_order;      // streaming variant: grid slot z handles row row_order[z] (null: row z)
+  const int4 *slots;         // decode steps of the engine: by rank of length {row, tokens, stream, 0}, and the row's pages
+  const int *slot_pages;     // [rank][pps] (null: rows as they come, through row_pos, row_stream and page_table)
   int *err;                  // set to 1 if a bounded wait of the streaming variant expires (may be null)
+};
+
+// Row `z` of an attention grid and, lane for lane, its first 32 pages: by a warp, one round trip to L2 where `slots` is set.
+struct AttnRow {
+  int row, n_tok;
+  const int *pt;
+  int mine;
+  template <typename Args>
+  __device__ __forceinline__ AttnRow(const Args &a, int z) {
+    const int lane = threadIdx.x & 31;
+    if (a.slots) {
+      const int4 d = a.slots[z];
+      row = d.x; n_tok = d.y;
+      pt = a.slot_pages + (size_t)z * a.pps;
+    } else {
+      row = z; n_tok = a.row_pos[z] + 1;
+      pt = a.page_table + (size_t)a.row_stream[z] * a.pps;
+    }
+    mine = lane < a.pps ? pt[lane] : 0;
+  }
+  // place of a page in the pool; `page` the same in every lane of the warp
+  __device__ __forceinline__ int phys(int page) const { return page < 32 ? __shfl_sync(0xFFFFFFFFu, mine, page) : pt[page]; }
 };
 
 // ------------------------------------------------------------------------------------------
@@ -155,7 +179,7 @@ __device__ __forceinline__ void fold_page(PageLoad &pl, const float (&qv)[8], in
 // 4*page + quarter; a warp's batch holds 4 units u0, u0+stride, ... (slots 4j..4j+3 = unit j, tokens
 // tg, tg+4, tg+8, tg+12 of the quarter), so that even a short context keeps every warp of every
 // CTA of the cluster busy with 32 loads in flight.
-__device__ __forceinline__ uint32_t load_quarters(PageLoad &pl, const uint16_t *kv_layer, const int *pt, int H, int h,
+__device__ __forceinline__ uint32_t load_quarters(PageLoad &pl, const uint16_t *kv_layer, const AttnRow &ar, int H, int h,
                                                   int u0, int stride, int n_units, int n_tok, int tg, int sub,
                                                   int &ng) {
   uint32_t vmask = 0u;
@@ -166,7 +190,7 @@ __device__ __forceinline__ uint32_t load_quarters(PageLoad &pl, const uint16_t *
     if (u < n_units) {
       ng = j + 1;
       const int page = u >> 2, qt = u & 3;
-      const int phys = pt[page];
+      const int phys = ar.phys(page);
       const uint16_t *K = kv_layer + (((size_t)phys * 2 + 0) * H + h) * kPageElems + (size_t)(16 * qt) * kHeadDim;
       const uint16_t *V = kv_layer + (((size_t)phys * 2 + 1) * H + h) * kPageElems + (size_t)(16 * qt) * kHeadDim;
       const int left = n_tok - page * kPageTokens - 16 * qt;   // tokens of the row from this quarter on
@@ -230,15 +254,15 @@ __device__ __forceinline__ void cta_merge(float m, float l, float (&o)[8], int w
 // every instruction once: instruction fetch shows up in their stall reasons)
 template <bool CLUSTER>
 __global__ void __launch_bounds__(kAttnWarps * 32) attention_kernel(const AttnArgs a) {
-  const int S = CLUSTER ? gridDim.x : 1, c = blockIdx.x, h = blockIdx.y, r = blockIdx.z;
+  const int S = CLUSTER ? gridDim.x : 1, c = blockIdx.x, h = blockIdx.y;
   trace_mark(a.trace, a.trace_slot, 0);
   // The row table and page table were written before the first kernel of the step started, so
   // they may be read ahead of the dependency wait.
-  const int n_tok = a.row_pos[r] + 1;
+  const AttnRow ar(a, blockIdx.z);
+  const int r = ar.row, n_tok = ar.n_tok;
   const int n_pages = (n_tok + kPageTokens - 1) / kPageTokens;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tg = lane >> 3, sub = lane & 7;
-  const int *pt = a.page_table + (size_t)a.row_stream[r] * a.pps;
 
   __shared__ float sm_m[kAttnWarps], sm_l[kAttnWarps], sm_o[kAttnWarps][kHeadDim];
   __shared__ float cl_all[kAttnMaxCluster][kAttnPartialFloats];  // rank 0: every rank's (M, L, O[64])
@@ -261,15 +285,15 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attention_kernel(const AttnAr
     const bool early = a.old_pages_final && gw < n_units;
     uint32_t vmask = 0u;
     int ng = 0;
-    if (early) vmask = load_quarters(pl, a.kv_layer, pt, a.H, h, gw, GW, n_units, n_tok, tg, sub, ng);
+    if (early) vmask = load_quarters(pl, a.kv_layer, ar, a.H, h, gw, GW, n_units, n_tok, tg, sub, ng);
     pdl_launch_dependents();
     pdl_wait();
     trace_mark(a.trace, a.trace_slot, 1);
     load_q(qv, a.q + (size_t)r * a.H * kHeadDim + h * kHeadDim + 8 * sub);
     if (early) {
       const int us = 4 * (n_pages - 1) + (tn >> 4);   // unit of the new token
+      const int phys = ar.phys(n_pages - 1);
       if (us % GW == gw && us / GW < 4 && (tn & 3) == tg) {
-        const int phys = pt[n_pages - 1];
         const uint4 kn = ld_cg_u4(a.kv_layer + (((size_t)phys * 2 + 0) * a.H + h) * kPageElems + (size_t)tn * kHeadDim + 8 * sub);
         const uint4 vn = ld_cg_u4(a.kv_layer + (((size_t)phys * 2 + 1) * a.H + h) * kPageElems + (size_t)tn * kHeadDim + 8 * sub);
         const int sel = 4 * (us / GW) + ((tn & 15) >> 2);
@@ -285,7 +309,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attention_kernel(const AttnAr
     }
     bool loaded = early;
     for (int u0 = gw; u0 < n_units; u0 += 4 * GW) {
-      if (!loaded) vmask = load_quarters(pl, a.kv_layer, pt, a.H, h, u0, GW, n_units, n_tok, tg, sub, ng);
+      if (!loaded) vmask = load_quarters(pl, a.kv_layer, ar, a.H, h, u0, GW, n_units, n_tok, tg, sub, ng);
       loaded = false;
       fold_slots(pl, qv, vmask, ng, m, l, o);
     }
@@ -295,7 +319,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attention_kernel(const AttnAr
     const bool early = a.old_pages_final && page < n_pages;
     const uint16_t *K0 = nullptr, *V0 = nullptr;
     if (early) {
-      const int phys = pt[page];
+      const int phys = ar.phys(page);
       K0 = a.kv_layer + (((size_t)phys * 2 + 0) * a.H + h) * kPageElems;
       V0 = a.kv_layer + (((size_t)phys * 2 + 1) * a.H + h) * kPageElems;
       load_page(pl, K0, V0, tg, sub);
@@ -320,7 +344,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attention_kernel(const AttnAr
     bool loaded = early;
     for (; page < n_pages; page += kAttnWarps) {
       if (!loaded) {
-        const int phys = pt[page];
+        const int phys = ar.phys(page);
         load_page(pl, a.kv_layer + (((size_t)phys * 2 + 0) * a.H + h) * kPageElems,
                   a.kv_layer + (((size_t)phys * 2 + 1) * a.H + h) * kPageElems, tg, sub);
       }
@@ -394,20 +418,19 @@ inline int attention_cluster_size(int R, int H, int n_sm, int fill = 1) {
 // 1730 (int4 weights) 0.674 -> 0.640, 10 rows of 930 0.895 -> 0.843.
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kAttnWarps * 32, 4) attention_half_kernel(const AttnArgs a) {
-  const int S = gridDim.x, c = blockIdx.x, h = blockIdx.y, r = blockIdx.z;
+  const int S = gridDim.x, c = blockIdx.x, h = blockIdx.y;
   trace_mark(a.trace, a.trace_slot, 0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tg = lane >> 3, sub = lane & 7;
   __shared__ float sm_m[kAttnWarps], sm_l[kAttnWarps], sm_o[kAttnWarps][kHeadDim];
   __shared__ float cl_all[kAttnMaxCluster][kAttnPartialFloats];   // rank 0: every split's (M, L, O[64])
   // row and page tables are final before the step's first kernel starts
-  const int n_tok = a.row_pos[r] + 1, n_half = (n_tok + 31) >> 5;
+  const AttnRow ar(a, blockIdx.z);
+  const int r = ar.row, n_tok = ar.n_tok, n_half = (n_tok + 31) >> 5;
   const int per = (n_half + S - 1) / S, n_chunks = (n_half + per - 1) / per;   // half pages per split, splits that have some
   const int first = c * per + warp, end = min(n_half, (c + 1) * per);
-  const int *pt = a.page_table + (size_t)a.row_stream[r] * a.pps;
   auto half_of = [&](int i) { return first + i * kAttnWarps; };
-  const int my_phys = half_of(lane) < end ? pt[half_of(lane) >> 1] : 0;        // page of the warp's item `lane`
   auto block = [&](int i) {                                                    // K rows of item i; V: v_off elements on
-    const int u = half_of(i), phys = i < 32 ? __shfl_sync(0xFFFFFFFFu, my_phys, i) : pt[u >> 1];
+    const int u = half_of(i), phys = ar.phys(u >> 1);
     return a.kv_layer + ((size_t)phys * 2 * a.H + h) * kPageElems + (u & 1) * (32 * kHeadDim);
   };
   const size_t v_off = (size_t)a.H * kPageElems;
@@ -544,42 +567,122 @@ inline cudaError_t launch_attention(const AttnArgs &a, int R, int cluster, cudaS
 
 // ------------------------------------------------------------------------------------------
 // streaming variant (the engine's path once there are enough (row, head) pairs to fill the GPU
-// several times): one CTA per (row, head), warp w takes pages w, w+4, ...  A page's K and V blocks
-// (8 KB each, contiguous in the pool) come in by two bulk asynchronous copies into the warp's own
-// 16 KB stage of shared memory; as soon as the warp has pulled the stage into registers, lane 0
-// requests the warp's next page into the same stage, so that the copy runs under the arithmetic
-// of the current page and every resident warp keeps 16 KB in flight with no registers tied up by
+// several times): a CTA works on one pair, or (attention_queue_kernel: three CTAs per SM) on one pair after the other, warp
+// w taking pages w, w+4, ... of each.
+// A page's K and V blocks (8 KB each, contiguous in the pool) come in by two bulk asynchronous copies into the warp's own
+// 16 KB stage of shared memory; as soon as the warp has pulled the stage into registers, lane 0 requests the warp's next
+// page into the same stage, be it of this pair or of the CTA's next one, so that the copy runs under the arithmetic and
+// the merge of the present pair and every resident warp keeps 16 KB in flight with no registers tied up by
 // outstanding loads.  Only the tokens that exist are copied from a partial last page.
+// Bound: HBM.  With a CTA per pair every CTA began with three dependent reads and a copy in front of its first product,
+// and ended in a merge, its stages empty meanwhile: 128 rows of 200 to 1200 tokens (455 MB a layer) 81.5 us, 5.6 TB/s; through
+// the queue 74.7, 6.1 TB/s.  (Copies alone, with nothing done to the pages: 67.)  The order of sums is the same either way.
 // ------------------------------------------------------------------------------------------
 constexpr uint32_t kAttnHalfStage = kPageElems * 2;          // one K or V block: 8 KB
 constexpr uint32_t kAttnStageBytes = 2 * kAttnHalfStage;
 constexpr unsigned long long kAttnWaitNs = 2000000000ull;
+constexpr int kAttnStreamCtas = 3;                           // resident per SM: 12 warps with 16 KB each
 
-__device__ __forceinline__ void stream_issue(const AttnArgs &a, const int *pt, int h, int page, int n_tok,
-                                             unsigned char *stage, uint64_t *bar) {
-  const int n_here = min(kPageTokens, n_tok - page * kPageTokens);
+// The (row, head) pairs of a launch in the order they are handed out: rows longest first, a row's heads next to each other.
+// A CTA starts with pairs blockIdx.x and blockIdx.x + gridDim.x and takes further ones from a counter in global memory, two
+// pairs ahead of the one it works on, until the first that does not exist: pairs - 2 gridDim.x successful takes and one
+// failing take per CTA, behind which the counter has wrapped to zero for the next launch.  Which CTA takes a pair changes
+// nothing in its result.
+struct AttnQueue {
+  unsigned int *next;                                        // zero between launches
+  unsigned int wrap;                                         // takes of a launch - 1
+  int n_pair;                                                // at least 2 gridDim.x
+};
+inline AttnQueue attn_queue(unsigned int *counter, int n_pair, int grid) {
+  return AttnQueue{counter, (unsigned int)(n_pair - 2 * grid + grid - 1), n_pair};
+}
+constexpr int kAttnListPages = 32;
+struct AttnPair {
+  int row, head, n_tok, slot;                                // row < 0: none
+  int phys[kAttnListPages];                                  // its first pages' places in the pool
+};
+// by a warp: pair i into shared memory
+template <typename Args>
+__device__ __forceinline__ void attn_pair(AttnPair &p, const AttnQueue &qu, int i, const Args &a) {
+  const int lane = threadIdx.x & 31;
+  if (i >= qu.n_pair) {
+    if (lane == 0) { p.row = -1; p.head = 0; p.n_tok = 0; p.slot = 0; }
+    return;
+  }
+  const int slot = i / a.H;
+  const int4 d = a.slots[slot];
+  const int phys = lane < a.pps ? a.slot_pages[slot * a.pps + lane] : 0;
+  if (lane == 0) { p.row = d.x; p.head = i - slot * a.H; p.n_tok = d.y; p.slot = slot; }
+  p.phys[lane] = phys;
+}
+// by one lane: index of a further pair (not to be called again once it has returned one that does not exist)
+__device__ __forceinline__ int attn_take(const AttnQueue &qu) { return 2 * (int)gridDim.x + (int)atomicInc(qu.next, qu.wrap); }
+
+__device__ __forceinline__ void stream_issue(const AttnArgs &a, int phys, int h, int n_here, unsigned char *stage, uint64_t *bar) {
   const uint32_t bytes = (uint32_t)n_here * kHeadDim * 2;
-  const int phys = pt[page];
   const uint16_t *K = a.kv_layer + (((size_t)phys * 2 + 0) * a.H + h) * kPageElems;
-  const uint16_t *V = a.kv_layer + (((size_t)phys * 2 + 1) * a.H + h) * kPageElems;
   mbar_expect_tx(bar, 2 * bytes);
   bulk_copy_g2s(stage, K, bytes, bar);
-  bulk_copy_g2s(stage + kAttnHalfStage, V, bytes, bar);
+  bulk_copy_g2s(stage + kAttnHalfStage, K + (size_t)a.H * kPageElems, bytes, bar);
 }
 
-__global__ void __launch_bounds__(kAttnWarps * 32, 3) attention_stream_kernel(const AttnArgs a) {
+// A page in a warp's stage into the warp's running softmax: scores, then V into registers, then `refill` (the stage is free),
+// then the weighted values.  PATCH: the rows of token `tn`, copied before the kernel in front had written them, are kn, vn.
+template <typename Refill>
+__device__ __forceinline__ void stream_fold(const unsigned char *stage, int n_here, bool patch, int tn, const uint4 &kn, const uint4 &vn, int tg, int sub,
+                                            const float (&qv)[8], float &m, float &l, float (&o)[8], Refill refill) {
+  uint32_t vmask = 0u;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) vmask |= (tg + 4 * i < n_here) ? (1u << i) : 0u;
+  const int sel = tn >> 2;
+  uint4 kk[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    kk[i] = *reinterpret_cast<const uint4 *>(stage + (size_t)(tg + 4 * i) * (kHeadDim * 2) + 16 * sub);
+    if (patch && i == sel) kk[i] = kn;
+  }
+  float s[16];
+  const float pm = score_slots<16>(kk, qv, vmask, s);
+  uint4 vv[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    vv[i] = *reinterpret_cast<const uint4 *>(stage + kAttnHalfStage + (size_t)(tg + 4 * i) * (kHeadDim * 2) + 16 * sub);
+    if (patch && i == sel) vv[i] = vn;
+  }
+  // The stage may be overwritten only after every read of it has returned: the K reads have (the
+  // scores consumed them); one word of every V read is folded into a value that the fence below
+  // takes as an operand, so the copy cannot be issued ahead of those reads either.
+  uint32_t seen = 0u;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) seen ^= vv[i].x;
+  __syncwarp();   // every lane has read the stage
+  if ((threadIdx.x & 31) == 0) asm volatile("fence.proxy.async.shared::cta; // after %0" ::"r"(seen) : "memory");
+  refill();
+  accum_slots<16>(vv, s, pm, vmask, m, l, o);
+}
+__device__ __forceinline__ void attn_write_out(const AttnArgs &a, int row, int col, float v) {
+  uint16_t *out = a.out_image ? reinterpret_cast<uint16_t *>(reinterpret_cast<unsigned char *>(a.out) + act_image_offset_tiled(row, col, a.H * kHeadDim))
+                              : a.out + (size_t)row * a.H * kHeadDim + col;
+  *out = float_to_bf16_bits(v);
+}
+
+// a CTA per pair
+__global__ void __launch_bounds__(kAttnWarps * 32, kAttnStreamCtas) attention_stream_kernel(const AttnArgs a) {
   extern __shared__ __align__(128) unsigned char attn_stages[];   // [warp][K 8 KB | V 8 KB]
   __shared__ __align__(8) uint64_t bars[kAttnWarps];
   __shared__ float sm_m[kAttnWarps], sm_l[kAttnWarps], sm_o[kAttnWarps][kHeadDim];
-  const int h = blockIdx.y, r = a.row_order ? a.row_order[blockIdx.z] : blockIdx.z;
   trace_mark(a.trace, a.trace_slot, 0);
-  const int n_tok = a.row_pos[r] + 1;   // row and page tables are final before the step's first kernel starts
+  const AttnRow ar(a, blockIdx.z);   // row and page tables are final before the step's first kernel starts
+  const int h = blockIdx.y, n_tok = ar.n_tok;
   const int n_pages = (n_tok + kPageTokens - 1) / kPageTokens;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tg = lane >> 3, sub = lane & 7;
-  const int *pt = a.page_table + (size_t)a.row_stream[r] * a.pps;
   unsigned char *stage = attn_stages + (size_t)warp * kAttnStageBytes;
   uint64_t *bar = bars + warp;
+  auto request = [&](int page) {
+    const int phys = ar.phys(page);
+    if (lane == 0) stream_issue(a, phys, h, min(kPageTokens, n_tok - page * kPageTokens), stage, bar);
+  };
 
   float m = -INFINITY, l = 0.f;
   float o[8];
@@ -592,18 +695,16 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 3) attention_stream_kernel(co
   // warp's first page is requested ahead of the dependency wait and those two rows are read again
   // afterwards if the page holds them.
   const bool early = a.old_pages_final && page < n_pages;
-  if (lane == 0) {
-    mbar_init(bar, 1);
-    if (early) stream_issue(a, pt, h, page, n_tok, stage, bar);
-  }
+  if (lane == 0) mbar_init(bar, 1);
   __syncwarp();
+  if (early) request(page);
   pdl_launch_dependents();
   pdl_wait();
   trace_mark(a.trace, a.trace_slot, 1);
-  load_q(qv, a.q + (size_t)r * a.H * kHeadDim + h * kHeadDim + 8 * sub);
-  if (!early && page < n_pages && lane == 0) stream_issue(a, pt, h, page, n_tok, stage, bar);
+  load_q(qv, a.q + (size_t)ar.row * a.H * kHeadDim + h * kHeadDim + 8 * sub);
+  if (!early && page < n_pages) request(page);
   uint32_t phase = 0;
-  bool first = true;
+#pragma unroll 1
   for (; page < n_pages; page += kAttnWarps) {
     if (!mbar_wait_bounded(bar, phase, kAttnWaitNs)) {
       if (a.err) atomicExch(a.err, 1);
@@ -611,59 +712,108 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 3) attention_stream_kernel(co
       break;
     }
     phase ^= 1u;
-    const int n_here = min(kPageTokens, n_tok - page * kPageTokens);
-    uint32_t vmask = 0u;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) vmask |= (tg + 4 * i < n_here) ? (1u << i) : 0u;
-    // the new token's rows, if this page was copied before the kernel in front had written them
-    const bool patch = first && early && page == n_pages - 1 && (tn & 3) == tg;
-    const int sel = tn >> 2;
+    const bool last = page == n_pages - 1, patch = early && page == warp && last && (tn & 3) == tg;
     uint4 kn = make_uint4(0, 0, 0, 0), vn = kn;
-    if (patch) {
-      const int phys = pt[page];
-      kn = ld_cg_u4(a.kv_layer + (((size_t)phys * 2 + 0) * a.H + h) * kPageElems + (size_t)tn * kHeadDim + 8 * sub);
-      vn = ld_cg_u4(a.kv_layer + (((size_t)phys * 2 + 1) * a.H + h) * kPageElems + (size_t)tn * kHeadDim + 8 * sub);
+    if (early && page == warp && last) {
+      const uint16_t *K = a.kv_layer + (((size_t)ar.phys(page) * 2 + 0) * a.H + h) * kPageElems + (size_t)tn * kHeadDim + 8 * sub;
+      if (patch) { kn = ld_cg_u4(K); vn = ld_cg_u4(K + (size_t)a.H * kPageElems); }
     }
-    first = false;
-    uint4 kk[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      kk[i] = *reinterpret_cast<const uint4 *>(stage + (size_t)(tg + 4 * i) * (kHeadDim * 2) + 16 * sub);
-      if (patch && i == sel) kk[i] = kn;
-    }
-    float s[16];
-    const float pm = score_slots<16>(kk, qv, vmask, s);
-    uint4 vv[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      vv[i] = *reinterpret_cast<const uint4 *>(stage + kAttnHalfStage + (size_t)(tg + 4 * i) * (kHeadDim * 2) + 16 * sub);
-      if (patch && i == sel) vv[i] = vn;
-    }
-    // The stage may be overwritten only after every read of it has returned: the K reads have (the
-    // scores consumed them); one word of every V read is folded into a value that the fence below
-    // takes as an operand, so the copy cannot be issued ahead of those reads either.
-    uint32_t seen = 0u;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) seen ^= vv[i].x;
-    __syncwarp();   // every lane has read the stage
-    if (page + kAttnWarps < n_pages && lane == 0) {
-      asm volatile("fence.proxy.async.shared::cta; // after %0" ::"r"(seen) : "memory");
-      stream_issue(a, pt, h, page + kAttnWarps, n_tok, stage, bar);
-    }
-    accum_slots<16>(vv, s, pm, vmask, m, l, o);
+    stream_fold(stage, min(kPageTokens, n_tok - page * kPageTokens), patch, tn, kn, vn, tg, sub, qv, m, l, o,
+                [&]() { if (page + kAttnWarps < n_pages) request(page + kAttnWarps); });
   }
   trace_mark(a.trace, a.trace_slot, 3);
-  const int e = threadIdx.x;
   float M, L, O;
   cta_merge(m, l, o, warp, tg, sub, sm_m, sm_l, sm_o, M, L, O);
-  if (e < kHeadDim) {
-    uint16_t *out = a.out_image ? reinterpret_cast<uint16_t *>(reinterpret_cast<unsigned char *>(a.out) + act_image_offset_tiled(r, h * kHeadDim + e, a.H * kHeadDim))
-                                : a.out + (size_t)r * a.H * kHeadDim + h * kHeadDim + e;
-    *out = float_to_bf16_bits(O / L);
-  }
+  if (threadIdx.x < kHeadDim) attn_write_out(a, ar.row, h * kHeadDim + threadIdx.x, O / L);
   trace_mark(a.trace, a.trace_slot, 2);
 }
 
+// three CTAs per SM working through the pairs (decode steps of the engine)
+__global__ void __launch_bounds__(kAttnWarps * 32, kAttnStreamCtas) attention_queue_kernel(const AttnArgs a, const AttnQueue qu) {
+  extern __shared__ __align__(128) unsigned char attn_stages[];   // [warp][K 8 KB | V 8 KB]
+  __shared__ __align__(8) uint64_t bars[kAttnWarps];
+  __shared__ AttnPair pairs[4];                                   // pair number k of the CTA in slot k % 4
+  __shared__ float sm_m[2][kAttnWarps], sm_l[2][kAttnWarps], sm_o[2][kAttnWarps][kHeadDim];
+  __shared__ int sm_dead;                                         // some warp's wait has expired
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tg = lane >> 3, sub = lane & 7;
+  unsigned char *stage = attn_stages + (size_t)warp * kAttnStageBytes;
+  uint64_t *bar = bars + warp;
+  trace_mark(a.trace, a.trace_slot, 0);
+  if (lane == 0) mbar_init(bar, 1);
+  if (threadIdx.x == 0) sm_dead = 0;
+  if (warp < 2) attn_pair(pairs[warp], qu, blockIdx.x + warp * gridDim.x, a);
+  __syncthreads();
+  bool pending = false;                         // a page of this warp is in the stage or on its way there
+  auto request = [&](const AttnPair &p, int page) {   // the page of a pair, if there is one
+    pending = page * kPageTokens < p.n_tok;
+    if (pending && lane == 0) {
+      const int phys = page < kAttnListPages ? p.phys[page] : a.slot_pages[p.slot * a.pps + page];
+      stream_issue(a, phys, p.head, min(kPageTokens, p.n_tok - page * kPageTokens), stage, bar);
+    }
+  };
+  request(pairs[0], warp);                      // as above: ahead of the dependency wait
+  pdl_launch_dependents();
+  pdl_wait();
+  trace_mark(a.trace, a.trace_slot, 1);
+  uint32_t phase = 0;
+  bool more = true;                             // the last warp: the counter has not run out
+#pragma unroll 1
+  for (int k = 0; pairs[k & 3].row >= 0; ++k) {
+    const AttnPair &cur = pairs[k & 3], &next = pairs[(k + 1) & 3];
+    if (warp == kAttnWarps - 1) {               // the warp with the fewest pages looks up the pair behind the next one
+      int i = qu.n_pair;
+      if (more && lane == 0) i = attn_take(qu);
+      i = __shfl_sync(0xFFFFFFFFu, i, 0);
+      more = i < qu.n_pair;
+      attn_pair(pairs[(k + 2) & 3], qu, i, a);
+    }
+    const int row = cur.row, head = cur.head, n_tok = cur.n_tok, n_pages = (n_tok + kPageTokens - 1) / kPageTokens;
+    float m = -INFINITY, l = 0.f;
+    float o[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) o[e] = 0.f;
+    float qv[8];
+    load_q(qv, a.q + (size_t)row * a.H * kHeadDim + head * kHeadDim + 8 * sub);
+    const int tn = (n_tok - 1) & (kPageTokens - 1);   // the new token's slot in the last page
+    if (warp >= n_pages) request(next, warp);   // no page of this pair for the warp: on to the next
+#pragma unroll 1
+    for (int page = warp; page < n_pages; page += kAttnWarps) {
+      if (!mbar_wait_bounded(bar, phase, kAttnWaitNs)) {
+        if (a.err) atomicExch(a.err, 1);
+        mbar_wait_bounded(bar, phase, kAttnWaitNs);   // a last chance for the copy in flight towards this CTA
+        sm_dead = 1;
+        pending = false;
+        break;
+      }
+      phase ^= 1u;
+      const bool patch = k == 0 && page == warp && page == n_pages - 1 && (tn & 3) == tg;
+      uint4 kn = make_uint4(0, 0, 0, 0), vn = kn;
+      if (patch) {
+        const uint16_t *K = a.kv_layer + (((size_t)cur.phys[page] * 2 + 0) * a.H + head) * kPageElems + (size_t)tn * kHeadDim + 8 * sub;
+        kn = ld_cg_u4(K); vn = ld_cg_u4(K + (size_t)a.H * kPageElems);
+      }
+      stream_fold(stage, min(kPageTokens, n_tok - page * kPageTokens), patch, tn, kn, vn, tg, sub, qv, m, l, o, [&]() {
+        if (page + kAttnWarps < n_pages) request(cur, page + kAttnWarps);
+        else request(next, warp);
+      });
+    }
+    if (k == 0) trace_mark(a.trace, a.trace_slot, 3);
+    float M, L, O;
+    cta_merge(m, l, o, warp, tg, sub, sm_m[k & 1], sm_l[k & 1], sm_o[k & 1], M, L, O);   // its barrier also publishes pairs[]
+    if (sm_dead) break;                         // (a wait expires after seconds: every thread has read the mark of the pair in front by then)
+    if (threadIdx.x < kHeadDim) attn_write_out(a, row, head * kHeadDim + threadIdx.x, O / L);
+  }
+  if (pending) mbar_wait_bounded(bar, phase, kAttnWaitNs);   // behind an expired wait: no copy may be in flight towards a CTA that has left
+  if (warp == kAttnWarps - 1 && lane == 0 && sm_dead)
+    while (more) more = attn_take(qu) < qu.n_pair;           // the counter returns to zero all the same
+  trace_mark(a.trace, a.trace_slot, 2);
+}
+
+// Pairs from which they are handed out by a queue instead of a CTA each.  us per layer, a CTA per pair / queue, ragged rows:
+// 37 rows of 50 to 1100 tokens 21.2 / 25.4 (the long pairs' CTAs hold a second one from the start), 64 of 200 to 800 33.9 /
+// 34.0, 90 of 200 to 1200 58.5 / 55.5, 128 of 200 to 1200 81.5 / 74.7.
+inline bool attention_use_queue(int n_pair, int n_sm) { return n_pair > 10 * n_sm; }
 // (row, head) pairs from which the streaming variant is used where the kernels above and that of the middle batches are not
 // (sampled steps, batches of more than ten pairs per SM): the GPU is then covered four times over with one CTA per pair.
 inline bool attention_use_stream(int R, int H, int n_sm) { return R * H >= 4 * n_sm; }
@@ -673,6 +823,15 @@ inline cudaError_t launch_attention_stream(const AttnArgs &a, int R, cudaStream_
   const size_t smem = (size_t)kAttnWarps * kAttnStageBytes;
   if (const cudaError_t e = opt_in(attention_stream_kernel, smem)) return e;
   return launch_kernel(attention_stream_kernel, dim3(1, a.H, R), dim3(kAttnWarps * 32), smem, st, pdl, a);
+}
+
+// Decode steps with `slots` and at least two pairs.  counter: zero between launches.
+inline cudaError_t launch_attention_queue(const AttnArgs &a, int R, unsigned int *counter, int n_sm, cudaStream_t st, bool pdl) {
+  static SmemOptIn opt_in;
+  const size_t smem = (size_t)kAttnWarps * kAttnStageBytes;
+  if (const cudaError_t e = opt_in(attention_queue_kernel, smem)) return e;
+  const int n_pair = R * a.H, grid = std::min(n_pair / 2, kAttnStreamCtas * n_sm);
+  return launch_kernel(attention_queue_kernel, dim3(grid), dim3(kAttnWarps * 32), smem, st, pdl, a, attn_queue(counter, n_pair, grid));
 }
 
 // ------------------------------------------------------------------------------------------

@@ -26,7 +26,9 @@ struct RowTable {
   const uint16_t **row_emb;   // bf16 [d] embedding of a prefix row
   int *out_rows;              // rows whose logits are wanted, compacted
   int *out_slot;              // position of that row's results in the caller's output arrays
-  int *row_order;             // decode steps: rows by descending context length (longest first)
+  // decode steps, by rank of context length (longest first):
+  int4 *slots;                // {row, tokens with the step's own, stream, 0}
+  int *slot_pages;            // [rank][pps] the row's pages
 };
 
 // x[r,:] = tok_emb[token] + pos_emb[posidx]   (generated tokens take a positional embedding from

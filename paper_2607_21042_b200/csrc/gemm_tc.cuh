@@ -333,10 +333,6 @@ __device__ __forceinline__ void tc_linger(volatile int *failed) {
   while (__any_sync(0xFFFFFFFFu, global_timer_ns() - t0 <= kTcLingerNs)) {}
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
 // GROUPED (int4 weights): the MMAs of each 128-column group accumulate into one of two 32-column
 // tensor-memory buffers; while the next group runs in the other buffer, the epilogue warps read the
 // finished group out, multiply it by the group's scale of their weight row and add it to fp32

@@ -109,7 +109,8 @@ struct Fp8AttnArgs {
   float *partials;                // [R][H][kAttnMaxChunks][66]
   unsigned int *tickets;          // [R][H], zero between launches
   int H, pps, out_image;
-  const int *row_order;           // streaming variant: rows by descending context length, or null
+  const int4 *slots;              // see AttnArgs
+  const int *slot_pages;
   int *err;                       // streaming variant: set when a bounded wait ran out
   const uint16_t *stage;          // decode variant: the step's new K/V rows, bf16 [R][2][H*64]
   int whole_pages;                // decode variant, 1: the ticket kernel's split into whole pages and its order of sums
@@ -287,7 +288,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attention_fp8_kernel(const Fp
 // Per step, against the encoding kernel and the ticket kernel: 1 row of 930 tokens 0.633 -> 0.493 ms, 3 rows 0.731 -> 0.610,
 // 9 rows 0.807 -> 0.758, 12 rows 0.951 -> 0.841, 28 rows of 730 tokens 1.254 -> 0.989.
 __global__ void __launch_bounds__(kAttnWarps * 32) attention_fp8_decode_kernel(const Fp8AttnArgs a) {
-  const int c = blockIdx.x, S = gridDim.x, h = blockIdx.y, r = blockIdx.z;
+  const int c = blockIdx.x, S = gridDim.x, h = blockIdx.y;
   trace_mark(a.trace, a.trace_slot, 0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tg = lane >> 2, sub = lane & 3;
@@ -295,20 +296,18 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attention_fp8_decode_kernel(c
   __shared__ float cl_all[kAttnMaxChunks][kAttnPartialFloats];          // rank 0: every split's (M, L, O[64])
   __shared__ __align__(16) unsigned char sm_new[2][kHeadDim];           // the new token's codes
   // row and page tables are final before the step's first kernel starts
-  const int n_tok = min(a.row_pos[r] + 1, a.pps * kPageTokens);
+  const AttnRow ar(a, blockIdx.z);
+  const int r = ar.row, n_tok = min(ar.n_tok, a.pps * kPageTokens);
   // The row is cut into half pages of 32 tokens, dealt in runs to the splits and round-robin to the warps of a split; with
   // whole_pages a warp takes both halves of a page.  Item i of this warp is half page first + (i >> sh) * step + (i & sh).
   const int sh = a.whole_pages, n_half = (n_tok + 31) / 32, n_unit = sh ? (n_half + 1) >> 1 : n_half;
   const int per = (n_unit + S - 1) / S;                    // units per split
   const int n_chunks = (n_unit + per - 1) / per;           // splits that have units
   const int first = (c * per + warp) << sh, step = kAttnWarps << sh, end = min(n_half, ((c + 1) * per) << sh);
-  const int *pt = a.page_table + (size_t)a.row_stream[r] * a.pps;
   const size_t v_off = (size_t)a.H * kFp8BlockBytes;
   auto half_of = [&](int i) { return first + (i >> sh) * step + (i & sh); };
-  const int my_phys = half_of(lane) < end ? pt[half_of(lane) >> 1] : 0;     // page of item `lane`
   auto block = [&](int i) {                                                 // K block of item i's page; V: v_off on
-    const int phys = i < 32 ? __shfl_sync(0xFFFFFFFFu, my_phys, i) : pt[half_of(i) >> 1];
-    return a.kv_layer + ((size_t)phys * 2 * a.H + h) * kFp8BlockBytes;
+    return a.kv_layer + ((size_t)ar.phys(half_of(i) >> 1) * 2 * a.H + h) * kFp8BlockBytes;
   };
 
   uint4 kk[4], vv[4];
@@ -354,7 +353,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attention_fp8_decode_kernel(c
     const uint16_t *st = a.stage + (size_t)r * 2 * a.H * kHeadDim + h * kHeadDim + 2 * lane;
     const uint16_t kc = e4m3_encode_row(__ldcg(reinterpret_cast<const unsigned int *>(st)), new_ks);
     const uint16_t vc = e4m3_encode_row(__ldcg(reinterpret_cast<const unsigned int *>(st + a.H * kHeadDim)), new_vs);
-    unsigned char *blk = const_cast<unsigned char *>(a.kv_layer) + ((size_t)pt[newest >> 1] * 2 * a.H + h) * kFp8BlockBytes;
+    unsigned char *blk = const_cast<unsigned char *>(a.kv_layer) + ((size_t)ar.phys(newest >> 1) * 2 * a.H + h) * kFp8BlockBytes;
     *reinterpret_cast<uint16_t *>(blk + (size_t)tn * kHeadDim + 2 * lane) = kc;
     *reinterpret_cast<uint16_t *>(blk + v_off + (size_t)tn * kHeadDim + 2 * lane) = vc;
     if (lane < 2) *reinterpret_cast<float *>(blk + lane * v_off + kPageTokens * kHeadDim + 4 * tn) = lane ? new_vs : new_ks;
@@ -503,8 +502,7 @@ inline cudaError_t launch_kv_dequant_pages(const unsigned char *kv_layer, uint16
 constexpr uint32_t kFp8StageBytes = 2 * kFp8BlockBytes;   // K block | V block
 constexpr int kFp8Stages = 2;
 
-__device__ __forceinline__ void fp8_stream_issue(const Fp8AttnArgs &a, const int *pt, int h, int page, unsigned char *stage, uint64_t *bar) {
-  const int phys = pt[page];
+__device__ __forceinline__ void fp8_stream_issue(const Fp8AttnArgs &a, int phys, int h, unsigned char *stage, uint64_t *bar) {
   const unsigned char *K = a.kv_layer + (((size_t)phys * 2 + 0) * a.H + h) * kFp8BlockBytes;
   mbar_expect_tx(bar, kFp8StageBytes);
   bulk_copy_g2s(stage, K, kFp8BlockBytes, bar);
@@ -515,36 +513,34 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 3) attention_fp8_stream_kerne
   extern __shared__ __align__(128) unsigned char fp8_stages[];   // [warp][stage][K block | V block]
   __shared__ __align__(8) uint64_t bars[kAttnWarps][kFp8Stages];
   __shared__ float sm_m[kAttnWarps], sm_l[kAttnWarps], sm_o[kAttnWarps][kHeadDim];
-  const int h = blockIdx.y, r = a.row_order ? a.row_order[blockIdx.z] : blockIdx.z;
+  const int h = blockIdx.y;
   trace_mark(a.trace, a.trace_slot, 0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tg = lane >> 2, sub = lane & 3;
-  const int n_tok = min(a.row_pos[r] + 1, a.pps * kPageTokens);   // row and page tables are final before the step's first kernel starts
+  const AttnRow ar(a, blockIdx.z);
+  const int r = ar.row, n_tok = min(ar.n_tok, a.pps * kPageTokens);   // row and page tables are final before the step's first kernel starts
   const int n_pages = (n_tok + kPageTokens - 1) / kPageTokens;
-  const int *pt = a.page_table + (size_t)a.row_stream[r] * a.pps;
   unsigned char *stages = fp8_stages + (size_t)warp * (kFp8Stages * kFp8StageBytes);
   // pages of this warp: warp, warp + 4, ...; iteration it uses stage it % 2
-  bool issued[kFp8Stages] = {false, false};
+  auto request = [&](int page, int s) {
+    const int phys = ar.phys(page);
+    if (lane == 0) fp8_stream_issue(a, phys, h, stages + s * kFp8StageBytes, &bars[warp][s]);
+  };
   if (lane == 0) {
 #pragma unroll
     for (int s = 0; s < kFp8Stages; ++s) mbar_init(&bars[warp][s], 1);
-#pragma unroll
-    for (int s = 0; s < kFp8Stages; ++s) {
-      const int page = warp + kAttnWarps * s;
-      if (page < n_pages - 1) { fp8_stream_issue(a, pt, h, page, stages + s * kFp8StageBytes, &bars[warp][s]); issued[s] = true; }
-    }
   }
+  __syncwarp();
+#pragma unroll
+  for (int s = 0; s < kFp8Stages; ++s)
+    if (warp + kAttnWarps * s < n_pages - 1) request(warp + kAttnWarps * s, s);
   __syncwarp();
   pdl_launch_dependents();
   pdl_wait();
   trace_mark(a.trace, a.trace_slot, 1);
-  if (lane == 0) {
 #pragma unroll
-    for (int s = 0; s < kFp8Stages; ++s) {
-      const int page = warp + kAttnWarps * s;
-      if (!issued[s] && page < n_pages) fp8_stream_issue(a, pt, h, page, stages + s * kFp8StageBytes, &bars[warp][s]);
-    }
-  }
+  for (int s = 0; s < kFp8Stages; ++s)
+    if (warp + kAttnWarps * s == n_pages - 1) request(n_pages - 1, s);
   float qv[16];
   {
     const float qs = 0.125f * 1.4426950408889634f;   // scores in log2 units
@@ -589,10 +585,8 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 3) attention_fp8_stream_kerne
     // The stage may be refilled only after every lane's reads of it have returned: the ballot needs a value
     // that every lane computed from what it read, and the fence takes the ballot as an operand.
     const unsigned int done = __ballot_sync(0xFFFFFFFFu, o[0] == o[0] || l >= 0.f);
-    if (page + kFp8Stages * kAttnWarps < n_pages && lane == 0) {
-      asm volatile("fence.proxy.async.shared::cta; // after %0" ::"r"(done) : "memory");
-      fp8_stream_issue(a, pt, h, page + kFp8Stages * kAttnWarps, stages + s * kFp8StageBytes, bar);
-    }
+    if (lane == 0) asm volatile("fence.proxy.async.shared::cta; // after %0" ::"r"(done) : "memory");
+    if (page + kFp8Stages * kAttnWarps < n_pages) request(page + kFp8Stages * kAttnWarps, s);
   }
   trace_mark(a.trace, a.trace_slot, 3);
   // warp result: sum over the 8 token groups

@@ -32,7 +32,7 @@ __global__ void init_pages_kernel(PageState ps) {
   if (i == 0) *ps.free_top = ps.n_pages;
 }
 
-// exclusive prefix sum of one int per thread over a block of kMaxRows threads
+// exclusive prefix sum of one int per thread over the first kMaxRows threads of a block
 __device__ __forceinline__ int block_exclusive_scan_128(int v, int *total) {
   __shared__ int warp_tot[kMaxRows / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -42,7 +42,7 @@ __device__ __forceinline__ int block_exclusive_scan_128(int v, int *total) {
     const int n = __shfl_up_sync(0xFFFFFFFFu, incl, o);
     if (lane >= o) incl += n;
   }
-  if (lane == 31) warp_tot[warp] = incl;
+  if (lane == 31 && warp < kMaxRows / 32) warp_tot[warp] = incl;
   __syncthreads();
   int base = 0, tot = 0;
   for (int w = 0; w < kMaxRows / 32; ++w) { if (w < warp) base += warp_tot[w]; tot += warp_tot[w]; }
@@ -58,15 +58,28 @@ struct StepParams {
 
 // One decode step: each stream whose context length sits on a page boundary pops a page (streams
 // in call order take pages in stack order), then the row table is written and ctx_len advances.
-__global__ void __launch_bounds__(kMaxRows) step_setup_kernel(const StepParams p, PageState ps, RowTable rt, StepIO *io) {
+// Attention's CTAs find what they work on in `slots` and `slot_pages`, by rank of the row's length: one round trip to L2
+// where row order, position, stream and page table were three, in front of the first page request of every CTA of 24 layers.
+constexpr int kSetupThreads = 512, kSetupPages = kMaxRows * 32 / kSetupThreads;   // page-table entries per thread: max_context is at most 2048
+__global__ void __launch_bounds__(kSetupThreads) step_setup_kernel(const StepParams p, PageState ps, RowTable rt, StepIO *io) {
   const int i = threadIdx.x;
+  __shared__ int len_s[kMaxRows], new_s[kMaxRows], rank_s[kMaxRows];
+  // the page lists, row by row: asked for together with everything else
+  int page[kSetupPages];
+#pragma unroll
+  for (int q = 0; q < kSetupPages; ++q) {
+    const int j = i + q * kSetupThreads, r = j / ps.pps;
+    page[q] = r < p.n ? ps.page_table[(size_t)p.stream_ids[r] * ps.pps + (j - r * ps.pps)] : 0;
+  }
   int s = 0, t = 0, need = 0;
   if (i < p.n) { s = p.stream_ids[i]; t = ps.ctx_len[s]; need = (t % kPageTokens) == 0; }
+  if (i < kMaxRows) len_s[i] = i < p.n ? t : -1;
   int total;
   const int rank = block_exclusive_scan_128(need, &total);
   const int top = *ps.free_top;
   if (i < p.n) {
-    if (need) ps.page_table[(size_t)s * ps.pps + t / kPageTokens] = ps.free_list[top - 1 - rank];
+    const int fresh = need ? ps.free_list[top - 1 - rank] : -1;
+    if (need) ps.page_table[(size_t)s * ps.pps + t / kPageTokens] = fresh;
     rt.row_stream[i] = s;
     rt.row_pos[i] = t;
     rt.row_token[i] = p.io.in_tokens ? max(p.io.in_tokens[i], 0) : ps.last_token[s];
@@ -75,17 +88,20 @@ __global__ void __launch_bounds__(kMaxRows) step_setup_kernel(const StepParams p
     rt.out_slot[i] = i;
     ps.ctx_len[s] = t + 1;
     ps.pos_next[s] += 1;
-  }
-  // attention works through the rows longest first, so that the short ones fill the tail of its grid
-  __shared__ int len_s[kMaxRows];
-  len_s[i] = i < p.n ? t : -1;
-  __syncthreads();
-  if (i < p.n) {
+    // attention works through the rows longest first, so that the short ones fill the tail of its grid
     int before = 0;
     for (int j = 0; j < p.n; ++j) before += (len_s[j] > t || (len_s[j] == t && j < i)) ? 1 : 0;
-    rt.row_order[before] = i;
+    rt.slots[before] = make_int4(i, t + 1, s, 0);
+    rank_s[i] = before;
+    new_s[i] = fresh;
   }
   if (i == 0) { *ps.free_top = top - total; *io = p.io; }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < kSetupPages; ++q) {
+    const int j = i + q * kSetupThreads, r = j / ps.pps, at = j - r * ps.pps;
+    if (r < p.n) rt.slot_pages[rank_s[r] * ps.pps + at] = new_s[r] >= 0 && at == len_s[r] / kPageTokens ? new_s[r] : page[q];
+  }
 }
 
 struct PrefillParams {

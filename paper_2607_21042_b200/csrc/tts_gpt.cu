@@ -124,6 +124,7 @@ struct tts_gpt {
   bool use_attn_half = true;     // half-page attention of decode steps (option "attn_half")
   bool use_attn_decode = true;   // unit-split tensor-pipe attention of decode steps (option "attn_decode")
   bool use_attn_stream = true;   // streaming attention for large batches (option "attn_stream")
+  int attn_queue = 1;            // 0: a CTA per pair, 1: as attention_use_queue says, 2: a queue of pairs (option "attn_queue")
   int attn_cluster_fill = 1;     // clusters grow until the grid covers the GPU this many times
   int attn_stream_min_pairs = 0; // (row, head) pairs from which it is used; 0: attention_use_stream decides
   int tc_min_rows = 17; // rows from which the tensor-core path is taken (option "tc_min_rows")
@@ -267,7 +268,8 @@ size_t carve(tts_gpt *h, void *base) {
   rt.row_emb = cv.take<const uint16_t *>(kMaxPassRows);
   rt.out_rows = cv.take<int>(kMaxRows);
   rt.out_slot = cv.take<int>(kMaxRows);
-  rt.row_order = cv.take<int>(kMaxRows);
+  rt.slots = cv.take<int4>(kMaxRows);
+  rt.slot_pages = cv.take<int>((size_t)kMaxRows * h->pps);
   h->io = cv.take<StepIO>(1);
   h->x = cv.take<float>(pass_rows * d);
   h->logits = cv.take<float>((size_t)kMaxRows * V);
@@ -373,6 +375,7 @@ void trace_attach(tts_gpt *h, Args &a) {
 // Attention for R rows: clusters while (row, head) pairs are scarce, one streaming CTA per pair
 // once they cover the GPU several times.
 cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool pdl) {
+  if (aa.old_pages_final) { aa.slots = h->rt.slots; aa.slot_pages = h->rt.slot_pages; }   // written by the decode step's set-up kernel
   if (h->kv_fp8) {
     // 8-bit cache: the QKV linear left the new K/V rows in the staging area; encode them into their page
     // slots, then attend over e4m3 pages (the same kernel for prefill passes and decode steps)
@@ -401,7 +404,7 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
       e = launch_kv_dequant_pages(kvl, h->kv_scratch, h->scratch_src, h->scratch_ntok, h->pass_scratch, aa.H, st, pdl);
       if (e != cudaSuccess) return e;
       h->launches += 1;
-      aa.kv_layer = h->kv_scratch; aa.page_table = h->scratch_table; aa.err = h->dev_err; aa.row_order = nullptr;
+      aa.kv_layer = h->kv_scratch; aa.page_table = h->scratch_table; aa.err = h->dev_err;
       if (h->use_attn_tc && R > kMaxRows) return launch_attention_prefill_tc(aa, R, h->n_sm, st, pdl);
       return launch_attention_prefill_mma(aa, R, st, pdl);
     }
@@ -410,9 +413,8 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
     fa.q = aa.q; fa.kv_layer = kvl; fa.page_table = aa.page_table; fa.row_stream = aa.row_stream; fa.row_pos = aa.row_pos;
     fa.out = aa.out; fa.partials = h->attn_partials; fa.tickets = h->attn_tickets; fa.H = aa.H; fa.pps = aa.pps;
     fa.out_image = aa.out_image; fa.trace = aa.trace; fa.trace_slot = aa.trace_slot;
-    fa.err = h->dev_err;
+    fa.err = h->dev_err; fa.slots = aa.slots; fa.slot_pages = aa.slot_pages;
     if (stream) {
-      fa.row_order = h->rt.row_order;
       return launch_attention_fp8_stream(fa, R, st, pdl);
     }
     fa.stage = h->kv_stage; fa.whole_pages = h->ordered ? 1 : 0;
@@ -420,7 +422,6 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
     return launch_attention_fp8(fa, R, attention_fp8_splits(R, aa.H, h->n_sm), st, pdl);
   }
   aa.err = h->dev_err;
-  aa.row_order = aa.old_pages_final ? h->rt.row_order : nullptr;   // written by the decode step's set-up kernel
   // prefill passes: rows of one stream share their pages (one CTA per 16 rows and head on the tensor cores;
   // the CUDA-core variant with 8 rows per CTA stays selectable)
   // (passes of several row tiles: 128 rows per CTA on tcgen05)
@@ -432,7 +433,11 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
   if (aa.old_pages_final && h->use_attn_half && !h->ordered && h->attn_stream_min_pairs == 0 && attention_use_half(R, aa.H, h->n_sm))
     return launch_attention_half(aa, R, attention_half_splits(R, aa.H, h->n_sm), st, pdl);
   const bool stream = h->attn_stream_min_pairs > 0 ? R * aa.H >= h->attn_stream_min_pairs : attention_use_stream(R, aa.H, h->n_sm);
-  if (h->use_attn_stream && stream) return launch_attention_stream(aa, R, st, pdl);
+  if (h->use_attn_stream && stream) {
+    const int n_pair = R * aa.H;
+    const bool queue = aa.slots && n_pair >= 2 && (h->attn_queue == 2 || (h->attn_queue == 1 && attention_use_queue(n_pair, h->n_sm)));
+    return queue ? launch_attention_queue(aa, R, h->attn_tickets, h->n_sm, st, pdl) : launch_attention_stream(aa, R, st, pdl);
+  }
   return launch_attention(aa, R, attention_cluster_size(R, aa.H, h->n_sm, h->attn_cluster_fill), st, pdl);
 }
 
@@ -1048,7 +1053,7 @@ int32_t tts_gpt_decode_step(tts_gpt_t *h, int32_t n, const int32_t *stream_ids, 
   sp.io.out_hidden = (uint16_t *)out_hidden; sp.io.top_k = top_k; sp.io.temperature = temperature; sp.io.n_out = n;
   h->ordered = top_k > 1;
   auto enqueue = [&]() -> int {
-    step_setup_kernel<<<1, kMaxRows, 0, h->stream>>>(sp, h->ps, h->rt, h->io);
+    step_setup_kernel<<<1, kSetupThreads, 0, h->stream>>>(sp, h->ps, h->rt, h->io);
     CUDA_TRY(h, cudaGetLastError());
     h->launches += 1;
     int r = run_embed(h, n);
@@ -1084,7 +1089,7 @@ int32_t tts_gpt_decode_step(tts_gpt_t *h, int32_t n, const int32_t *stream_ids, 
     cudaKernelNodeParams kp;
     memset(&kp, 0, sizeof kp);
     kp.func = (void *)step_setup_kernel;
-    kp.gridDim = dim3(1); kp.blockDim = dim3(kMaxRows); kp.kernelParams = args;
+    kp.gridDim = dim3(1); kp.blockDim = dim3(kSetupThreads); kp.kernelParams = args;
     CUDA_TRY(h, cudaGraphExecKernelNodeSetParams(sg->exec, sg->setup, &kp));
   }
   for (int i = 0; i < n; ++i) { h->ctx[stream_ids[i]] += 1; h->pos_next[stream_ids[i]] += 1; }
@@ -1293,6 +1298,7 @@ int32_t tts_gpt_debug_set_option(tts_gpt_t *h, const char *name, int32_t value) 
   else if (k == "attn_stream") h->use_attn_stream = on;
   else if (k == "attn_stream_min_pairs") h->attn_stream_min_pairs = value > 0 ? value : 0;
   else if (k == "attn_cluster_fill") h->attn_cluster_fill = value > 0 ? value : 1;
+  else if (k == "attn_queue") { if (value < 0 || value > 2) return fail(h, TTS_GPT_E_ARG, "attn_queue must be 0 (off), 1 (by the number of pairs) or 2 (always)"); h->attn_queue = value; }
   else if (k == "fc2_ksplit") h->use_fc2_ksplit = on;
   else if (k == "poison_free_pages") {
     h->poison_free = on;

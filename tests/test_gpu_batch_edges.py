@@ -71,6 +71,34 @@ def test_unit_split_decode_attention(S):
     eng.destroy()
 
 
+@pytest.mark.parametrize("S", [1, 3, 40, 128])
+def test_queued_attention_has_the_bits_of_a_cta_per_pair(S):
+    """Pairs handed out by a queue (2 to 444 CTAs, one pair or many behind the first two): pages with one token and with 64, rows
+    whose warps have no page, a long context among short ones, several launches on one counter."""
+    edges = [700, 1, 63, 64, 65, 127, 128, 129, 255, 256, 257, 320]
+    lens = [edges[i] if i < 12 else 2 + (37 * i) % 300 for i in range(S)]
+    cfg = C.tiny_config(max_streams=S, n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=768)
+    w = C.make_weights(cfg, seed=51)
+    model = O.OracleModel(cfg, w)
+    eng = B.TtsGpt(cfg, w, DEV)
+    for name, value in (("poison_free_pages", 1), ("attn_decode", 0), ("attn_half", 0), ("attn_stream_min_pairs", 1)):
+        eng.set_option(name, value)
+    prefixes = C.make_prefixes(cfg, lens, seed=52)
+    eng.set_option("attn_queue", 2)
+    lg, tk = _run(eng, prefixes, 4)
+    _check(model, prefixes, lg, tk, list(range(min(S, 6))) + [S - 1], "queued attention")
+    eng.set_option("attn_queue", 0)
+    lg2, tk2 = _run(eng, prefixes, 4)
+    assert np.array_equal(lg, lg2) and np.array_equal(tk, tk2)
+    eng.set_option("attn_queue", 2)
+    u = torch.full((S,), 0.4, device=DEV)
+    lg3, _ = _run(eng, prefixes, 4, top_k=30, uniforms=u)
+    eng.set_option("attn_queue", 0)
+    assert np.array_equal(lg3, _run(eng, prefixes, 4, top_k=30, uniforms=u)[0])
+    assert eng.check_canaries() == 0
+    eng.destroy()
+
+
 @pytest.mark.parametrize("wfmt", [C.W_BF16, C.W_INT8_PC, C.W_INT4_G128])
 @pytest.mark.parametrize("lens", [[1025], [700, 3, 450, 128, 1], [1279, 1281, 5, 31]])
 def test_prefill_passes_of_the_pair_kernel(wfmt, lens):
