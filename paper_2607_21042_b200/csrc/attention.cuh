@@ -524,9 +524,12 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 4) attention_half_kernel(cons
 inline bool attention_half_fits(int R, int H, int splits, int n_sm) { return R * H * splits <= 4 * n_sm; }
 inline int attention_half_splits(int R, int H, int n_sm) {
   const int s = std::max(1, std::min(kAttnMaxCluster, 4 * n_sm / (R * H)));
-  // clusters of seven leave places free: 4 rows, on seven / on six, ms per step at 100, 530 and 1400 tokens: 0.642 / 0.586, 0.653 /
-  // 0.605, 0.733 / 0.678; 8-bit cache 0.671 / 0.587, 0.680 / 0.607, 0.747 / 0.663
-  return s == 7 ? 6 : s;
+  // Clusters of seven and eight leave places free and take longer to meet: ms per step at 500 and 1400 tokens, on eight / on
+  // six: 3 rows 0.551 / 0.540, 0.615 / 0.614, 8-bit cache 0.573 / 0.562; 4 rows on seven / on six 0.653 / 0.605, 0.733 / 0.678;
+  // two rows level.  And where CTAs of more than two would take over nine tenths of the places, some wait for a second
+  // wave: 7 rows on four (560 of 592) / on three 0.667 / 0.635, 0.780 / 0.743.
+  if (R > 2 && s >= 7) return 6;
+  return s >= 3 && 10 * R * H * s > 37 * n_sm ? s - 1 : s;
 }
 // Two rows and more whose pairs the kernel above spreads over every SM, up to the middle batches' kernel.  Here / clusters of
 // whole pages (attention_kernel), ms per step at contexts of 100, 530 and 1400 tokens: 1 row 0.467 / 0.470, 0.470 / 0.484,

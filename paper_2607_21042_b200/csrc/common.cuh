@@ -147,16 +147,22 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
-// The same with `cluster` neighbouring CTAs of grid.x as a thread-block cluster (1: none).
+__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+// writes the word at `p`'s place in the shared memory of a CTA of the cluster
+__device__ __forceinline__ void st_shared_of_rank(float *p, uint32_t rank, float v) {
+  asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, %1;\n\tst.shared::cluster.f32 [a], %2;\n\t}" ::"r"(smem_u32(p)), "r"(rank), "f"(v) : "memory");
+}
+
+// The same with `cluster` neighbouring CTAs as a thread-block cluster (one: none).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_kernel_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, cudaStream_t st, bool pdl, Args... args) {
+inline cudaError_t launch_kernel_cluster_dims(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, dim3 cluster, cudaStream_t st, bool pdl, Args... args) {
   cudaLaunchConfig_t cfg;
-  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = 0; cfg.stream = st;
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
   cudaLaunchAttribute at[2];
   int n = 0;
-  if (cluster > 1) {
+  if (cluster.x * cluster.y * cluster.z > 1) {
     at[n].id = cudaLaunchAttributeClusterDimension;
-    at[n].val.clusterDim.x = cluster; at[n].val.clusterDim.y = 1; at[n].val.clusterDim.z = 1;
+    at[n].val.clusterDim.x = cluster.x; at[n].val.clusterDim.y = cluster.y; at[n].val.clusterDim.z = cluster.z;
     ++n;
   }
   if (pdl) {
@@ -167,6 +173,11 @@ inline cudaError_t launch_kernel_cluster(void (*kernel)(KArgs...), dim3 grid, di
   cfg.attrs = at;
   cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_kernel_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, cudaStream_t st, bool pdl, Args... args) {
+  return launch_kernel_cluster_dims(kernel, grid, block, 0, dim3(cluster), st, pdl, args...);
 }
 
 // 128-bit load served by L2 (never by a possibly stale L1 line).

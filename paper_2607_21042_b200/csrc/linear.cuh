@@ -32,9 +32,9 @@ enum { EPI_F32 = 0, EPI_QKV = 1, EPI_RESID = 2, EPI_GELU = 3 };
 constexpr int kLinearWarps = 10;  // divides the k-tile counts of K=1280 and K=5120 in every format
 constexpr int kLinearThreads = kLinearWarps * 32;
 constexpr int kSmallKSplit = 4;     // k-ranges of FC2 from 2 to 16 rows (partial sums folded by the next LayerNorm)
-constexpr int kLnFuseMaxRows = 1;   // LayerNorm is fused into the linear up to this batch: every CTA repeats it, which
-                                    // beats a separate launch for a single row only
+constexpr int kLnFuseMaxRows = 10;  // LayerNorm is fused into the linear up to this batch, every CTA repeating it: a warp per row
 constexpr int kLnFuseMaxRowsOrdered = 4;   // the same for launches that keep the order of sums of the FMA path
+constexpr int kLnFuseMaxK = 4 * kLinearThreads;   // one row: a float4 per thread; more: ten float4 per lane of the row's warp
 
 __host__ __device__ inline int k_per_tile(int wf) { return wf == WF_BF16 ? 32 : (wf == WF_INT8 ? 64 : 128); }
 __host__ __device__ inline int row_tiles(int N) { return (N + 7) / 8; }
@@ -150,6 +150,7 @@ struct LinearArgs {
   int *err;                   // optional device error word: set to 1 if the weight copy never arrives
   int ksplit;                 // 0 or 1: whole K per CTA; n > 1 (EPI_RESID only, no fused LN): gridDim.y = n k-ranges,
                               // out_f32 = partial sums [n][kMaxRows][N] without bias, folded by the next LayerNorm
+  int cluster;                // with ksplit (up to 16 rows, tensor-pipe path): the k-ranges of a tile are a cluster and add into out_f32 themselves
 };
 
 // exact int8 (biased byte) -> float via the 2^23 magic number
@@ -181,10 +182,13 @@ constexpr int kLinearSmemBudget = 108 * 1024;  // per CTA, so that two CTAs shar
 // NB: 0 = tensor-pipe path (any batch, 16 rows per m-tile); 1 or 4 = CUDA-core path for at most NB rows.  The fp32 FMAs
 // on the widened weights are cheaper for a single row, where MMAs are fifteen sixteenths padding.  From two rows on the
 // MMAs win: FMAs with LayerNorm fused in took 0.77 / 0.90 / 1.04 ms per step at 2 / 3 / 4 rows (bf16, context 530),
-// MMAs behind LayerNorm kernels of their own 0.59 / 0.63 / 0.71.  FMAs remain up to 4 rows where LinearArgs::ordered asks
+// MMAs behind LayerNorm kernels of their own 0.59 / 0.63 / 0.71 (with LayerNorm fused in 0.52 / 0.55 / 0.55).  FMAs remain up to 4 rows where LinearArgs::ordered asks
 // for their order of sums.
-template <int WF, int RT, int MODE, int NB>
+// CL: the k-ranges of a tile (gridDim.y of them) are the CTAs of a cluster and meet in its shared memory, so that the rows they
+// add into are complete when the kernel ends and the LayerNorm behind it can be fused into its consumer.
+template <int WF, int RT, int MODE, int NB, bool CL = false>
 __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearArgs a) {
+  static_assert(!CL || (NB == 0 && MODE == ACT_STAGED), "clusters: up to 16 staged rows on the tensor pipe");
   constexpr bool LN = MODE == ACT_LN;
   constexpr bool STAGED = MODE != ACT_DIRECT;
   constexpr int KT = WF == WF_BF16 ? 32 : (WF == WF_INT8 ? 64 : 128);
@@ -262,13 +266,34 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
   }
   uint2 ln_gg = make_uint2(0, 0), ln_bb = make_uint2(0, 0);
   const int lc = threadIdx.x * 4;               // fused LN: this thread's 4 columns (K <= 1280)
-  if (LN && lc < a.K) {
+  if (LN && NB > 0 && lc < a.K) {
     ln_gg = *reinterpret_cast<const uint2 *>(a.ln_g + lc);
     ln_bb = *reinterpret_cast<const uint2 *>(a.ln_b + lc);
+  }
+  // several rows: gamma | beta wait in the partial sums' memory, which is idle until the products are done
+  constexpr bool LN_ROWS = LN && NB == 0;
+  uint16_t *gb = reinterpret_cast<uint16_t *>(red);   // K <= 1280: 5120 bytes, the smallest `red`
+  if (LN_ROWS && threadIdx.x < a.K / 8) {
+    reinterpret_cast<uint4 *>(gb)[threadIdx.x] = *reinterpret_cast<const uint4 *>(a.ln_g + 8 * threadIdx.x);
+    reinterpret_cast<uint4 *>(gb + a.K)[threadIdx.x] = *reinterpret_cast<const uint4 *>(a.ln_b + 8 * threadIdx.x);
+  }
+  if (LN_ROWS) __syncthreads();
+  // cluster of k-ranges: the outputs this CTA finishes, one per thread (a quarter of the tile's), and their bias
+  __shared__ float cl_part[CL ? kSmallKSplit : 1][CL ? 4 * C : 1];   // every range's sums of this CTA's share
+  __shared__ int cl_here[kSmallKSplit];                                  // ... have been written
+  const int cl_share = CL ? (a.B * C + (int)gridDim.y - 1) / (int)gridDim.y : 1, cl_o = (int)blockIdx.y * cl_share + (int)threadIdx.x;
+  const bool cl_mine = CL && threadIdx.x < cl_share && cl_o < a.B * C && tile0 * 8 + cl_o % C < a.N;
+  float cl_bias = 0.f;
+  if (CL) {
+    if (cl_mine && a.bias) cl_bias = bf16_bits_to_float(a.bias[tile0 * 8 + cl_o % C]);
+    if (threadIdx.x < kSmallKSplit) cl_here[threadIdx.x] = 0;
+    cluster_arrive_release();
   }
   pdl_launch_dependents();
   pdl_wait();
   trace_mark(a.trace, a.trace_slot, 1);
+  float cl_old = 0.f;
+  if (cl_mine) cl_old = a.out_f32[(size_t)(cl_o / C) * a.out_stride + tile0 * 8 + cl_o % C];
 
   // ---- optional fused LayerNorm: the CTA splits each row over all threads (4 columns each) and
   //      handles up to RPR rows per round.  Each thread forms the mean and the centered sum of
@@ -276,8 +301,43 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
   //      (mean = (ma+mb)/2, M2 = M2a + M2b + (mb-ma)^2 * n/2), first by shuffles, then across the
   //      warps through shared memory: one block barrier, no cancellation.
   const int stride = ln_stage_stride(WF, KB * KT);   // staged columns: this CTA's k-range
-  constexpr int RPR = NB == 1 ? 1 : kLnFuseMaxRowsOrdered;   // rows per LayerNorm round (a one-row launch carries the code of one row only)
-  if (LN) {
+  constexpr int RPR = NB <= 1 ? 1 : kLnFuseMaxRowsOrdered;   // rows per LayerNorm round (a one-row launch carries the code of one row only)
+  if (LN_ROWS) {
+    // a warp per row: lane l owns columns 4 l + 128 j .. + 3; two passes over registers, no block barrier in between
+    for (int b = warp; b < a.B; b += kLinearWarps) {
+      const float *src = a.ln_x + (size_t)(a.ln_gather ? a.ln_gather[b] : b) * a.K + 4 * lane;
+      float4 xv[kLnFuseMaxK / 128];
+      float sum = 0.f, m2 = 0.f;
+#pragma unroll
+      for (int j = 0; j < kLnFuseMaxK / 128; ++j) {
+        xv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (128 * j < a.K) xv[j] = *reinterpret_cast<const float4 *>(src + 128 * j);
+      }
+#pragma unroll
+      for (int j = 0; j < kLnFuseMaxK / 128; ++j) sum += (xv[j].x + xv[j].y) + (xv[j].z + xv[j].w);
+      const float mu = warp_sum(sum) / a.K;
+#pragma unroll
+      for (int j = 0; j < kLnFuseMaxK / 128; ++j)
+        if (128 * j < a.K) {
+          const float d0 = xv[j].x - mu, d1 = xv[j].y - mu, d2 = xv[j].z - mu, d3 = xv[j].w - mu;
+          m2 += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
+        }
+      const float rstd = rsqrtf(warp_sum(m2) / a.K + a.ln_eps);
+      uint16_t *hid = blockIdx.x == 0 && a.ln_io && a.ln_io->out_hidden ? a.ln_io->out_hidden + (size_t)(a.ln_out_slot ? a.ln_out_slot[b] : b) * a.K : nullptr;
+#pragma unroll
+      for (int j = 0; j < kLnFuseMaxK / 128; ++j)
+        if (128 * j < a.K) {
+          const int col = 128 * j + 4 * lane;
+          const uint2 g2 = *reinterpret_cast<const uint2 *>(gb + col), b2 = *reinterpret_cast<const uint2 *>(gb + a.K + col);
+          uint2 y;
+          y.x = pack_bf16x2((xv[j].x - mu) * rstd * bf16_lo(g2.x) + bf16_lo(b2.x), (xv[j].y - mu) * rstd * bf16_hi(g2.x) + bf16_hi(b2.x));
+          y.y = pack_bf16x2((xv[j].z - mu) * rstd * bf16_lo(g2.y) + bf16_lo(b2.y), (xv[j].w - mu) * rstd * bf16_hi(g2.y) + bf16_hi(b2.y));
+          *reinterpret_cast<uint2 *>(stage + (size_t)b * stride + col) = y;
+          if (hid) *reinterpret_cast<uint2 *>(hid + col) = y;
+        }
+    }
+    __syncthreads();
+  } else if (LN) {
     float2 *lnred = reinterpret_cast<float2 *>(red);  // [warps][RPR] (mean, M2), reused later for the partial sums
     const int nw_used = (a.K / 4 + 31) / 32;           // warps that hold columns (K is a multiple of 128)
     const float inv_nw = 1.0f / nw_used, inv_k = 1.0f / a.K;
@@ -362,10 +422,13 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
   trace_mark(a.trace, a.trace_slot, 3);
 
   // ---- the weights must have landed by now (they were requested before the dependency wait) ----
-  if (!mbar_wait_bounded(wbar, 0, 2000000000ull)) {
+  bool arrived = mbar_wait_bounded(wbar, 0, 2000000000ull);
+  if (CL) arrived = __syncthreads_and(arrived);   // the CTA goes one way, and stays for the others' sums if its weights did not come
+  if (!arrived) {
     if (a.err) atomicExch(a.err, 1);
     // give the copies still in flight towards this CTA's shared memory a last chance to finish
     mbar_wait_bounded(wbar, 0, 2000000000ull);
+    if (CL) { cluster_wait(); cluster_arrive_release(); cluster_wait(); }
     return;
   }
   const uint4 *wtile = reinterpret_cast<const uint4 *>(wsm);   // tile (j, kb) at ((j*KB + kb)*32 + lane)
@@ -546,6 +609,7 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
     }
     __syncthreads();
     trace_mark(a.trace, a.trace_slot, 5);
+    if (CL) cluster_wait();   // the others run and have cleared their marks
 #pragma unroll
     for (int e = 0; e < ER; ++e) {
       const int o = threadIdx.x < EPT ? threadIdx.x + e * EPT : 16 * C;
@@ -556,6 +620,11 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
 #pragma unroll
         for (int w = 0; w < kLinearWarps; ++w) v += red[((size_t)w * 16 + bl) * C + ecol];
         if (WF == WF_INT8) v *= e_scale;
+        if (CL) {              // partial sum of this k-range, to the CTA that finishes the output
+          const int rank = o / cl_share;
+          st_shared_of_rank(&cl_part[CL ? (int)blockIdx.y : 0][CL ? o - rank * cl_share : 0], rank, v);
+          continue;
+        }
         if (gridDim.y > 1) {   // partial sum of this k-range; bias and residual are added by the folding LayerNorm
           a.out_f32[((size_t)blockIdx.y * kMaxRows + b) * a.N + n] = v;
           continue;
@@ -590,6 +659,18 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
       }
     }
     __syncthreads();
+  }
+  if (CL) {   // the k-ranges' sums in order, each CTA for its share of the tile's outputs
+    if (threadIdx.x < kSmallKSplit) st_shared_of_rank(reinterpret_cast<float *>(&cl_here[blockIdx.y]), threadIdx.x, __int_as_float(1));
+    cluster_arrive_release();
+    cluster_wait();
+    if (cl_mine) {
+      float v = cl_part[0][threadIdx.x];
+      int here = cl_here[0];
+#pragma unroll
+      for (int k = 1; k < (CL ? kSmallKSplit : 1); ++k) { v += cl_part[k][threadIdx.x]; here &= cl_here[k]; }
+      if (here) a.out_f32[(size_t)(cl_o / C) * a.out_stride + tile0 * 8 + cl_o % C] = cl_old + (v + cl_bias);
+    }
   }
   trace_mark(a.trace, a.trace_slot, 2);
 }
@@ -628,6 +709,13 @@ inline cudaError_t launch_linear_nb(const LinearArgs &a, int grid, cudaStream_t 
   const size_t smem = linear_smem_bytes(WF, RT, MODE, a.B, a.K / ks);
   static SmemOptIn opt_in;
   if (const cudaError_t e = opt_in(linear_kernel<WF, RT, MODE, NB>, 200 * 1024)) return e;
+  if constexpr (NB == 0 && MODE == ACT_STAGED) {
+    if (a.cluster) {
+      static SmemOptIn opt_in_cl;
+      if (const cudaError_t e = opt_in_cl(linear_kernel<WF, RT, MODE, NB, true>, 200 * 1024)) return e;
+      return launch_kernel_cluster_dims(linear_kernel<WF, RT, MODE, NB, true>, dim3(grid, ks), dim3(kLinearThreads), smem, dim3(1, ks), st, pdl, a);
+    }
+  }
   return launch_kernel(linear_kernel<WF, RT, MODE, NB>, dim3(grid, ks), dim3(kLinearThreads), smem, st, pdl, a);
 }
 
@@ -652,9 +740,9 @@ inline cudaError_t launch_linear_wf(const LinearArgs &a, int max_ctas, cudaStrea
   return launch_linear_inst<WF, 4, MODE>(a, p.grid, st, pdl);
 }
 
-// Whether LayerNorm can be fused in front of a linear with this shape (one float4 of the row per thread).
-inline bool can_fuse_ln(int B, int K, bool ordered) {
-  return B <= (ordered ? kLnFuseMaxRowsOrdered : kLnFuseMaxRows) && K <= 4 * kLinearThreads;
+// Whether LayerNorm can be fused in front of a linear with this shape.
+inline bool can_fuse_ln(int B, int K, bool ordered, int max_rows = kLnFuseMaxRows) {
+  return B <= (ordered ? kLnFuseMaxRowsOrdered : max_rows) && K <= kLnFuseMaxK;
 }
 
 template <int WF>
@@ -667,7 +755,8 @@ inline cudaError_t launch_linear_mode(const LinearArgs &a, int max_ctas, cudaStr
 
 // K must be a multiple of 128.
 inline cudaError_t launch_linear(int wf, const LinearArgs &a, cudaStream_t st, bool pdl, int max_ctas) {
-  if (a.ln_x && !can_fuse_ln(a.B, a.K, a.ordered)) return cudaErrorInvalidValue;
+  if (a.ln_x && !can_fuse_ln(a.B, a.K, a.ordered, 16)) return cudaErrorInvalidValue;
+  if (a.cluster && (a.ksplit != kSmallKSplit || a.B < 2 || a.B > 16 || a.ordered || (size_t)a.B * ln_stage_stride(wf, a.K / a.ksplit) * sizeof(uint16_t) > (size_t)kStageMaxBytes)) return cudaErrorInvalidValue;
   if (a.ksplit > 1 && (a.ln_x || a.mode != EPI_RESID || (a.K / k_per_tile(wf)) % a.ksplit != 0)) return cudaErrorInvalidValue;
   if (wf == WF_BF16) return launch_linear_mode<WF_BF16>(a, max_ctas, st, pdl);
   if (wf == WF_INT8) return launch_linear_mode<WF_INT8>(a, max_ctas, st, pdl);

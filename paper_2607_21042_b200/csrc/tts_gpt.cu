@@ -100,6 +100,7 @@ struct tts_gpt {
   std::map<int, StepGraph> graphs;
   bool use_graph;
   bool use_pdl;
+  int ln_fuse_rows = kLnFuseMaxRows;   // rows up to which LayerNorm is fused into its consumer (option "ln_fuse_rows")
   bool use_fc2_ksplit = true;   // 2-16 rows: FC2 splits K (option "fc2_ksplit")
   int pending_parts = 0;        // k-range partial sums of the last FC2 still to be folded into x
   size_t partials_floats = 0;
@@ -562,6 +563,18 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
   return TTS_GPT_OK;
 }
 
+// Whether LayerNorm is fused into the linears of up to 16 rows; FC2's k-ranges then meet in clusters, so that x is complete.
+// Five kernels per layer instead of seven; the price is x read by every CTA (5 KB a row) and a cluster barrier.  ms per
+// step, kernels of their own / fused, contexts of 500 tokens (bf16, int4, bf16 weights over the 8-bit cache) and 1400 (bf16):
+// 2 rows 0.552 / 0.520, 0.542 / 0.522, 0.574 / 0.547, 0.598 / 0.571; 4 rows 0.596 / 0.552, 0.591 / 0.552, 0.633 / 0.585, 0.671 /
+// 0.638; 6 rows 0.666 / 0.601, 0.648 / 0.596, 0.688 / 0.642, 0.758 / 0.703; 7 rows 0.659 / 0.633, 0.654 / 0.624, 0.698 / 0.679,
+// 0.784 / 0.741; 8 rows 0.638 / 0.647, 0.639 / 0.620, 0.673 / 0.677, 0.754 / 0.792 (kernels of their own but for int4); 9 rows
+// 0.705 / 0.699, 0.692 / 0.664, 0.746 / 0.730, 0.875 / 0.845; 10 rows 0.756 / 0.717, 0.695 / 0.674, 0.825 / 0.799, 0.947 / 0.924;
+// 11 rows 0.777 / 0.799, 0.728 / 0.748, 0.852 / 0.868, 0.993 / 1.010; 14 rows 0.891 / 1.001, 0.798 / 0.804, 0.997 / 1.098.
+bool fuse_layernorm(const tts_gpt *h, int R) {
+  return can_fuse_ln(R, h->cfg.d_model, h->ordered, h->ln_fuse_rows) && (h->ordered || R != 8 || h->cfg.wfmt == WF_INT4);
+}
+
 // Final LayerNorm (folding the last FC2's partial sums), LM head, sampling after run_layers_tc.
 int run_head_tc(tts_gpt *h, int n_out) {
   const tts_gpt_config_t &c = h->cfg;
@@ -601,10 +614,12 @@ int run_layers(tts_gpt *h, int R, bool decode) {
   const int d = c.d_model;
   cudaStream_t st = h->stream;
   const bool pdl = h->use_pdl;
-  const bool fuse_ln = can_fuse_ln(R, d, h->ordered);
+  const bool fuse_ln = fuse_layernorm(h, R);
   // 2 to 16 rows: FC2 (K = d_ff) splits K over kSmallKSplit CTAs per row tile, so that a CTA stages a
   // quarter of the wide activation rows; its partial sums are folded into x by the next LayerNorm
-  const int fc2_ks = (!fuse_ln && h->use_fc2_ksplit && (c.d_ff / k_per_tile(c.wfmt)) % kSmallKSplit == 0 &&
+  // (with LayerNorm fused into its consumer the k-ranges are a cluster, which adds into x itself)
+  const bool cluster = fuse_ln && R > 1 && !h->ordered;
+  const int fc2_ks = ((!fuse_ln || cluster) && h->use_fc2_ksplit && (c.d_ff / k_per_tile(c.wfmt)) % kSmallKSplit == 0 &&
                       (size_t)kSmallKSplit * kMaxRows * d <= h->partials_floats) ? kSmallKSplit : 1;
   h->pending_parts = 0;
   for (int l = 0; l < c.n_layer; ++l) {
@@ -655,12 +670,12 @@ int run_layers(tts_gpt *h, int R, bool decode) {
     CUDA_TRY(h, launch_linear(c.wfmt, f1, st, pdl, 2 * h->n_sm));
     LinearArgs f2 = linear_args(h, L.fc2, h->hbuf, R, EPI_RESID);
     f2.out_f32 = h->x; f2.out_stride = d;
-    if (fc2_ks > 1) { f2.ksplit = fc2_ks; f2.out_f32 = h->partials; }
+    if (fc2_ks > 1) { f2.ksplit = fc2_ks; f2.cluster = cluster ? 1 : 0; if (!cluster) f2.out_f32 = h->partials; }
     trace_attach(h, f2);
     CUDA_TRY(h, launch_linear(c.wfmt, f2, st, pdl, 2 * h->n_sm));
     h->launches += 5;
   }
-  h->pending_parts = fc2_ks > 1 ? fc2_ks : 0;   // the last FC2's partial sums: folded by the head's LayerNorm
+  h->pending_parts = fc2_ks > 1 && !cluster ? fc2_ks : 0;   // the last FC2's partial sums: folded by the head's LayerNorm
   return TTS_GPT_OK;
 }
 
@@ -679,7 +694,7 @@ int run_head(tts_gpt *h, int n_out, int R) {
                           h->rt.out_slot, h->io, 0);
     if (rc) return rc;
     h->pending_parts = 0;
-  } else if (can_fuse_ln(n_out, c.d_model, h->ordered)) {
+  } else if (fuse_layernorm(h, n_out)) {
     ha.ln_x = h->x; ha.ln_g = h->lnf_g; ha.ln_b = h->lnf_b; ha.ln_eps = c.ln_eps;
     ha.ln_gather = h->rt.out_rows; ha.ln_out_slot = h->rt.out_slot; ha.ln_io = h->io;
   } else {
@@ -1299,6 +1314,7 @@ int32_t tts_gpt_debug_set_option(tts_gpt_t *h, const char *name, int32_t value) 
   else if (k == "attn_stream_min_pairs") h->attn_stream_min_pairs = value > 0 ? value : 0;
   else if (k == "attn_cluster_fill") h->attn_cluster_fill = value > 0 ? value : 1;
   else if (k == "attn_queue") { if (value < 0 || value > 2) return fail(h, TTS_GPT_E_ARG, "attn_queue must be 0 (off), 1 (by the number of pairs) or 2 (always)"); h->attn_queue = value; }
+  else if (k == "ln_fuse_rows") { if (value < 1 || value > 16) return fail(h, TTS_GPT_E_ARG, "ln_fuse_rows must be in 1..16"); h->ln_fuse_rows = value; }
   else if (k == "fc2_ksplit") h->use_fc2_ksplit = on;
   else if (k == "poison_free_pages") {
     h->poison_free = on;

@@ -71,6 +71,31 @@ def test_unit_split_decode_attention(S):
     eng.destroy()
 
 
+@pytest.mark.parametrize("wfmt", [C.W_BF16, C.W_INT8_PC, C.W_INT4_G128])
+@pytest.mark.parametrize("S,d", [(2, 1280), (5, 384), (7, 256), (10, 1280)])
+def test_layernorm_fused_into_linears_of_several_rows(S, d, wfmt):
+    """A warp per row in every CTA (2, 3 and 10 float4 per lane), FC2's k-ranges added up by a cluster (shares that do and do not
+    divide evenly), hidden rows from the fused head; against the oracle, and against LayerNorm kernels of their own."""
+    cfg = C.tiny_config(d_model=d, n_head=d // 64, d_ff=4 * d if d < 1280 else 1536, wfmt=wfmt, max_streams=S, n_pages=3 * S)
+    w = C.make_weights(cfg, seed=53)
+    model = O.OracleModel(cfg, w)
+    eng = B.TtsGpt(cfg, w, DEV)
+    prefixes = C.make_prefixes(cfg, [20 + 9 * i for i in range(S)], seed=54)
+    hid = torch.zeros((2, S, d), dtype=torch.bfloat16, device=DEV)
+    lg, tk = _run(eng, prefixes, 3, out_hidden=hid[0])
+    _check(model, prefixes, lg, tk, range(S), "fused LayerNorm")
+    assert np.array_equal(lg, _run(eng, prefixes, 3)[0])
+    eng.set_option("ln_fuse_rows", 1)
+    lg2, tk2 = _run(eng, prefixes, 3, out_hidden=hid[1])
+    _check(model, prefixes, lg2, tk2, range(S), "LayerNorm kernels")
+    # rows of unit variance whose bf16 operands round along two orders of sums: a few bf16 steps (2^-8 of a value), one in the mean
+    same = np.array([np.array_equal(a, b) for a, b in zip(tk, tk2)])
+    a, b = hid[0].float().cpu().numpy()[same], hid[1].float().cpu().numpy()[same]
+    assert same.any() and np.linalg.norm(a - b) <= 2.0 ** -7 * np.linalg.norm(a)
+    assert eng.check_canaries() == 0
+    eng.destroy()
+
+
 @pytest.mark.parametrize("S", [1, 3, 40, 128])
 def test_queued_attention_has_the_bits_of_a_cta_per_pair(S):
     """Pairs handed out by a queue (2 to 444 CTAs, one pair or many behind the first two): pages with one token and with 64, rows
