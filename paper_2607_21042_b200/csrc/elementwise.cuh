@@ -27,6 +27,7 @@ struct RowTable {
   int *out_rows;              // rows whose logits are wanted, compacted
   int *out_slot;              // position of that row's results in the caller's output arrays
   // decode steps, by rank of context length (longest first):
+  int *row_order;
   int4 *slots;                // {row, tokens with the step's own, stream, 0}
   int *slot_pages;            // [rank][pps] the row's pages
 };

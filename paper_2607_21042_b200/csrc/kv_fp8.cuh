@@ -109,6 +109,7 @@ struct Fp8AttnArgs {
   float *partials;                // [R][H][kAttnMaxChunks][66]
   unsigned int *tickets;          // [R][H], zero between launches
   int H, pps, out_image;
+  const int *row_order;
   const int4 *slots;              // see AttnArgs
   const int *slot_pages;
   int *err;                       // streaming variant: set when a bounded wait ran out
@@ -502,7 +503,8 @@ inline cudaError_t launch_kv_dequant_pages(const unsigned char *kv_layer, uint16
 constexpr uint32_t kFp8StageBytes = 2 * kFp8BlockBytes;   // K block | V block
 constexpr int kFp8Stages = 2;
 
-__device__ __forceinline__ void fp8_stream_issue(const Fp8AttnArgs &a, int phys, int h, unsigned char *stage, uint64_t *bar) {
+__device__ __forceinline__ void fp8_stream_issue(const Fp8AttnArgs &a, const int *pt, int h, int page, unsigned char *stage, uint64_t *bar) {
+  const int phys = pt[page];
   const unsigned char *K = a.kv_layer + (((size_t)phys * 2 + 0) * a.H + h) * kFp8BlockBytes;
   mbar_expect_tx(bar, kFp8StageBytes);
   bulk_copy_g2s(stage, K, kFp8BlockBytes, bar);
@@ -513,34 +515,36 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 3) attention_fp8_stream_kerne
   extern __shared__ __align__(128) unsigned char fp8_stages[];   // [warp][stage][K block | V block]
   __shared__ __align__(8) uint64_t bars[kAttnWarps][kFp8Stages];
   __shared__ float sm_m[kAttnWarps], sm_l[kAttnWarps], sm_o[kAttnWarps][kHeadDim];
-  const int h = blockIdx.y;
+  const int h = blockIdx.y, r = a.row_order ? a.row_order[blockIdx.z] : blockIdx.z;
   trace_mark(a.trace, a.trace_slot, 0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tg = lane >> 2, sub = lane & 3;
-  const AttnRow ar(a, blockIdx.z);
-  const int r = ar.row, n_tok = min(ar.n_tok, a.pps * kPageTokens);   // row and page tables are final before the step's first kernel starts
+  const int n_tok = min(a.row_pos[r] + 1, a.pps * kPageTokens);   // row and page tables are final before the step's first kernel starts
   const int n_pages = (n_tok + kPageTokens - 1) / kPageTokens;
+  const int *pt = a.page_table + (size_t)a.row_stream[r] * a.pps;
   unsigned char *stages = fp8_stages + (size_t)warp * (kFp8Stages * kFp8StageBytes);
   // pages of this warp: warp, warp + 4, ...; iteration it uses stage it % 2
-  auto request = [&](int page, int s) {
-    const int phys = ar.phys(page);
-    if (lane == 0) fp8_stream_issue(a, phys, h, stages + s * kFp8StageBytes, &bars[warp][s]);
-  };
+  bool issued[kFp8Stages] = {false, false};
   if (lane == 0) {
 #pragma unroll
     for (int s = 0; s < kFp8Stages; ++s) mbar_init(&bars[warp][s], 1);
-  }
-  __syncwarp();
 #pragma unroll
-  for (int s = 0; s < kFp8Stages; ++s)
-    if (warp + kAttnWarps * s < n_pages - 1) request(warp + kAttnWarps * s, s);
+    for (int s = 0; s < kFp8Stages; ++s) {
+      const int page = warp + kAttnWarps * s;
+      if (page < n_pages - 1) { fp8_stream_issue(a, pt, h, page, stages + s * kFp8StageBytes, &bars[warp][s]); issued[s] = true; }
+    }
+  }
   __syncwarp();
   pdl_launch_dependents();
   pdl_wait();
   trace_mark(a.trace, a.trace_slot, 1);
+  if (lane == 0) {
 #pragma unroll
-  for (int s = 0; s < kFp8Stages; ++s)
-    if (warp + kAttnWarps * s == n_pages - 1) request(n_pages - 1, s);
+    for (int s = 0; s < kFp8Stages; ++s) {
+      const int page = warp + kAttnWarps * s;
+      if (!issued[s] && page < n_pages) fp8_stream_issue(a, pt, h, page, stages + s * kFp8StageBytes, &bars[warp][s]);
+    }
+  }
   float qv[16];
   {
     const float qs = 0.125f * 1.4426950408889634f;   // scores in log2 units
@@ -585,8 +589,10 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 3) attention_fp8_stream_kerne
     // The stage may be refilled only after every lane's reads of it have returned: the ballot needs a value
     // that every lane computed from what it read, and the fence takes the ballot as an operand.
     const unsigned int done = __ballot_sync(0xFFFFFFFFu, o[0] == o[0] || l >= 0.f);
-    if (lane == 0) asm volatile("fence.proxy.async.shared::cta; // after %0" ::"r"(done) : "memory");
-    if (page + kFp8Stages * kAttnWarps < n_pages) request(page + kFp8Stages * kAttnWarps, s);
+    if (page + kFp8Stages * kAttnWarps < n_pages && lane == 0) {
+      asm volatile("fence.proxy.async.shared::cta; // after %0" ::"r"(done) : "memory");
+      fp8_stream_issue(a, pt, h, page + kFp8Stages * kAttnWarps, stages + s * kFp8StageBytes, bar);
+    }
   }
   trace_mark(a.trace, a.trace_slot, 3);
   // warp result: sum over the 8 token groups

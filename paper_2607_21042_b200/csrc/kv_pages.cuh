@@ -91,6 +91,7 @@ __global__ void __launch_bounds__(kSetupThreads) step_setup_kernel(const StepPar
     // attention works through the rows longest first, so that the short ones fill the tail of its grid
     int before = 0;
     for (int j = 0; j < p.n; ++j) before += (len_s[j] > t || (len_s[j] == t && j < i)) ? 1 : 0;
+    rt.row_order[before] = i;
     rt.slots[before] = make_int4(i, t + 1, s, 0);
     rank_s[i] = before;
     new_s[i] = fresh;

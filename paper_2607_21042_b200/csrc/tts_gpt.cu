@@ -270,6 +270,7 @@ size_t carve(tts_gpt *h, void *base) {
   rt.out_rows = cv.take<int>(kMaxRows);
   rt.out_slot = cv.take<int>(kMaxRows);
   rt.slots = cv.take<int4>(kMaxRows);
+  rt.row_order = cv.take<int>(kMaxRows);
   rt.slot_pages = cv.take<int>((size_t)kMaxRows * h->pps);
   h->io = cv.take<StepIO>(1);
   h->x = cv.take<float>(pass_rows * d);
@@ -416,6 +417,7 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
     fa.out_image = aa.out_image; fa.trace = aa.trace; fa.trace_slot = aa.trace_slot;
     fa.err = h->dev_err; fa.slots = aa.slots; fa.slot_pages = aa.slot_pages;
     if (stream) {
+      fa.row_order = h->rt.row_order;
       return launch_attention_fp8_stream(fa, R, st, pdl);
     }
     fa.stage = h->kv_stage; fa.whole_pages = h->ordered ? 1 : 0;
