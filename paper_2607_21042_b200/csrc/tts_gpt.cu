@@ -464,10 +464,23 @@ GemmTcArgs gemm_args(tts_gpt *h, const PackedLinear &pl, const void *act_img, in
 // One prefill call of the 24-layer model, one-CTA kernel / pairs, ms: one stream of 300 rows 1.42 / 1.69, 640 1.71 / 1.95,
 // 777 1.80 / 2.24, 896 1.83 / 2.28, 1000 2.47 / 2.48, 1024 2.45 / 2.46, 1100 2.64 / 2.80, 1280 2.84 / 2.91, 1400 3.07 / 3.04,
 // 1536 3.15 / 3.09, 2000 4.22 / 4.09; eight streams of 640 rows together 1.67 / 1.91, 1024 2.18 / 2.14, 1152 2.28 / 2.49, 1536
-// 2.87 / 2.66, 1792 3.03 / 2.79 (int8 weights within 2 % of these).  The two cross between 1000 and 1400 rows, up and down
-// with how full the last wave of either is; a rule by the two kernels' waves could gain up to 9 % there.
-constexpr int kPairMinRows = 1024;
-bool use_pairs(const tts_gpt *h, int R) { return R > kPairMinRows && !(h->cfg.wfmt == WF_INT4 && h->w4_exact); }
+// 2.87 / 2.66, 1792 3.03 / 2.79 (int8 weights within 2 % of these).  Up to 1280 rows the pairs' 256-row tiles of QKV leave the
+// second wave nearly empty; from 1400 on they are the faster.
+constexpr int kPairMinRows = 1280;
+bool can_pair(const tts_gpt *h) { return !(h->cfg.wfmt == WF_INT4 && h->w4_exact); }
+bool use_pairs(const tts_gpt *h, int R) { return R > kPairMinRows && can_pair(h); }
+
+// FC2 alone goes to pairs where its one-CTA tiles begin a second wave and its pairs need one: 897 to 1024 rows, of which it
+// takes 17.2 us a layer on pairs and 23.0 on single CTAs (QKV 13.3 there against 15.5 on pairs, the O projection 9.3 against
+// 11.6, FC1 level).  Beyond, the two are level (1152 rows 22.9 / 22.2, 1280 rows 23.2 / 29.0).
+bool pair_fc2(const tts_gpt *h, int R) {
+  const tts_gpt_config_t &c = h->cfg;
+  if (use_pairs(h, R)) return true;
+  if (!can_pair(h) || h->ordered || R <= kMaxRows || R > kMaxSplitRows) return false;
+  const int tiles = (R + kMaxRows - 1) / kMaxRows, single = (c.d_model + 127) / 128 * tcw_ksplit_resid(c.d_ff) * tiles;
+  const PwPlan p = pw_plan(c.d_model, c.d_ff, R, true, h->n_sm);
+  return single > 2 * h->n_sm && (tiles + 1) / 2 * ((c.d_model + p.bn - 1) / p.bn) * p.ksplit <= h->n_sm / 2;
+}
 
 int launch_ln_tc(tts_gpt *h, int rows, const uint16_t *g, const uint16_t *b, int n_part, const uint16_t *add_bias,
                  void *out_img, uint16_t *out_plain, const int *gather, const int *out_slot, const StepIO *io,
@@ -498,9 +511,9 @@ int launch_ln_tc(tts_gpt *h, int rows, const uint16_t *g, const uint16_t *b, int
   return TTS_GPT_OK;
 }
 
-int launch_gemm(tts_gpt *h, const GemmTcArgs &a, const CUtensorMap &w_map, const CUtensorMap &x_map, bool wide, cudaStream_t st, bool pdl) {
+int launch_gemm(tts_gpt *h, const GemmTcArgs &a, const CUtensorMap &w_map, const CUtensorMap &x_map, bool wide, bool pairs, cudaStream_t st, bool pdl) {
   if (!wide) CUDA_TRY(h, launch_gemm_tc(a, h->n_sm, st, pdl));
-  else if (!use_pairs(h, a.B)) CUDA_TRY(h, launch_gemm_tcw(a, h->n_sm, st, pdl));
+  else if (!pairs) CUDA_TRY(h, launch_gemm_tcw(a, h->n_sm, st, pdl));
   else {
     const CUtensorMap *out = a.mode != EPI_RESID ? nullptr : a.ksplit > 1 ? &h->part_map : &h->xrow_map;
     CUDA_TRY(h, launch_gemm_pw(a, w_map, x_map, out, pw_plan(a.N, a.K, a.B, a.mode == EPI_RESID, h->n_sm, a.ksplit).bn, h->n_sm, st, pdl));
@@ -517,10 +530,10 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
   cudaStream_t st = h->stream;
   const bool pdl = h->use_pdl;
   const bool wide = R > kMaxRows;
-  const bool pairs = use_pairs(h, R);
-  const bool free_ks = pairs && !h->ordered;   // ordered passes keep the k-ranges of the one-CTA wide kernel
+  const bool pairs = use_pairs(h, R), pairs2 = wide && pair_fc2(h, R);
+  const bool free_ks = pairs && !h->ordered, free_ks2 = pairs2 && !h->ordered;   // ordered passes keep the k-ranges of the one-CTA wide kernel
   const int o_ks = !wide ? kTcKSplit : free_ks ? pw_plan(d, d, R, true, h->n_sm).ksplit : tcw_ksplit_resid(d);
-  const int f2_ks = !wide ? kTcKSplit : free_ks ? pw_plan(d, c.d_ff, R, true, h->n_sm).ksplit : tcw_ksplit_resid(c.d_ff);
+  const int f2_ks = !wide ? kTcKSplit : free_ks2 ? pw_plan(d, c.d_ff, R, true, h->n_sm).ksplit : tcw_ksplit_resid(c.d_ff);
   const int o_parts = o_ks > 1 ? o_ks : 0, f2_parts = f2_ks > 1 ? f2_ks : 0;   // 0: the linear added into x itself
   for (int l = 0; l < c.n_layer; ++l) {
     LayerW &L = h->layers[l];
@@ -537,7 +550,7 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
     const bool q_img = wide && h->use_attn_tc && h->use_attn_mma && (!h->kv_fp8 || h->pass_scratch > 0);   // the tcgen05 attention follows
     qa.q_img = q_img ? h->q_img : nullptr;
     trace_attach(h, qa);
-    if ((rc = launch_gemm(h, qa, L.qkv.w_map, h->a_map, wide, st, pdl))) return rc;
+    if ((rc = launch_gemm(h, qa, L.qkv.w_map, h->a_map, wide, pairs, st, pdl))) return rc;
     AttnArgs aa;
     memset(&aa, 0, sizeof aa);
     aa.q = h->q; aa.kv_layer = kvl; aa.page_table = h->ps.page_table; aa.row_stream = h->rt.row_stream;
@@ -548,17 +561,17 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
     GemmTcArgs oa = gemm_args(h, L.o, h->o_img, R, EPI_RESID, o_ks);
     oa.out_f32 = o_parts ? h->partials : h->x; oa.out_stride = d;
     trace_attach(h, oa);
-    if ((rc = launch_gemm(h, oa, L.o.w_map, h->o_map, wide, st, pdl))) return rc;
+    if ((rc = launch_gemm(h, oa, L.o.w_map, h->o_map, wide, pairs, st, pdl))) return rc;
     rc = launch_ln_tc(h, R, L.ln2_g, L.ln2_b, o_parts, o_parts ? L.o.bias : nullptr, h->a_img, nullptr, nullptr, nullptr, nullptr, 1);
     if (rc) return rc;
     GemmTcArgs f1 = gemm_args(h, L.fc1, h->a_img, R, EPI_GELU, 1);
     f1.out_img = h->h_img; f1.gelu_tanh = c.gelu_tanh;
     trace_attach(h, f1);
-    if ((rc = launch_gemm(h, f1, L.fc1.w_map, h->a_map, wide, st, pdl))) return rc;
+    if ((rc = launch_gemm(h, f1, L.fc1.w_map, h->a_map, wide, pairs, st, pdl))) return rc;
     GemmTcArgs f2 = gemm_args(h, L.fc2, h->h_img, R, EPI_RESID, f2_ks);
     f2.out_f32 = f2_parts ? h->partials : h->x; f2.out_stride = d;
     trace_attach(h, f2);
-    if ((rc = launch_gemm(h, f2, L.fc2.w_map, h->h_map, wide, st, pdl))) return rc;
+    if ((rc = launch_gemm(h, f2, L.fc2.w_map, h->h_map, wide, pairs2, st, pdl))) return rc;
     h->launches += 5;
   }
   h->tc_tail_parts = f2_parts;
@@ -953,10 +966,11 @@ static int prefill_impl(tts_gpt_t *h, int32_t n, const void *const *emb, const i
   h->ordered = top_k > 1;
   // Ordered passes: what a row's sums look like depends on the pass of `unit` rows it lies in by its last tile (a pass of up
   // to 128 rows has kernels of its own) and by the rows whose logits are wanted together.  Several units run as one pass,
-  // with a last unit of up to 128 rows apart and the head unit by unit.  (Over the 8-bit cache a pass is one unit: how many
-  // pages it reaches decides which attention it takes.)
+  // with a last unit of up to 128 rows apart and the head unit by unit.  (Over the 8-bit cache too: its rows attend over
+  // decoded pages, of which a unit and a pass of several reach at most one stream's old ones and those of their own rows.)
   const int unit = h->ordered ? std::min(pass_rows, h->ordered_pass_rows) : 0;
-  if (unit) pass_rows = h->kv_fp8 ? unit : std::max(unit, std::min(pass_rows, kMaxOrderedRows) / unit * unit);
+  static_assert(2048 / kPageTokens + kMaxOrderedRows / kPageTokens + kMaxRows <= kScratchPages, "a pass over the 8-bit cache never reaches more pages than can be decoded");
+  if (unit) pass_rows = std::max(unit, std::min(pass_rows, kMaxOrderedRows) / unit * unit);
   int left = 0;            // rows not yet in a pass
   for (int i = 0; i < n; ++i) left += plen[i];
   PassParams ps;

@@ -268,6 +268,41 @@ def test_sampled_passes_of_several_units_give_the_bits_of_single_units(form, wfm
     eng.destroy()
 
 
+@pytest.mark.parametrize("form", list(ONE_UNIT_OF_MORE))
+def test_sampled_passes_of_several_units_over_the_8bit_cache(form):
+    """The same over the 8-bit cache, whose passes decode the pages they attend over."""
+    model, unit, lens = ONE_UNIT_OF_MORE[form]
+    kw = dict(kv_fmt=C.KV_FP8_E4M3, max_streams=len(lens), n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=2048, max_pos=2048)
+    if model == "wide":
+        kw.update(d_model=1280, n_head=20, d_ff=5120)
+    cfg = C.tiny_config(**kw)
+    eng = B.TtsGpt(cfg, C.make_weights(cfg, seed=57), DEV)
+    prefixes = C.make_prefixes(cfg, lens, seed=58)
+    u = dict(top_k=30, uniforms=torch.rand(len(lens), generator=torch.Generator(DEV).manual_seed(4), device=DEV))
+    steps = 2 if max(lens) <= 2040 else 0
+    lg, tk = _run(eng, prefixes, steps, **u)
+    eng.set_option("prefill_pass_rows", unit)
+    lg1, tk1 = _run(eng, prefixes, steps, **u)
+    assert np.array_equal(lg, lg1) and np.array_equal(tk, tk1)
+    assert eng.check_canaries() == 0
+    eng.destroy()
+
+
+@pytest.mark.parametrize("wfmt,lens", [(C.W_BF16, [897]), (C.W_INT8_PC, [500, 520]), (C.W_INT4_G128, [1024]), (C.W_BF16, [640, 512, 128])])
+def test_prefill_passes_around_the_pair_kernels_lines(wfmt, lens):
+    """897, 1020 and 1024 rows: FC2 alone on pairs, the other linears on single CTAs; 1280: all on single CTAs."""
+    cfg = C.tiny_config(wfmt=wfmt, d_model=1280, n_head=20, d_ff=5120, max_streams=len(lens), n_pages=sum(x // 64 + 2 for x in lens),
+                        max_context=1088, max_pos=1088)
+    w = C.make_weights(cfg, seed=59)
+    model = O.OracleModel(cfg, w)
+    eng = B.TtsGpt(cfg, w, DEV)
+    prefixes = C.make_prefixes(cfg, lens, seed=60)
+    lg, tk = _run(eng, prefixes, 1)
+    _check(model, prefixes, lg, tk, range(len(lens)), "around the lines")
+    assert np.array_equal(lg, _run(eng, prefixes, 1)[0])
+    eng.destroy()
+
+
 @pytest.mark.parametrize("S", [1, 21, 30, 40, 60, 80])
 def test_8bit_decode_attention_splits(S):
     """8, 6, 4, 3, 2 and 1 CTAs per (row, head) over the 8-bit cache: contexts at the edges of half pages and pages, splits
