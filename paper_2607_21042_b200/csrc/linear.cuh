@@ -279,8 +279,9 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
   }
   if (LN_ROWS) __syncthreads();
   // cluster of k-ranges: the outputs this CTA finishes, one per thread (a quarter of the tile's), and their bias
-  __shared__ float cl_part[CL ? kSmallKSplit : 1][CL ? 4 * C : 1];   // every range's sums of this CTA's share
-  __shared__ int cl_here[kSmallKSplit];                                  // ... have been written
+  // (behind the activation rows: a static array would move every kernel's shared memory)
+  float *cl_part = reinterpret_cast<float *>(stage + (size_t)a.B * ln_stage_stride(WF, KB * KT));   // [range][4 C] every range's sums of this CTA's share
+  int *cl_here = reinterpret_cast<int *>(cl_part + kSmallKSplit * 4 * C);                           // [range] ... have been written
   const int cl_share = CL ? (a.B * C + (int)gridDim.y - 1) / (int)gridDim.y : 1, cl_o = (int)blockIdx.y * cl_share + (int)threadIdx.x;
   const bool cl_mine = CL && threadIdx.x < cl_share && cl_o < a.B * C && tile0 * 8 + cl_o % C < a.N;
   float cl_bias = 0.f;
@@ -622,7 +623,7 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
         if (WF == WF_INT8) v *= e_scale;
         if (CL) {              // partial sum of this k-range, to the CTA that finishes the output
           const int rank = o / cl_share;
-          st_shared_of_rank(&cl_part[CL ? (int)blockIdx.y : 0][CL ? o - rank * cl_share : 0], rank, v);
+          st_shared_of_rank(cl_part + (int)blockIdx.y * 4 * C + o - rank * cl_share, rank, v);
           continue;
         }
         if (gridDim.y > 1) {   // partial sum of this k-range; bias and residual are added by the folding LayerNorm
@@ -665,10 +666,10 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
     cluster_arrive_release();
     cluster_wait();
     if (cl_mine) {
-      float v = cl_part[0][threadIdx.x];
+      float v = cl_part[threadIdx.x];
       int here = cl_here[0];
 #pragma unroll
-      for (int k = 1; k < (CL ? kSmallKSplit : 1); ++k) { v += cl_part[k][threadIdx.x]; here &= cl_here[k]; }
+      for (int k = 1; k < kSmallKSplit; ++k) { v += cl_part[k * 4 * C + threadIdx.x]; here &= cl_here[k]; }
       if (here) a.out_f32[(size_t)(cl_o / C) * a.out_stride + tile0 * 8 + cl_o % C] = cl_old + (v + cl_bias);
     }
   }
@@ -713,7 +714,7 @@ inline cudaError_t launch_linear_nb(const LinearArgs &a, int grid, cudaStream_t 
     if (a.cluster) {
       static SmemOptIn opt_in_cl;
       if (const cudaError_t e = opt_in_cl(linear_kernel<WF, RT, MODE, NB, true>, 200 * 1024)) return e;
-      return launch_kernel_cluster_dims(linear_kernel<WF, RT, MODE, NB, true>, dim3(grid, ks), dim3(kLinearThreads), smem, dim3(1, ks), st, pdl, a);
+      return launch_kernel_cluster_dims(linear_kernel<WF, RT, MODE, NB, true>, dim3(grid, ks), dim3(kLinearThreads), smem + (kSmallKSplit * 4 * 8 * RT + kSmallKSplit) * sizeof(float), dim3(1, ks), st, pdl, a);
     }
   }
   return launch_kernel(linear_kernel<WF, RT, MODE, NB>, dim3(grid, ks), dim3(kLinearThreads), smem, st, pdl, a);
