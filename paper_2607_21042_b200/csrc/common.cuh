@@ -189,6 +189,28 @@ __device__ __forceinline__ uint4 ld_cg_u4(const void *p) {
 
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
+// Pages of a decode step's next attention, asked into L2 while the linears leave the memory idle: by one warp of every CTA.
+struct KvPrefetch {
+  const unsigned char *layer;   // the layer's slice of the page pool; null: nothing to ask for
+  uint32_t block_bytes;         // one (page, K|V, head) block
+  int blocks;                   // blocks of a page, contiguous
+  const int4 *slots;            // rows by rank of length, and their pages (AttnArgs)
+  const int *slot_pages;
+  int pps, rows, cap;           // up to `cap` complete pages of every row
+  int part, n_parts;            // this kernel's share of the blocks
+};
+__device__ __forceinline__ void kv_prefetch(const KvPrefetch &p, int cta, int n_cta) {
+  const int lane = threadIdx.x & 31;
+  const int total = p.rows * p.cap * p.blocks;
+#pragma unroll 1
+  for (int u = (cta * 32 + lane) * p.n_parts + p.part; u < total; u += n_cta * 32 * p.n_parts) {
+    const int t = u / p.blocks, b = u - t * p.blocks, z = t / p.cap, j = t - z * p.cap;
+    const int phys = p.slot_pages[z * p.pps + j];
+    if (j >= (p.slots[z].y - 1) / kPageTokens) continue;
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.layer + ((size_t)phys * p.blocks + b) * p.block_bytes), "r"(p.block_bytes) : "memory");
+  }
+}
+
 // D(16x8,f32) += A(16x16,bf16,row) * B(16x8,bf16,col).  Fragment layout (g = lane/4, t = lane%4):
 // a0=(row g, k 2t..2t+1) a1=(row g+8, same k) a2=(row g, k 2t+8..2t+9) a3=(row g+8, same);
 // b0=(k 2t..2t+1, col g) b1=(k 2t+8..2t+9, col g); c0,c1=(row g, cols 2t,2t+1) c2,c3=(row g+8).

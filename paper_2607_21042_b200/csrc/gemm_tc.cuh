@@ -269,6 +269,7 @@ struct GemmTcArgs {
   unsigned long long issue_wait_ns;   // -1: the producer of a pair's CTA 1 comes to each of its tiles that much late; 0: none
   unsigned long long *trace;  // optional timeline trace (see trace_mark)
   int trace_slot;
+  KvPrefetch pf;
 };
 
 // One lane of a converged warp, known to the compiler as such.  tcgen05 and bulk-copy instructions take their operands
@@ -414,6 +415,7 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
     }
   }
   pdl_launch_dependents();
+  if (a.pf.layer && warp == 9) kv_prefetch(a.pf, (bc + gridDim.y * ks) * gridDim.x + nt, gridDim.x * gridDim.y * gridDim.z);
   pdl_wait();
   trace_mark(a.trace, a.trace_slot, 1);
   if (warp == 0) {

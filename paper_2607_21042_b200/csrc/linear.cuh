@@ -150,6 +150,7 @@ struct LinearArgs {
   int *err;                   // optional device error word: set to 1 if the weight copy never arrives
   int ksplit;                 // 0 or 1: whole K per CTA; n > 1 (EPI_RESID only, no fused LN): gridDim.y = n k-ranges,
                               // out_f32 = partial sums [n][kMaxRows][N] without bias, folded by the next LayerNorm
+  KvPrefetch pf;              // tensor-pipe path
   int cluster;                // with ksplit (up to 16 rows, tensor-pipe path): the k-ranges of a tile are a cluster and add into out_f32 themselves
 };
 
@@ -291,6 +292,7 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
     cluster_arrive_release();
   }
   pdl_launch_dependents();
+  if (NB == 0 && a.pf.layer && warp == kLinearWarps - 1) kv_prefetch(a.pf, blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y);
   pdl_wait();
   trace_mark(a.trace, a.trace_slot, 1);
   float cl_old = 0.f;

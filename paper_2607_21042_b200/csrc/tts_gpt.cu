@@ -129,6 +129,7 @@ struct tts_gpt {
   int attn_cluster_fill = 1;     // clusters grow until the grid covers the GPU this many times
   int attn_stream_min_pairs = 0; // (row, head) pairs from which it is used; 0: attention_use_stream decides
   int tc_min_rows = 17; // rows from which the tensor-core path is taken (option "tc_min_rows")
+  bool kv_prefetch = true;       // pages of the next attention asked into L2 by the linears in between (option "kv_prefetch")
   bool poison_free = false;     // option "poison_free_pages": released pages are filled with NaN
   unsigned char *canary_lo = nullptr, *canary_hi = nullptr;   // guard regions either side of the KV pool
   int n_sm = 148;
@@ -444,6 +445,39 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
   return launch_attention(aa, R, attention_cluster_size(R, aa.H, h->n_sm, h->attn_cluster_fill), st, pdl);
 }
 
+// Whether LayerNorm is fused into the linears of up to 16 rows; FC2's k-ranges then meet in clusters, so that x is complete.
+// Five kernels per layer instead of seven; the price is x read by every CTA (5 KB a row) and a cluster barrier.  ms per
+// step, kernels of their own / fused, contexts of 500 tokens (bf16, int4, bf16 weights over the 8-bit cache) and 1400 (bf16):
+// 2 rows 0.552 / 0.520, 0.542 / 0.522, 0.574 / 0.547, 0.598 / 0.571; 4 rows 0.596 / 0.552, 0.591 / 0.552, 0.633 / 0.585, 0.671 /
+// 0.638; 6 rows 0.666 / 0.601, 0.648 / 0.596, 0.688 / 0.642, 0.758 / 0.703; 7 rows 0.659 / 0.633, 0.654 / 0.624, 0.698 / 0.679,
+// 0.784 / 0.741; 8 rows 0.638 / 0.647, 0.639 / 0.620, 0.673 / 0.677, 0.754 / 0.792 (kernels of their own but for int4); 9 rows
+// 0.705 / 0.699, 0.692 / 0.664, 0.746 / 0.730, 0.875 / 0.845; 10 rows 0.756 / 0.717, 0.695 / 0.674, 0.825 / 0.799, 0.947 / 0.924;
+// 11 rows 0.777 / 0.799, 0.728 / 0.748, 0.852 / 0.868, 0.993 / 1.010; 14 rows 0.891 / 1.001, 0.798 / 0.804, 0.997 / 1.098.
+bool fuse_layernorm(const tts_gpt *h, int R) {
+  return can_fuse_ln(R, h->cfg.d_model, h->ordered, h->ln_fuse_rows) && (h->ordered || R != 8 || h->cfg.wfmt == WF_INT4);
+}
+
+// Part 0 (O projection), 1 (FC1) or 2 (FC2 of layer l) of the pages asked into L2 for the attention of the layer behind (behind
+// the last: the next step's first).  Between two attentions the memory is idle half of the time, and attention at these
+// sizes waits for it: ms per step without / with 16 MB of pages, 8 rows of 500 tokens 0.637 / 0.622, 12 rows of 900 0.904 /
+// 0.889, 16 rows of 500 0.851 / 0.839, 24 rows of 500 1.014 / 0.995, 37 rows of 575 1.208 / 1.187 (sampled 1.216 / 1.203); with
+// 48 MB the linears behind wait for theirs (24 rows 1.034).  Not with LayerNorm fused (3 rows of 1700 0.619 / 0.620), not over
+// the 8-bit cache (9 rows 0.734 / 0.750, 24 rows level), and from 49 rows on a page per row is more than the budget.
+constexpr long long kPrefetchBytes = 16000000;
+KvPrefetch kv_prefetch_args(const tts_gpt *h, int R, int l, int part, bool decode) {
+  KvPrefetch p;
+  memset(&p, 0, sizeof p);
+  if (!decode || !h->kv_prefetch || h->kv_fp8 || R < 2 || fuse_layernorm(h, R)) return p;
+  p.cap = (int)std::min<long long>(h->pps, kPrefetchBytes / ((long long)R * h->kv_page_elems * 2));
+  if (p.cap < 1) return p;
+  p.layer = reinterpret_cast<const unsigned char *>(h->kv + h->kv_layer_elems * ((l + 1) % h->cfg.n_layer));
+  p.blocks = 2 * h->cfg.n_head;
+  p.block_bytes = kPageElems * 2;
+  p.slots = h->rt.slots; p.slot_pages = h->rt.slot_pages; p.pps = h->pps;
+  p.rows = R; p.part = part; p.n_parts = 3;
+  return p;
+}
+
 // The transformer blocks for R rows already described by the row table, x holding the input rows.
 // Every kernel after the first of a step is launched with programmatic dependent launch, so its
 // weight loads overlap the tail of its predecessor.
@@ -561,33 +595,24 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
     GemmTcArgs oa = gemm_args(h, L.o, h->o_img, R, EPI_RESID, o_ks);
     oa.out_f32 = o_parts ? h->partials : h->x; oa.out_stride = d;
     trace_attach(h, oa);
+    oa.pf = kv_prefetch_args(h, R, l, 0, decode);
     if ((rc = launch_gemm(h, oa, L.o.w_map, h->o_map, wide, pairs, st, pdl))) return rc;
     rc = launch_ln_tc(h, R, L.ln2_g, L.ln2_b, o_parts, o_parts ? L.o.bias : nullptr, h->a_img, nullptr, nullptr, nullptr, nullptr, 1);
     if (rc) return rc;
     GemmTcArgs f1 = gemm_args(h, L.fc1, h->a_img, R, EPI_GELU, 1);
     f1.out_img = h->h_img; f1.gelu_tanh = c.gelu_tanh;
     trace_attach(h, f1);
+    f1.pf = kv_prefetch_args(h, R, l, 1, decode);
     if ((rc = launch_gemm(h, f1, L.fc1.w_map, h->a_map, wide, pairs, st, pdl))) return rc;
     GemmTcArgs f2 = gemm_args(h, L.fc2, h->h_img, R, EPI_RESID, f2_ks);
     f2.out_f32 = f2_parts ? h->partials : h->x; f2.out_stride = d;
     trace_attach(h, f2);
+    f2.pf = kv_prefetch_args(h, R, l, 2, decode);
     if ((rc = launch_gemm(h, f2, L.fc2.w_map, h->h_map, wide, pairs2, st, pdl))) return rc;
     h->launches += 5;
   }
   h->tc_tail_parts = f2_parts;
   return TTS_GPT_OK;
-}
-
-// Whether LayerNorm is fused into the linears of up to 16 rows; FC2's k-ranges then meet in clusters, so that x is complete.
-// Five kernels per layer instead of seven; the price is x read by every CTA (5 KB a row) and a cluster barrier.  ms per
-// step, kernels of their own / fused, contexts of 500 tokens (bf16, int4, bf16 weights over the 8-bit cache) and 1400 (bf16):
-// 2 rows 0.552 / 0.520, 0.542 / 0.522, 0.574 / 0.547, 0.598 / 0.571; 4 rows 0.596 / 0.552, 0.591 / 0.552, 0.633 / 0.585, 0.671 /
-// 0.638; 6 rows 0.666 / 0.601, 0.648 / 0.596, 0.688 / 0.642, 0.758 / 0.703; 7 rows 0.659 / 0.633, 0.654 / 0.624, 0.698 / 0.679,
-// 0.784 / 0.741; 8 rows 0.638 / 0.647, 0.639 / 0.620, 0.673 / 0.677, 0.754 / 0.792 (kernels of their own but for int4); 9 rows
-// 0.705 / 0.699, 0.692 / 0.664, 0.746 / 0.730, 0.875 / 0.845; 10 rows 0.756 / 0.717, 0.695 / 0.674, 0.825 / 0.799, 0.947 / 0.924;
-// 11 rows 0.777 / 0.799, 0.728 / 0.748, 0.852 / 0.868, 0.993 / 1.010; 14 rows 0.891 / 1.001, 0.798 / 0.804, 0.997 / 1.098.
-bool fuse_layernorm(const tts_gpt *h, int R) {
-  return can_fuse_ln(R, h->cfg.d_model, h->ordered, h->ln_fuse_rows) && (h->ordered || R != 8 || h->cfg.wfmt == WF_INT4);
 }
 
 // Final LayerNorm (folding the last FC2's partial sums), LM head, sampling after run_layers_tc.
@@ -670,6 +695,7 @@ int run_layers(tts_gpt *h, int R, bool decode) {
     LinearArgs oa = linear_args(h, L.o, h->o, R, EPI_RESID);
     oa.out_f32 = h->x; oa.out_stride = d;
     trace_attach(h, oa);
+    oa.pf = kv_prefetch_args(h, R, l, 0, decode);
     CUDA_TRY(h, launch_linear(c.wfmt, oa, st, pdl, 2 * h->n_sm));
     LinearArgs f1 = linear_args(h, L.fc1, h->a, R, EPI_GELU);
     if (fuse_ln) {
@@ -682,11 +708,13 @@ int run_layers(tts_gpt *h, int R, bool decode) {
     }
     f1.out_bf16 = h->hbuf; f1.gelu_tanh = c.gelu_tanh;
     trace_attach(h, f1);
+    f1.pf = kv_prefetch_args(h, R, l, 1, decode);
     CUDA_TRY(h, launch_linear(c.wfmt, f1, st, pdl, 2 * h->n_sm));
     LinearArgs f2 = linear_args(h, L.fc2, h->hbuf, R, EPI_RESID);
     f2.out_f32 = h->x; f2.out_stride = d;
     if (fc2_ks > 1) { f2.ksplit = fc2_ks; f2.cluster = cluster ? 1 : 0; if (!cluster) f2.out_f32 = h->partials; }
     trace_attach(h, f2);
+    f2.pf = kv_prefetch_args(h, R, l, 2, decode);
     CUDA_TRY(h, launch_linear(c.wfmt, f2, st, pdl, 2 * h->n_sm));
     h->launches += 5;
   }
@@ -1084,7 +1112,7 @@ int32_t tts_gpt_decode_step(tts_gpt_t *h, int32_t n, const int32_t *stream_ids, 
   sp.io.out_hidden = (uint16_t *)out_hidden; sp.io.top_k = top_k; sp.io.temperature = temperature; sp.io.n_out = n;
   h->ordered = top_k > 1;
   auto enqueue = [&]() -> int {
-    step_setup_kernel<<<1, kSetupThreads, 0, h->stream>>>(sp, h->ps, h->rt, h->io);
+    step_setup_kernel<<<1, setup_threads(n), 0, h->stream>>>(sp, h->ps, h->rt, h->io);
     CUDA_TRY(h, cudaGetLastError());
     h->launches += 1;
     int r = run_embed(h, n);
@@ -1120,7 +1148,7 @@ int32_t tts_gpt_decode_step(tts_gpt_t *h, int32_t n, const int32_t *stream_ids, 
     cudaKernelNodeParams kp;
     memset(&kp, 0, sizeof kp);
     kp.func = (void *)step_setup_kernel;
-    kp.gridDim = dim3(1); kp.blockDim = dim3(kSetupThreads); kp.kernelParams = args;
+    kp.gridDim = dim3(1); kp.blockDim = dim3(setup_threads(n)); kp.kernelParams = args;
     CUDA_TRY(h, cudaGraphExecKernelNodeSetParams(sg->exec, sg->setup, &kp));
   }
   for (int i = 0; i < n; ++i) { h->ctx[stream_ids[i]] += 1; h->pos_next[stream_ids[i]] += 1; }
@@ -1331,6 +1359,7 @@ int32_t tts_gpt_debug_set_option(tts_gpt_t *h, const char *name, int32_t value) 
   else if (k == "attn_cluster_fill") h->attn_cluster_fill = value > 0 ? value : 1;
   else if (k == "attn_queue") { if (value < 0 || value > 2) return fail(h, TTS_GPT_E_ARG, "attn_queue must be 0 (off), 1 (by the number of pairs) or 2 (always)"); h->attn_queue = value; }
   else if (k == "ln_fuse_rows") { if (value < 1 || value > 16) return fail(h, TTS_GPT_E_ARG, "ln_fuse_rows must be in 1..16"); h->ln_fuse_rows = value; }
+  else if (k == "kv_prefetch") h->kv_prefetch = on;
   else if (k == "fc2_ksplit") h->use_fc2_ksplit = on;
   else if (k == "poison_free_pages") {
     h->poison_free = on;

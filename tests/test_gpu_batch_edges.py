@@ -268,6 +268,21 @@ def test_sampled_passes_of_several_units_give_the_bits_of_single_units(form, wfm
     eng.destroy()
 
 
+@pytest.mark.parametrize("S", [11, 40, 128])
+def test_pages_asked_into_l2_change_nothing(S):
+    """The linears of a step ask the next attention's complete pages into L2: the same bits with and without, contexts with and
+    without a complete page, more pages than the budget takes."""
+    lens = [1, 63, 64, 65, 129, 700][:min(S, 6)] + [3 + (13 * i) % 200 for i in range(S - 6)]
+    cfg = C.tiny_config(max_streams=S, n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=768)
+    eng = B.TtsGpt(cfg, C.make_weights(cfg, seed=61), DEV)
+    prefixes = C.make_prefixes(cfg, lens, seed=62)
+    lg, tk = _run(eng, prefixes, 3)
+    eng.set_option("kv_prefetch", 0)
+    lg2, tk2 = _run(eng, prefixes, 3)
+    assert np.array_equal(lg, lg2) and np.array_equal(tk, tk2)
+    eng.destroy()
+
+
 @pytest.mark.parametrize("form", list(ONE_UNIT_OF_MORE))
 def test_sampled_passes_of_several_units_over_the_8bit_cache(form):
     """The same over the 8-bit cache, whose passes decode the pages they attend over."""
