@@ -190,7 +190,7 @@ __device__ __forceinline__ uint32_t load_quarters(PageLoad &pl, const uint16_t *
     if (u < n_units) {
       ng = j + 1;
       const int page = u >> 2, qt = u & 3;
-      const int phys = ar.phys(page);
+      const int phys = ar.pt[page];
       const uint16_t *K = kv_layer + (((size_t)phys * 2 + 0) * H + h) * kPageElems + (size_t)(16 * qt) * kHeadDim;
       const uint16_t *V = kv_layer + (((size_t)phys * 2 + 1) * H + h) * kPageElems + (size_t)(16 * qt) * kHeadDim;
       const int left = n_tok - page * kPageTokens - 16 * qt;   // tokens of the row from this quarter on
@@ -292,8 +292,8 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attention_kernel(const AttnAr
     load_q(qv, a.q + (size_t)r * a.H * kHeadDim + h * kHeadDim + 8 * sub);
     if (early) {
       const int us = 4 * (n_pages - 1) + (tn >> 4);   // unit of the new token
-      const int phys = ar.phys(n_pages - 1);
       if (us % GW == gw && us / GW < 4 && (tn & 3) == tg) {
+        const int phys = ar.pt[n_pages - 1];
         const uint4 kn = ld_cg_u4(a.kv_layer + (((size_t)phys * 2 + 0) * a.H + h) * kPageElems + (size_t)tn * kHeadDim + 8 * sub);
         const uint4 vn = ld_cg_u4(a.kv_layer + (((size_t)phys * 2 + 1) * a.H + h) * kPageElems + (size_t)tn * kHeadDim + 8 * sub);
         const int sel = 4 * (us / GW) + ((tn & 15) >> 2);

@@ -60,16 +60,19 @@ struct StepParams {
 // in call order take pages in stack order), then the row table is written and ctx_len advances.
 // Attention's CTAs find what they work on in `slots` and `slot_pages`, by rank of the row's length: one round trip to L2
 // where row order, position, stream and page table were three, in front of the first page request of every CTA of 24 layers.
-constexpr int kSetupRows = 8;   // page lists per warp, lane = page (max_context is at most 2048)
+// ROWS: page lists per warp, lane = page (max_context is at most 2048).  Little code where there are few rows: it runs once per
+// step, fetched cold.
+constexpr int kSetupRows = 8;
 inline int setup_threads(int n) { return n <= kSetupRows * kMaxRows / 32 ? kMaxRows : kMaxRows / kSetupRows * 32; }
+template <int ROWS>
 __global__ void __launch_bounds__(kMaxRows / kSetupRows * 32) step_setup_kernel(const StepParams p, PageState ps, RowTable rt, StepIO *io) {
   const int i = threadIdx.x;
   __shared__ int len_s[kMaxRows], new_s[kMaxRows], rank_s[kMaxRows];
   // the page lists, a row per warp at a time: asked for together with everything else
   const int warp = i >> 5, lane = i & 31, n_warp = blockDim.x >> 5;
-  int page[kSetupRows];
+  int page[ROWS];
 #pragma unroll
-  for (int q = 0; q < kSetupRows; ++q) {
+  for (int q = 0; q < ROWS; ++q) {
     const int r = warp + q * n_warp;
     page[q] = 0;
     if (r < p.n && lane < ps.pps) page[q] = ps.page_table[p.stream_ids[r] * ps.pps + lane];
@@ -102,7 +105,7 @@ __global__ void __launch_bounds__(kMaxRows / kSetupRows * 32) step_setup_kernel(
   if (i == 0) { *ps.free_top = top - total; *io = p.io; }
   __syncthreads();
 #pragma unroll
-  for (int q = 0; q < kSetupRows; ++q) {
+  for (int q = 0; q < ROWS; ++q) {
     const int r = warp + q * n_warp;
     if (r < p.n && lane < ps.pps) rt.slot_pages[rank_s[r] * ps.pps + lane] = new_s[r] >= 0 && lane == len_s[r] / kPageTokens ? new_s[r] : page[q];
   }

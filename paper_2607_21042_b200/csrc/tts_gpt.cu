@@ -1111,8 +1111,9 @@ int32_t tts_gpt_decode_step(tts_gpt_t *h, int32_t n, const int32_t *stream_ids, 
   sp.io.in_tokens = in_tokens; sp.io.uniforms = uniforms; sp.io.out_tokens = out_tokens; sp.io.out_logits = out_logits;
   sp.io.out_hidden = (uint16_t *)out_hidden; sp.io.top_k = top_k; sp.io.temperature = temperature; sp.io.n_out = n;
   h->ordered = top_k > 1;
+  const auto setup = n <= kMaxRows / 32 ? step_setup_kernel<1> : step_setup_kernel<kSetupRows>;   // one page list per warp, or more
   auto enqueue = [&]() -> int {
-    step_setup_kernel<<<1, setup_threads(n), 0, h->stream>>>(sp, h->ps, h->rt, h->io);
+    setup<<<1, setup_threads(n), 0, h->stream>>>(sp, h->ps, h->rt, h->io);
     CUDA_TRY(h, cudaGetLastError());
     h->launches += 1;
     int r = run_embed(h, n);
@@ -1147,7 +1148,7 @@ int32_t tts_gpt_decode_step(tts_gpt_t *h, int32_t n, const int32_t *stream_ids, 
     void *args[] = {&sp, &h->ps, &h->rt, &h->io};
     cudaKernelNodeParams kp;
     memset(&kp, 0, sizeof kp);
-    kp.func = (void *)step_setup_kernel;
+    kp.func = (void *)setup;
     kp.gridDim = dim3(1); kp.blockDim = dim3(setup_threads(n)); kp.kernelParams = args;
     CUDA_TRY(h, cudaGraphExecKernelNodeSetParams(sg->exec, sg->setup, &kp));
   }
