@@ -269,8 +269,10 @@ struct GemmTcArgs {
   unsigned long long issue_wait_ns;   // -1: the producer of a pair's CTA 1 comes to each of its tiles that much late; 0: none
   unsigned long long *trace;  // optional timeline trace (see trace_mark)
   int trace_slot;
-  KvPrefetch pf;
 };
+// Steps whose linears ask for pages have a kernel of their own, the same for all four linears of a layer: its arguments cost
+// the other steps 0.1 us a linear (47 rows over the 8-bit cache 1 %), and two kernels in turn fetch their code cold (24 rows 5 %).
+struct GemmTcPrefetchArgs : GemmTcArgs { KvPrefetch pf; };
 
 // One lane of a converged warp, known to the compiler as such.  tcgen05 and bulk-copy instructions take their operands
 // from the warp's uniform registers: issued under `if (lane == 0)` inside single-thread code, each operand is first
@@ -339,8 +341,8 @@ __device__ __forceinline__ void tc_linger(volatile int *failed) {
 // finished group out, multiply it by the group's scale of their weight row and add it to fp32
 // registers.  Otherwise one 32-column accumulator collects the whole k-range.
 // CN: batch rows per CTA (the N operand), 32 or 64.
-template <bool GROUPED, int CN>
-__global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a) {
+template <bool GROUPED, int CN, typename Args>
+__global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const Args a) {
   static_assert(CN == 32 || !GROUPED, "the group buffers hold 32 columns");
   constexpr uint32_t kStage = kTcABytes + CN * 128;   // a stage: 128 weight rows | CN batch rows
   const int n_stage = a.stages;                       // even: a stage is always consumed by the same issuer
@@ -415,7 +417,9 @@ __global__ void __launch_bounds__(kTcThreads) gemm_tc_kernel(const GemmTcArgs a)
     }
   }
   pdl_launch_dependents();
-  if (a.pf.layer && warp == 9) kv_prefetch(a.pf, (bc + gridDim.y * ks) * gridDim.x + nt, gridDim.x * gridDim.y * gridDim.z);
+  if constexpr (sizeof(Args) > sizeof(GemmTcArgs)) {
+    if (a.pf.layer && warp == 9) kv_prefetch(a.pf, (bc + gridDim.y * ks) * gridDim.x + nt, gridDim.x * gridDim.y * gridDim.z);
+  }
   pdl_wait();
   trace_mark(a.trace, a.trace_slot, 1);
   if (warp == 0) {
@@ -940,19 +944,20 @@ __global__ void fold_partials_kernel(const float *__restrict__ part, int n_part,
 
 inline size_t gemm_tc_smem_bytes(int cn, int stages) { return (size_t)stages * (kTcABytes + cn * 128) + 1024 + 1024; }
 
-template <bool GROUPED, int CN>
-inline cudaError_t launch_gemm_tc_as(GemmTcArgs a, int stages, cudaStream_t st, bool pdl) {
+template <bool GROUPED, int CN, typename Args>
+inline cudaError_t launch_gemm_tc_as(Args a, int stages, cudaStream_t st, bool pdl) {
   static SmemOptIn opt_in;
-  if (const cudaError_t e = opt_in(gemm_tc_kernel<GROUPED, CN>, gemm_tc_smem_bytes(CN, kTcMaxStages))) return e;
+  if (const cudaError_t e = opt_in(gemm_tc_kernel<GROUPED, CN, Args>, gemm_tc_smem_bytes(CN, kTcMaxStages))) return e;
   a.stages = stages;
   dim3 grid((a.N + kTcTileM - 1) / kTcTileM, (a.B + CN - 1) / CN, a.ksplit);
-  return launch_kernel(gemm_tc_kernel<GROUPED, CN>, grid, dim3(kTcThreads), gemm_tc_smem_bytes(CN, stages), st, pdl, a);
+  return launch_kernel(gemm_tc_kernel<GROUPED, CN, Args>, grid, dim3(kTcThreads), gemm_tc_smem_bytes(CN, stages), st, pdl, a);
 }
 
 // n_sm: SMs of the device.  With chunks of 32 batch rows a linear of more than 64 rows has more CTAs than SMs, which share
 // an SM, its bandwidth from L2 (20 KB per k-chunk and CTA, the weights four times over) and a ring of half the depth;
 // chunks of 64 rows leave one CTA per SM with eight stages in flight.
-inline cudaError_t launch_gemm_tc(const GemmTcArgs &a, int n_sm, cudaStream_t st, bool pdl) {
+template <typename Args>
+inline cudaError_t launch_gemm_tc(const Args &a, int n_sm, cudaStream_t st, bool pdl) {
   if (a.wfmt == WF_INT4) return launch_gemm_tc_as<true, 32>(a, kTcStages, st, pdl);
   const int tiles = (a.N + kTcTileM - 1) / kTcTileM * a.ksplit;
   if (tiles * ((a.B + 31) / 32) <= n_sm) return launch_gemm_tc_as<false, 32>(a, kTcMaxStages, st, pdl);

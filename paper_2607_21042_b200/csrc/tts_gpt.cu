@@ -457,7 +457,7 @@ bool fuse_layernorm(const tts_gpt *h, int R) {
   return can_fuse_ln(R, h->cfg.d_model, h->ordered, h->ln_fuse_rows) && (h->ordered || R != 8 || h->cfg.wfmt == WF_INT4);
 }
 
-// Part 0 (O projection), 1 (FC1) or 2 (FC2 of layer l) of the pages asked into L2 for the attention of the layer behind (behind
+// Part 0 (O projection), 1 (FC1), 2 (FC2 of layer l) or none (-1: QKV, which runs the same kernel) of the pages asked into L2 for the attention of the layer behind (behind
 // the last: the next step's first).  Between two attentions the memory is idle half of the time, and attention at these
 // sizes waits for it: ms per step without / with 16 MB of pages, 8 rows of 500 tokens 0.637 / 0.622, 12 rows of 900 0.904 /
 // 0.889, 16 rows of 500 0.851 / 0.839, 24 rows of 500 1.014 / 0.995, 37 rows of 575 1.208 / 1.187 (sampled 1.216 / 1.203); with
@@ -470,11 +470,13 @@ KvPrefetch kv_prefetch_args(const tts_gpt *h, int R, int l, int part, bool decod
   if (!decode || !h->kv_prefetch || h->kv_fp8 || R < 2 || fuse_layernorm(h, R)) return p;
   p.cap = (int)std::min<long long>(h->pps, kPrefetchBytes / ((long long)R * h->kv_page_elems * 2));
   if (p.cap < 1) return p;
+  p.rows = R;   // the step asks for pages
+  if (part < 0) return p;
   p.layer = reinterpret_cast<const unsigned char *>(h->kv + h->kv_layer_elems * ((l + 1) % h->cfg.n_layer));
   p.blocks = 2 * h->cfg.n_head;
   p.block_bytes = kPageElems * 2;
   p.slots = h->rt.slots; p.slot_pages = h->rt.slot_pages; p.pps = h->pps;
-  p.rows = R; p.part = part; p.n_parts = 3;
+  p.part = part; p.n_parts = 3;
   return p;
 }
 
@@ -545,8 +547,15 @@ int launch_ln_tc(tts_gpt *h, int rows, const uint16_t *g, const uint16_t *b, int
   return TTS_GPT_OK;
 }
 
-int launch_gemm(tts_gpt *h, const GemmTcArgs &a, const CUtensorMap &w_map, const CUtensorMap &x_map, bool wide, bool pairs, cudaStream_t st, bool pdl) {
-  if (!wide) CUDA_TRY(h, launch_gemm_tc(a, h->n_sm, st, pdl));
+int launch_gemm(tts_gpt *h, const GemmTcArgs &a, const CUtensorMap &w_map, const CUtensorMap &x_map, bool wide, bool pairs, cudaStream_t st, bool pdl,
+                const KvPrefetch &pf = KvPrefetch{}) {
+  if (!wide && pf.rows > 0) {
+    GemmTcPrefetchArgs p;
+    static_cast<GemmTcArgs &>(p) = a;
+    p.pf = pf;
+    CUDA_TRY(h, launch_gemm_tc(p, h->n_sm, st, pdl));
+  }
+  else if (!wide) CUDA_TRY(h, launch_gemm_tc(a, h->n_sm, st, pdl));
   else if (!pairs) CUDA_TRY(h, launch_gemm_tcw(a, h->n_sm, st, pdl));
   else {
     const CUtensorMap *out = a.mode != EPI_RESID ? nullptr : a.ksplit > 1 ? &h->part_map : &h->xrow_map;
@@ -584,7 +593,7 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
     const bool q_img = wide && h->use_attn_tc && h->use_attn_mma && (!h->kv_fp8 || h->pass_scratch > 0);   // the tcgen05 attention follows
     qa.q_img = q_img ? h->q_img : nullptr;
     trace_attach(h, qa);
-    if ((rc = launch_gemm(h, qa, L.qkv.w_map, h->a_map, wide, pairs, st, pdl))) return rc;
+    if ((rc = launch_gemm(h, qa, L.qkv.w_map, h->a_map, wide, pairs, st, pdl, kv_prefetch_args(h, R, l, -1, decode)))) return rc;
     AttnArgs aa;
     memset(&aa, 0, sizeof aa);
     aa.q = h->q; aa.kv_layer = kvl; aa.page_table = h->ps.page_table; aa.row_stream = h->rt.row_stream;
@@ -595,20 +604,17 @@ int run_layers_tc(tts_gpt *h, int R, bool decode) {
     GemmTcArgs oa = gemm_args(h, L.o, h->o_img, R, EPI_RESID, o_ks);
     oa.out_f32 = o_parts ? h->partials : h->x; oa.out_stride = d;
     trace_attach(h, oa);
-    oa.pf = kv_prefetch_args(h, R, l, 0, decode);
-    if ((rc = launch_gemm(h, oa, L.o.w_map, h->o_map, wide, pairs, st, pdl))) return rc;
+    if ((rc = launch_gemm(h, oa, L.o.w_map, h->o_map, wide, pairs, st, pdl, kv_prefetch_args(h, R, l, 0, decode)))) return rc;
     rc = launch_ln_tc(h, R, L.ln2_g, L.ln2_b, o_parts, o_parts ? L.o.bias : nullptr, h->a_img, nullptr, nullptr, nullptr, nullptr, 1);
     if (rc) return rc;
     GemmTcArgs f1 = gemm_args(h, L.fc1, h->a_img, R, EPI_GELU, 1);
     f1.out_img = h->h_img; f1.gelu_tanh = c.gelu_tanh;
     trace_attach(h, f1);
-    f1.pf = kv_prefetch_args(h, R, l, 1, decode);
-    if ((rc = launch_gemm(h, f1, L.fc1.w_map, h->a_map, wide, pairs, st, pdl))) return rc;
+    if ((rc = launch_gemm(h, f1, L.fc1.w_map, h->a_map, wide, pairs, st, pdl, kv_prefetch_args(h, R, l, 1, decode)))) return rc;
     GemmTcArgs f2 = gemm_args(h, L.fc2, h->h_img, R, EPI_RESID, f2_ks);
     f2.out_f32 = f2_parts ? h->partials : h->x; f2.out_stride = d;
     trace_attach(h, f2);
-    f2.pf = kv_prefetch_args(h, R, l, 2, decode);
-    if ((rc = launch_gemm(h, f2, L.fc2.w_map, h->h_map, wide, pairs2, st, pdl))) return rc;
+    if ((rc = launch_gemm(h, f2, L.fc2.w_map, h->h_map, wide, pairs2, st, pdl, kv_prefetch_args(h, R, l, 2, decode)))) return rc;
     h->launches += 5;
   }
   h->tc_tail_parts = f2_parts;
