@@ -99,21 +99,27 @@ __device__ __forceinline__ void load_page(PageLoad &pl, const uint16_t *K, const
 template <int NS, int N>
 __device__ __forceinline__ float score_slots(const uint4 (&kk)[N], const float (&qv)[8], uint32_t vmask, float (&s)[N]) {
   float pm = -INFINITY;
+  static_assert(NS % 2 == 0, "slots go in pairs: two fp32 products per instruction, each rounded as a scalar one");
 #pragma unroll
-  for (int i = 0; i < NS; ++i) {
-    float d = qv[0] * bf16_lo(kk[i].x);
-    d = fmaf(qv[1], bf16_hi(kk[i].x), d);
-    d = fmaf(qv[2], bf16_lo(kk[i].y), d);
-    d = fmaf(qv[3], bf16_hi(kk[i].y), d);
-    d = fmaf(qv[4], bf16_lo(kk[i].z), d);
-    d = fmaf(qv[5], bf16_hi(kk[i].z), d);
-    d = fmaf(qv[6], bf16_lo(kk[i].w), d);
-    d = fmaf(qv[7], bf16_hi(kk[i].w), d);
-    d += __shfl_xor_sync(0xFFFFFFFFu, d, 1);
-    d += __shfl_xor_sync(0xFFFFFFFFu, d, 2);
-    d += __shfl_xor_sync(0xFFFFFFFFu, d, 4);
-    s[i] = ((vmask >> i) & 1u) ? d : -INFINITY;
-    pm = fmaxf(pm, s[i]);
+  for (int i = 0; i < NS; i += 2) {
+    const uint32_t a[4] = {kk[i].x, kk[i].y, kk[i].z, kk[i].w}, b[4] = {kk[i + 1].x, kk[i + 1].y, kk[i + 1].z, kk[i + 1].w};
+    unsigned long long d2 = mul_f32x2(pack_f32x2(qv[0], qv[0]), pack_f32x2(bf16_lo(a[0]), bf16_lo(b[0])));
+    d2 = fma_f32x2(pack_f32x2(qv[1], qv[1]), pack_f32x2(bf16_hi(a[0]), bf16_hi(b[0])), d2);
+#pragma unroll
+    for (int e = 1; e < 4; ++e) {
+      d2 = fma_f32x2(pack_f32x2(qv[2 * e], qv[2 * e]), pack_f32x2(bf16_lo(a[e]), bf16_lo(b[e])), d2);
+      d2 = fma_f32x2(pack_f32x2(qv[2 * e + 1], qv[2 * e + 1]), pack_f32x2(bf16_hi(a[e]), bf16_hi(b[e])), d2);
+    }
+    float d[2];
+    unpack_f32x2(d2, d[0], d[1]);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      d[j] += __shfl_xor_sync(0xFFFFFFFFu, d[j], 1);
+      d[j] += __shfl_xor_sync(0xFFFFFFFFu, d[j], 2);
+      d[j] += __shfl_xor_sync(0xFFFFFFFFu, d[j], 4);
+      s[i + j] = ((vmask >> (i + j)) & 1u) ? d[j] : -INFINITY;
+      pm = fmaxf(pm, s[i + j]);
+    }
   }
   pm = fmaxf(pm, __shfl_xor_sync(0xFFFFFFFFu, pm, 8));
   pm = fmaxf(pm, __shfl_xor_sync(0xFFFFFFFFu, pm, 16));
@@ -127,22 +133,22 @@ __device__ __forceinline__ void accum_slots(uint4 (&vv)[N], const float (&s)[N],
   const float m_new = fmaxf(m, pm);           // finite: the caller only folds batches with a valid token
   const float rescale = exp2f(m - m_new);     // first batch: exp2(-inf) = 0
   float lp = 0.f;
+  unsigned long long o2[4];                   // two fp32 products per instruction, each rounded as a scalar one
 #pragma unroll
-  for (int e = 0; e < 8; ++e) o[e] *= rescale;
+  for (int e = 0; e < 4; ++e) o2[e] = mul_f32x2(pack_f32x2(o[2 * e], o[2 * e + 1]), pack_f32x2(rescale, rescale));
 #pragma unroll
   for (int i = 0; i < NS; ++i) {
     if (!((vmask >> i) & 1u)) vv[i] = make_uint4(0, 0, 0, 0);  // stale page contents may hold NaN: 0 * NaN must not reach o
     const float p = exp2f(s[i] - m_new);  // masked tokens: exp2(-inf) = 0
     lp += p;
-    o[0] = fmaf(p, bf16_lo(vv[i].x), o[0]);
-    o[1] = fmaf(p, bf16_hi(vv[i].x), o[1]);
-    o[2] = fmaf(p, bf16_lo(vv[i].y), o[2]);
-    o[3] = fmaf(p, bf16_hi(vv[i].y), o[3]);
-    o[4] = fmaf(p, bf16_lo(vv[i].z), o[4]);
-    o[5] = fmaf(p, bf16_hi(vv[i].z), o[5]);
-    o[6] = fmaf(p, bf16_lo(vv[i].w), o[6]);
-    o[7] = fmaf(p, bf16_hi(vv[i].w), o[7]);
+    const unsigned long long p2 = pack_f32x2(p, p);
+    o2[0] = fma_f32x2(p2, pack_f32x2(bf16_lo(vv[i].x), bf16_hi(vv[i].x)), o2[0]);
+    o2[1] = fma_f32x2(p2, pack_f32x2(bf16_lo(vv[i].y), bf16_hi(vv[i].y)), o2[1]);
+    o2[2] = fma_f32x2(p2, pack_f32x2(bf16_lo(vv[i].z), bf16_hi(vv[i].z)), o2[2]);
+    o2[3] = fma_f32x2(p2, pack_f32x2(bf16_lo(vv[i].w), bf16_hi(vv[i].w)), o2[3]);
   }
+#pragma unroll
+  for (int e = 0; e < 4; ++e) unpack_f32x2(o2[e], o[2 * e], o[2 * e + 1]);
   lp += __shfl_xor_sync(0xFFFFFFFFu, lp, 8);
   lp += __shfl_xor_sync(0xFFFFFFFFu, lp, 16);
   l = l * rescale + lp;
