@@ -499,13 +499,13 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
             }
 #pragma unroll
             for (int b = 0; b < NBA; ++b) {
-              // two independent chains of four products keep the FMA pipe busy
-              float s0 = (WF == WF_INT4) ? tacc[j][b] : facc[j][b];
+              // two independent chains of four products, in step: chain 0 a product ahead, then two per instruction
               float s1 = wv[4] * xf[b][4];
-              s0 = fmaf(wv[0], xf[b][0], s0); s1 = fmaf(wv[5], xf[b][5], s1);
-              s0 = fmaf(wv[1], xf[b][1], s0); s1 = fmaf(wv[6], xf[b][6], s1);
-              s0 = fmaf(wv[2], xf[b][2], s0); s1 = fmaf(wv[7], xf[b][7], s1);
-              s0 = fmaf(wv[3], xf[b][3], s0);
+              float s0 = fmaf(wv[0], xf[b][0], (WF == WF_INT4) ? tacc[j][b] : facc[j][b]);
+              unsigned long long s2 = pack_f32x2(s0, s1);
+#pragma unroll
+              for (int e = 1; e < 4; ++e) s2 = fma_f32x2(pack_f32x2(wv[e], wv[4 + e]), pack_f32x2(xf[b][e], xf[b][4 + e]), s2);
+              unpack_f32x2(s2, s0, s1);
               s0 += s1;
               if (WF == WF_INT4) tacc[j][b] = s0; else facc[j][b] = s0;
             }
