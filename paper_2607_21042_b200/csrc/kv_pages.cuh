@@ -60,8 +60,9 @@ struct StepParams {
 // in call order take pages in stack order), then the row table is written and ctx_len advances.
 // Attention's CTAs find what they work on in `slots` and `slot_pages`, by rank of the row's length: one round trip to L2
 // where row order, position, stream and page table were three, in front of the first page request of every CTA of 24 layers.
-// ROWS: page lists per warp, lane = page (max_context is at most 2048).  Little code where there are few rows: it runs once per
-// step, fetched cold.
+// ROWS: page lists per warp, lane = page (max_context is at most 2048); 0: one row, whose attention finds its work itself, without
+// rank tables (with them the two-layer model took 0.3 us more of 39 a step).  Little code where there are few rows: it runs once
+// per step, fetched cold.
 constexpr int kSetupRows = 8;
 inline int setup_threads(int n) { return n <= kSetupRows * kMaxRows / 32 ? kMaxRows : kMaxRows / kSetupRows * 32; }
 template <int ROWS>
@@ -70,7 +71,7 @@ __global__ void __launch_bounds__(kMaxRows / kSetupRows * 32) step_setup_kernel(
   __shared__ int len_s[kMaxRows], new_s[kMaxRows], rank_s[kMaxRows];
   // the page lists, a row per warp at a time: asked for together with everything else
   const int warp = i >> 5, lane = i & 31, n_warp = blockDim.x >> 5;
-  int page[ROWS];
+  int page[ROWS > 0 ? ROWS : 1];
 #pragma unroll
   for (int q = 0; q < ROWS; ++q) {
     const int r = warp + q * n_warp;
@@ -98,12 +99,10 @@ __global__ void __launch_bounds__(kMaxRows / kSetupRows * 32) step_setup_kernel(
     int before = 0;
     for (int j = 0; j < p.n; ++j) before += (len_s[j] > t || (len_s[j] == t && j < i)) ? 1 : 0;
     rt.row_order[before] = i;
-    rt.slots[before] = make_int4(i, t + 1, s, 0);
-    rank_s[i] = before;
-    new_s[i] = fresh;
+    if (ROWS > 0) { rt.slots[before] = make_int4(i, t + 1, s, 0); rank_s[i] = before; new_s[i] = fresh; }
   }
   if (i == 0) { *ps.free_top = top - total; *io = p.io; }
-  __syncthreads();
+  if (ROWS > 0) __syncthreads();
 #pragma unroll
   for (int q = 0; q < ROWS; ++q) {
     const int r = warp + q * n_warp;

@@ -378,7 +378,7 @@ void trace_attach(tts_gpt *h, Args &a) {
 // Attention for R rows: clusters while (row, head) pairs are scarce, one streaming CTA per pair
 // once they cover the GPU several times.
 cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool pdl) {
-  if (aa.old_pages_final) { aa.slots = h->rt.slots; aa.slot_pages = h->rt.slot_pages; }   // written by the decode step's set-up kernel
+  if (aa.old_pages_final && R > 1) { aa.slots = h->rt.slots; aa.slot_pages = h->rt.slot_pages; }   // written by the decode step's set-up kernel
   if (h->kv_fp8) {
     // 8-bit cache: the QKV linear left the new K/V rows in the staging area; encode them into their page
     // slots, then attend over e4m3 pages (the same kernel for prefill passes and decode steps)
@@ -1117,7 +1117,7 @@ int32_t tts_gpt_decode_step(tts_gpt_t *h, int32_t n, const int32_t *stream_ids, 
   sp.io.in_tokens = in_tokens; sp.io.uniforms = uniforms; sp.io.out_tokens = out_tokens; sp.io.out_logits = out_logits;
   sp.io.out_hidden = (uint16_t *)out_hidden; sp.io.top_k = top_k; sp.io.temperature = temperature; sp.io.n_out = n;
   h->ordered = top_k > 1;
-  const auto setup = n <= kMaxRows / 32 ? step_setup_kernel<1> : step_setup_kernel<kSetupRows>;   // one page list per warp, or more
+  const auto setup = n == 1 ? step_setup_kernel<0> : n <= kMaxRows / 32 ? step_setup_kernel<1> : step_setup_kernel<kSetupRows>;
   auto enqueue = [&]() -> int {
     setup<<<1, setup_threads(n), 0, h->stream>>>(sp, h->ps, h->rt, h->io);
     CUDA_TRY(h, cudaGetLastError());
