@@ -179,6 +179,7 @@ __host__ __device__ inline int ln_stage_stride(int wf, int K) { return K + (wf =
 enum { ACT_DIRECT = 0, ACT_STAGED = 1, ACT_LN = 2 };
 constexpr int kStageMaxBytes = 44 * 1024;
 constexpr int kLinearSmemBudget = 108 * 1024;  // per CTA, so that two CTAs share an SM
+constexpr int kLinearSmemMax = 200 * 1024;     // per CTA, where one tile of a long K needs more
 
 // NB: 0 = tensor-pipe path (any batch, 16 rows per m-tile); 1 or 4 = CUDA-core path for at most NB rows.  The fp32 FMAs
 // on the widened weights are cheaper for a single row, where MMAs are fifteen sixteenths padding.  From two rows on the
@@ -706,17 +707,29 @@ inline LinearPlan plan_linear(int wf, int N, int K, int B, int mode, int max_cta
   return p;
 }
 
+// What a clustered linear needs of shared memory besides: every range's sums of a CTA's share, and their marks.
+inline size_t cluster_smem_bytes(int rt) { return (kSmallKSplit * 4 * 8 * rt + kSmallKSplit) * sizeof(float); }
+
+// Whether the kSmallKSplit k-ranges of a linear can be a cluster: whole tiles in each, and the activation rows of a range in
+// the staging area (bf16 weights, 10 rows: K up to 8832), beside the weights of the smallest plan.
+inline bool can_cluster(int wf, int B, int K) {
+  const int range = K / kSmallKSplit;
+  return B >= 2 && B <= 16 && (K / k_per_tile(wf)) % kSmallKSplit == 0 &&
+         (size_t)B * ln_stage_stride(wf, range) * sizeof(uint16_t) <= (size_t)kStageMaxBytes &&
+         linear_smem_bytes(wf, 1, ACT_STAGED, B, range) + cluster_smem_bytes(1) <= (size_t)kLinearSmemMax;
+}
+
 template <int WF, int RT, int MODE, int NB>
 inline cudaError_t launch_linear_nb(const LinearArgs &a, int grid, cudaStream_t st, bool pdl) {
   const int ks = a.ksplit > 1 ? a.ksplit : 1;
   const size_t smem = linear_smem_bytes(WF, RT, MODE, a.B, a.K / ks);
   static SmemOptIn opt_in;
-  if (const cudaError_t e = opt_in(linear_kernel<WF, RT, MODE, NB>, 200 * 1024)) return e;
+  if (const cudaError_t e = opt_in(linear_kernel<WF, RT, MODE, NB>, kLinearSmemMax)) return e;
   if constexpr (NB == 0 && MODE == ACT_STAGED) {
     if (a.cluster) {
       static SmemOptIn opt_in_cl;
-      if (const cudaError_t e = opt_in_cl(linear_kernel<WF, RT, MODE, NB, true>, 200 * 1024)) return e;
-      return launch_kernel_cluster_dims(linear_kernel<WF, RT, MODE, NB, true>, dim3(grid, ks), dim3(kLinearThreads), smem + (kSmallKSplit * 4 * 8 * RT + kSmallKSplit) * sizeof(float), dim3(1, ks), st, pdl, a);
+      if (const cudaError_t e = opt_in_cl(linear_kernel<WF, RT, MODE, NB, true>, kLinearSmemMax)) return e;
+      return launch_kernel_cluster_dims(linear_kernel<WF, RT, MODE, NB, true>, dim3(grid, ks), dim3(kLinearThreads), smem + cluster_smem_bytes(RT), dim3(1, ks), st, pdl, a);
     }
   }
   return launch_kernel(linear_kernel<WF, RT, MODE, NB>, dim3(grid, ks), dim3(kLinearThreads), smem, st, pdl, a);
@@ -736,7 +749,7 @@ template <int WF, int MODE>
 inline cudaError_t launch_linear_wf(const LinearArgs &a, int max_ctas, cudaStream_t st, bool pdl) {
   const int ks = a.ksplit > 1 ? a.ksplit : 1;
   const LinearPlan p = plan_linear(WF, a.N, a.K / ks, a.B, MODE, max_ctas / ks);
-  if (linear_smem_bytes(WF, p.rt, MODE, a.B, a.K / ks) > 200 * 1024) return cudaErrorInvalidValue;
+  if (linear_smem_bytes(WF, p.rt, MODE, a.B, a.K / ks) > (size_t)kLinearSmemMax) return cudaErrorInvalidValue;
   if (p.rt == 1) return launch_linear_inst<WF, 1, MODE>(a, p.grid, st, pdl);
   if (p.rt == 2) return launch_linear_inst<WF, 2, MODE>(a, p.grid, st, pdl);
   if (p.rt == 3) return launch_linear_inst<WF, 3, MODE>(a, p.grid, st, pdl);
@@ -759,7 +772,7 @@ inline cudaError_t launch_linear_mode(const LinearArgs &a, int max_ctas, cudaStr
 // K must be a multiple of 128.
 inline cudaError_t launch_linear(int wf, const LinearArgs &a, cudaStream_t st, bool pdl, int max_ctas) {
   if (a.ln_x && !can_fuse_ln(a.B, a.K, a.ordered, 16)) return cudaErrorInvalidValue;
-  if (a.cluster && (a.ksplit != kSmallKSplit || a.B < 2 || a.B > 16 || a.ordered || (size_t)a.B * ln_stage_stride(wf, a.K / a.ksplit) * sizeof(uint16_t) > (size_t)kStageMaxBytes)) return cudaErrorInvalidValue;
+  if (a.cluster && (a.ksplit != kSmallKSplit || a.ordered || !can_cluster(wf, a.B, a.K))) return cudaErrorInvalidValue;
   if (a.ksplit > 1 && (a.ln_x || a.mode != EPI_RESID || (a.K / k_per_tile(wf)) % a.ksplit != 0)) return cudaErrorInvalidValue;
   if (wf == WF_BF16) return launch_linear_mode<WF_BF16>(a, max_ctas, st, pdl);
   if (wf == WF_INT8) return launch_linear_mode<WF_INT8>(a, max_ctas, st, pdl);

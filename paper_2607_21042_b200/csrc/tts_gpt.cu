@@ -445,6 +445,12 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
   return launch_attention(aa, R, attention_cluster_size(R, aa.H, h->n_sm, h->attn_cluster_fill), st, pdl);
 }
 
+// Whether FC2 of 2 to 16 rows is split over K.
+bool splits_fc2(const tts_gpt *h) {
+  return h->use_fc2_ksplit && (h->cfg.d_ff / k_per_tile(h->cfg.wfmt)) % kSmallKSplit == 0 &&
+         (size_t)kSmallKSplit * kMaxRows * h->cfg.d_model <= h->partials_floats;
+}
+
 // Whether LayerNorm is fused into the linears of up to 16 rows; FC2's k-ranges then meet in clusters, so that x is complete.
 // Five kernels per layer instead of seven; the price is x read by every CTA (5 KB a row) and a cluster barrier.  ms per
 // step, kernels of their own / fused, contexts of 500 tokens (bf16, int4, bf16 weights over the 8-bit cache) and 1400 (bf16):
@@ -453,7 +459,9 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
 // 0.784 / 0.741; 8 rows 0.638 / 0.647, 0.639 / 0.620, 0.673 / 0.677, 0.754 / 0.792 (kernels of their own but for int4); 9 rows
 // 0.705 / 0.699, 0.692 / 0.664, 0.746 / 0.730, 0.875 / 0.845; 10 rows 0.756 / 0.717, 0.695 / 0.674, 0.825 / 0.799, 0.947 / 0.924;
 // 11 rows 0.777 / 0.799, 0.728 / 0.748, 0.852 / 0.868, 0.993 / 1.010; 14 rows 0.891 / 1.001, 0.798 / 0.804, 0.997 / 1.098.
+// Where FC2 splits K but its k-ranges cannot be clusters, it leaves partial sums, which only a LayerNorm kernel folds.
 bool fuse_layernorm(const tts_gpt *h, int R) {
+  if (R > 1 && !h->ordered && splits_fc2(h) && !can_cluster(h->cfg.wfmt, R, h->cfg.d_ff)) return false;
   return can_fuse_ln(R, h->cfg.d_model, h->ordered, h->ln_fuse_rows) && (h->ordered || R != 8 || h->cfg.wfmt == WF_INT4);
 }
 
@@ -665,8 +673,7 @@ int run_layers(tts_gpt *h, int R, bool decode) {
   // quarter of the wide activation rows; its partial sums are folded into x by the next LayerNorm
   // (with LayerNorm fused into its consumer the k-ranges are a cluster, which adds into x itself)
   const bool cluster = fuse_ln && R > 1 && !h->ordered;
-  const int fc2_ks = ((!fuse_ln || cluster) && h->use_fc2_ksplit && (c.d_ff / k_per_tile(c.wfmt)) % kSmallKSplit == 0 &&
-                      (size_t)kSmallKSplit * kMaxRows * d <= h->partials_floats) ? kSmallKSplit : 1;
+  const int fc2_ks = (!fuse_ln || cluster) && splits_fc2(h) ? kSmallKSplit : 1;
   h->pending_parts = 0;
   for (int l = 0; l < c.n_layer; ++l) {
     LayerW &L = h->layers[l];

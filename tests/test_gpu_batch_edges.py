@@ -96,6 +96,22 @@ def test_layernorm_fused_into_linears_of_several_rows(S, d, wfmt):
     eng.destroy()
 
 
+@pytest.mark.parametrize("wfmt,S,d_ff", [(C.W_BF16, 10, 8832), (C.W_BF16, 10, 8960), (C.W_BF16, 9, 10240), (C.W_INT8_PC, 10, 10240), (C.W_INT4_G128, 10, 10240)])
+def test_fc2_whose_rows_do_not_fit_a_cluster(wfmt, S, d_ff):
+    """Small batches on either side of the longest K whose staged rows a cluster holds, in decode steps and in a prefill pass
+    of as many rows."""
+    cfg = C.tiny_config(d_ff=d_ff, wfmt=wfmt, max_streams=S, n_pages=2 * S)
+    w = C.make_weights(cfg, seed=55)
+    model = O.OracleModel(cfg, w)
+    eng = B.TtsGpt(cfg, w, DEV)
+    for lens in ([1] * S, [5 + i for i in range(S)]):   # the first: a pass of S rows
+        prefixes = C.make_prefixes(cfg, lens, seed=56)
+        lg, tk = _run(eng, prefixes, 3)
+        _check(model, prefixes, lg, tk, range(S), "FC2 of K = %d" % d_ff)
+    assert eng.check_canaries() == 0
+    eng.destroy()
+
+
 @pytest.mark.parametrize("S", [1, 3, 40, 128])
 def test_queued_attention_has_the_bits_of_a_cta_per_pair(S):
     """Pairs handed out by a queue (2 to 444 CTAs, one pair or many behind the first two): pages with one token and with 64, rows
