@@ -334,10 +334,11 @@ def test_prefill_passes_around_the_pair_kernels_lines(wfmt, lens):
     eng.destroy()
 
 
-@pytest.mark.parametrize("S", [1, 21, 30, 40, 60, 80])
+@pytest.mark.parametrize("S", [1, 21, 30, 40, 60, 80, 100])
 def test_8bit_decode_attention_splits(S):
     """8, 6, 4, 3, 2 and 1 CTAs per (row, head) over the 8-bit cache: contexts at the edges of half pages and pages, splits
-    without tokens, stale pages; against the streaming kernel on the same history, greedy and sampled order."""
+    without tokens, stale pages; against the streaming kernel on the same history, greedy and sampled order (a ticket kernel of
+    five CTAs per SM up to 80 rows, of four at 100)."""
     edges = [700, 1, 30, 31, 32, 33, 62, 63, 64, 65, 95, 96, 127, 128, 161]
     lens = [edges[i % len(edges)] if i < 30 else 2 + (11 * i) % 60 for i in range(S)]
     cfg = C.tiny_config(kv_fmt=C.KV_FP8_E4M3, max_streams=S, n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=768)
