@@ -505,14 +505,31 @@ GemmTcArgs gemm_args(tts_gpt *h, const PackedLinear &pl, const void *act_img, in
 }
 
 // Passes of up to kPairMinRows rows stay with the one-CTA wide kernel (two CTAs per SM): their tiles are too few for pairs.
-// One prefill call of the 24-layer model, one-CTA kernel / pairs, ms: one stream of 300 rows 1.42 / 1.69, 640 1.71 / 1.95,
-// 777 1.80 / 2.24, 896 1.83 / 2.28, 1000 2.47 / 2.48, 1024 2.45 / 2.46, 1100 2.64 / 2.80, 1280 2.84 / 2.91, 1400 3.07 / 3.04,
-// 1536 3.15 / 3.09, 2000 4.22 / 4.09; eight streams of 640 rows together 1.67 / 1.91, 1024 2.18 / 2.14, 1152 2.28 / 2.49, 1536
-// 2.87 / 2.66, 1792 3.03 / 2.79 (int8 weights within 2 % of these).  Up to 1280 rows the pairs' 256-row tiles of QKV leave the
-// second wave nearly empty; from 1400 on they are the faster.
-constexpr int kPairMinRows = 1280;
+// From kPairAlwaysRows on every pass takes pairs.  One prefill call of the 24-layer model, one-CTA kernel / pairs, ms: one
+// stream of 300 rows 1.42 / 1.69, 640 1.71 / 1.95, 777 1.80 / 2.24, 896 1.83 / 2.28, 1000 2.47 / 2.48, 1400 3.07 / 3.04, 1536 3.15 /
+// 3.09, 2000 4.22 / 4.09; eight streams of 640 rows together 1.67 / 1.91, 1360 2.82 / 2.65, 1792 3.03 / 2.79.
+// In between the waves decide.  Both kernels put as many outputs into a wave (two 128 x 128 tiles per SM, a 256 x 256 tile per
+// pair), so what differs is how a pass is rounded up to tiles and waves.  One CTA where FC1's last wave of pairs is less than half
+// full and QKV or FC1 takes fewer waves of one-CTA tiles (24-layer model: nine row tiles, QKV 270 of 296 places against 75
+// of 74): one stream of 1100 rows 2.65 / 2.81, eight of 1152 2.29 / 2.48, one of 1152 over the 8-bit cache 2.73 / 2.90; but one of
+// 1216 there 3.35 / 3.18, eight of 1280 2.68 / 2.67, one of 1280 2.86 / 2.90 (pairs).  Other widths (d_ff = 4 d, fewer layers), one
+// stream of 1152 and of 1280 rows: 512 0.59 / 0.55, 0.65 / 0.58; 1024 0.61 / 0.76, 0.86 / 0.84; 1536 0.84 / 0.78, 0.95 / 0.83;
+// 2048 0.75 / 0.78, 0.95 / 0.85.  Sampled passes, which keep the one-CTA kernel's k-ranges on pairs too, take one CTA wherever
+// that last wave is less than half full: 1152 rows 2.58 / 2.82, 1280 2.87 / 3.04 (8-bit cache 3.33 / 3.32); 1280 rows at widths 512
+// 0.66 / 0.61, 1024 0.87 / 0.92, 1152 0.92 / 0.98, 1408 0.87 / 0.89, 1536 0.96 / 0.94.
+constexpr int kPairMinRows = 1024, kPairAlwaysRows = 1280;
 bool can_pair(const tts_gpt *h) { return !(h->cfg.wfmt == WF_INT4 && h->w4_exact); }
-bool use_pairs(const tts_gpt *h, int R) { return R > kPairMinRows && can_pair(h); }
+bool use_pairs(const tts_gpt *h, int R) {
+  if (R <= kPairMinRows || !can_pair(h)) return false;
+  if (R > kPairAlwaysRows) return true;
+  auto ceil_div = [](int a, int b) { return (a + b - 1) / b; };
+  const int tiles = ceil_div(R, kMaxRows), n_pair = std::max(1, h->n_sm / 2);
+  auto pair_tiles = [&](int N) { return ceil_div(N, 256) * ceil_div(tiles, 2); };
+  auto fewer_waves = [&](int N) { return ceil_div(ceil_div(N, 128) * tiles, 2 * h->n_sm) < ceil_div(pair_tiles(N), n_pair); };
+  const int fc1 = pair_tiles(h->cfg.d_ff);
+  const bool nearly_empty = fc1 > n_pair && (fc1 - 1) % n_pair + 1 <= n_pair / 2;
+  return !(nearly_empty && (h->ordered || fewer_waves(3 * h->cfg.d_model) || fewer_waves(h->cfg.d_ff)));
+}
 
 // FC2 alone goes to pairs where its one-CTA tiles begin a second wave and its pairs need one: 897 to 1024 rows, of which it
 // takes 17.2 us a layer on pairs and 23.0 on single CTAs (QKV 13.3 there against 15.5 on pairs, the O projection 9.3 against

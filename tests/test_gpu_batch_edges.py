@@ -319,9 +319,11 @@ def test_sampled_passes_of_several_units_over_the_8bit_cache(form):
     eng.destroy()
 
 
-@pytest.mark.parametrize("wfmt,lens", [(C.W_BF16, [897]), (C.W_INT8_PC, [500, 520]), (C.W_INT4_G128, [1024]), (C.W_BF16, [640, 512, 128])])
+@pytest.mark.parametrize("wfmt,lens", [(C.W_BF16, [897]), (C.W_INT8_PC, [500, 520]), (C.W_INT4_G128, [1024]), (C.W_BF16, [640, 512, 128]),
+                                       (C.W_INT8_PC, [640, 512]), (C.W_BF16, [640, 513])])
 def test_prefill_passes_around_the_pair_kernels_lines(wfmt, lens):
-    """897, 1020 and 1024 rows: FC2 alone on pairs, the other linears on single CTAs; 1280: all on single CTAs."""
+    """897, 1020 and 1024 rows: FC2 alone on pairs, the other linears on single CTAs; 1152: all on single CTAs; 1153 and 1280: all
+    on pairs."""
     cfg = C.tiny_config(wfmt=wfmt, d_model=1280, n_head=20, d_ff=5120, max_streams=len(lens), n_pages=sum(x // 64 + 2 for x in lens),
                         max_context=1088, max_pos=1088)
     w = C.make_weights(cfg, seed=59)
