@@ -748,7 +748,11 @@ inline cudaError_t launch_linear_inst(const LinearArgs &a, int grid, cudaStream_
 template <int WF, int MODE>
 inline cudaError_t launch_linear_wf(const LinearArgs &a, int max_ctas, cudaStream_t st, bool pdl) {
   const int ks = a.ksplit > 1 ? a.ksplit : 1;
-  const LinearPlan p = plan_linear(WF, a.N, a.K / ks, a.B, MODE, max_ctas / ks);
+  // Clusters of four find fewer places than CTAs, since each lies within a group of SMs: 71 of 74 on 148 SMs at two CTAs each, so
+  // the rule counts on nine tenths.  The 72 clusters of width 1152 began a second wave, 16 layers 0.382 ms a step at 2 rows and 0.465
+  // at 8; on three tiles per CTA (48 clusters) 0.341 and 0.417.
+  const int places = a.cluster ? max_ctas / 10 * 9 : max_ctas;
+  const LinearPlan p = plan_linear(WF, a.N, a.K / ks, a.B, MODE, places / ks);
   if (linear_smem_bytes(WF, p.rt, MODE, a.B, a.K / ks) > (size_t)kLinearSmemMax) return cudaErrorInvalidValue;
   if (p.rt == 1) return launch_linear_inst<WF, 1, MODE>(a, p.grid, st, pdl);
   if (p.rt == 2) return launch_linear_inst<WF, 2, MODE>(a, p.grid, st, pdl);

@@ -72,7 +72,7 @@ def test_unit_split_decode_attention(S):
 
 
 @pytest.mark.parametrize("wfmt", [C.W_BF16, C.W_INT8_PC, C.W_INT4_G128])
-@pytest.mark.parametrize("S,d", [(2, 1280), (5, 384), (7, 256), (10, 1280)])
+@pytest.mark.parametrize("S,d", [(2, 1280), (5, 384), (7, 256), (10, 1280), (6, 1152)])
 def test_layernorm_fused_into_linears_of_several_rows(S, d, wfmt):
     """A warp per row in every CTA (2, 3 and 10 float4 per lane), FC2's k-ranges added up by a cluster (shares that do and do not
     divide evenly), hidden rows from the fused head; against the oracle, and against LayerNorm kernels of their own."""
