@@ -100,7 +100,7 @@ struct tts_gpt {
   std::map<int, StepGraph> graphs;
   bool use_graph;
   bool use_pdl;
-  int ln_fuse_rows = kLnFuseMaxRows;   // rows up to which LayerNorm is fused into its consumer (option "ln_fuse_rows")
+  int ln_fuse_rows = 0;         // rows up to which LayerNorm is fused into its consumer (option "ln_fuse_rows"); 0: see fuse_layernorm
   bool use_fc2_ksplit = true;   // 2-16 rows: FC2 splits K (option "fc2_ksplit")
   int pending_parts = 0;        // k-range partial sums of the last FC2 still to be folded into x
   size_t partials_floats = 0;
@@ -452,17 +452,23 @@ bool splits_fc2(const tts_gpt *h) {
 }
 
 // Whether LayerNorm is fused into the linears of up to 16 rows; FC2's k-ranges then meet in clusters, so that x is complete.
-// Five kernels per layer instead of seven; the price is x read by every CTA (5 KB a row) and a cluster barrier.  ms per
-// step, kernels of their own / fused, contexts of 500 tokens (bf16, int4, bf16 weights over the 8-bit cache) and 1400 (bf16):
-// 2 rows 0.552 / 0.520, 0.542 / 0.522, 0.574 / 0.547, 0.598 / 0.571; 4 rows 0.596 / 0.552, 0.591 / 0.552, 0.633 / 0.585, 0.671 /
-// 0.638; 6 rows 0.666 / 0.601, 0.648 / 0.596, 0.688 / 0.642, 0.758 / 0.703; 7 rows 0.659 / 0.633, 0.654 / 0.624, 0.698 / 0.679,
-// 0.784 / 0.741; 8 rows 0.638 / 0.647, 0.639 / 0.620, 0.673 / 0.677, 0.754 / 0.792 (kernels of their own but for int4); 9 rows
-// 0.705 / 0.699, 0.692 / 0.664, 0.746 / 0.730, 0.875 / 0.845; 10 rows 0.756 / 0.717, 0.695 / 0.674, 0.825 / 0.799, 0.947 / 0.924;
-// 11 rows 0.777 / 0.799, 0.728 / 0.748, 0.852 / 0.868, 0.993 / 1.010; 14 rows 0.891 / 1.001, 0.798 / 0.804, 0.997 / 1.098.
+// Five kernels per layer instead of seven; the price is x read by every CTA (4 d bytes a row) and a cluster barrier, and decode
+// steps over the bf16 cache give up the pages asked into L2 (kv_prefetch_args).  ms per step of the 24-layer model, kernels of
+// their own / fused, contexts of 500 and 1400 tokens.  bf16 weights: 2 rows 0.552 / 0.520, 0.598 / 0.571; 4 rows 0.596 / 0.552,
+// 0.671 / 0.638; 6 rows 0.643 / 0.605, 0.723 / 0.704; 7 rows 0.645 / 0.631, 0.755 / 0.737; 8 rows 0.630 / 0.652, 0.742 / 0.798;
+// 9 rows 0.680 / 0.703, 0.819 / 0.851; 10 rows 0.717 / 0.724, 0.922 / 0.909.  int8: 7 rows 0.662 / 0.650, 8 rows 0.639 / 0.654, 9 rows
+// 0.695 / 0.700, 10 rows 0.692 / 0.716.  int4: 8 rows level, 9 rows 0.671 / 0.666, 0.794 / 0.781; 10 rows 0.676 / 0.680, 0.840 /
+// 0.826.  8-bit cache, bf16 and int4 weights: 7 rows 0.654 / 0.632, 0.660 / 0.625; 8 rows 0.637 / 0.641, 0.635 / 0.624; 9 rows
+// 0.676 / 0.676, 0.692 / 0.664; 10 rows 0.707 / 0.686, 0.684 / 0.677.  11 rows, the second round of a CTA's ten warps: bf16 0.740 /
+// 0.813, int4 over the 8-bit cache 0.715 / 0.738.  Narrower models, whose rows cost a CTA less, at 500 tokens (bf16): width 512 8
+// rows 0.241 / 0.230, 10 rows 0.247 / 0.237; width 1024 8 rows 0.395 / 0.379, 10 rows 0.397 / 0.394; width 1152 8 rows 0.438 / 0.417,
+// 10 rows 0.458 / 0.449.
 // Where FC2 splits K but its k-ranges cannot be clusters, it leaves partial sums, which only a LayerNorm kernel folds.
-bool fuse_layernorm(const tts_gpt *h, int R) {
+bool fuse_layernorm(const tts_gpt *h, int R, bool decode) {
   if (R > 1 && !h->ordered && splits_fc2(h) && !can_cluster(h->cfg.wfmt, R, h->cfg.d_ff)) return false;
-  return can_fuse_ln(R, h->cfg.d_model, h->ordered, h->ln_fuse_rows) && (h->ordered || R != 8 || h->cfg.wfmt == WF_INT4);
+  const bool gives_up_pages = decode && !h->kv_fp8 && h->cfg.wfmt != WF_INT4 && h->cfg.d_model > 1152;
+  const int max_rows = h->ln_fuse_rows ? h->ln_fuse_rows : gives_up_pages ? 7 : kLnFuseMaxRows;
+  return can_fuse_ln(R, h->cfg.d_model, h->ordered, max_rows);
 }
 
 // Part 0 (O projection), 1 (FC1), 2 (FC2 of layer l) or none (-1: QKV, which runs the same kernel) of the pages asked into L2 for the attention of the layer behind (behind
@@ -475,7 +481,7 @@ constexpr long long kPrefetchBytes = 16000000;
 KvPrefetch kv_prefetch_args(const tts_gpt *h, int R, int l, int part, bool decode) {
   KvPrefetch p;
   memset(&p, 0, sizeof p);
-  if (!decode || !h->kv_prefetch || h->kv_fp8 || R < 2 || fuse_layernorm(h, R)) return p;
+  if (!decode || !h->kv_prefetch || h->kv_fp8 || R < 2 || fuse_layernorm(h, R, decode)) return p;
   p.cap = (int)std::min<long long>(h->pps, kPrefetchBytes / ((long long)R * h->kv_page_elems * 2));
   if (p.cap < 1) return p;
   p.rows = R;   // the step asks for pages
@@ -685,7 +691,7 @@ int run_layers(tts_gpt *h, int R, bool decode) {
   const int d = c.d_model;
   cudaStream_t st = h->stream;
   const bool pdl = h->use_pdl;
-  const bool fuse_ln = fuse_layernorm(h, R);
+  const bool fuse_ln = fuse_layernorm(h, R, decode);
   // 2 to 16 rows: FC2 (K = d_ff) splits K over kSmallKSplit CTAs per row tile, so that a CTA stages a
   // quarter of the wide activation rows; its partial sums are folded into x by the next LayerNorm
   // (with LayerNorm fused into its consumer the k-ranges are a cluster, which adds into x itself)
@@ -767,7 +773,7 @@ int run_head(tts_gpt *h, int n_out, int R) {
                           h->rt.out_slot, h->io, 0);
     if (rc) return rc;
     h->pending_parts = 0;
-  } else if (fuse_layernorm(h, n_out)) {
+  } else if (can_fuse_ln(n_out, c.d_model, h->ordered, h->ln_fuse_rows ? h->ln_fuse_rows : kLnFuseMaxRows)) {
     ha.ln_x = h->x; ha.ln_g = h->lnf_g; ha.ln_b = h->lnf_b; ha.ln_eps = c.ln_eps;
     ha.ln_gather = h->rt.out_rows; ha.ln_out_slot = h->rt.out_slot; ha.ln_io = h->io;
   } else {

@@ -96,6 +96,28 @@ def test_layernorm_fused_into_linears_of_several_rows(S, d, wfmt):
     eng.destroy()
 
 
+@pytest.mark.parametrize("S,d,wfmt,kv,fused", [
+    (7, 1280, C.W_BF16, C.KV_BF16, True), (8, 1280, C.W_BF16, C.KV_BF16, False), (10, 1280, C.W_INT8_PC, C.KV_BF16, False), (8, 1280, C.W_INT4_G128, C.KV_BF16, True),
+    (8, 1280, C.W_BF16, C.KV_FP8_E4M3, True), (8, 1024, C.W_INT8_PC, C.KV_BF16, True), (10, 256, C.W_BF16, C.KV_BF16, True), (11, 256, C.W_BF16, C.KV_BF16, False)])
+def test_rule_of_the_fused_layernorm(S, d, wfmt, kv, fused):
+    """Steps on either side of the rule's lines have the bits of the form it names, and those of the other form (up to 16 rows: two
+    per warp) pass the oracle's bars too."""
+    cfg = C.tiny_config(d_model=d, n_head=d // 64, d_ff=1536, wfmt=wfmt, kv_fmt=kv, max_streams=S, n_pages=3 * S)
+    w = C.make_weights(cfg, seed=63)
+    model = O.OracleModel(cfg, w)
+    prefixes = C.make_prefixes(cfg, [40 + 5 * i for i in range(S)], seed=64)
+    out = {}
+    for rows in (None, 1, 16):
+        eng = B.TtsGpt(cfg, w, DEV)
+        if rows:
+            eng.set_option("ln_fuse_rows", rows)
+        out[rows] = _run(eng, prefixes, 3)
+        (_check_e4m3 if kv == C.KV_FP8_E4M3 else _check)(model, prefixes, *out[rows], range(S), "ln_fuse_rows %s" % rows)
+        eng.destroy()
+    assert np.array_equal(out[None][0], out[16 if fused else 1][0])
+    assert not np.array_equal(out[1][0], out[16][0])
+
+
 @pytest.mark.parametrize("wfmt,S,d_ff", [(C.W_BF16, 10, 8832), (C.W_BF16, 10, 8960), (C.W_BF16, 9, 10240), (C.W_INT8_PC, 10, 10240), (C.W_INT4_G128, 10, 10240)])
 def test_fc2_whose_rows_do_not_fit_a_cluster(wfmt, S, d_ff):
     """Small batches on either side of the longest K whose staged rows a cluster holds, in decode steps and in a prefill pass
