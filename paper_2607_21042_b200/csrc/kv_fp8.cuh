@@ -171,7 +171,7 @@ __device__ __forceinline__ void fp8_fold4(const uint4 (&kk)[4], const uint4 (&vv
 // CTAS: resident per SM, five with 96 registers and four with 116 (more loads in flight).  Five where a launch of more than four per
 // SM then stays one wave, ms per sampled step on four / on five: 11 rows of 500 tokens (660 CTAs on 148 SMs) 0.902 / 0.836, 17
 // rows of 1300 (680) 1.272 / 1.144; with two waves either way four are the faster: 14 rows of 1300 (840) 1.236 / 1.277, 24 (960)
-// 1.338 / 1.393.
+// 1.338 / 1.393; and so they are in prefill passes of up to 7 rows, whose contexts seldom have tokens for every split (2 %).
 template <int CTAS>
 __global__ void __launch_bounds__(kAttnWarps * 32, CTAS) attention_fp8_kernel(const Fp8AttnArgs a) {
   const int c = blockIdx.x, S = gridDim.x, h = blockIdx.y, r = blockIdx.z;
@@ -662,9 +662,9 @@ inline cudaError_t launch_kv_quantize(const uint16_t *stage, unsigned char *kv_l
   return launch_kernel(kv_quantize_kernel, dim3(H, R), dim3(64), 0, st, pdl, stage, kv_layer, page_table, row_stream, row_pos, pps, H);
 }
 
-inline cudaError_t launch_attention_fp8(const Fp8AttnArgs &a, int R, int splits, int n_sm, cudaStream_t st, bool pdl) {
+inline cudaError_t launch_attention_fp8(const Fp8AttnArgs &a, int R, int splits, bool step, int n_sm, cudaStream_t st, bool pdl) {
   const int n_cta = splits * a.H * R;
-  return launch_kernel(n_cta > 4 * n_sm && n_cta <= 5 * n_sm ? attention_fp8_kernel<5> : attention_fp8_kernel<4>, dim3(splits, a.H, R),
+  return launch_kernel(step && n_cta > 4 * n_sm && n_cta <= 5 * n_sm ? attention_fp8_kernel<5> : attention_fp8_kernel<4>, dim3(splits, a.H, R),
                        dim3(kAttnWarps * 32), 0, st, pdl, a);
 }
 

@@ -423,7 +423,7 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
     }
     fa.stage = h->kv_stage; fa.whole_pages = h->ordered ? 1 : 0;
     if (small) return launch_attention_fp8_decode(fa, R, n_split, st, pdl);
-    return launch_attention_fp8(fa, R, attention_fp8_splits(R, aa.H, h->n_sm), h->n_sm, st, pdl);
+    return launch_attention_fp8(fa, R, attention_fp8_splits(R, aa.H, h->n_sm), aa.old_pages_final != 0, h->n_sm, st, pdl);
   }
   aa.err = h->dev_err;
   // prefill passes: rows of one stream share their pages (one CTA per 16 rows and head on the tensor cores;
