@@ -217,16 +217,22 @@ struct KvPrefetch {
   int pps, rows, cap;           // up to `cap` complete pages of every row
   int part, n_parts;            // this kernel's share of the blocks
 };
+// The blocks are numbered rank by rank, page by page; a lane takes the number it starts with and every stride-th behind it.
+__host__ __device__ __forceinline__ int kv_prefetch_first(const KvPrefetch &p, int cta, int lane) { return (cta * 32 + lane) * p.n_parts + p.part; }
+__host__ __device__ __forceinline__ int kv_prefetch_stride(const KvPrefetch &p, int n_cta) { return n_cta * 32 * p.n_parts; }
+__host__ __device__ __forceinline__ int kv_prefetch_total(const KvPrefetch &p) { return p.rows * p.cap * p.blocks; }
+// address of block number u, or null: that page is not complete
+__host__ __device__ __forceinline__ const unsigned char *kv_prefetch_address(const KvPrefetch &p, int u) {
+  const int t = u / p.blocks, b = u - t * p.blocks, z = t / p.cap, j = t - z * p.cap;
+  const int phys = p.slot_pages[z * p.pps + j];
+  if (j >= (p.slots[z].y - 1) / kPageTokens) return nullptr;
+  return p.layer + ((size_t)phys * p.blocks + b) * p.block_bytes;
+}
 __device__ __forceinline__ void kv_prefetch(const KvPrefetch &p, int cta, int n_cta) {
-  const int lane = threadIdx.x & 31;
-  const int total = p.rows * p.cap * p.blocks;
+  const int total = kv_prefetch_total(p), stride = kv_prefetch_stride(p, n_cta);
 #pragma unroll 1
-  for (int u = (cta * 32 + lane) * p.n_parts + p.part; u < total; u += n_cta * 32 * p.n_parts) {
-    const int t = u / p.blocks, b = u - t * p.blocks, z = t / p.cap, j = t - z * p.cap;
-    const int phys = p.slot_pages[z * p.pps + j];
-    if (j >= (p.slots[z].y - 1) / kPageTokens) continue;
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.layer + ((size_t)phys * p.blocks + b) * p.block_bytes), "r"(p.block_bytes) : "memory");
-  }
+  for (int u = kv_prefetch_first(p, cta, threadIdx.x & 31); u < total; u += stride)
+    if (const unsigned char *q = kv_prefetch_address(p, u)) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(q), "r"(p.block_bytes) : "memory");
 }
 
 // D(16x8,f32) += A(16x16,bf16,row) * B(16x8,bf16,col).  Fragment layout (g = lane/4, t = lane%4):

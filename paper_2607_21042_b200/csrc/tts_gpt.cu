@@ -445,6 +445,10 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
   return launch_attention(aa, R, attention_cluster_size(R, aa.H, h->n_sm, h->attn_cluster_fill), st, pdl);
 }
 
+bool use_tc_path(const tts_gpt *h, int R) {
+  return h->have_tc && h->use_tc && R >= h->tc_min_rows;
+}
+
 // Whether FC2 of 2 to 16 rows is split over K.
 bool splits_fc2(const tts_gpt *h) {
   return h->use_fc2_ksplit && (h->cfg.d_ff / k_per_tile(h->cfg.wfmt)) % kSmallKSplit == 0 &&
@@ -471,17 +475,34 @@ bool fuse_layernorm(const tts_gpt *h, int R, bool decode) {
   return can_fuse_ln(R, h->cfg.d_model, h->ordered, max_rows);
 }
 
-// Part 0 (O projection), 1 (FC1), 2 (FC2 of layer l) or none (-1: QKV, which runs the same kernel) of the pages asked into L2 for the attention of the layer behind (behind
-// the last: the next step's first).  Between two attentions the memory is idle half of the time, and attention at these
-// sizes waits for it: ms per step without / with 16 MB of pages, 8 rows of 500 tokens 0.637 / 0.622, 12 rows of 900 0.904 /
-// 0.889, 16 rows of 500 0.851 / 0.839, 24 rows of 500 1.014 / 0.995, 37 rows of 575 1.208 / 1.187 (sampled 1.216 / 1.203); with
-// 48 MB the linears behind wait for theirs (24 rows 1.034).  Not with LayerNorm fused (3 rows of 1700 0.619 / 0.620), not over
-// the 8-bit cache (9 rows 0.734 / 0.750, 24 rows level), and from 49 rows on a page per row is more than the budget.
+// Whether the linears of a decode step ask pages of the next attention into L2.  Between two attentions the memory is idle
+// half of the time, and attention at these sizes waits for it; what the linears lose is their own loads' bandwidth.  Not with
+// LayerNorm fused (3 rows of 1700 0.619 / 0.620) and not over the 8-bit cache (9 rows 0.734 / 0.750).  ms per step without / with,
+// contexts of 500 and 1300 tokens, 24-layer model unless a width is given (fewer layers).
+// Greedy steps of up to 16 rows from width 512 on: 9 rows bf16 0.737 / 0.706, 12 rows 0.789 / 0.762, int4 0.741 / 0.724, 1.011 / 1.001;
+// width 512 16 rows 0.278 / 0.275; width 256 0.160 / 0.161.  The tcgen05 linears of larger greedy steps at widths 1024 to 1280: 24 rows
+// 0.986 / 0.974, 37 rows 1.157 / 1.138, width 1152 24 rows 0.631 / 0.623, 44 rows 0.758 / 0.763 (from 49 rows on a page per row is
+// more than the budget); narrower and wider 0 to 3 % behind (512 24 rows 0.315 / 0.318, 1408 32 rows 0.615 / 0.620, 2048 24 rows
+// 0.503 / 0.509).
+// Sampled steps from width 1280 on (1152: 8 rows 3 % behind): 5 rows bf16 0.653 / 0.641, 12 rows 0.787 / 0.766, 16 rows 0.951 / 0.943;
+// int8 5 rows 0.675 / 0.668, 12 rows 0.757 / 0.761, 0.944 / 0.961, 16 rows 0.868 / 0.862.  Behind where each pair has a CTA of its own
+// in one wave, most so with quantized weights, whose linears are soon done; level from 17 rows on.
+bool asks_for_pages(const tts_gpt *h, int R) {
+  const int d = h->cfg.d_model;
+  if (!h->kv_prefetch || h->kv_fp8 || R < 2 || fuse_layernorm(h, R, true)) return false;
+  const bool small = !use_tc_path(h, R);
+  if (!h->ordered) return small ? d >= 512 : d >= 1024 && d <= 1280;
+  return small && d >= 1280 && (R <= (h->cfg.wfmt == WF_BF16 ? 12 : 9) || R * h->cfg.n_head > 2 * h->n_sm);
+}
+
+// Part 0 (O projection), 1 (FC1), 2 (FC2 of layer l) or none (-1: QKV, which runs the same kernel) of the pages asked for: up
+// to 16 MB of complete pages (with 48 MB the linears behind wait for theirs, 24 rows 1.034 ms) of the layer behind, and behind
+// the last layer of the first one, for a step that may follow.
 constexpr long long kPrefetchBytes = 16000000;
 KvPrefetch kv_prefetch_args(const tts_gpt *h, int R, int l, int part, bool decode) {
   KvPrefetch p;
   memset(&p, 0, sizeof p);
-  if (!decode || !h->kv_prefetch || h->kv_fp8 || R < 2 || fuse_layernorm(h, R, decode)) return p;
+  if (!decode || !asks_for_pages(h, R)) return p;
   p.cap = (int)std::min<long long>(h->pps, kPrefetchBytes / ((long long)R * h->kv_page_elems * 2));
   if (p.cap < 1) return p;
   p.rows = R;   // the step asks for pages
@@ -678,10 +699,6 @@ int run_head_tc(tts_gpt *h, int n_out) {
   CUDA_TRY(h, launch_kernel(sample_kernel, dim3(n_out), dim3(kSampleThreads), (size_t)c.vocab * sizeof(float), st, pdl, sa));
   h->launches += 2;
   return TTS_GPT_OK;
-}
-
-bool use_tc_path(const tts_gpt *h, int R) {
-  return h->have_tc && h->use_tc && R >= h->tc_min_rows;
 }
 
 int run_layers(tts_gpt *h, int R, bool decode) {

@@ -306,17 +306,18 @@ def test_sampled_passes_of_several_units_give_the_bits_of_single_units(form, wfm
     eng.destroy()
 
 
-@pytest.mark.parametrize("S", [11, 40, 128])
-def test_pages_asked_into_l2_change_nothing(S):
-    """The linears of a step ask the next attention's complete pages into L2: the same bits with and without, contexts with and
-    without a complete page, more pages than the budget takes."""
+@pytest.mark.parametrize("S,d,top_k", [(11, 512, 0), (9, 1280, 0), (12, 1280, 30), (40, 1280, 0), (47, 1024, 0)])
+def test_pages_asked_into_l2_change_nothing(S, d, top_k):
+    """The linears of a step ask the next attention's complete pages into L2 (at these rows and widths): the same bits with and
+    without, contexts with and without a complete page, more pages than the budget takes."""
     lens = [1, 63, 64, 65, 129, 700][:min(S, 6)] + [3 + (13 * i) % 200 for i in range(S - 6)]
-    cfg = C.tiny_config(max_streams=S, n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=768)
+    cfg = C.tiny_config(d_model=d, n_head=d // 64, d_ff=1536, max_streams=S, n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=768)
     eng = B.TtsGpt(cfg, C.make_weights(cfg, seed=61), DEV)
     prefixes = C.make_prefixes(cfg, lens, seed=62)
-    lg, tk = _run(eng, prefixes, 3)
+    kw = dict(top_k=top_k, uniforms=torch.full((S,), 0.3, device=DEV)) if top_k else {}
+    lg, tk = _run(eng, prefixes, 3, **kw)
     eng.set_option("kv_prefetch", 0)
-    lg2, tk2 = _run(eng, prefixes, 3)
+    lg2, tk2 = _run(eng, prefixes, 3, **kw)
     assert np.array_equal(lg, lg2) and np.array_equal(tk, tk2)
     eng.destroy()
 
