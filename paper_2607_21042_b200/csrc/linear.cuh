@@ -150,9 +150,10 @@ struct LinearArgs {
   int *err;                   // optional device error word: set to 1 if the weight copy never arrives
   int ksplit;                 // 0 or 1: whole K per CTA; n > 1 (EPI_RESID only, no fused LN): gridDim.y = n k-ranges,
                               // out_f32 = partial sums [n][kMaxRows][N] without bias, folded by the next LayerNorm
-  KvPrefetch pf;              // tensor-pipe path
   int cluster;                // with ksplit (up to 16 rows, tensor-pipe path): the k-ranges of a tile are a cluster and add into out_f32 themselves
 };
+// Steps whose linears ask for pages (tensor-pipe path, LayerNorm not fused) have kernels of their own, as in the tcgen05 linears.
+struct LinearPrefetchArgs : LinearArgs { KvPrefetch pf; };
 
 // exact int8 (biased byte) -> float via the 2^23 magic number
 __device__ __forceinline__ float biased_byte_to_float(uint32_t word, int i) {
@@ -188,8 +189,8 @@ constexpr int kLinearSmemMax = 200 * 1024;     // per CTA, where one tile of a l
 // for their order of sums.
 // CL: the k-ranges of a tile (gridDim.y of them) are the CTAs of a cluster and meet in its shared memory, so that the rows they
 // add into are complete when the kernel ends and the LayerNorm behind it can be fused into its consumer.
-template <int WF, int RT, int MODE, int NB, bool CL = false>
-__global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearArgs a) {
+template <int WF, int RT, int MODE, int NB, bool CL, typename Args>
+__global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const Args a) {
   static_assert(!CL || (NB == 0 && MODE == ACT_STAGED), "clusters: up to 16 staged rows on the tensor pipe");
   constexpr bool LN = MODE == ACT_LN;
   constexpr bool STAGED = MODE != ACT_DIRECT;
@@ -293,7 +294,9 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const LinearA
     cluster_arrive_release();
   }
   pdl_launch_dependents();
-  if (NB == 0 && a.pf.layer && warp == kLinearWarps - 1) kv_prefetch(a.pf, blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y);
+  if constexpr (sizeof(Args) > sizeof(LinearArgs)) {
+    if (a.pf.layer && warp == kLinearWarps - 1) kv_prefetch(a.pf, blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y);
+  }
   pdl_wait();
   trace_mark(a.trace, a.trace_slot, 1);
   float cl_old = 0.f;
@@ -719,34 +722,42 @@ inline bool can_cluster(int wf, int B, int K) {
          linear_smem_bytes(wf, 1, ACT_STAGED, B, range) + cluster_smem_bytes(1) <= (size_t)kLinearSmemMax;
 }
 
+template <int WF, int RT, int MODE, int NB, bool CL, typename Args>
+inline cudaError_t launch_linear_kernel(const Args &a, int grid, int ks, size_t smem, cudaStream_t st, bool pdl) {
+  static SmemOptIn opt_in;
+  if (const cudaError_t e = opt_in(linear_kernel<WF, RT, MODE, NB, CL, Args>, kLinearSmemMax)) return e;
+  return launch_kernel_cluster_dims(linear_kernel<WF, RT, MODE, NB, CL, Args>, dim3(grid, ks), dim3(kLinearThreads), smem, dim3(1, CL ? ks : 1), st, pdl, a);
+}
+
+// pf: the pages to ask for, or null (see LinearPrefetchArgs)
 template <int WF, int RT, int MODE, int NB>
-inline cudaError_t launch_linear_nb(const LinearArgs &a, int grid, cudaStream_t st, bool pdl) {
+inline cudaError_t launch_linear_nb(const LinearArgs &a, const KvPrefetch *pf, int grid, cudaStream_t st, bool pdl) {
   const int ks = a.ksplit > 1 ? a.ksplit : 1;
   const size_t smem = linear_smem_bytes(WF, RT, MODE, a.B, a.K / ks);
-  static SmemOptIn opt_in;
-  if (const cudaError_t e = opt_in(linear_kernel<WF, RT, MODE, NB>, kLinearSmemMax)) return e;
-  if constexpr (NB == 0 && MODE == ACT_STAGED) {
-    if (a.cluster) {
-      static SmemOptIn opt_in_cl;
-      if (const cudaError_t e = opt_in_cl(linear_kernel<WF, RT, MODE, NB, true>, kLinearSmemMax)) return e;
-      return launch_kernel_cluster_dims(linear_kernel<WF, RT, MODE, NB, true>, dim3(grid, ks), dim3(kLinearThreads), smem + cluster_smem_bytes(RT), dim3(1, ks), st, pdl, a);
+  if constexpr (NB == 0 && MODE == ACT_STAGED)
+    if (a.cluster) return launch_linear_kernel<WF, RT, MODE, NB, true>(a, grid, ks, smem + cluster_smem_bytes(RT), st, pdl);
+  if constexpr (NB == 0 && MODE != ACT_LN)
+    if (pf) {
+      LinearPrefetchArgs p;
+      static_cast<LinearArgs &>(p) = a;
+      p.pf = *pf;
+      return launch_linear_kernel<WF, RT, MODE, NB, false>(p, grid, ks, smem, st, pdl);
     }
-  }
-  return launch_kernel(linear_kernel<WF, RT, MODE, NB>, dim3(grid, ks), dim3(kLinearThreads), smem, st, pdl, a);
+  return launch_linear_kernel<WF, RT, MODE, NB, false>(a, grid, ks, smem, st, pdl);
 }
 
 template <int WF, int RT, int MODE>
-inline cudaError_t launch_linear_inst(const LinearArgs &a, int grid, cudaStream_t st, bool pdl) {
+inline cudaError_t launch_linear_inst(const LinearArgs &a, const KvPrefetch *pf, int grid, cudaStream_t st, bool pdl) {
   if (MODE != ACT_DIRECT) {  // batches of up to 4 rows always fit the staging buffer
     constexpr int M = MODE == ACT_DIRECT ? ACT_STAGED : MODE;
-    if (a.B == 1) return launch_linear_nb<WF, RT, M, 1>(a, grid, st, pdl);
-    if (a.ordered && a.B <= kLnFuseMaxRowsOrdered) return launch_linear_nb<WF, RT, M, 4>(a, grid, st, pdl);
+    if (a.B == 1) return launch_linear_nb<WF, RT, M, 1>(a, pf, grid, st, pdl);
+    if (a.ordered && a.B <= kLnFuseMaxRowsOrdered) return launch_linear_nb<WF, RT, M, 4>(a, pf, grid, st, pdl);
   }
-  return launch_linear_nb<WF, RT, MODE, 0>(a, grid, st, pdl);
+  return launch_linear_nb<WF, RT, MODE, 0>(a, pf, grid, st, pdl);
 }
 
 template <int WF, int MODE>
-inline cudaError_t launch_linear_wf(const LinearArgs &a, int max_ctas, cudaStream_t st, bool pdl) {
+inline cudaError_t launch_linear_wf(const LinearArgs &a, const KvPrefetch *pf, int max_ctas, cudaStream_t st, bool pdl) {
   const int ks = a.ksplit > 1 ? a.ksplit : 1;
   // Clusters of four find fewer places than CTAs, since each lies within a group of SMs: 71 of 74 on 148 SMs at two CTAs each, so
   // the rule counts on nine tenths.  The 72 clusters of width 1152 began a second wave, 16 layers 0.382 ms a step at 2 rows and 0.465
@@ -754,10 +765,10 @@ inline cudaError_t launch_linear_wf(const LinearArgs &a, int max_ctas, cudaStrea
   const int places = a.cluster ? max_ctas / 10 * 9 : max_ctas;
   const LinearPlan p = plan_linear(WF, a.N, a.K / ks, a.B, MODE, places / ks);
   if (linear_smem_bytes(WF, p.rt, MODE, a.B, a.K / ks) > (size_t)kLinearSmemMax) return cudaErrorInvalidValue;
-  if (p.rt == 1) return launch_linear_inst<WF, 1, MODE>(a, p.grid, st, pdl);
-  if (p.rt == 2) return launch_linear_inst<WF, 2, MODE>(a, p.grid, st, pdl);
-  if (p.rt == 3) return launch_linear_inst<WF, 3, MODE>(a, p.grid, st, pdl);
-  return launch_linear_inst<WF, 4, MODE>(a, p.grid, st, pdl);
+  if (p.rt == 1) return launch_linear_inst<WF, 1, MODE>(a, pf, p.grid, st, pdl);
+  if (p.rt == 2) return launch_linear_inst<WF, 2, MODE>(a, pf, p.grid, st, pdl);
+  if (p.rt == 3) return launch_linear_inst<WF, 3, MODE>(a, pf, p.grid, st, pdl);
+  return launch_linear_inst<WF, 4, MODE>(a, pf, p.grid, st, pdl);
 }
 
 // Whether LayerNorm can be fused in front of a linear with this shape.
@@ -766,21 +777,21 @@ inline bool can_fuse_ln(int B, int K, bool ordered, int max_rows = kLnFuseMaxRow
 }
 
 template <int WF>
-inline cudaError_t launch_linear_mode(const LinearArgs &a, int max_ctas, cudaStream_t st, bool pdl) {
-  if (a.ln_x) return launch_linear_wf<WF, ACT_LN>(a, max_ctas, st, pdl);
+inline cudaError_t launch_linear_mode(const LinearArgs &a, const KvPrefetch *pf, int max_ctas, cudaStream_t st, bool pdl) {
+  if (a.ln_x) return launch_linear_wf<WF, ACT_LN>(a, pf, max_ctas, st, pdl);
   if ((size_t)a.B * ln_stage_stride(WF, a.K / (a.ksplit > 1 ? a.ksplit : 1)) * sizeof(uint16_t) <= (size_t)kStageMaxBytes)
-    return launch_linear_wf<WF, ACT_STAGED>(a, max_ctas, st, pdl);
-  return launch_linear_wf<WF, ACT_DIRECT>(a, max_ctas, st, pdl);
+    return launch_linear_wf<WF, ACT_STAGED>(a, pf, max_ctas, st, pdl);
+  return launch_linear_wf<WF, ACT_DIRECT>(a, pf, max_ctas, st, pdl);
 }
 
 // K must be a multiple of 128.
-inline cudaError_t launch_linear(int wf, const LinearArgs &a, cudaStream_t st, bool pdl, int max_ctas) {
+inline cudaError_t launch_linear(int wf, const LinearArgs &a, cudaStream_t st, bool pdl, int max_ctas, const KvPrefetch *pf = nullptr) {
   if (a.ln_x && !can_fuse_ln(a.B, a.K, a.ordered, 16)) return cudaErrorInvalidValue;
   if (a.cluster && (a.ksplit != kSmallKSplit || a.ordered || !can_cluster(wf, a.B, a.K))) return cudaErrorInvalidValue;
   if (a.ksplit > 1 && (a.ln_x || a.mode != EPI_RESID || (a.K / k_per_tile(wf)) % a.ksplit != 0)) return cudaErrorInvalidValue;
-  if (wf == WF_BF16) return launch_linear_mode<WF_BF16>(a, max_ctas, st, pdl);
-  if (wf == WF_INT8) return launch_linear_mode<WF_INT8>(a, max_ctas, st, pdl);
-  return launch_linear_mode<WF_INT4>(a, max_ctas, st, pdl);
+  if (wf == WF_BF16) return launch_linear_mode<WF_BF16>(a, pf, max_ctas, st, pdl);
+  if (wf == WF_INT8) return launch_linear_mode<WF_INT8>(a, pf, max_ctas, st, pdl);
+  return launch_linear_mode<WF_INT4>(a, pf, max_ctas, st, pdl);
 }
 
 inline cudaError_t launch_pack(int wf, int N, int K, const void *w, const void *s, void *dst_w, void *dst_s,

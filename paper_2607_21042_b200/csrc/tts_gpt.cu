@@ -715,6 +715,10 @@ int run_layers(tts_gpt *h, int R, bool decode) {
   const bool cluster = fuse_ln && R > 1 && !h->ordered;
   const int fc2_ks = (!fuse_ln || cluster) && splits_fc2(h) ? kSmallKSplit : 1;
   h->pending_parts = 0;
+  auto launch_small = [&](const LinearArgs &a, int part, int l) {   // part: see kv_prefetch_args
+    const KvPrefetch pf = kv_prefetch_args(h, R, l, part, decode);
+    return launch_linear(c.wfmt, a, st, pdl, 2 * h->n_sm, pf.rows > 0 ? &pf : nullptr);
+  };
   for (int l = 0; l < c.n_layer; ++l) {
     LayerW &L = h->layers[l];
     uint16_t *kvl = h->kv + h->kv_layer_elems * l;
@@ -736,7 +740,7 @@ int run_layers(tts_gpt *h, int R, bool decode) {
       qa.row_stream = h->rt.row_stream; qa.row_pos = h->rt.row_pos; qa.pps = h->pps; qa.d = d; qa.H = c.n_head;
       qa.kv_stage = h->kv_stage;
       trace_attach(h, qa);
-      CUDA_TRY(h, launch_linear(c.wfmt, qa, st, pdl, 2 * h->n_sm));
+      CUDA_TRY(h, launch_small(qa, -1, l));
       AttnArgs aa;
       memset(&aa, 0, sizeof aa);
       aa.q = h->q; aa.kv_layer = kvl; aa.page_table = h->ps.page_table; aa.row_stream = h->rt.row_stream;
@@ -748,8 +752,7 @@ int run_layers(tts_gpt *h, int R, bool decode) {
     LinearArgs oa = linear_args(h, L.o, h->o, R, EPI_RESID);
     oa.out_f32 = h->x; oa.out_stride = d;
     trace_attach(h, oa);
-    oa.pf = kv_prefetch_args(h, R, l, 0, decode);
-    CUDA_TRY(h, launch_linear(c.wfmt, oa, st, pdl, 2 * h->n_sm));
+    CUDA_TRY(h, launch_small(oa, 0, l));
     LinearArgs f1 = linear_args(h, L.fc1, h->a, R, EPI_GELU);
     if (fuse_ln) {
       f1.ln_x = h->x; f1.ln_g = L.ln2_g; f1.ln_b = L.ln2_b; f1.ln_eps = c.ln_eps;
@@ -761,14 +764,12 @@ int run_layers(tts_gpt *h, int R, bool decode) {
     }
     f1.out_bf16 = h->hbuf; f1.gelu_tanh = c.gelu_tanh;
     trace_attach(h, f1);
-    f1.pf = kv_prefetch_args(h, R, l, 1, decode);
-    CUDA_TRY(h, launch_linear(c.wfmt, f1, st, pdl, 2 * h->n_sm));
+    CUDA_TRY(h, launch_small(f1, 1, l));
     LinearArgs f2 = linear_args(h, L.fc2, h->hbuf, R, EPI_RESID);
     f2.out_f32 = h->x; f2.out_stride = d;
     if (fc2_ks > 1) { f2.ksplit = fc2_ks; f2.cluster = cluster ? 1 : 0; if (!cluster) f2.out_f32 = h->partials; }
     trace_attach(h, f2);
-    f2.pf = kv_prefetch_args(h, R, l, 2, decode);
-    CUDA_TRY(h, launch_linear(c.wfmt, f2, st, pdl, 2 * h->n_sm));
+    CUDA_TRY(h, launch_small(f2, 2, l));
     h->launches += 5;
   }
   h->pending_parts = fc2_ks > 1 && !cluster ? fc2_ks : 0;   // the last FC2's partial sums: folded by the head's LayerNorm
