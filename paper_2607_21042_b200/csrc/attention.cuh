@@ -605,23 +605,24 @@ struct AttnQueue {
 inline AttnQueue attn_queue(unsigned int *counter, int n_pair, int grid) {
   return AttnQueue{counter, (unsigned int)(n_pair - 2 * grid + grid - 1), n_pair};
 }
-constexpr int kAttnListPages = 32;
+constexpr int kAttnListPages = 32;                           // pages of a stream of the engine: a lane each
+static_assert(kAttnMaxChunks * kAttnWarps <= kAttnListPages, "max_context: the set-up kernel's page lists and AttnPair have a page per lane");
 struct AttnPair {
-  int row, head, n_tok, slot;                                // row < 0: none
-  int phys[kAttnListPages];                                  // its first pages' places in the pool
+  int row, head, n_tok;                                      // row < 0: none
+  int phys[kAttnListPages];                                  // its pages' places in the pool
 };
 // by a warp: pair i into shared memory
 template <typename Args>
 __device__ __forceinline__ void attn_pair(AttnPair &p, const AttnQueue &qu, int i, const Args &a) {
   const int lane = threadIdx.x & 31;
   if (i >= qu.n_pair) {
-    if (lane == 0) { p.row = -1; p.head = 0; p.n_tok = 0; p.slot = 0; }
+    if (lane == 0) { p.row = -1; p.head = 0; p.n_tok = 0; }
     return;
   }
   const int slot = i / a.H;
   const int4 d = a.slots[slot];
   const int phys = lane < a.pps ? a.slot_pages[slot * a.pps + lane] : 0;
-  if (lane == 0) { p.row = d.x; p.head = i - slot * a.H; p.n_tok = d.y; p.slot = slot; }
+  if (lane == 0) { p.row = d.x; p.head = i - slot * a.H; p.n_tok = d.y; }
   p.phys[lane] = phys;
 }
 // by one lane: index of a further pair (not to be called again once it has returned one that does not exist)
@@ -757,8 +758,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnStreamCtas) attention_qu
   auto request = [&](const AttnPair &p, int page) {   // the page of a pair, if there is one
     pending = page * kPageTokens < p.n_tok;
     if (pending && lane == 0) {
-      const int phys = page < kAttnListPages ? p.phys[page] : a.slot_pages[p.slot * a.pps + page];
-      stream_issue(a, phys, p.head, min(kPageTokens, p.n_tok - page * kPageTokens), stage, bar);
+      stream_issue(a, p.phys[page], p.head, min(kPageTokens, p.n_tok - page * kPageTokens), stage, bar);
     }
   };
   request(pairs[0], warp);                      // as above: ahead of the dependency wait

@@ -60,7 +60,7 @@ struct StepParams {
 // in call order take pages in stack order), then the row table is written and ctx_len advances.
 // Attention's CTAs find what they work on in `slots` and `slot_pages`, by rank of the row's length: one round trip to L2
 // where row order, position, stream and page table were three, in front of the first page request of every CTA of 24 layers.
-// ROWS: page lists per warp, lane = page (max_context is at most 2048); 0: one row, whose attention finds its work itself, without
+// ROWS: page lists per warp, lane = page (kAttnListPages of them are all that max_context allows); 0: one row, whose attention finds its work itself, without
 // rank tables (with them the two-layer model took 0.3 us more of 39 a step).  Little code where there are few rows: it runs once
 // per step, fetched cold.
 constexpr int kSetupRows = 8;

@@ -439,7 +439,7 @@ cudaError_t run_attention(tts_gpt *h, AttnArgs &aa, int R, cudaStream_t st, bool
   const bool stream = h->attn_stream_min_pairs > 0 ? R * aa.H >= h->attn_stream_min_pairs : attention_use_stream(R, aa.H, h->n_sm);
   if (h->use_attn_stream && stream) {
     const int n_pair = R * aa.H;
-    const bool queue = aa.slots && n_pair >= 2 && (h->attn_queue == 2 || (h->attn_queue == 1 && attention_use_queue(n_pair, h->n_sm)));
+    const bool queue = aa.slots && (h->attn_queue == 2 || (h->attn_queue == 1 && attention_use_queue(n_pair, h->n_sm)));
     return queue ? launch_attention_queue(aa, R, h->attn_tickets, h->n_sm, st, pdl) : launch_attention_stream(aa, R, st, pdl);
   }
   return launch_attention(aa, R, attention_cluster_size(R, aa.H, h->n_sm, h->attn_cluster_fill), st, pdl);
@@ -1051,7 +1051,7 @@ static int prefill_impl(tts_gpt_t *h, int32_t n, const void *const *emb, const i
   // with a last unit of up to 128 rows apart and the head unit by unit.  (Over the 8-bit cache too: its rows attend over
   // decoded pages, of which a unit and a pass of several reach at most one stream's old ones and those of their own rows.)
   const int unit = h->ordered ? std::min(pass_rows, h->ordered_pass_rows) : 0;
-  static_assert(2048 / kPageTokens + kMaxOrderedRows / kPageTokens + kMaxRows <= kScratchPages, "a pass over the 8-bit cache never reaches more pages than can be decoded");
+  static_assert(kAttnListPages + kMaxOrderedRows / kPageTokens + kMaxRows <= kScratchPages, "a pass over the 8-bit cache never reaches more pages than can be decoded");
   if (unit) pass_rows = std::max(unit, std::min(pass_rows, kMaxOrderedRows) / unit * unit);
   int left = 0;            // rows not yet in a pass
   for (int i = 0; i < n; ++i) left += plen[i];
