@@ -234,7 +234,7 @@ int32_t tts_gpt_debug_check_canaries(tts_gpt_t *h, int32_t *bad_bytes);
  * from the SM count and the model width, 3584 for the 24-layer model on 148 SMs; passes of more than 128 rows need
  * the tensor-core path; sampled calls take a multiple of a unit of rows, 896 for the 24-layer model), "w4_tc_exact" (int4 weights only: by default the operand images of the tensor-core path, used for more than 16 rows,
  * hold code x group scale rounded once to bf16; 1 rewrites them as integer codes and the kernels scale fp32 sums per
- * 128-column group, 0 writes the default back), "attn_tc", "attn_mma", "attn_prefill", "attn_half", "attn_decode", "attn_stream", "attn_stream_min_pairs", "attn_queue" (0, 1: by the number of pairs, 2), "attn_cluster_fill", "ln_fuse_rows" (1..16), "kv_prefetch",
+ * 128-column group, 0 writes the default back), "attn_tc", "attn_mma", "attn_prefill", "attn_half", "attn_decode", "attn_stream", "attn_stream_min_pairs", "attn_queue" (0, 1: by the number of pairs, 2: every streaming step of more than one row), "attn_cluster_fill", "ln_fuse_rows" (1..16), "kv_prefetch",
  * "fc2_ksplit"; "poison_free_pages" (test aid standing in for a memory checker: every free page, and
  * from then on every released page, is filled with NaN in all layers, so that a kernel reading a slot no
  * token was written to poisons its result).  Unknown name or value out of range: TTS_GPT_E_ARG. */

@@ -813,6 +813,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnStreamCtas) attention_qu
     if (sm_dead) break;                         // (a wait expires after seconds: every thread has read the mark of the pair in front by then)
     if (threadIdx.x < kHeadDim) attn_write_out(a, row, head * kHeadDim + threadIdx.x, O / L);
   }
+  trace_mark(a.trace, a.trace_slot, 4);         // (of the attentions this one only) behind the CTA's last pair
   if (pending) mbar_wait_bounded(bar, phase, kAttnWaitNs);   // behind an expired wait: no copy may be in flight towards a CTA that has left
   if (warp == kAttnWarps - 1 && lane == 0 && sm_dead)
     while (more) more = attn_take(qu) < qu.n_pair;           // the counter returns to zero all the same

@@ -134,30 +134,50 @@ def test_fc2_whose_rows_do_not_fit_a_cluster(wfmt, S, d_ff):
     eng.destroy()
 
 
-@pytest.mark.parametrize("S", [1, 3, 40, 128])
+@pytest.mark.parametrize("S", [2, 45, 80, 128])
 def test_queued_attention_has_the_bits_of_a_cta_per_pair(S):
-    """Pairs handed out by a queue (2 to 444 CTAs, one pair or many behind the first two): pages with one token and with 64, rows
-    whose warps have no page, a long context among short ones, several launches on one counter."""
+    """40 pairs on 20 CTAs (all handed out by position), 900, 1600 and 2560 on 444 (12, 712 and 1672 taken from the counter): pages
+    with one token and with 64, rows whose warps have no page, a long context among short ones, several launches on one
+    counter; greedy and sampled, whose steps of more than ten pairs per SM come to the queue by the rule."""
     edges = [700, 1, 63, 64, 65, 127, 128, 129, 255, 256, 257, 320]
     lens = [edges[i] if i < 12 else 2 + (37 * i) % 300 for i in range(S)]
-    cfg = C.tiny_config(max_streams=S, n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=768)
+    cfg = C.tiny_config(d_model=1280, n_head=20, d_ff=1536, max_streams=S, n_pages=sum((x + 8 + 63) // 64 for x in lens), max_context=768)
     w = C.make_weights(cfg, seed=51)
     model = O.OracleModel(cfg, w)
     eng = B.TtsGpt(cfg, w, DEV)
-    for name, value in (("poison_free_pages", 1), ("attn_decode", 0), ("attn_half", 0), ("attn_stream_min_pairs", 1)):
-        eng.set_option(name, value)
     prefixes = C.make_prefixes(cfg, lens, seed=52)
-    eng.set_option("attn_queue", 2)
-    lg, tk = _run(eng, prefixes, 4)
-    _check(model, prefixes, lg, tk, list(range(min(S, 6))) + [S - 1], "queued attention")
-    eng.set_option("attn_queue", 0)
-    lg2, tk2 = _run(eng, prefixes, 4)
-    assert np.array_equal(lg, lg2) and np.array_equal(tk, tk2)
-    eng.set_option("attn_queue", 2)
     u = torch.full((S,), 0.4, device=DEV)
-    lg3, _ = _run(eng, prefixes, 4, top_k=30, uniforms=u)
-    eng.set_option("attn_queue", 0)
-    assert np.array_equal(lg3, _run(eng, prefixes, 4, top_k=30, uniforms=u)[0])
+    trace = torch.zeros(8 * eng.set_trace(None), dtype=torch.int64, device=DEV)
+
+    def run(queue, **kw):   # logits, tokens, and in how many kernels of a step CTA 0 left a mark that of the attention only the queue's does
+        if queue is not None:
+            eng.set_option("attn_queue", queue)
+        lg, tk = _run(eng, prefixes, 4, **kw)
+        out = torch.zeros(S, dtype=torch.int32, device=DEV)
+        ids, _ = eng.prefill([bits_dev(p) for p in prefixes], out_tokens=out, **kw)
+        eng.set_trace(trace)
+        trace.zero_()
+        eng.wait_for_caller()
+        eng.decode_step(ids, out, **kw)
+        eng.sync()
+        eng.set_trace(None)
+        for s in ids:
+            eng.release_stream(s)
+        return lg, tk, int((trace.view(-1, 8)[:, 4] != 0).sum())
+
+    by_rule = run(None, top_k=30, uniforms=u)
+    eng.set_option("poison_free_pages", 1)
+    sampled = [run(q, top_k=30, uniforms=u) for q in (0, 1)]
+    for x in (by_rule, sampled[1]):
+        assert np.array_equal(x[0], sampled[0][0]) and np.array_equal(x[1], sampled[0][1])
+        assert x[2] == sampled[0][2] + (cfg.n_layer if 20 * S > 10 * 148 else 0)
+    for name, value in (("attn_decode", 0), ("attn_half", 0), ("attn_stream_min_pairs", 1)):
+        eng.set_option(name, value)
+    single, queued = run(0), run(2)
+    _check(model, prefixes, queued[0], queued[1], list(range(min(S, 4))) + [S - 1], "queued attention")
+    assert np.array_equal(single[0], queued[0]) and np.array_equal(single[1], queued[1])
+    assert queued[2] == single[2] + cfg.n_layer
+    assert np.array_equal(run(0, top_k=30, uniforms=u)[0], run(2, top_k=30, uniforms=u)[0])
     assert eng.check_canaries() == 0
     eng.destroy()
 
