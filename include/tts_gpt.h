@@ -254,7 +254,10 @@ int32_t tts_gpt_debug_expire_wait(tts_gpt_t *h, uint32_t limit_us);
  * are announced 16 bytes longer than they are, its issuing warps give up after limit_us microseconds (1..100000;
  * kernel 1: after the 2 s that every wait has), the tile is not stored, nor (kernel 2) are the pair's later ones, and the next tts_gpt_sync returns TTS_GPT_E_TIMEOUT once.
  * tile -1: a whole run.  tile -2 (kernel 2): a whole run, on tiles of 256 features, in which the second CTA of a pair
- * comes to each of its tiles limit_us late (nothing expires).  Nothing hangs or faults. */
+ * comes to each of its tiles limit_us late (nothing expires).
+ * kernel 3: FC2 of layer 0 as steps of 2..16 rows run it, its k-ranges in clusters, on the activation rows of the last such
+ * step; adds into out (DEVICE fp32 [rows][d]).  tile -1: a whole run; tile >= 0: the second k-range of the tile-th CTA gives up
+ * after the 2 s that every wait has, and its cluster stores nothing.  Nothing hangs or faults. */
 int32_t tts_gpt_debug_expire_linear(tts_gpt_t *h, int32_t kernel, int32_t rows, int32_t tile, uint32_t limit_us, float *out);
 
 /* ---------------------------------------------------------------------------------------------

@@ -150,7 +150,8 @@ struct LinearArgs {
   int *err;                   // optional device error word: set to 1 if the weight copy never arrives
   int ksplit;                 // 0 or 1: whole K per CTA; n > 1 (EPI_RESID only, no fused LN): gridDim.y = n k-ranges,
                               // out_f32 = partial sums [n][kMaxRows][N] without bias, folded by the next LayerNorm
-  int cluster;                // with ksplit (up to 16 rows, tensor-pipe path): the k-ranges of a tile are a cluster and add into out_f32 themselves
+  int cluster;                // with ksplit (up to 16 rows, tensor-pipe path), not 0: the k-ranges of a tile are a cluster and add into out_f32
+                              // themselves (test aid, 2 + x: the second range of CTA x announces 16 bytes more than it copies)
 };
 // Steps whose linears ask for pages (tensor-pipe path, LayerNorm not fused) have kernels of their own, as in the tcgen05 linears.
 struct LinearPrefetchArgs : LinearArgs { KvPrefetch pf; };
@@ -220,7 +221,7 @@ __global__ void __launch_bounds__(kLinearThreads, 2) linear_kernel(const Args a)
     const uint32_t wbytes = (uint32_t)n_valid * KB * 512u;
     const uint32_t sbytes = WF == WF_INT4 ? (uint32_t)n_valid * KB * 16u : 0u;
     mbar_init(wbar, 1);
-    mbar_expect_tx(wbar, wbytes + sbytes);
+    mbar_expect_tx(wbar, wbytes + sbytes + (CL && a.cluster == 2 + (int)blockIdx.x && blockIdx.y == 1 ? 16u : 0u));
     if (gridDim.y == 1) {   // all of K: the CTA's tiles are one contiguous range
       const unsigned char *gw = reinterpret_cast<const unsigned char *>(a.w) + (size_t)tile0 * KB * 512;
       for (uint32_t off = 0; off < wbytes; off += 32768u)

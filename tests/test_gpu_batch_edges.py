@@ -118,6 +118,33 @@ def test_rule_of_the_fused_layernorm(S, d, wfmt, kv, fused):
     assert not np.array_equal(out[1][0], out[16][0])
 
 
+@pytest.mark.parametrize("wfmt,S,d,cols", [(C.W_BF16, 5, 256, 8), (C.W_INT8_PC, 10, 1280, 24), (C.W_INT4_G128, 2, 1280, 24)])
+def test_a_cluster_stores_nothing_behind_an_expired_wait(wfmt, S, d, cols):
+    """The weights of one k-range do not arrive: its cluster's columns (one and three 8-row tiles per CTA) are not stored by any of its
+    CTAs, all others are whole, the error is reported once and the engine goes on."""
+    cfg = C.tiny_config(d_model=d, n_head=d // 64, d_ff=4 * d, wfmt=wfmt, max_streams=S, n_pages=2 * S)
+    eng = B.TtsGpt(cfg, C.make_weights(cfg, seed=67), DEV)
+    prefixes = C.make_prefixes(cfg, [7 + i for i in range(S)], seed=68)
+    lg, tk = _run(eng, prefixes, 2)
+    mark = torch.arange(S * d, device=DEV, dtype=torch.float32).view(S, d) / 7
+    whole, out = mark.clone(), mark.clone()
+    eng.wait_for_caller()
+    eng.debug_expire_linear(3, S, -1, 1000, whole)
+    eng.sync()
+    assert not bool((whole == mark).all(0).any()) and bool(torch.isfinite(whole).all())
+    eng.debug_expire_linear(3, S, 2, 1000, out)
+    with pytest.raises(B.TtsGptError) as e:
+        eng.sync()
+    assert e.value.code == B.E_TIMEOUT
+    lost = torch.zeros(d, dtype=torch.bool, device=DEV)
+    lost[2 * cols:3 * cols] = True
+    assert torch.equal(out[:, lost], mark[:, lost]) and torch.equal(out[:, ~lost], whole[:, ~lost])
+    eng.sync()
+    lg2, tk2 = _run(eng, prefixes, 2)
+    assert np.array_equal(lg, lg2) and np.array_equal(tk, tk2)
+    eng.destroy()
+
+
 @pytest.mark.parametrize("wfmt,S,d_ff", [(C.W_BF16, 10, 8832), (C.W_BF16, 10, 8960), (C.W_BF16, 9, 10240), (C.W_INT8_PC, 10, 10240), (C.W_INT4_G128, 10, 10240)])
 def test_fc2_whose_rows_do_not_fit_a_cluster(wfmt, S, d_ff):
     """Small batches on either side of the longest K whose staged rows a cluster holds, in decode steps and in a prefill pass
