@@ -147,11 +147,11 @@ int32_t tts_gpt_prefill_tokens(tts_gpt_t *h, int32_t n, const void *const *cond_
  * top_k 0 or 1 = greedy (lowest index on ties); top_k in 2..64 = softmax over the top_k logits
  * at `temperature`, inverse CDF with uniforms[i].  Afterwards ctx_i += 1.
  * Reproducibility: the same sequence of calls on a fresh engine gives the same results bit for bit, greedy or
- * sampled (same library, same kind of GPU); no sum depends on timing.  The order of a sum does depend on the rows of
- * the call (decode: 1, 2-4, 5-16, 17 and more rows, in some kernels the contexts of the other rows too; prefill: the rows
- * prefilled together), so a stream that goes on in a
- * batch of another size sees logits rounded differently (about 0.5 % relative after 24 layers), and a sampled token
- * whose uniform falls that close to an edge of the distribution may change.  Sampled calls (prefill and decode, top_k > 1)
+ * sampled (same library, same kind of GPU); no sum depends on timing.  The order of a sum does depend on the number of
+ * rows of the call (decode: any two counts may differ, in particular every two up to 11 and either side of 17, by width and
+ * formats; in some kernels on the contexts of the other rows too; prefill: on the rows prefilled together), so a stream
+ * that goes on in a batch of another size, as one does whose neighbours end, sees logits rounded differently (about 0.5 %
+ * relative after 24 layers), and a sampled token whose uniform falls that close to an edge of the distribution may change.  Sampled calls (prefill and decode, top_k > 1)
  * keep, for each number of rows, the orders of sums of earlier versions of this library; greedy calls take faster
  * kernels with other orders where there are some.
  * Errors: E_ARG, E_STREAM (unknown / duplicate id), E_CTX_OVERFLOW (ctx_i + 1 > max_context),
@@ -229,15 +229,20 @@ int32_t tts_gpt_debug_check_canaries(tts_gpt_t *h, int32_t *bad_bytes);
 
 /* Experiments and tests: switches a kernel schedule of this engine on or off (value 0 / 1) or sets
  * a threshold.  Defaults are what the measurements use.  Waits for the stream and drops captured
- * step graphs.  Names: "graph", "pdl", "tc" and "tc_min_rows" (tensor-core
- * linears), "prefill_pass_rows" (rows per prefill pass: a multiple of 128 up to 4096; the default is chosen at creation
- * from the SM count and the model width, 3584 for the 24-layer model on 148 SMs; passes of more than 128 rows need
- * the tensor-core path; sampled calls take a multiple of a unit of rows, 896 for the 24-layer model), "w4_tc_exact" (int4 weights only: by default the operand images of the tensor-core path, used for more than 16 rows,
- * hold code x group scale rounded once to bf16; 1 rewrites them as integer codes and the kernels scale fp32 sums per
- * 128-column group, 0 writes the default back), "attn_tc", "attn_mma", "attn_prefill", "attn_half", "attn_decode", "attn_stream", "attn_stream_min_pairs", "attn_queue" (0, 1: by the number of pairs, 2: every streaming step of more than one row), "attn_cluster_fill", "ln_fuse_rows" (1..16), "kv_prefetch",
- * "fc2_ksplit"; "poison_free_pages" (test aid standing in for a memory checker: every free page, and
- * from then on every released page, is filled with NaN in all layers, so that a kernel reading a slot no
- * token was written to poisons its result).  Unknown name or value out of range: TTS_GPT_E_ARG. */
+ * step graphs.  Names:
+ *   "graph", "pdl", "attn_tc", "attn_mma", "attn_prefill", "attn_half", "attn_decode", "attn_stream", "kv_prefetch", "fc2_ksplit";
+ *   "tc" and "tc_min_rows" (tensor-core linears), "attn_stream_min_pairs", "attn_cluster_fill";
+ *   "prefill_pass_rows": rows per prefill pass, a multiple of 128 up to 4096; the default is chosen at creation from the SM
+ *     count and the model width, 3584 for the 24-layer model on 148 SMs; passes of more than 128 rows need the tensor-core
+ *     path; sampled calls take a multiple of a unit of rows, 896 for the 24-layer model;
+ *   "attn_queue": 0, 1 (by the number of pairs) or 2 (every streaming step of more than one row over the bf16 cache);
+ *   "ln_fuse_rows": 1..16, LayerNorm fused into the linears up to that many rows, in place of the rule by rows and formats;
+ *   "w4_tc_exact" (int4 weights only): by default the operand images of the tensor-core path, used for more than 16 rows,
+ *     hold code x group scale rounded once to bf16; 1 rewrites them as integer codes and the kernels scale fp32 sums per
+ *     128-column group, 0 writes the default back;
+ *   "poison_free_pages" (test aid standing in for a memory checker): every free page, and from then on every released
+ *     page, is filled with NaN in all layers, so that a kernel reading a slot no token was written to poisons its result.
+ * Unknown name or value out of range: TTS_GPT_E_ARG. */
 int32_t tts_gpt_debug_set_option(tts_gpt_t *h, const char *name, int32_t value);
 
 /* Test aid for the device-side error path: enqueues a one-thread kernel that waits, with the same

@@ -78,14 +78,13 @@ __global__ void __launch_bounds__(kAdWarps * 32, 1) attention_decode_kernel(cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int cid = blockIdx.x, n_cta = gridDim.x;
   const int P = (ad.n_pair - cid + n_cta - 1) / n_cta;   // pair i of this CTA: cid + i * n_cta
-  auto pair_of = [&](int i) { return cid + i * n_cta; };
   trace_mark(a.trace, a.trace_slot, 0);
 
   // ---- the CTA's unit list (row, page and order tables are final before the step's first kernel starts) ----
   if (threadIdx.x < kAdMaxPairs) {
     int n = 0;
     if ((int)threadIdx.x < P) {
-      const int slot = pair_of(threadIdx.x) / a.H;
+      const int slot = (cid + (int)threadIdx.x * n_cta) / a.H;
       const int4 d = a.slots ? a.slots[slot] : make_int4(slot, a.row_pos[slot] + 1, a.row_stream[slot], 0);
       n = d.y;
       sh.row[threadIdx.x] = d.x;
@@ -123,7 +122,7 @@ __global__ void __launch_bounds__(kAdWarps * 32, 1) attention_decode_kernel(cons
       const int k = u - sh.first_unit[lo];
       my_pair = lo;
       my_left = sh.n_tok[lo] - k * kAdUnit;
-      const int h = pair_of(lo) % a.H;
+      const int h = (cid + lo * n_cta) % a.H;
       const int phys = sh.pt[lo][k >> 1];
       my_row_k = ad.layer_row + ((phys * 2) * a.H + h) * kPageTokens + (k & 1) * kAdUnit;
     }
@@ -161,7 +160,7 @@ __global__ void __launch_bounds__(kAdWarps * 32, 1) attention_decode_kernel(cons
   }
   // the queries of the CTA's pairs, in log2 units: times 1/sqrt(64) * log2(e)
   for (int i = threadIdx.x; i < P * (kHeadDim / 4); i += kAdWarps * 32) {
-    const int pr = i / (kHeadDim / 4), c = i % (kHeadDim / 4), h = pair_of(pr) % a.H;
+    const int pr = i / (kHeadDim / 4), c = i % (kHeadDim / 4), h = (cid + pr * n_cta) % a.H;
     const float qs = 0.125f * 1.4426950408889634f;
     const float4 x = *reinterpret_cast<const float4 *>(a.q + (size_t)sh.row[pr] * a.H * kHeadDim + h * kHeadDim + 4 * c);
     *reinterpret_cast<float4 *>(&sh.q[pr][4 * c]) = make_float4(x.x * qs, x.y * qs, x.z * qs, x.w * qs);
@@ -175,7 +174,7 @@ __global__ void __launch_bounds__(kAdWarps * 32, 1) attention_decode_kernel(cons
   bool dead = false;
 
   auto write_out = [&](int pr, const float (&o)[4][2], float inv) {   // lane t of a quad writes dimensions 16 t + g and + 8
-    const int h = pair_of(pr) % a.H, r = sh.row[pr];
+    const int h = (cid + pr * n_cta) % a.H, r = sh.row[pr];
     const float x0 = (t == 0 ? o[0][0] : t == 1 ? o[1][0] : t == 2 ? o[2][0] : o[3][0]) * inv;
     const float x1 = (t == 0 ? o[0][1] : t == 1 ? o[1][1] : t == 2 ? o[2][1] : o[3][1]) * inv;
 #pragma unroll
@@ -342,7 +341,7 @@ __global__ void __launch_bounds__(kAdWarps * 32, 1) attention_decode_kernel(cons
       O1 = fmaf(f, o[lane + 32], O1);
     }
     if (!sh.dead) {
-      const int h = pair_of(pair) % a.H, r = sh.row[pair];
+      const int h = (cid + pair * n_cta) % a.H, r = sh.row[pair];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         const int dim = h * kHeadDim + lane + 32 * e;

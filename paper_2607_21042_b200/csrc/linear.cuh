@@ -31,8 +31,9 @@ enum { EPI_F32 = 0, EPI_QKV = 1, EPI_RESID = 2, EPI_GELU = 3 };
 
 constexpr int kLinearWarps = 10;  // divides the k-tile counts of K=1280 and K=5120 in every format
 constexpr int kLinearThreads = kLinearWarps * 32;
-constexpr int kSmallKSplit = 4;     // k-ranges of FC2 from 2 to 16 rows (partial sums folded by the next LayerNorm)
-constexpr int kLnFuseMaxRows = 10;  // LayerNorm is fused into the linear up to this batch, every CTA repeating it: a warp per row
+constexpr int kSmallKSplit = 4;     // k-ranges of FC2 from 2 to 16 rows: partial sums folded by the next LayerNorm, or (LayerNorm
+                                    // fused into its consumer) added up by a cluster
+constexpr int kLnFuseMaxRows = 10;  // LayerNorm is fused into the linear up to this batch at most, every CTA repeating it: a warp per row
 constexpr int kLnFuseMaxRowsOrdered = 4;   // the same for launches that keep the order of sums of the FMA path
 constexpr int kLnFuseMaxK = 4 * kLinearThreads;   // one row: a float4 per thread; more: ten float4 per lane of the row's warp
 
@@ -148,7 +149,7 @@ struct LinearArgs {
   unsigned long long *trace;  // optional timeline trace (see trace_mark)
   int trace_slot;
   int *err;                   // optional device error word: set to 1 if the weight copy never arrives
-  int ksplit;                 // 0 or 1: whole K per CTA; n > 1 (EPI_RESID only, no fused LN): gridDim.y = n k-ranges,
+  int ksplit;                 // 0 or 1: whole K per CTA; n > 1 (EPI_RESID only, no fused LN): gridDim.y = n k-ranges, without `cluster`
                               // out_f32 = partial sums [n][kMaxRows][N] without bias, folded by the next LayerNorm
   int cluster;                // with ksplit (up to 16 rows, tensor-pipe path), not 0: the k-ranges of a tile are a cluster and add into out_f32
                               // themselves (test aid, 2 + x: the second range of CTA x announces 16 bytes more than it copies)
@@ -186,8 +187,8 @@ constexpr int kLinearSmemMax = 200 * 1024;     // per CTA, where one tile of a l
 // NB: 0 = tensor-pipe path (any batch, 16 rows per m-tile); 1 or 4 = CUDA-core path for at most NB rows.  The fp32 FMAs
 // on the widened weights are cheaper for a single row, where MMAs are fifteen sixteenths padding.  From two rows on the
 // MMAs win: FMAs with LayerNorm fused in took 0.77 / 0.90 / 1.04 ms per step at 2 / 3 / 4 rows (bf16, context 530),
-// MMAs behind LayerNorm kernels of their own 0.59 / 0.63 / 0.71 (with LayerNorm fused in 0.52 / 0.55 / 0.55).  FMAs remain up to 4 rows where LinearArgs::ordered asks
-// for their order of sums.
+// MMAs behind LayerNorm kernels of their own 0.59 / 0.63 / 0.71 (with LayerNorm fused in 0.52 / 0.55 / 0.55).  FMAs remain up
+// to 4 rows where LinearArgs::ordered asks for their order of sums.
 // CL: the k-ranges of a tile (gridDim.y of them) are the CTAs of a cluster and meet in its shared memory, so that the rows they
 // add into are complete when the kernel ends and the LayerNorm behind it can be fused into its consumer.
 template <int WF, int RT, int MODE, int NB, bool CL, typename Args>

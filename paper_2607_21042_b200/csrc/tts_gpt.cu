@@ -359,8 +359,6 @@ LinearArgs linear_args(const PackedLinear &pl, const uint16_t *act, int B, int m
   a.N = pl.N; a.K = pl.K; a.B = B; a.mode = mode;
   return a;
 }
-LinearArgs linear_args(tts_gpt *h, const PackedLinear &pl, const uint16_t *act, int B, int mode);
-
 LinearArgs linear_args(tts_gpt *h, const PackedLinear &pl, const uint16_t *act, int B, int mode) {
   LinearArgs a = linear_args(pl, act, B, mode);
   a.err = h->dev_err;
