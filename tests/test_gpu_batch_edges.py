@@ -126,6 +126,7 @@ def test_a_cluster_stores_nothing_behind_an_expired_wait(wfmt, S, d, cols):
     eng = B.TtsGpt(cfg, C.make_weights(cfg, seed=67), DEV)
     prefixes = C.make_prefixes(cfg, [7 + i for i in range(S)], seed=68)
     lg, tk = _run(eng, prefixes, 2)
+    _run(eng, prefixes, 1, top_k=4, uniforms=torch.zeros(S, device=DEV))   # a sampled call in front changes nothing here
     mark = torch.arange(S * d, device=DEV, dtype=torch.float32).view(S, d) / 7
     whole, out = mark.clone(), mark.clone()
     eng.wait_for_caller()
