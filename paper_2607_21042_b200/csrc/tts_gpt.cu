@@ -1372,7 +1372,7 @@ int32_t tts_gpt_debug_expire_linear(tts_gpt_t *h, int32_t kernel, int32_t rows, 
   if (kernel == 3) {   // FC2 of 2 to 16 rows in clusters
     if (tile < -1 || tile >= (c.d_model + 7) / 8 || limit_us < 1 || limit_us > 100000 || !out || (uintptr_t)out % 16 || !splits_fc2(h) || !can_cluster(c.wfmt, rows, c.d_ff))
       return fail(h, TTS_GPT_E_ARG, "expire_linear: bad or misaligned argument");
-    LinearArgs f2 = linear_args(h->layers[0].fc2, h->hbuf, rows, EPI_RESID);
+    LinearArgs f2 = linear_args(h, h->layers[0].fc2, h->hbuf, rows, EPI_RESID);
     f2.ordered = 0; f2.out_f32 = out; f2.out_stride = c.d_model; f2.ksplit = kSmallKSplit; f2.cluster = 2 + tile;
     CUDA_TRY(h, launch_linear(c.wfmt, f2, h->stream, false, 2 * h->n_sm));
     return TTS_GPT_OK;
